@@ -211,6 +211,7 @@ struct rbe_ctx {
     double* d_kcoef = nullptr;                // coef_scale / k^2 per k
     bool mh = false;                          // paper's MH sampler (chains in the handle)
     int mh_words = 0;                         // largest 2M+1 (MH tables staged per block)
+    int m_max() const { return (mh_words - 1) / 2; }   // largest M over the systems
     uint64_t* d_mh_tq = nullptr;              // MH proposal thresholds, all systems
     double* d_mh_rho = nullptr;               // MH acceptance ratios, all systems
     int4* d_mh_state = nullptr;               // per system: current (m_x, m_y, m_z)
@@ -463,9 +464,8 @@ int auto_list_split(long long ntot) {
     return r;
 }
 
-// Threads per particle of the FP64 real-space pass: the largest power of two
-// not above the mixed path's.
-int real_split64(int r) { return r >= 8 ? 8 : (r >= 2 ? 2 : 1); }
+// Threads per particle of the FP64 real-space pass, from the mixed path's.
+int real_split64(int r) { return r >= 8 ? 16 : (r >= 2 ? 8 : 4); }
 
 // Cells along x per real-space block: enough blocks to fill the GPU, and a
 // staged neighbourhood (9 rows of seg + 2 cells) of about 2500 records.
@@ -938,18 +938,18 @@ RealArgs make_real_args(const rbe_ctx* h, int parts) {
 // Structure factors: per-chunk partials added to the fixed-point rho(k).
 void launch_rho(const rbe_ctx* h, cudaStream_t st, bool mixed, bool pdl = false) {
     const bool one = !h->batch;
-    const int kt = mixed ? kRhoKT : kLTile;           // wave vectors per tile
-    const int ltiles = (h->pmax + kt - 1) / kt;
+    const int ltiles = (h->pmax + kRhoKT - 1) / kRhoKT;
     const Work w = make_work(h, h->d_chunks, h->cur_chunk, 1);
     if (mixed)
         launch_rho_mixed(st, one, w, h->nchunks, ltiles, h->d_ksamp, h->d_kcoef, h->d_fx,
                          h->d_rho_fx, h->d_kcnt, h->d_kab, pdl);
     else
-        launch_rho_f64(st, one, w, h->nchunks, ltiles, h->d_ksamp, h->d_fx64, h->d_rho_fx);
+        launch_rho_f64(st, one, w, h->nchunks, h->cur_chunk, h->pmax, h->m_max(), h->d_ksamp,
+                       h->d_fx64, h->d_rho_fx);
 }
 
 void launch_force(const rbe_ctx* h, cudaStream_t st, bool mixed, const MdOut& md = MdOut{},
-                  bool pdl = false) {
+                  bool pdl = false, bool phi = true) {
     const bool one = !h->batch;
     if (mixed) {
         const Work w = make_work(h, h->split == 1 ? h->d_pblk : h->d_fblk, kBlockP / h->split, 0);
@@ -957,8 +957,8 @@ void launch_force(const rbe_ctx* h, cudaStream_t st, bool mixed, const MdOut& md
                                    h->d_fx, h->d_ksamp, h->d_kab, h->d_fs, md, pdl);
     } else {
         const Work w = make_work(h, h->d_pblk, kBlockP, 0);
-        launch_fourier_force_f64(st, one, w, h->npblk, h->d_fx64, h->d_ksamp, h->d_rho_fx,
-                                 h->d_fs64);
+        launch_fourier_force_f64(st, one, w, h->npblk, h->m_max(), phi, h->d_fx64, h->d_ksamp,
+                                 h->d_kcoef, h->d_rho_fx, h->d_fs64);
     }
 }
 
@@ -1037,8 +1037,8 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
             launch_prep_mixed(st, one, wp, h->npblk, a.pos, h->d_fx, h->d_cid, h->d_rank,
                               h->d_cell_cnt, pa);
         else
-            launch_prep_f64(st, one, wp, h->npblk, a.pos64, h->d_fx64, h->d_cid, h->d_rank,
-                            h->d_cell_cnt, pa);
+            launch_prep_f64(st, one, wp, h->npblk, a.pos64, h->d_fx64, h->d_fx, h->d_cid,
+                            h->d_rank, h->d_cell_cnt, pa);
     });
     if (a.list) {
         // list step: prep -> structure factors -> Fourier force on st with
@@ -1073,7 +1073,9 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
         cudaEventRecord(h->ev_fork, st);
         cudaStreamWaitEvent(st2, h->ev_fork, 0);
         run(RBE_K_RHO, st2, [&] { launch_rho(h, st2, mixed); });
-        run(RBE_K_FOURIER_FORCE, st2, [&] { launch_force(h, st2, mixed); });
+        run(RBE_K_FOURIER_FORCE, st2, [&] {
+            launch_force(h, st2, mixed, MdOut{}, false, mixed || a.phi64);
+        });
         cudaEventRecord(h->ev_join, st2);
     }
     // the cell list; on a list step the (usually no-op) rebuild runs on a
@@ -1099,8 +1101,8 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
                        h->d_err);
     });
     run(RBE_K_CELL_ORDER, sc, [&] {
-        launch_order(sc, n, h->d_cid, h->d_cell_start, h->d_perm_tmp, mixed ? h->d_fx : nullptr,
-                     h->d_spos, mixed ? nullptr : h->d_fx64, h->d_spos64, h->d_perm, lflag,
+        launch_order(sc, n, h->d_cid, h->d_cell_start, h->d_perm_tmp, h->d_fx, h->d_spos,
+                     mixed ? nullptr : h->d_fx64, h->d_spos64, h->d_perm, lflag,
                      lst ? h->d_iperm : nullptr, h->d_err);
     });
     if (lst)

@@ -374,8 +374,9 @@ __device__ __forceinline__ int cell_of_f64(double w, double invL, int ncd) {
 template <bool ONE>
 __global__ void __launch_bounds__(kBlockP)
 k_prep_f64(const __grid_constant__ Work w, const double4* __restrict__ pos_q,
-           double4* __restrict__ fx64, int* __restrict__ cid, int* __restrict__ rank,
-           int* __restrict__ cell_cnt, const __grid_constant__ PrepArgs pa) {
+           double4* __restrict__ fx64, uint4* __restrict__ fx, int* __restrict__ cid,
+           int* __restrict__ rank, int* __restrict__ cell_cnt,
+           const __grid_constant__ PrepArgs pa) {
     // the k-sampling blocks come first, so that their table staging and
     // searches run alongside the particle blocks instead of after them
     const int nsb = (int)gridDim.x - pa.npblk;
@@ -407,6 +408,11 @@ k_prep_f64(const __grid_constant__ Work w, const double4* __restrict__ pos_q,
         cid[i] = c;
         rank[i] = RBE_IN_BOUNDS(c, pa.ncell, pa.err) ? atomicAdd(cell_cnt + c, 1) : 0;
         fx64[i] = make_double4(x, y, z, p.w);
+        // fixed-point record for the real-space pass's candidate test (x < L; a
+        // fraction that rounds up to 1 wraps to 0)
+        fx[i] = make_uint4((uint32_t)__double2ull_rz(x * S.invL * 4294967296.0),
+                           (uint32_t)__double2ull_rz(y * S.invL * 4294967296.0),
+                           (uint32_t)__double2ull_rz(z * S.invL * 4294967296.0), 0u);
         qs = p.w;
         q2s = p.w * p.w;
     }
@@ -518,10 +524,9 @@ __global__ void k_scatter(int n, const int* __restrict__ cid, const int* __restr
 }
 
 // Canonical order inside each cell: the particle at atomic slot s goes to
-// cell_start + (number of members of its cell that precede it).  The mixed
-// path orders by fixed-point x (ties by caller index), which the real-space
-// kernel's x windows rely on; the FP64 path by caller index.  One thread per
-// particle; cells hold a handful of particles.
+// cell_start + (number of members of its cell that precede it), by fixed-point
+// x (ties by caller index), which the mixed real-space kernel's x windows rely
+// on.  One thread per particle; cells hold a handful of particles.
 __global__ void k_order(int n, const int* __restrict__ cid, const int* __restrict__ cell_start,
                         const int* __restrict__ perm_tmp, const uint4* __restrict__ fx,
                         uint4* __restrict__ spos, const double4* __restrict__ fx64,
@@ -535,22 +540,17 @@ __global__ void k_order(int n, const int* __restrict__ cid, const int* __restric
     const int c = cid[i];
     const int b = cell_start[c], e = cell_start[c + 1];
     int r = 0;
-    if (fx) {
-        // mixed path: ascending fixed-point x, ties by index
-        const uint32_t xi = fx[i].x;
-        for (int k = b; k < e; ++k) {
-            const int j = __ldg(perm_tmp + k);
-            const uint32_t xj = __ldg(&fx[j].x);
-            r += (xj < xi || (xj == xi && j < i)) ? 1 : 0;
-        }
-    } else {
-        for (int k = b; k < e; ++k) r += (__ldg(perm_tmp + k) < i) ? 1 : 0;
+    const uint32_t xi = fx[i].x;
+    for (int k = b; k < e; ++k) {
+        const int j = __ldg(perm_tmp + k);
+        const uint32_t xj = __ldg(&fx[j].x);
+        r += (xj < xi || (xj == xi && j < i)) ? 1 : 0;
     }
     const int dst = b + r;
     if (!RBE_IN_BOUNDS(dst, n, err)) return;
     perm[dst] = i;
     if (iperm) iperm[i] = dst;
-    if (fx) spos[dst] = fx[i];
+    spos[dst] = fx[i];
     if (fx64) spos64[dst] = fx64[i];
 }
 
@@ -569,16 +569,17 @@ void launch_prep_mixed(cudaStream_t st, bool one, const Work& w, int nblk, const
 }
 
 void launch_prep_f64(cudaStream_t st, bool one, const Work& w, int nblk, const double4* pos_q,
-                     double4* fx64, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa) {
+                     double4* fx64, uint4* fx, int* cid, int* rank, int* cell_cnt,
+                     const PrepArgs& pa) {
     // particle blocks, then sampling blocks: one per system (MH chains) or one per kBlockP samples
     if (pa.ktot > 0) nblk += pa.mh ? pa.nsys : (pa.ktot + kBlockP - 1) / kBlockP;
     if (nblk <= 0) return;
     const size_t smem = pa.mh ? (sizeof(double) + sizeof(uint32_t)) * (size_t)pa.mh_words
                               : sizeof(uint32_t) * (size_t)pa.tab_words;
     if (one)
-        k_prep_f64<true><<<nblk, kBlockP, smem, st>>>(w, pos_q, fx64, cid, rank, cell_cnt, pa);
+        k_prep_f64<true><<<nblk, kBlockP, smem, st>>>(w, pos_q, fx64, fx, cid, rank, cell_cnt, pa);
     else
-        k_prep_f64<false><<<nblk, kBlockP, smem, st>>>(w, pos_q, fx64, cid, rank, cell_cnt, pa);
+        k_prep_f64<false><<<nblk, kBlockP, smem, st>>>(w, pos_q, fx64, fx, cid, rank, cell_cnt, pa);
 }
 
 void launch_cell_assign(cudaStream_t st, bool one, const Work& w, int nblk, const uint4* fx,

@@ -44,17 +44,6 @@ __global__ void k_sample(const SysDev* __restrict__ sysv, int nsys, int ktot,
     ksamp[g] = sample_one(S, table + S.off_t, g - S.off_k, *cur_step, err);
 }
 
-// Force coefficients of wave vector m: coef = lB (S/P) 4 pi / (V k^2) times
-// (Im rho, Re rho), from the fixed-point rho(k) accumulator, in FP64.
-__device__ __forceinline__ double2 kcoef(const SysDev& S, int4 m,
-                                         const unsigned long long* __restrict__ rho) {
-    const double2 r = rho_read(rho, S.rho_inv_scale);
-    const double tp = 2.0 * M_PI * S.invL;
-    const double k2 = tp * tp * ((double)m.x * m.x + (double)m.y * m.y + (double)m.z * m.z);
-    const double coef = S.coef_scale / k2;
-    return make_double2(coef * r.y, coef * r.x);
-}
-
 // ----------------------------------------------------------------- rho (mixed)
 // Two threads per wave vector (threads t and t + kLTile), each over every
 // other particle of the chunk; their sums are added before the atomics.
@@ -237,41 +226,6 @@ k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
     list_body<R, ONE, false, false, 8>(a, b - r1, threadIdx.x);
 }
 
-// ----------------------------------------------------------------- rho (FP64)
-template <bool ONE>
-__global__ void __launch_bounds__(kLTile)
-k_rho_f64(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
-          const double4* __restrict__ fx64, unsigned long long* __restrict__ rho_fx) {
-    __shared__ double4 sp[kStage / 2];
-    const Tile ch = tile_of<ONE>(w);
-    const SysDev& S = sys_of<ONE>(w, ch.sys);
-    const int l = blockIdx.y * kLTile + threadIdx.x;
-    if (blockIdx.y * kLTile >= S.P) return;
-    const bool active = l < S.P;
-    int4 m = make_int4(0, 0, 0, 0);
-    if (active) m = ksamp[S.off_k + l];
-    const double tp = 2.0 * M_PI * S.invL;
-    const double kx = tp * m.x, ky = tp * m.y, kz = tp * m.z;
-    double re = 0.0, im = 0.0;
-    for (int base = 0; base < ch.count; base += kStage / 2) {
-        const int cnt = min(kStage / 2, ch.count - base);
-        __syncthreads();
-        for (int t = threadIdx.x; t < cnt; t += blockDim.x) sp[t] = fx64[ch.first + base + t];
-        __syncthreads();
-        if (active) {
-            for (int j = 0; j < cnt; ++j) {
-                const double4 p = sp[j];
-                const double th = kx * p.x + ky * p.y + kz * p.z;
-                double sn, cs;
-                sincos(th, &sn, &cs);
-                re += p.w * cs;
-                im += p.w * sn;
-            }
-        }
-    }
-    if (active) rho_accumulate(rho_fx + 2 * (S.off_k + l), re, im, S.rho_scale);
-}
-
 // ----------------------------------------------------------------- force (mixed)
 // Shared-memory record per wave vector: -m and phi (the phase of the
 // coefficient, 2^-32 turns) as integers, and R m (the direction scaled by the
@@ -432,51 +386,6 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
     }
 }
 
-// ----------------------------------------------------------------- force (FP64)
-template <bool ONE>
-__global__ void __launch_bounds__(kBlockP)
-k_force_f64(const __grid_constant__ Work w, const double4* __restrict__ rec64,
-            const int4* __restrict__ ksamp, const unsigned long long* __restrict__ rho_fx,
-            double4* __restrict__ fs64) {
-    constexpr int kKT = 256;
-    __shared__ double4 kk[kKT];     // kx, ky, kz, A
-    __shared__ double kb[kKT];      // B
-    const Tile tl = tile_of<ONE>(w);
-    const SysDev& S = sys_of<ONE>(w, tl.sys);
-    const int t = threadIdx.x;
-    const bool active = t < tl.count;
-    double4 p = make_double4(0, 0, 0, 0);
-    if (active) p = rec64[tl.first + t];
-    const double tp = 2.0 * M_PI * S.invL;
-    double fx = 0, fy = 0, fz = 0, ph = 0;
-    for (int base = 0; base < S.P; base += kKT) {
-        const int cnt = min(kKT, S.P - base);
-        __syncthreads();
-        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
-            const int4 m = ksamp[S.off_k + base + k];
-            const double2 ab = kcoef(S, m, rho_fx + 2 * (S.off_k + base + k));
-            kk[k] = make_double4(tp * m.x, tp * m.y, tp * m.z, ab.x);
-            kb[k] = ab.y;
-        }
-        __syncthreads();
-        if (active) {
-            for (int k = 0; k < cnt; ++k) {
-                const double4 kv = kk[k];
-                const double th = kv.x * p.x + kv.y * p.y + kv.z * p.z;
-                double sn, cs;
-                sincos(th, &sn, &cs);
-                const double B = kb[k];
-                const double g = cs * kv.w - sn * B;
-                fx += g * kv.x;
-                fy += g * kv.y;
-                fz += g * kv.z;
-                ph += cs * B + sn * kv.w;
-            }
-        }
-    }
-    if (active) fs64[tl.first + t] = make_double4(-p.w * fx, -p.w * fy, -p.w * fz, ph);
-}
-
 // ------------------------------------------------------------- launchers
 void launch_sample(cudaStream_t st, const SysDev* sys, int nsys, int ktot, const int* kstart,
                    const uint64_t* table, const uint64_t* cur_step, int4* ksamp, int* err) {
@@ -541,16 +450,6 @@ void launch_rho_list(cudaStream_t st, bool one, const Work& w, int nchunks, int 
     }
 }
 
-void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
-                    const int4* ksamp, const double4* fx64, unsigned long long* rho_fx) {
-    if (nchunks <= 0 || ltiles <= 0) return;
-    dim3 grid(nchunks, ltiles);
-    if (one)
-        k_rho_f64<true><<<grid, kLTile, 0, st>>>(w, ksamp, fx64, rho_fx);
-    else
-        k_rho_f64<false><<<grid, kLTile, 0, st>>>(w, ksamp, fx64, rho_fx);
-}
-
 template <int SPLIT, int PT>
 static void force_mixed_split(cudaStream_t st, bool one, const Work& w, int nblk, const uint4* fx,
                               const int4* ksamp, const float2* kab, float4* fs,
@@ -575,16 +474,6 @@ void launch_fourier_force_mixed(cudaStream_t st, bool one, const Work& w, int nb
         case 8: force_mixed_split<8, 1>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl); break;
         default: force_mixed_split<1, 2>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl); break;
     }
-}
-
-void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk,
-                              const double4* fx64, const int4* ksamp,
-                              const unsigned long long* rho_fx, double4* fs64) {
-    if (nblk <= 0) return;
-    if (one)
-        k_force_f64<true><<<nblk, kBlockP, 0, st>>>(w, fx64, ksamp, rho_fx, fs64);
-    else
-        k_force_f64<false><<<nblk, kBlockP, 0, st>>>(w, fx64, ksamp, rho_fx, fs64);
 }
 
 }  // namespace rbe

@@ -414,7 +414,7 @@ struct PrepArgs {
 void launch_prep_mixed(cudaStream_t st, bool one, const Work& w, int nblk, const float4* pos_q,
                        uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa);
 void launch_prep_f64(cudaStream_t st, bool one, const Work& w, int nblk, const double4* pos_q,
-                     double4* fx64, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa);
+                     double4* fx64, uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa);
 // Neighbour-list evaluations: cell ids and slots (cid, rank, cell_cnt) of the
 // particles from their fixed-point records, only when *list_flag is set.
 void launch_cell_assign(cudaStream_t st, bool one, const Work& w, int nblk, const uint4* fx,
@@ -473,8 +473,11 @@ __device__ __forceinline__ double2 rho_read(const unsigned long long* src, doubl
 void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
                       const int4* ksamp, const double* kcoef, const uint4* fx,
                       unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl = false);
-void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
-                    const int4* ksamp, const double4* fx64, unsigned long long* rho_fx);
+// FP64 path (rbe_fourier64.cu): chunk = particles per chunk, pmax and mcap the
+// largest P and sampler half width M over the systems; phi: also dE/dq.
+void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int chunk, int pmax,
+                    int mcap, const int4* ksamp, const double4* fx64,
+                    unsigned long long* rho_fx);
 // The last stage of a neighbour-list MD step, run by the Fourier-force
 // kernel: total force = Fourier + freal, then the thermostat.
 struct MdOut {
@@ -497,9 +500,10 @@ struct MdOut {
 void launch_fourier_force_mixed(cudaStream_t st, bool one, const Work& w, int nblk, int split,
                                 const uint4* fx, const int4* ksamp, const float2* kab,
                                 float4* fs, const MdOut& md = MdOut{}, bool pdl = false);
-void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk,
-                              const double4* fx64, const int4* ksamp,
-                              const unsigned long long* rho_fx, double4* fs64);
+void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int mcap,
+                              bool phi, const double4* fx64, const int4* ksamp,
+                              const double* kcoef, const unsigned long long* rho_fx,
+                              double4* fs64);
 
 // real space, LJ, Langevin, energies (rbe_real.cu)
 // Blocks per real-space segment (mixed path): the first takes the particles
@@ -512,7 +516,7 @@ struct RealArgs {
     Work w;                  // real-space tiles of kBlockP / split particles (FP64 path)
     int nrblk;
     int split;               // threads per particle, mixed path (1, 3 or 9)
-    int split64;             // threads per particle, FP64 path (power of two)
+    int split64;             // threads per particle, FP64 path (4, 8 or 16)
     int ncell;               // cells over all systems
     int nsys;
     const int* cstart;       // first cell of each system (nsys + 1), batch only

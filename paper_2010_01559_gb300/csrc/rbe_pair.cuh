@@ -10,6 +10,26 @@ namespace rbe {
 
 constexpr int kPartFourier = 1, kPartReal = 2, kPartLJ = 4;
 
+__device__ __forceinline__ int wrapc(int c, int n) { return c < 0 ? c + n : (c >= n ? c - n : c); }
+
+// The 27 neighbour cells as 9 rows (dz, dy) of three x-adjacent cells.  Cells
+// are numbered x fastest, so a row is one contiguous range of the sorted
+// particles unless it wraps around the box edge; then it is two ranges.
+__device__ __forceinline__ void row_ranges(const int* __restrict__ cs, int base, int cx, int ncd,
+                                           int& s0, int& e0, int& s1, int& e1) {
+    if (ncd < 3) {                                  // one cell per edge: the whole row once
+        s0 = __ldg(cs + base); e0 = __ldg(cs + base + ncd); s1 = 0; e1 = 0;
+    } else if (cx > 0 && cx < ncd - 1) {
+        s0 = __ldg(cs + base + cx - 1); e0 = __ldg(cs + base + cx + 2); s1 = 0; e1 = 0;
+    } else if (cx == 0) {
+        s0 = __ldg(cs + base); e0 = __ldg(cs + base + 2);
+        s1 = __ldg(cs + base + ncd - 1); e1 = __ldg(cs + base + ncd);
+    } else {
+        s0 = __ldg(cs + base + ncd - 2); e0 = __ldg(cs + base + ncd);
+        s1 = __ldg(cs + base); e1 = __ldg(cs + base + 1);
+    }
+}
+
 // Deterministic block sum of two doubles (fixed shuffle tree, then warps in
 // order); the result is valid in thread 0.
 __device__ __forceinline__ double2 block_sum2_real(double a, double b) {

@@ -11,8 +11,7 @@
 // pairs within r_c + skin (k_list_build, k_real_list); forces calls scan the
 // cells: one block per segment of x-adjacent cells with the neighbourhood
 // staged in shared memory and R = 1, 3 or 9 threads per particle, each scanning
-// 9/R neighbour rows (k_real_seg).  FP64 path: G threads per particle reading
-// the neighbours from global memory.
+// 9/R neighbour rows (k_real_seg).  FP64 path: rbe_real64.cu.
 //
 // Real-space pair terms for r < r_c (r_ij = r_j - r_i):
 //   F_i   += -lB q_i q_j G(r) r_ij / r,  G = erfc(sqrt(a) r)/r^2 + 2 sqrt(a) e^{-a r^2}/(sqrt(pi) r)
@@ -35,28 +34,6 @@
 #include "rbe_list_body.cuh"
 
 namespace rbe {
-
-
-
-__device__ __forceinline__ int wrapc(int c, int n) { return c < 0 ? c + n : (c >= n ? c - n : c); }
-
-// The 27 neighbour cells as 9 rows (dz, dy) of three x-adjacent cells.  Cells
-// are numbered x fastest, so a row is one contiguous range of the sorted
-// particles unless it wraps around the box edge; then it is two ranges.
-__device__ __forceinline__ void row_ranges(const int* __restrict__ cs, int base, int cx, int ncd,
-                                           int& s0, int& e0, int& s1, int& e1) {
-    if (ncd < 3) {                                  // one cell per edge: the whole row once
-        s0 = __ldg(cs + base); e0 = __ldg(cs + base + ncd); s1 = 0; e1 = 0;
-    } else if (cx > 0 && cx < ncd - 1) {
-        s0 = __ldg(cs + base + cx - 1); e0 = __ldg(cs + base + cx + 2); s1 = 0; e1 = 0;
-    } else if (cx == 0) {
-        s0 = __ldg(cs + base); e0 = __ldg(cs + base + 2);
-        s1 = __ldg(cs + base + ncd - 1); e1 = __ldg(cs + base + ncd);
-    } else {
-        s0 = __ldg(cs + base + ncd - 2); e0 = __ldg(cs + base + ncd);
-        s1 = __ldg(cs + base); e1 = __ldg(cs + base + 1);
-    }
-}
 
 // ----------------------------------------------------------------- mixed
 // One block per cell.  The block stages the records of the 27 neighbouring
@@ -478,171 +455,6 @@ __global__ void __launch_bounds__(kBlockP) k_list_build(const __grid_constant__ 
     if (blockIdx.x == 0 && t == 0) atomicAdd(la.stats, 1ull);
 }
 
-// ----------------------------------------------------------------- FP64
-template <int G, bool ONE>
-__global__ void __launch_bounds__(kBlockP)
-k_real_f64(const __grid_constant__ RealArgs a) {
-    const Tile tl = tile_of<ONE>(a.w);
-    const SysDev& S = sys_of<ONE>(a.w, tl.sys);
-    const int g = threadIdx.x % G;
-    const int t = threadIdx.x / G;
-    const bool active = t < tl.count;
-    const int i = tl.first + (tl.count > 0 ? min(t, tl.count - 1) : 0);
-    double4 pi = make_double4(0, 0, 0, 0);
-    if (tl.count > 0) pi = a.spos64[i];
-    const double qi = pi.w;
-    const bool do_real = (a.parts & kPartReal) != 0;
-    const bool do_lj = (a.parts & kPartLJ) != 0 && S.lj_eps != 0.0;
-    double fx = 0, fy = 0, fz = 0, phr = 0, ec = 0, elj = 0, wc = 0, wlj = 0;
-    const bool vir = a.blk_w != nullptr;
-    if (active && (do_real || do_lj)) {
-        const int ncd = S.ncd;
-        auto cell = [&](double w) {
-            const double u = w * S.invL * (double)ncd;
-            return (u >= 0.0 && u < (double)ncd) ? (int)u : 0;
-        };
-        const int cx = cell(pi.x), cy = cell(pi.y), cz = cell(pi.z);
-        const double L = S.L, invL = S.invL;
-        const double rc2 = do_real ? S.r_c * S.r_c : 0.0;
-        const double lj_rc2 = do_lj ? S.lj_rcut2 : 0.0;
-        const double two_sa_spi = 2.0 * S.sqrt_alpha / sqrt(M_PI);
-        const int dlo = ncd < 3 ? 0 : -1, dhi = ncd < 3 ? 0 : 1;   // one cell: all pairs once
-        for (int dz = dlo; dz <= dhi; ++dz) {
-            const int zz = wrapc(cz + dz, ncd);
-            for (int dy = dlo; dy <= dhi; ++dy) {
-                const int yy = wrapc(cy + dy, ncd);
-                int s0, e0, s1, e1;
-                row_ranges(a.cell_start, S.off_c + (zz * ncd + yy) * ncd, cx, ncd, s0, e0, s1, e1);
-                for (int r = 0; r < 2; ++r) {
-                    const int s = r ? s1 : s0, e = r ? e1 : e0;
-                    for (int j = s + g; j < e; j += G) {
-                        if (j == i) continue;
-                        const double4 pj = a.spos64[j];
-                        double ddx = pj.x - pi.x, ddy = pj.y - pi.y, ddz = pj.z - pi.z;
-                        ddx -= L * rint(ddx * invL);
-                        ddy -= L * rint(ddy * invL);
-                        ddz -= L * rint(ddz * invL);
-                        const double r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-                        if (r2 < rc2) {
-                            const double r = sqrt(r2);
-                            const double erfc_v = erfc(S.sqrt_alpha * r);
-                            const double G_ = erfc_v / r2 + two_sa_spi * exp(-S.alpha * r2) / r;
-                            const double s_ = -S.lB * qi * pj.w * G_ / r;
-                            fx += s_ * ddx; fy += s_ * ddy; fz += s_ * ddz;
-                            phr += S.lB * pj.w * erfc_v / r;
-                            ec += 0.5 * S.lB * qi * pj.w * erfc_v / r;
-                            if (vir)
-                                wc += 0.5 * S.lB * qi * pj.w *
-                                      (erfc_v / r + two_sa_spi * exp(-S.alpha * r2));
-                        }
-                        if (r2 < lj_rc2) {
-                            const double sr2 = S.lj_sigma2 / r2;
-                            const double sr6 = sr2 * sr2 * sr2;
-                            const double mag = 24.0 * S.lj_eps * (2.0 * sr6 * sr6 - sr6) / r2;
-                            fx -= mag * ddx; fy -= mag * ddy; fz -= mag * ddz;
-                            elj += 0.5 * (4.0 * S.lj_eps * (sr6 * sr6 - sr6) + S.lj_shift);
-                            if (vir) wlj += 0.5 * mag * r2;
-                        }
-                    }
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        fx += __shfl_down_sync(0xffffffffu, fx, o, G);
-        fy += __shfl_down_sync(0xffffffffu, fy, o, G);
-        fz += __shfl_down_sync(0xffffffffu, fz, o, G);
-        phr += __shfl_down_sync(0xffffffffu, phr, o, G);
-        ec += __shfl_down_sync(0xffffffffu, ec, o, G);
-        elj += __shfl_down_sync(0xffffffffu, elj, o, G);
-        wc += __shfl_down_sync(0xffffffffu, wc, o, G);
-        wlj += __shfl_down_sync(0xffffffffu, wlj, o, G);
-    }
-    const bool owner = active && g == 0;
-    if (owner) {
-        double phi = phr;
-        const int o = a.perm[i];
-        if (a.parts & kPartFourier) {
-            const double4 f = a.fs64[o];
-            fx += f.x; fy += f.y; fz += f.z;
-            if (a.phi_out64) {
-                const double qs = (double)(long long)__ldcg(a.qsum_fx + tl.sys) / kQScale;
-                phi += f.w - 2.0 * S.self_coef * qi - S.bg_coef * qs;
-            }
-        }
-        if (a.F_out64) a.F_out64[o] = make_double4(fx, fy, fz, 0.0);
-        if (a.phi_out64) a.phi_out64[o] = phi;
-        if (a.md_pos64 && a.nh && S.thermostat == RBE_THERMO_NOSE_HOOVER) {
-            // Nose-Hoover leapfrog: v <- (v a + (dt/m) F) b, drift, wrap
-            const double na = a.nh[tl.sys].a, nb = a.nh[tl.sys].b;
-            const double F3[3] = {fx, fy, fz};
-            double4 v = a.md_vel64[o];
-            double4 rp = a.md_pos64[o];
-            double* vv[3] = {&v.x, &v.y, &v.z};
-            double* rr[3] = {&rp.x, &rp.y, &rp.z};
-            double v2 = 0.0;
-            for (int d = 0; d < 3; ++d) {
-                const double vd = (*vv[d] * na + S.dt_over_m * F3[d]) * nb;
-                double rd = *rr[d] + S.dt * vd;
-                rd -= S.L * floor(rd / S.L);
-                *vv[d] = vd;
-                *rr[d] = rd;
-                v2 += vd * vd;
-            }
-            a.md_vel64[o] = v;
-            a.md_pos64[o] = rp;
-            atomicAdd(&a.nh[tl.sys].k2, __double2ull_rn(v2 * S.nh_k2scale));
-        } else if (a.md_pos64) {
-            const uint64_t step = *a.cur_step;
-            const uint2 key = make_uint2((uint32_t)S.seed, (uint32_t)(S.seed >> 32));
-            const uint32_t pid = (uint32_t)(o - S.off_p);
-            const bool andersen = S.thermostat == RBE_THERMO_ANDERSEN;
-            // Langevin: normals of the OU step; Andersen: collision word, then normals
-            const uint4 c = philox4x32_10(make_uint4(pid, 0u, (uint32_t)step,
-                                                     (S.stream << 8) | (andersen ? 0x07u : 0x02u)),
-                                          key);
-            const bool hit = andersen && (uint64_t)c.x < S.andersen_thr;
-            const uint4 w = andersen ? philox4x32_10(make_uint4(pid, 1u, (uint32_t)step,
-                                                                (S.stream << 8) | 0x07u), key)
-                                     : c;
-            const double u1 = ((double)w.x + 1.0) / 4294967296.0;
-            const double u2 = (double)w.y / 4294967296.0;
-            const double u3 = ((double)w.z + 1.0) / 4294967296.0;
-            const double u4 = (double)w.w / 4294967296.0;
-            const double r1 = sqrt(-2.0 * log(u1)), r3 = sqrt(-2.0 * log(u3));
-            const double xi[3] = {r1 * cos(2.0 * M_PI * u2), r1 * sin(2.0 * M_PI * u2),
-                                  r3 * cos(2.0 * M_PI * u4)};
-            const double F3[3] = {fx, fy, fz};
-            double4 v = a.md_vel64[o];
-            double4 rp = a.md_pos64[o];
-            double* vv[3] = {&v.x, &v.y, &v.z};
-            double* rr[3] = {&rp.x, &rp.y, &rp.z};
-            const double L = S.L;
-            for (int d = 0; d < 3; ++d) {
-                double vd = *vv[d] + S.dt_over_m * F3[d];
-                if (!andersen) vd = S.c1 * vd + S.c2 * xi[d];
-                double rd = *rr[d] + S.dt * vd;
-                rd -= L * floor(rd / L);
-                if (hit) vd = S.vsd * xi[d];           // Andersen collision after the drift
-                *vv[d] = vd;
-                *rr[d] = rd;
-            }
-            a.md_vel64[o] = v;
-            a.md_pos64[o] = rp;
-        }
-    }
-    if (a.blk_e) {
-        const double2 r = block_sum2_real(owner ? ec : 0.0, owner ? elj : 0.0);
-        if (threadIdx.x == 0) a.blk_e[blockIdx.x] = r;
-    }
-    if (vir) {
-        __syncthreads();                                // the partial buffers are reused
-        const double2 r = block_sum2_real(owner ? wc : 0.0, owner ? wlj : 0.0);
-        if (threadIdx.x == 0) a.blk_w[blockIdx.x] = r;
-    }
-}
-
 // ----------------------------------------------------------------- energy
 // One block per system: fixed-order FP64 sums of the per-k energy terms and the
 // per-block real-space / LJ partials, plus the self and background terms.
@@ -751,12 +563,6 @@ static void real_mixed_r(cudaStream_t st, bool one, const RealArgs& a) {
     else real_mixed_rn<R, 64>(st, one, a);
 }
 
-template <int G>
-static void real_f64_g(cudaStream_t st, bool one, const RealArgs& a) {
-    if (one) k_real_f64<G, true><<<a.nrblk, kBlockP, 0, st>>>(a);
-    else k_real_f64<G, false><<<a.nrblk, kBlockP, 0, st>>>(a);
-}
-
 void launch_real_mixed(cudaStream_t st, bool one, const RealArgs& a) {
     if (a.nseg <= 0) return;
     switch (a.split) {
@@ -791,18 +597,6 @@ void launch_list_build(cudaStream_t st, bool one, const ListArgs& la) {
     if (la.nblk <= 0) return;
     if (one) k_list_build<true><<<la.nblk, kBlockP, 0, st>>>(la);
     else k_list_build<false><<<la.nblk, kBlockP, 0, st>>>(la);
-}
-
-void launch_real_f64(cudaStream_t st, bool one, const RealArgs& a) {
-    if (a.nrblk <= 0) return;
-    switch (a.split64) {
-        case 2: real_f64_g<2>(st, one, a); break;
-        case 4: real_f64_g<4>(st, one, a); break;
-        case 8: real_f64_g<8>(st, one, a); break;
-        case 16: real_f64_g<16>(st, one, a); break;
-        case 32: real_f64_g<32>(st, one, a); break;
-        default: real_f64_g<1>(st, one, a); break;
-    }
 }
 
 void launch_energy(cudaStream_t st, bool one, const Work& w, int nsys, const int4* ksamp,

@@ -1,0 +1,299 @@
+// rbe_real64.cu -- real-space Coulomb, shifted Lennard-Jones, the assembly of
+// the total force / dE/dq and the MD update on the FP64 path (formulas:
+// rbe_real.cu), over the cell list.
+//
+// What bounds it: the FP64 pipe (two lanes per SM and clock).  The pair terms
+// cost about a hundred FP64 instructions, and only about one candidate of the
+// 27 cells in ten is within the cutoff, so a warp that tested and evaluated in
+// one loop spent them on nearly every candidate.  Here G lanes per particle
+// first test the candidates' 32-bit fixed-point records (integer and FP32 work
+// only, with a margin that keeps every pair the FP64 test would) and collect
+// the survivors' indices in shared memory; then the G lanes evaluate them
+// densely in FP64, which applies the cutoffs themselves.  erfc is
+// e^{-x^2} erfcx(x) with the Gaussian the force needs anyway, and one
+// reciprocal square root serves every division.  The closing MD update runs
+// one thread per particle after the block's pair sums.
+// Measured (events around the kernel, launch included): N = 1000, r_c = 5, MD
+// step: 298 -> 39 us; N = 8001, r_c = 6, forces with energy and dE/dq: 930 ->
+// 153 us.
+#include <cmath>
+
+#include "rbe_internal.cuh"
+#include "rbe_pair.cuh"
+
+namespace rbe {
+
+constexpr int kHitCap = 96;           // listed candidates per particle before a flush
+
+struct Pair64 {
+    double fx, fy, fz, phr, ec, elj, wc, wlj;
+};
+
+struct Const64 {
+    double rc2, lj_rc2, lj_sigma2, lj_eps, lj_shift, alpha, sqrt_alpha, two_sa_spi, lB, lBqi;
+    double L, halfL;
+};
+
+__device__ __forceinline__ double min_image(double d, const Const64& c) {
+    return fabs(d) > c.halfL ? d - copysign(c.L, d) : d;
+}
+
+// EN: also the potential, energies and virials.
+template <bool EN>
+__device__ __forceinline__ void pair64(const double4& pi, const double4& pj, const Const64& c,
+                                       Pair64& a) {
+    const double dx = min_image(pj.x - pi.x, c), dy = min_image(pj.y - pi.y, c),
+                 dz = min_image(pj.z - pi.z, c);
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const bool in = r2 < c.rc2, lj = r2 < c.lj_rc2;
+    if (!in && !lj) return;
+    const double inv_r = rsqrt(r2), inv_r2 = inv_r * inv_r;
+    double s = 0.0;
+    if (in) {
+        const double ex = exp(-c.alpha * r2);
+        const double pot = ex * erfcx(c.sqrt_alpha * (r2 * inv_r)) * inv_r;     // erfc / r
+        const double g = fma(c.two_sa_spi, ex, pot);
+        const double qq = c.lBqi * pj.w;
+        s = -qq * g * inv_r2;
+        if constexpr (EN) {
+            a.phr = fma(c.lB * pj.w, pot, a.phr);
+            a.ec = fma(0.5 * qq, pot, a.ec);
+            a.wc = fma(0.5 * qq, g, a.wc);
+        }
+    }
+    if (lj) {
+        const double sr2 = c.lj_sigma2 * inv_r2;
+        const double sr6 = sr2 * sr2 * sr2;
+        const double mag = 24.0 * c.lj_eps * fma(2.0 * sr6, sr6, -sr6) * inv_r2;
+        s -= mag;
+        if constexpr (EN) {
+            a.elj += 0.5 * fma(4.0 * c.lj_eps, fma(sr6, sr6, -sr6), c.lj_shift);
+            a.wlj = fma(0.5 * mag, r2, a.wlj);
+        }
+    }
+    a.fx = fma(s, dx, a.fx);
+    a.fy = fma(s, dy, a.fy);
+    a.fz = fma(s, dz, a.fz);
+}
+
+// r wrapped into [0, L): inside the box floor(r / L) is 0, so the division is
+// only taken outside it
+__device__ __forceinline__ double wrap_box(double r, double L) {
+    return (r >= 0.0 && r < L) ? r : r - L * floor(r / L);
+}
+
+template <int G, bool ONE, bool EN>
+__global__ void __launch_bounds__(kBlockP)
+k_real_f64(const __grid_constant__ RealArgs a) {
+    constexpr int T = kBlockP / G;               // particles per block
+    __shared__ int s_hit[T][kHitCap];
+    __shared__ double4 s_f[T];
+    const Tile tl = tile_of<ONE>(a.w);
+    const SysDev& S = sys_of<ONE>(a.w, tl.sys);
+    const int g = threadIdx.x % G, t = threadIdx.x / G;
+    const bool active = t < tl.count;
+    const int i = tl.first + (tl.count > 0 ? min(t, tl.count - 1) : 0);
+    const bool do_real = (a.parts & kPartReal) != 0;
+    const bool do_lj = (a.parts & kPartLJ) != 0 && S.lj_eps != 0.0;
+    Pair64 acc{0, 0, 0, 0, 0, 0, 0, 0};
+    if (tl.count > 0 && (do_real || do_lj)) {
+        const double4 pi = a.spos64[i];
+        Const64 c;
+        c.rc2 = do_real ? S.r_c * S.r_c : 0.0;
+        c.lj_rc2 = do_lj ? S.lj_rcut2 : 0.0;
+        c.lj_sigma2 = S.lj_sigma2;
+        c.lj_eps = S.lj_eps;
+        c.lj_shift = S.lj_shift;
+        c.alpha = S.alpha;
+        c.sqrt_alpha = S.sqrt_alpha;
+        c.two_sa_spi = 2.0 * S.sqrt_alpha * 0.5641895835477563;      // 1 / sqrt(pi)
+        c.lB = S.lB;
+        c.lBqi = S.lB * pi.w;
+        c.L = S.L;
+        c.halfL = 0.5 * S.L;
+        // the candidate test: fixed-point records are within a unit of the FP64
+        // positions, and the widened cutoff covers that and the FP32 rounding
+        const float Lu = S.L_over_2_32;
+        const float cut2 = fmaxf(do_real ? S.f_rc2 : 0.f, do_lj ? S.f_lj_rc2 : 0.f) * 1.0001f;
+        const uint4 si = a.spos[i];
+        const unsigned lane = threadIdx.x & 31;
+        const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane & ~(G - 1u));
+        const unsigned below = gmask & ((1u << lane) - 1u);
+        int* hit = s_hit[t];
+        int nhit = 0;                            // the same in every lane of the group
+        auto dense = [&](int n) {                // the first n listed pairs, G at a time
+            for (int k = g; k < n; k += G) pair64<EN>(pi, a.spos64[hit[k]], c, acc);
+        };
+        const int ncd = S.ncd;
+        auto cell = [&](double w) {
+            const double u = w * S.invL * (double)ncd;
+            return (u >= 0.0 && u < (double)ncd) ? (int)u : 0;
+        };
+        if (active) {
+            const int cx = cell(pi.x), cy = cell(pi.y), cz = cell(pi.z);
+            const int nrow = ncd < 3 ? 1 : 9;    // one cell: every pair once
+#pragma unroll 1
+            for (int r = 0; r < nrow; ++r) {
+                const int dz = ncd < 3 ? 0 : r / 3 - 1, dy = ncd < 3 ? 0 : r % 3 - 1;
+                const int zz = wrapc(cz + dz, ncd), yy = wrapc(cy + dy, ncd);
+                int s0, e0, s1, e1;
+                row_ranges(a.cell_start, S.off_c + (zz * ncd + yy) * ncd, cx, ncd, s0, e0, s1, e1);
+                const int n0 = e0 - s0, n = n0 + (e1 - s1);
+                for (int k0 = 0; k0 < n; k0 += G) {
+                    const int k = k0 + g;
+                    const int j = k < n0 ? s0 + k : s1 + (k - n0);
+                    bool near = false;
+                    if (k < n) {
+                        const uint4 sj = __ldg(a.spos + j);
+                        const float dx = (float)(int32_t)(sj.x - si.x) * Lu;
+                        const float dyy = (float)(int32_t)(sj.y - si.y) * Lu;
+                        const float dzz = (float)(int32_t)(sj.z - si.z) * Lu;
+                        near = fmaf(dx, dx, fmaf(dyy, dyy, dzz * dzz)) < cut2 && j != i;
+                    }
+                    const unsigned m = __ballot_sync(gmask, near) & gmask;
+                    if (near) hit[nhit + __popc(m & below)] = j;
+                    nhit += __popc(m);
+                    if (nhit > kHitCap - G) {    // crowded: evaluate what is listed
+                        __syncwarp(gmask);
+                        dense(nhit);
+                        __syncwarp(gmask);
+                        nhit = 0;
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        // dense rounds, the warp's groups together
+        const int rounds = (int)__reduce_max_sync(0xffffffffu, (unsigned)(nhit + G - 1) / G);
+        for (int q = 0; q < rounds; ++q) {
+            const int k = q * G + g;
+            if (k < nhit) pair64<EN>(pi, a.spos64[hit[k]], c, acc);
+        }
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) {
+        acc.fx += __shfl_down_sync(0xffffffffu, acc.fx, o, G);
+        acc.fy += __shfl_down_sync(0xffffffffu, acc.fy, o, G);
+        acc.fz += __shfl_down_sync(0xffffffffu, acc.fz, o, G);
+        if constexpr (EN) {
+            acc.phr += __shfl_down_sync(0xffffffffu, acc.phr, o, G);
+            acc.ec += __shfl_down_sync(0xffffffffu, acc.ec, o, G);
+            acc.elj += __shfl_down_sync(0xffffffffu, acc.elj, o, G);
+            acc.wc += __shfl_down_sync(0xffffffffu, acc.wc, o, G);
+            acc.wlj += __shfl_down_sync(0xffffffffu, acc.wlj, o, G);
+        }
+    }
+    const bool owner = active && g == 0;
+    if (owner) s_f[t] = make_double4(acc.fx, acc.fy, acc.fz, acc.phr);
+    __syncthreads();
+    if ((int)threadIdx.x < min(T, tl.count)) {
+        // one thread per particle: total force, outputs, MD update
+        const int ii = tl.first + threadIdx.x;
+        const double4 fr = s_f[threadIdx.x];
+        double fx = fr.x, fy = fr.y, fz = fr.z, phi = fr.w;
+        const int o = a.perm[ii];
+        if (a.parts & kPartFourier) {
+            const double4 f = a.fs64[o];
+            fx += f.x; fy += f.y; fz += f.z;
+            if (a.phi_out64) {
+                const double qs = (double)(long long)__ldcg(a.qsum_fx + tl.sys) / kQScale;
+                phi += f.w - 2.0 * S.self_coef * a.spos64[ii].w - S.bg_coef * qs;
+            }
+        }
+        if (a.F_out64) a.F_out64[o] = make_double4(fx, fy, fz, 0.0);
+        if (a.phi_out64) a.phi_out64[o] = phi;
+        if (a.md_pos64 && a.nh && S.thermostat == RBE_THERMO_NOSE_HOOVER) {
+            // Nose-Hoover leapfrog: v <- (v a + (dt/m) F) b, drift, wrap
+            const double na = a.nh[tl.sys].a, nb = a.nh[tl.sys].b;
+            const double F3[3] = {fx, fy, fz};
+            double4 v = a.md_vel64[o];
+            double4 rp = a.md_pos64[o];
+            double* vv[3] = {&v.x, &v.y, &v.z};
+            double* rr[3] = {&rp.x, &rp.y, &rp.z};
+            double v2 = 0.0;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const double vd = (*vv[d] * na + S.dt_over_m * F3[d]) * nb;
+                *rr[d] = wrap_box(*rr[d] + S.dt * vd, S.L);
+                *vv[d] = vd;
+                v2 += vd * vd;
+            }
+            a.md_vel64[o] = v;
+            a.md_pos64[o] = rp;
+            atomicAdd(&a.nh[tl.sys].k2, __double2ull_rn(v2 * S.nh_k2scale));
+        } else if (a.md_pos64) {
+            const uint64_t step = *a.cur_step;
+            const uint2 key = make_uint2((uint32_t)S.seed, (uint32_t)(S.seed >> 32));
+            const uint32_t pid = (uint32_t)(o - S.off_p);
+            const bool andersen = S.thermostat == RBE_THERMO_ANDERSEN;
+            // Langevin: normals of the OU step; Andersen: collision word, then normals
+            const uint4 cw = philox4x32_10(make_uint4(pid, 0u, (uint32_t)step,
+                                                      (S.stream << 8) | (andersen ? 0x07u : 0x02u)),
+                                           key);
+            const bool coll = andersen && (uint64_t)cw.x < S.andersen_thr;
+            double xi[3] = {0.0, 0.0, 0.0};
+            if (!andersen || coll) {
+                const uint4 w = andersen ? philox4x32_10(make_uint4(pid, 1u, (uint32_t)step,
+                                                                    (S.stream << 8) | 0x07u), key)
+                                         : cw;
+                const double u1 = ((double)w.x + 1.0) * 0x1p-32, u2 = (double)w.y * 0x1p-32;
+                const double u3 = ((double)w.z + 1.0) * 0x1p-32, u4 = (double)w.w * 0x1p-32;
+                const double r1 = sqrt(-2.0 * log(u1)), r3 = sqrt(-2.0 * log(u3));
+                double s2, c2;
+                sincospi(2.0 * u2, &s2, &c2);
+                xi[0] = r1 * c2;
+                xi[1] = r1 * s2;
+                xi[2] = r3 * cospi(2.0 * u4);
+            }
+            const double F3[3] = {fx, fy, fz};
+            double4 v = a.md_vel64[o];
+            double4 rp = a.md_pos64[o];
+            double* vv[3] = {&v.x, &v.y, &v.z};
+            double* rr[3] = {&rp.x, &rp.y, &rp.z};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                double vd = *vv[d] + S.dt_over_m * F3[d];
+                if (!andersen) vd = S.c1 * vd + S.c2 * xi[d];
+                *rr[d] = wrap_box(*rr[d] + S.dt * vd, S.L);
+                if (coll) vd = S.vsd * xi[d];          // Andersen collision after the drift
+                *vv[d] = vd;
+            }
+            a.md_vel64[o] = v;
+            a.md_pos64[o] = rp;
+        }
+    }
+    if constexpr (EN) {
+        if (a.blk_e) {
+            const double2 r = block_sum2_real(owner ? acc.ec : 0.0, owner ? acc.elj : 0.0);
+            if (threadIdx.x == 0) a.blk_e[blockIdx.x] = r;
+        }
+        if (a.blk_w) {
+            __syncthreads();                            // the partial buffers are reused
+            const double2 r = block_sum2_real(owner ? acc.wc : 0.0, owner ? acc.wlj : 0.0);
+            if (threadIdx.x == 0) a.blk_w[blockIdx.x] = r;
+        }
+    }
+}
+
+template <int G>
+static void real_f64_g(cudaStream_t st, bool one, const RealArgs& a) {
+    const bool en = a.phi_out64 || a.blk_e || a.blk_w;
+    if (one) {
+        if (en) k_real_f64<G, true, true><<<a.nrblk, kBlockP, 0, st>>>(a);
+        else k_real_f64<G, true, false><<<a.nrblk, kBlockP, 0, st>>>(a);
+    } else {
+        if (en) k_real_f64<G, false, true><<<a.nrblk, kBlockP, 0, st>>>(a);
+        else k_real_f64<G, false, false><<<a.nrblk, kBlockP, 0, st>>>(a);
+    }
+}
+
+void launch_real_f64(cudaStream_t st, bool one, const RealArgs& a) {
+    if (a.nrblk <= 0) return;
+    switch (a.split64) {
+        case 4: real_f64_g<4>(st, one, a); break;
+        case 8: real_f64_g<8>(st, one, a); break;
+        default: real_f64_g<16>(st, one, a); break;
+    }
+}
+
+}  // namespace rbe
