@@ -298,7 +298,7 @@ typedef struct {
     int32_t force_split;   /* threads per particle in the Fourier-force pass: 1, 2, 4 or 8     */
     int32_t real_split;    /* threads per particle in the mixed real-space pass: 1, 3 or 9,
                               each scanning 9 / real_split of the 9 neighbour rows (the FP64
-                              pass then uses 4, 8 or 16 threads per particle)              */
+                              pass then uses 4, 8, or 16 to 32 threads per particle)       */
     int32_t real_seg;      /* cells along x per real-space block: 1 .. cells per edge           */
     int32_t list_split;    /* threads per particle in the neighbour-list pass of rbe_step:
                               1, 2, 4 or 8                                                   */

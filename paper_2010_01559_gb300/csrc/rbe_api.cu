@@ -223,6 +223,7 @@ struct rbe_ctx {
     int list_split = 0, cur_lsplit = -1;      // lanes per particle of the list pass (0 = auto)
     int lsplit = 1, nlblk = 0, max_lblk = 0;
     int list_cap = 0;                         // entries per particle
+    int small_n = -1, small_cs = 0;           // one-cluster MD steps: blocks for small_n particles
     Tile* d_lblk = nullptr;
     int* d_nbr = nullptr;                     // [slot * ntot + sorted index]
     int* d_ncnt = nullptr;
@@ -464,8 +465,12 @@ int auto_list_split(long long ntot) {
     return r;
 }
 
-// Threads per particle of the FP64 real-space pass, from the mixed path's.
-int real_split64(int r) { return r >= 8 ? 16 : (r >= 2 ? 8 : 4); }
+// Threads per particle of the FP64 real-space pass, from the mixed path's: with
+// 9 of those, 32 up to 16 warps per SM (fewer serial rounds where latency
+// bounds the pass: N = 1000 REAL32) and 16 above (fuller rounds).
+int real_split64(int r, long long ntot) {
+    return r >= 8 ? (ntot <= 152LL * 16 ? 32 : 16) : (r >= 2 ? 8 : 4);
+}
 
 // Cells along x per real-space block: enough blocks to fill the GPU, and a
 // staged neighbourhood (9 rows of seg + 2 cells) of about 2500 records.
@@ -499,7 +504,7 @@ rbe_status prepare(rbe_ctx* h, int n) {
     std::vector<Tile> pblk, fblk, rblk, chunks, lblk;
     const int ltile = kBlockP / lsplit;
     const int ftile = kBlockP / split;
-    const int rtile = kBlockP / real_split64(rsplit);
+    const int rtile = kBlockP / real_split64(rsplit, ntot);
     int off_part = 0;
     for (int s = 0; s < h->nsys; ++s) {
         SysHost& sh = h->sys[s];
@@ -910,10 +915,11 @@ Work make_work(const rbe_ctx* h, const Tile* tiles, int tile, int aux_stride) {
 
 RealArgs make_real_args(const rbe_ctx* h, int parts) {
     RealArgs r{};
-    r.w = make_work(h, h->d_rblk, kBlockP / real_split64(h->rsplit), 0);
+    const int split64 = real_split64(h->rsplit, h->batch ? h->ntot : h->cur_n);
+    r.w = make_work(h, h->d_rblk, kBlockP / split64, 0);
     r.nrblk = h->nrblk;
     r.split = h->rsplit;
-    r.split64 = real_split64(h->rsplit);
+    r.split64 = split64;
     r.ncell = h->ncell;
     r.nsys = h->nsys;
     r.cstart = h->d_cstart;
@@ -1369,6 +1375,26 @@ struct HostIO {
     float* vel;
 };
 
+// Whether the MD steps of a single list system of n particles run as one
+// cluster (rbe_small.cu).  The cluster's blocks share the work of the whole
+// GPU, so its step grows with n P where the separate kernels' hardly does:
+// SMALL_RULE
+constexpr int kSmallStepsPerLaunch = 512;
+constexpr long long kSmallMaxNP = 1000000;
+
+bool small_steps(rbe_ctx* h, int n) {
+    if (h->batch || h->mh || !h->list) return false;
+    const SysHost& sh = h->sys[0];
+    if ((long long)n * sh.p.P > kSmallMaxNP) return false;
+    if (h->small_n != n) {                       // asked once per particle count
+        h->small_n = n;
+        h->small_cs = 0;
+        for (int cs = 16; cs >= 8 && !h->small_cs; cs >>= 1)
+            if (small_md_fits(n, sh.p.P, sh.M, h->list_cap, cs)) h->small_cs = cs;
+    }
+    return h->small_cs > 0;
+}
+
 rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nsteps,
                      uint64_t* step_dev, float* F_out = nullptr, const HostIO* io = nullptr,
                      unsigned long long* done = nullptr) {
@@ -1419,6 +1445,45 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
         }
         cudaMemcpyAsync(h->h_pin + 1, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, sq);
     };
+    if (a.list && nsteps > 0 && !h->prof_on && small_steps(h, n)) {
+        // a small system: the steps of the call as one cluster, a few hundred
+        // steps per launch so that no launch holds its SMs for long
+        if (io) copy_in(h->stream);
+        for (int k = 0; k < nsteps; k += kSmallStepsPerLaunch) {
+            SmallArgs sa{};
+            sa.S = h->sysdev[0];
+            sa.n = n;
+            sa.cs = h->small_cs;
+            sa.nsteps = std::min(kSmallStepsPerLaunch, nsteps - k);
+            sa.pos = (float4*)pos;
+            sa.vel = (float4*)vel;
+            sa.F_out = (float4*)F_out;
+            sa.step_dev = step_dev;
+            sa.table = h->d_table;
+            const double ks = sa.S.coef_scale / (4.0 * M_PI * M_PI * sa.S.invL * sa.S.invL);
+            sa.kscale_hi = (float)ks;
+            sa.kscale_lo = (float)(ks - (double)sa.kscale_hi);
+            sa.nh = h->d_nh;
+            sa.list_flag = h->d_list_flag;
+            sa.sref = h->d_sref;
+            sa.perm = h->d_perm;
+            sa.iperm = h->d_iperm;
+            sa.nbr = h->d_nbr;
+            sa.ncnt = h->d_ncnt;
+            sa.stride = std::max(h->ntot, 1);
+            sa.cap = h->list_cap;
+            sa.stats = h->d_list_stats;
+            sa.err = h->d_err;
+            if (a.done && k + sa.nsteps == nsteps) {
+                sa.done_host = a.done;
+                sa.err_host = (int*)(a.done - 1);
+            }
+            RBE_CUDA(h, launch_small_md(h->stream, sa));
+            ++h->kernel_count;
+        }
+        if (io) copy_out(h->stream);
+        return finish(h, "rbe_step");
+    }
     // a host-buffer call replays one graph holding copies and steps (up to 4)
     const bool host_graph = io && nsteps <= 4;
     if (!h->use_graph || h->prof_on) {
@@ -1530,6 +1595,10 @@ rbe_status report_err(rbe_ctx* h) {
             return fail(h, RBE_ERR_NONFINITE, "a position or charge of the input was NaN or "
                                               "infinite (the results of those calls are not "
                                               "meaningful)");
+        if (err & kErrWait)
+            return fail(h, RBE_ERR_TIMEOUT, "the blocks of a one-cluster MD step did not hear "
+                                            "from each other (the results of that call are not "
+                                            "meaningful)");
         if (err & kErrBounds)
             return fail(h, RBE_ERR_BOUNDS, "the bounds-checked build found an index outside its "
                                            "array (the access was skipped)");

@@ -39,6 +39,7 @@ constexpr int kMaxAttempts = 32;  // bound on the (0,0,0) rejection loop
 constexpr int kErrSampler = 1;    // bits in the device error word
 constexpr int kErrList = 2;       // a neighbour list overflowed
 constexpr int kErrNonfinite = 4;  // a position or charge of the input was NaN or infinite
+constexpr int kErrWait = 16;      // blocks of a cluster did not hear from each other
 constexpr int kErrBounds = 8;     // (bounds-checked build) an index fell outside its array
 constexpr double kQScale = 4294967296.0;           // 2^32: fixed point of sum q
 
@@ -123,6 +124,27 @@ __device__ __forceinline__ bool rbe_in_bounds(long long i, long long n, int* err
 __device__ __forceinline__ void latch_any(bool cond, int* err, int bit) {
     const unsigned m = __ballot_sync(__activemask(), cond);
     if (m && err && (int)(threadIdx.x & 31) == __ffs(m) - 1) atomicOr(err, bit);
+}
+
+// Fixed-point fraction round(2^32 x / L) mod 2^32 of a coordinate (see
+// rbe_cells.cu); hi + lo = 2^32 / L.
+// FP32 and 32-bit integer work only (64-bit conversions would go through the
+// FP64 pipe, which is narrow on this part): the integer pr is first reduced
+// modulo 2^32 in FP32, exactly, to r in [-2^31, 2^31] (for |pr| >= 2^31 the
+// result is a multiple of ulp(pr) >= 2^8 below 2^31 in magnitude, so it is a
+// float; below that pr is left as it is).  Same fraction as the 64-bit sum
+// ip + ic mod 2^32 for |x| < 2^31 L.
+__device__ __forceinline__ uint32_t to_fixed(float x, float hi, float lo) {
+    const float p = x * hi;
+    const float e = fmaf(x, hi, -p);       // exact: x * hi = p + e
+    float corr = fmaf(x, lo, e);
+    const float pr = rintf(p);
+    corr += (p - pr);                      // exact (p and pr differ by < 1 ulp-scale)
+    const float n = rintf(pr * 2.3283064365386963e-10f);        // pr / 2^32, nearest
+    const float r = fmaf(-4294967296.0f, n, pr);                 // exact, |r| <= 2^31
+    // 2^31 and -2^31 are the same fraction; the conversion saturates at 2^31 - 1
+    const uint32_t ur = r >= 2147483648.0f ? 0x80000000u : (uint32_t)__float2int_rz(r);
+    return ur + (uint32_t)__float2int_rn(corr);
 }
 
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two 32x32
@@ -516,7 +538,7 @@ struct RealArgs {
     Work w;                  // real-space tiles of kBlockP / split particles (FP64 path)
     int nrblk;
     int split;               // threads per particle, mixed path (1, 3 or 9)
-    int split64;             // threads per particle, FP64 path (4, 8 or 16)
+    int split64;             // threads per particle, FP64 path (4, 8, 16 or 32)
     int ncell;               // cells over all systems
     int nsys;
     const int* cstart;       // first cell of each system (nsys + 1), batch only
@@ -571,6 +593,32 @@ void launch_rho_list(cudaStream_t st, bool one, const Work& w, int nchunks, int 
                      const int4* ksamp, const double* kcoef, const uint4* fx,
                      unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
                      bool pdl);
+// MD steps of a small single system, all of a call in one cluster (rbe_small.cu).
+struct SmallArgs {
+    SysDev S;
+    int n, cs, nsteps;       // particles, blocks of the cluster, steps
+    float4* pos;
+    float4* vel;
+    float4* F_out;           // nullable: the last step's total force
+    uint64_t* step_dev;      // advanced by nsteps
+    const uint64_t* table;
+    float kscale_hi, kscale_lo;   // coef_scale / (2 pi / L)^2 as a float pair
+    NhState* nh;
+    int* list_flag;          // in: set if the handle's list does not stand; cleared
+    uint4* sref;             // the handle's list: build records, order, entries, counts
+    int* perm;
+    int* iperm;
+    int* nbr;
+    int* ncnt;
+    int stride, cap;
+    unsigned long long* stats;
+    int* err;
+    unsigned long long* done_host;   // nullable: completion word (as in MdOut)
+    int* err_host;
+};
+bool small_md_fits(int n, int P, int M, int cap, int cs);
+cudaError_t launch_small_md(cudaStream_t st, const SmallArgs& a);
+
 void launch_observables(cudaStream_t st, const SysDev& S, const uint4* fx, int first, int n,
                         const int4* mlist, int K, unsigned long long* rho_fx, double2* part,
                         const float4* pos_q, const float4* vel, const double* E_in,

@@ -292,6 +292,7 @@ void launch_real_f64(cudaStream_t st, bool one, const RealArgs& a) {
     switch (a.split64) {
         case 4: real_f64_g<4>(st, one, a); break;
         case 8: real_f64_g<8>(st, one, a); break;
+        case 32: real_f64_g<32>(st, one, a); break;
         default: real_f64_g<16>(st, one, a); break;
     }
 }

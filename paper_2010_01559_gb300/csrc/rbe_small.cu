@@ -1,0 +1,606 @@
+// rbe_small.cu -- MD steps of a small system in one launch: one thread-block
+// cluster runs all the steps of a call.
+//
+// What bounds a step of a few hundred to a few thousand particles is latency:
+// as separate kernels it is nine dependent launches of about 2 us each for
+// well under a microsecond of arithmetic.  Here the sixteen blocks of a
+// cluster keep the whole system in their shared memory and exchange it twice
+// per step with asynchronous remote stores that complete on an mbarrier of the
+// receiving block (no cluster-wide barrier in the loop):
+//
+//   records    rank c owns n/16 particles (position, velocity and build record
+//              stay in registers for the whole call); each owner thread sends
+//              its fixed-point record to all ranks
+//   k-batch    every warp draws the two wave vectors it will sum (while the
+//              records are under way), then sums their structure factors over
+//              a share of all n records; rank c holds P/16 wave vectors, so
+//              no sum crosses blocks.  A thread per wave vector forms the force
+//              coefficient and sends it to all ranks
+//   pairs      meanwhile R lanes per owned particle walk its neighbour list,
+//              then (coefficients in) a lane per particle and a warp per share
+//              of the wave vectors add the Fourier force; one thread per
+//              particle sums the partials in a fixed order and applies the
+//              thermostat.
+//
+// A block that runs ahead cannot overwrite what another still reads, nor count
+// on a barrier phase that has not begun: to send the records of step s + 1 it
+// needs every rank's coefficients of step s, to send coefficients every rank's
+// records (a rank without particles or wave vectors sends a message all the
+// same), and the records alternate between two buffers.
+//
+// FP64 instructions are kept out of the loop (their latency on this part is
+// over a hundred cycles; the first form of this kernel, which summed a wave
+// vector's partials and its coefficient in FP64, spent 3500 to 10700 cycles a
+// step there): partial sums are added as float pairs, and the coefficient
+// (lB S/P 4 pi / V) / k^2 is a float-pair constant over the integer |m|^2.
+//
+// Neighbour list: the owned particles' neighbours within r_c + skin as 16-bit
+// caller indices in shared memory, read from the handle's list when that
+// stands and rebuilt (all pairs, in ascending order) when a particle has moved
+// more than skin/2 since the build, which also writes the handle's list
+// arrays (in the caller's order: perm is the identity).  List, displacement
+// test and build count thus carry over between calls and to the other paths
+// of the handle.
+//
+// Measured (one step, steps in one call): SMALL_FIGURES
+#include <algorithm>
+
+#include "rbe_internal.cuh"
+#include "rbe_pair.cuh"
+
+namespace rbe {
+
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t local_addr(const void* p) {
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+// shared::cluster address in block `rank` of this block's shared address a
+__device__ __forceinline__ uint32_t remote(uint32_t a, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+// 16 bytes into a block's shared memory, counted on that block's mbarrier
+__device__ __forceinline__ void send(uint32_t dst, const uint4& v, uint32_t bar) {
+    asm volatile(
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.u32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+            dst),
+        "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void bar_init(uint32_t bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+}
+// this phase of the barrier completes when `bytes` have come in
+__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
+                 : "memory");
+}
+// Waits for the phase of the given parity, for two seconds at most (a step takes
+// microseconds): false if it did not complete.
+__device__ __forceinline__ unsigned long long now_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
+    unsigned long long t0 = 0ull;
+    for (unsigned t = 0;; ++t) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if ((t & 63u) == 0u) {
+            const unsigned long long now = now_ns();
+            if (t == 0u) t0 = now;
+            else if (now - t0 > 2000000000ull) return false;
+        }
+    }
+}
+
+constexpr float kTurn = 1.4629180792671596e-09f;                     // 2 pi / 2^32
+constexpr int kSmallMaxKc = 2 * kSmallWarps;                         // wave vectors per rank
+constexpr int kSmallMaxCs = 16;                                      // blocks per cluster
+constexpr int kSmallOwnWarps = 8;                                    // owner warps per rank
+
+// Shared-memory layout of a block (byte offsets, 16-byte aligned).
+struct SmallLayout {
+    int np, kc, tab, npg, nks;   // owned particles, wave vectors per rank, table entries,
+                                 // particle groups of the Fourier force and warps on each
+    size_t rec, kv, part, list, table, end;
+};
+
+__host__ __device__ inline size_t small_align(size_t x) { return (x + 15) & ~size_t(15); }
+
+__host__ __device__ inline SmallLayout small_layout(int n, int P, int M, int cap, int cs, int R) {
+    SmallLayout L;
+    L.np = (n + cs - 1) / cs;
+    L.kc = (P + cs - 1) / cs;
+    L.tab = 2 * M + 1;
+    L.npg = (L.np + 31) / 32;
+    L.nks = kSmallWarps / L.npg;
+    L.rec = 0;                                                       // uint4 [2][n]
+    L.kv = L.rec + 32 * (size_t)n;                                   // uint4 [2][P]
+    L.part = L.kv + 32 * (size_t)P;                                  // float4 [R + nks][np]
+    L.list = L.part + 16 * (size_t)(R + L.nks) * L.np;               // u16 [np][cap]
+    L.table = L.list + small_align(2 * (size_t)L.np * cap);          // u32 [2M + 1]
+    L.end = L.table + small_align(4 * (size_t)L.tab);
+    return L;
+}
+
+// a + b as a float pair (s, e): s + e = a + b exactly (Knuth's two-sum).
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
+}
+
+// (ch + cl) (h + l) to FP32
+__device__ __forceinline__ float pair_mul(float ch, float cl, float2 v) {
+    const float p = __fmul_rn(ch, v.x);
+    return __fadd_rn(p, fmaf(ch, v.x, -p) + fmaf(ch, v.y, cl * v.x));
+}
+
+// Samples la and lb of the step's k-batch (as sample_one_smem draws them), by a
+// whole warp: six lanes look up one axis of one sample each.
+__device__ __forceinline__ void warp_sample2(const SysDev& S, const uint32_t* T, int la, int lb,
+                                             uint64_t step, int* err, int4& ma, int4& mb) {
+    const int lane = threadIdx.x & 31, ax = lane % 3;
+    const uint2 key = make_uint2((uint32_t)S.seed, (uint32_t)(S.seed >> 32));
+    bool oka = false, okb = false;
+    for (int a = 0; a < kMaxAttempts && !(oka && okb); ++a) {
+        const uint4 w = philox4x32_10(make_uint4((uint32_t)(lane < 3 ? la : lb), (uint32_t)a,
+                                                 (uint32_t)step, (S.stream << 8) | 0x01u), key);
+        const uint32_t u = ax == 0 ? w.x : (ax == 1 ? w.y : w.z);
+        int lo = 0, hi = 2 * S.M;                   // smallest j with u < T[j]
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (u < T[mid]) hi = mid; else lo = mid + 1;
+        }
+        const int v = lo - S.M;
+        const int x0 = __shfl_sync(0xffffffffu, v, 0), y0 = __shfl_sync(0xffffffffu, v, 1),
+                  z0 = __shfl_sync(0xffffffffu, v, 2), x1 = __shfl_sync(0xffffffffu, v, 3),
+                  y1 = __shfl_sync(0xffffffffu, v, 4), z1 = __shfl_sync(0xffffffffu, v, 5);
+        if (!oka) { ma = make_int4(x0, y0, z0, a + 1); oka = (x0 | y0 | z0) != 0; }
+        if (!okb) { mb = make_int4(x1, y1, z1, a + 1); okb = (x1 | y1 | z1) != 0; }
+    }
+    if (!oka) ma = make_int4(1, 0, 0, kMaxAttempts + 1);
+    if (!okb) mb = make_int4(1, 0, 0, kMaxAttempts + 1);
+    if (!(oka && okb) && lane == 0) atomicOr(err, kErrSampler);
+}
+
+template <int R>
+__global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_constant__ SmallArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ __align__(8) unsigned long long s_bar[2];        // records in, coefficients in
+    __shared__ float s_part[kSmallWarps][4];                    // structure-factor partials
+    __shared__ int4 s_m[kSmallMaxKc];                           // this rank's wave vectors
+    __shared__ uint4 s_token;                                   // from ranks without wave vectors
+    // from every rank's owner warps (at least its first warp): (particle moved,
+    // non-finite input, Nose-Hoover kinetic sum), by step parity
+    __shared__ uint4 s_msg[2][kSmallMaxCs * kSmallOwnWarps];
+    const SysDev& S = a.S;
+    const uint32_t rank = cluster_rank();
+    const int cs = a.cs, n = a.n, P = S.P, tid = threadIdx.x;
+    const int lane = tid & 31, warp = tid >> 5;
+    const SmallLayout L = small_layout(n, P, S.M, a.cap, cs, R);
+    uint4* rec = (uint4*)(smem + L.rec);
+    uint4* kv = (uint4*)(smem + L.kv);              // [l]: -m and phi; [P + l]: R m and R
+    float4* part = (float4*)(smem + L.part);
+    uint16_t* list = (uint16_t*)(smem + L.list);
+    uint32_t* table = (uint32_t*)(smem + L.table);
+    const int first = (int)rank * L.np;
+    const int np = max(0, min(L.np, n - first));    // owned particles (caller's order)
+    const int k0 = (int)rank * L.kc;
+    const int nk = max(0, min(L.kc, P - k0));       // owned wave vectors
+    const bool nhm = S.thermostat == RBE_THERMO_NOSE_HOOVER;
+    const bool owner = tid < np;                    // thread tid closes particle first + tid
+    const int o = first + tid;
+    const int p = tid / R, l = tid % R;             // pair lanes: particle p, lane l of R
+    const bool pairs = p < np;
+    const int pn = first + p;
+    const uint32_t bar_rec = local_addr(&s_bar[0]), bar_kv = local_addr(&s_bar[1]);
+    const uint64_t step0 = *a.step_dev;
+    const bool stale = *a.list_flag != 0;           // the handle's list does not stand
+    float4 pos = make_float4(0.f, 0.f, 0.f, 0.f), vel = pos;
+    uint4 ref = make_uint4(0, 0, 0, 0);
+    if (owner) {
+        pos = a.pos[o];
+        vel = a.vel[o];
+        ref = a.sref[o];
+    }
+    for (int j = tid; j < L.tab; j += kSmallThreads) table[j] = (uint32_t)a.table[j];
+    for (int j = tid; j < 2 * kSmallMaxCs * kSmallOwnWarps; j += kSmallThreads)
+        (&s_msg[0][0])[j] = make_uint4(0, 0, 0, 0);
+    int cnt = 0;                                    // list entries of particle p
+    if (pairs && !stale) {
+        // the handle's list, in sorted indices of its last build
+        const int i = a.iperm[pn];
+        cnt = min(a.ncnt[i], a.cap);
+        for (int k = l; k < cnt; k += R)
+            list[p * a.cap + k] = (uint16_t)a.perm[a.nbr[(size_t)k * a.stride + i]];
+    }
+    NhState nh{};
+    if (nhm) nh = *a.nh;
+    if (tid == 0) {
+        bar_init(bar_rec);
+        bar_init(bar_kv);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    cluster_sync();                                 // every rank's barriers are initialised
+
+    PairConst kc;
+    kc.rc2 = S.f_rc2;
+    kc.lj_rc2 = S.lj_eps != 0.0 ? S.f_lj_rc2 : 0.f;
+    kc.alpha = S.f_alpha;
+    kc.sa = S.f_sqrt_alpha;
+    kc.two_sa_spi = S.f_two_sa_spi;
+    kc.lB = S.f_lB;
+    kc.lj_s2 = S.f_lj_sigma2;
+    kc.lj_eps = S.f_lj_eps;
+    kc.lj_shift = S.f_lj_shift;
+    kc.vir = false;
+    const int kp = (nk + 1) / 2;                    // pairs of wave vectors, a group of warps each
+    const int wpp = kp > 0 ? kSmallWarps / kp : 0;
+    const bool sums = warp < kp * wpp;              // this warp sums pair pr, share sub of wpp
+    const int pr = sums ? warp % kp : 0, sub = sums ? warp / kp : 0;
+    const int pg = warp % L.npg, ks = warp / L.npg; // Fourier force: particle group, k share
+    // bytes a block receives per step: all records and all owner warps' messages
+    const int nfull = n / L.np, nrest = n - nfull * L.np;
+    const int nsend = nfull + (nrest > 0 ? 1 : 0);  // ranks with particles
+    const uint32_t rec_bytes =
+        16u * (uint32_t)(n + nfull * ((L.np + 31) / 32) + (nrest + 31) / 32 + (cs - nsend));
+    const uint32_t kv_bytes = 32u * (uint32_t)P + 16u * (uint32_t)(cs - (P + L.kc - 1) / L.kc);
+    unsigned long long k2w = 0ull;                  // this owner warp's kinetic sum
+    bool bad_seen = false;                          // some position or charge was not finite
+    bool late = false;                              // a wait gave up: no more waiting
+
+    for (int s = 0; s < a.nsteps; ++s) {
+        const uint64_t step = step0 + (uint64_t)s;
+        uint4* R_ = rec + (s & 1) * n;              // this step's records
+        const uint32_t par = (uint32_t)(s & 1);
+        if (tid == 0) {
+            bar_expect(bar_rec, rec_bytes);
+            bar_expect(bar_kv, kv_bytes);
+        }
+        // ---- fixed-point records and displacement test, to every rank
+        uint4 cur = make_uint4(0, 0, 0, 0);
+        if (warp * 32 < max(np, 1)) {
+            int moved = 0, bad = 0;
+            if (owner) {
+                cur = make_uint4(to_fixed(pos.x, S.fx_hi, S.fx_lo),
+                                 to_fixed(pos.y, S.fx_hi, S.fx_lo),
+                                 to_fixed(pos.z, S.fx_hi, S.fx_lo), __float_as_uint(pos.w));
+                const float dx = (float)(int32_t)(cur.x - ref.x) * S.L_over_2_32;
+                const float dy = (float)(int32_t)(cur.y - ref.y) * S.L_over_2_32;
+                const float dz = (float)(int32_t)(cur.z - ref.z) * S.L_over_2_32;
+                moved = (s == 0 && stale) || fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > S.f_half_skin2;
+                const uint32_t dst = local_addr(R_ + o);
+                for (int t = 0; t < cs; ++t) send(remote(dst, t), cur, remote(bar_rec, t));
+                bad = !(isfinite(pos.x) && isfinite(pos.y) && isfinite(pos.z) && isfinite(pos.w));
+                if (bad) atomicOr(a.err, kErrNonfinite);
+            }
+            moved = __any_sync(0xffffffffu, moved);
+            bad = __any_sync(0xffffffffu, bad);
+            if (lane < cs)
+                send(remote(local_addr(&s_msg[par][rank * kSmallOwnWarps + warp]), lane),
+                     make_uint4((uint32_t)moved, (uint32_t)bad, (uint32_t)k2w, (uint32_t)(k2w >> 32)),
+                     remote(bar_rec, lane));
+        }
+        // ---- this warp's wave vectors and the thermostat's noise meanwhile
+        int4 m0 = make_int4(0, 0, 0, 0), m1 = m0;
+        if (sums) {
+            warp_sample2(S, table, k0 + 2 * pr, k0 + min(2 * pr + 1, nk - 1), step, a.err, m0, m1);
+            if (sub == 0 && lane == 0) {
+                s_m[2 * pr] = m0;
+                s_m[2 * pr + 1] = m1;
+            }
+        }
+        MdNoise z{0.f, 0.f, 0.f, false};
+        if (owner && !nhm) z = md_noise(S, step, o);
+        if (!late && !bar_wait(bar_rec, par)) late = true;
+        bool rebuild = false;
+        for (int t = lane; t < kSmallMaxCs * kSmallOwnWarps; t += 32)
+        {
+            const uint4 v = s_msg[par][t];
+            rebuild |= v.x != 0u;
+            bad_seen |= v.y != 0u;
+        }
+        rebuild = __any_sync(0xffffffffu, rebuild);
+        bad_seen = __any_sync(0xffffffffu, bad_seen);
+        // ---- structure factors of two wave vectors over a share of all records
+        if (sums) {
+            float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
+#pragma unroll 2
+            for (int j = sub * 32 + lane; j < n; j += wpp * 32) {
+                const uint4 r = R_[j];
+                const float q = __uint_as_float(r.w);
+                float sn, cn;
+                __sincosf((float)(int32_t)((uint32_t)m0.x * r.x + (uint32_t)m0.y * r.y +
+                                           (uint32_t)m0.z * r.z) * kTurn, &sn, &cn);
+                re0 = fmaf(q, cn, re0);
+                im0 = fmaf(q, sn, im0);
+                __sincosf((float)(int32_t)((uint32_t)m1.x * r.x + (uint32_t)m1.y * r.y +
+                                           (uint32_t)m1.z * r.z) * kTurn, &sn, &cn);
+                re1 = fmaf(q, cn, re1);
+                im1 = fmaf(q, sn, im1);
+            }
+            // the four sums over the warp, halving the values with the lanes:
+            // lanes 0, 8, 16, 24 end with re0, im0, re1, im1
+            const bool up = lane & 16, up2 = lane & 8;
+            const float a0 = (up ? re1 : re0) + __shfl_xor_sync(0xffffffffu, up ? re0 : re1, 16);
+            const float a1 = (up ? im1 : im0) + __shfl_xor_sync(0xffffffffu, up ? im0 : im1, 16);
+            float v = (up2 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up2 ? a0 : a1, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 4);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            if ((lane & 7) == 0) s_part[sub * kp + pr][lane >> 3] = v;
+        }
+        __syncthreads();
+        if (tid < nk) {
+            float2 re = make_float2(0.f, 0.f), im = re;
+            for (int u = 0; u < wpp; ++u) {
+                const float* v = &s_part[u * kp + (tid >> 1)][(tid & 1) * 2];
+                const float2 x = two_sum(re.x, v[0]), y = two_sum(im.x, v[1]);
+                re = make_float2(x.x, re.y + x.y);
+                im = make_float2(y.x, im.y + y.y);
+            }
+            // c = coefficient scale / |m|^2 as a float pair (|m|^2 is exact)
+            const int4 m = s_m[tid];
+            const float m2 = (float)(m.x * m.x + m.y * m.y + m.z * m.z);
+            const float ch = a.kscale_hi / m2;
+            const float cl = (fmaf(-ch, m2, a.kscale_hi) + a.kscale_lo) / m2;
+            const float A = pair_mul(ch, cl, im), B = pair_mul(ch, cl, re), Rk = hypotf(A, B);
+            const float turns = atan2f(A, B) * 0.15915494309189535f;
+            const uint4 x = make_uint4(0u - (uint32_t)m.x, 0u - (uint32_t)m.y, 0u - (uint32_t)m.z,
+                                       (uint32_t)(long long)llrintf(turns * 4294967296.0f));
+            const uint4 y = make_uint4(__float_as_uint(Rk * (float)m.x),
+                                       __float_as_uint(Rk * (float)m.y),
+                                       __float_as_uint(Rk * (float)m.z), __float_as_uint(Rk));
+            const uint32_t dst = local_addr(kv + k0 + tid);
+            for (int t = 0; t < cs; ++t) {
+                const uint32_t d = remote(dst, t), b = remote(bar_kv, t);
+                send(d, x, b);
+                send(d + 16u * (uint32_t)P, y, b);
+            }
+        }
+        if (nk == 0 && tid == 0)
+            for (int t = 0; t < cs; ++t)
+                send(remote(local_addr(&s_token), t), make_uint4(0u, 0u, 0u, 0u),
+                     remote(bar_kv, t));
+        if (nhm && owner) {
+            // the friction, from the kinetic sums the messages carried
+            unsigned long long k2 = 0ull;
+            for (int t = 0; t < kSmallMaxCs * kSmallOwnWarps; ++t) {
+                const uint4 v = s_msg[par][t];
+                k2 += (unsigned long long)v.z | ((unsigned long long)v.w << 32);
+            }
+            if (s > 0) nh.k2 = k2;
+            if (!nh.first) nh.xi += S.nh_rate * ((double)nh.k2 * 0x1p-32 - 3.0 * (double)S.n);
+            nh.first = 0;
+            const double hx = 0.5 * nh.xi * S.dt;
+            nh.a = 1.0 - hx;
+            nh.b = 1.0 / (1.0 + hx);
+            nh.f_va = (float)(nh.a * nh.b);
+            nh.f_vf = (float)(S.dt_over_m * nh.b);
+        }
+        // ---- the list, rebuilt if any particle moved beyond half the skin
+        if (rebuild) {
+            const uint4 si = R_[min(pn, n - 1)];
+            cnt = 0;
+            const int gl = lane - l;                // first lane of the particle's group
+            for (int jb = 0; jb < n; jb += R) {
+                const int j = jb + l;
+                bool near = false;
+                if (pairs && j < n) {
+                    const uint4 sj = R_[j];
+                    const float dx = (float)(int32_t)(sj.x - si.x) * S.L_over_2_32;
+                    const float dy = (float)(int32_t)(sj.y - si.y) * S.L_over_2_32;
+                    const float dz = (float)(int32_t)(sj.z - si.z) * S.L_over_2_32;
+                    near = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < S.f_list_cut2 && j != pn;
+                }
+                const uint32_t bits = (__ballot_sync(0xffffffffu, near) >> gl) &
+                                      (R == 32 ? 0xffffffffu : (1u << (R & 31)) - 1u);
+                const int slot = cnt + __popc(bits & ((1u << l) - 1u));
+                if (near && slot < a.cap) {
+                    list[p * a.cap + slot] = (uint16_t)j;
+                    a.nbr[(size_t)slot * a.stride + pn] = j;
+                }
+                cnt += __popc(bits);
+            }
+            if (pairs && l == 0) {
+                a.ncnt[pn] = min(cnt, a.cap);
+                // (non-finite input has its own error; its neighbour counts mean nothing)
+                if (cnt > a.cap && !bad_seen) atomicOr(a.err, kErrList);
+                atomicMax(a.stats + 1, (unsigned long long)cnt);
+            }
+            cnt = min(cnt, a.cap);
+            if (owner) {
+                ref = cur;
+                a.sref[o] = cur;
+                a.perm[o] = o;
+                a.iperm[o] = o;
+            }
+            if (rank == 0 && tid == 0) atomicAdd(a.stats, 1ull);
+            __syncwarp();
+        }
+        // ---- real-space pairs
+        if (pairs) {
+            PairAcc acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            const uint4 si = R_[pn];
+            const float lbqi = kc.lB * __uint_as_float(si.w);
+            for (int k = l; k < cnt; k += R)
+                pair_fixed(si, R_[list[p * a.cap + k]], S.L_over_2_32, lbqi, kc, acc);
+            part[l * L.np + p] = make_float4(acc.fx, acc.fy, acc.fz, 0.f);
+        }
+        // ---- Fourier force: a lane per particle, a warp per share of the wave vectors
+        if (!late && !bar_wait(bar_kv, par)) late = true;
+        const int pf = pg * 32 + lane;
+        if (ks < L.nks && pf < np) {
+            const uint4 si = R_[first + pf];
+            float fx = 0.f, fy = 0.f, fz = 0.f;
+#pragma unroll 4
+            for (int k = ks; k < P; k += L.nks) {
+                const uint4 A = kv[k], B = kv[P + k];
+                const uint32_t d = A.w + A.x * si.x + A.y * si.y + A.z * si.z;
+                const float sn = __sinf((float)(int32_t)d * kTurn);
+                fx = fmaf(sn, __uint_as_float(B.x), fx);
+                fy = fmaf(sn, __uint_as_float(B.y), fy);
+                fz = fmaf(sn, __uint_as_float(B.z), fz);
+            }
+            const float sc = -__uint_as_float(si.w) * (float)(2.0 * M_PI) * S.f_invL;
+            part[(R + ks) * L.np + pf] = make_float4(sc * fx, sc * fy, sc * fz, 0.f);
+        }
+        __syncthreads();
+        // ---- total force, thermostat and drift
+        if (warp * 32 < np) {
+            unsigned long long k2 = 0ull;
+            if (owner) {
+                float fx = 0.f, fy = 0.f, fz = 0.f;
+#pragma unroll 8
+                for (int u = 0; u < R + L.nks; ++u) {
+                    const float4 v = part[u * L.np + tid];
+                    fx += v.x;
+                    fy += v.y;
+                    fz += v.z;
+                }
+                if (a.F_out && s == a.nsteps - 1) a.F_out[o] = make_float4(fx, fy, fz, 0.f);
+                if (nhm) k2 = nose_hoover_apply(S, nh.f_va, nh.f_vf, fx, fy, fz, vel, pos);
+                else md_apply(S, z, fx, fy, fz, vel, pos);
+            }
+            if (nhm) {
+                for (int d = 16; d > 0; d >>= 1) k2 += __shfl_xor_sync(0xffffffffu, k2, d);
+                k2w = k2;
+            }
+        }
+    }
+    if (owner) {
+        a.pos[o] = pos;
+        a.vel[o] = vel;
+    }
+    if (late && lane == 0) atomicOr(a.err, kErrWait);
+    // the last step's kinetic sums, for the friction of the next call (slots
+    // of the parity that no rank reads any more)
+    if (nhm && warp * 32 < np && lane == 0) {
+        const uint32_t d = remote(
+            local_addr(&s_msg[a.nsteps & 1][rank * kSmallOwnWarps + warp]), 0);
+        asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(d + 8u),
+                     "r"((uint32_t)k2w), "r"((uint32_t)(k2w >> 32))
+                     : "memory");
+    }
+    if (a.done_host) __threadfence_system();        // this thread's outputs
+    // orders those stores, and keeps every rank's shared memory alive until all are done
+    cluster_sync();
+    if (rank == 0 && tid == 0) {
+        if (nhm) {
+            unsigned long long k2 = 0ull;
+            for (int t = 0; t < kSmallMaxCs * kSmallOwnWarps; ++t) {
+                const uint4 v = s_msg[a.nsteps & 1][t];
+                k2 += (unsigned long long)v.z | ((unsigned long long)v.w << 32);
+            }
+            nh.k2 = k2;
+            *a.nh = nh;
+        }
+        *a.list_flag = 0;
+        *a.step_dev = step0 + (uint64_t)a.nsteps;
+        if (a.done_host) {
+            __threadfence_system();
+            *(volatile int*)a.err_host = *(const volatile int*)a.err;
+            __threadfence_system();
+            *(volatile unsigned long long*)a.done_host = step0 + (uint64_t)a.nsteps;
+        }
+    }
+}
+
+// Lanes per particle: as many as 1024 threads allow.
+static int small_lanes(int n, int cs) {
+    const int np = (n + cs - 1) / cs;
+    int r = 32;
+    while (r > 4 && np * r > kSmallThreads) r >>= 1;
+    return r;
+}
+
+template <int R>
+static bool small_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, cudaStream_t st,
+                         int cs, size_t smem) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(cs);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaFuncSetAttribute(k_small_md<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem) == cudaSuccess &&
+           cudaFuncSetAttribute(k_small_md<R>, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                1) == cudaSuccess;
+}
+
+template <int R>
+static bool small_fits(int cs, size_t smem) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    int clusters = 0;
+    const bool ok = small_config<R>(cfg, attr, nullptr, cs, smem) &&
+                    cudaOccupancyMaxActiveClusters(&clusters, k_small_md<R>, &cfg) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    return ok && clusters >= 1;
+}
+
+// Whether a system of n particles, P wave vectors, half width M and cap list
+// entries per particle runs as one cluster: it fits in the blocks' shared memory and the GPU can place the
+// cluster.  cs: blocks of the cluster.
+bool small_md_fits(int n, int P, int M, int cap, int cs) {
+    const int R = small_lanes(n, cs);
+    if (n < 1 || (n + cs - 1) / cs * R > kSmallThreads) return false;
+    if ((P + cs - 1) / cs > kSmallMaxKc || cs > kSmallMaxCs || M > 2000) return false;
+    if ((n + cs - 1) / cs > 32 * kSmallOwnWarps) return false;
+    const size_t smem = small_layout(n, P, M, cap, cs, R).end;
+    if (smem > 216 * 1024) return false;
+    switch (R) {
+        case 4: return small_fits<4>(cs, smem);
+        case 8: return small_fits<8>(cs, smem);
+        case 16: return small_fits<16>(cs, smem);
+        default: return small_fits<32>(cs, smem);
+    }
+}
+
+template <int R>
+static cudaError_t small_launch(cudaStream_t st, const SmallArgs& a, size_t smem) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    if (!small_config<R>(cfg, attr, st, a.cs, smem)) return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, k_small_md<R>, a);
+}
+
+cudaError_t launch_small_md(cudaStream_t st, const SmallArgs& a) {
+    const int R = small_lanes(a.n, a.cs);
+    const size_t smem = small_layout(a.n, a.S.P, a.S.M, a.cap, a.cs, R).end;
+    switch (R) {
+        case 4: return small_launch<4>(st, a, smem);
+        case 8: return small_launch<8>(st, a, smem);
+        case 16: return small_launch<16>(st, a, smem);
+        default: return small_launch<32>(st, a, smem);
+    }
+}
+
+}  // namespace rbe
