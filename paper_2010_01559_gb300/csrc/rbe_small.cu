@@ -9,18 +9,16 @@
 // receiving block (no cluster-wide barrier in the loop):
 //
 //   records    rank c owns n/16 particles (position, velocity and build record
-//              stay in registers for the whole call); each owner thread sends
-//              its fixed-point record to all ranks
-//   k-batch    every warp draws the two wave vectors it will sum (while the
-//              records are under way), then sums their structure factors over
-//              a share of all n records; rank c holds P/16 wave vectors, so
-//              no sum crosses blocks.  A thread per wave vector forms the force
+//              stay in registers of one thread each for the whole call); the
+//              block sends their fixed-point records to all ranks
+//   k-batch    rank c holds P/16 wave vectors, drawn while the records are
+//              under way; each warp sums the structure factors of two of them
+//              over a share of all n records (no sum crosses blocks); then a
+//              warp per wave vector adds the shares, forms the force
 //              coefficient and sends it to all ranks
 //   pairs      meanwhile R lanes per owned particle walk its neighbour list,
-//              then (coefficients in) a lane per particle and a warp per share
-//              of the wave vectors add the Fourier force; one thread per
-//              particle sums the partials in a fixed order and applies the
-//              thermostat.
+//              then (coefficients in) its wave vectors; the particle's thread
+//              applies the thermostat.
 //
 // A block that runs ahead cannot overwrite what another still reads, nor count
 // on a barrier phase that has not begun: to send the records of step s + 1 it
@@ -28,10 +26,11 @@
 // records (a rank without particles or wave vectors sends a message all the
 // same), and the records alternate between two buffers.
 //
-// FP64 instructions are kept out of the loop (their latency on this part is
-// over a hundred cycles; the first form of this kernel, which summed a wave
-// vector's partials and its coefficient in FP64, spent 3500 to 10700 cycles a
-// step there): partial sums are added as float pairs, and the coefficient
+// Serial chains are what counts.  FP64 instructions are kept out of the loop
+// (their latency on this part is over a hundred cycles; summing a wave vector's
+// shares and its coefficient in FP64 took 3500 to 10700 cycles a step); one
+// thread sending to 16 ranks in turn or adding 32 partial forces took 1200 to
+// 4000, which a thread per message and shuffles take to a few hundred.  Partial sums are added as float pairs, and the coefficient
 // (lB S/P 4 pi / V) / k^2 is a float-pair constant over the integer |m|^2.
 //
 // Neighbour list: the owned particles' neighbours within r_c + skin as 16-bit
@@ -116,28 +115,25 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
 constexpr float kTurn = 1.4629180792671596e-09f;                     // 2 pi / 2^32
 constexpr int kSmallMaxKc = 2 * kSmallWarps;                         // wave vectors per rank
 constexpr int kSmallMaxCs = 16;                                      // blocks per cluster
-constexpr int kSmallOwnWarps = 8;                                    // owner warps per rank
 
 // Shared-memory layout of a block (byte offsets, 16-byte aligned).
 struct SmallLayout {
-    int np, kc, tab, npg, nks;   // owned particles, wave vectors per rank, table entries,
-                                 // particle groups of the Fourier force and warps on each
-    size_t rec, kv, part, list, table, end;
+    int np, kc, tab;             // owned particles, wave vectors per rank, table entries
+    size_t rec, kv, own, frc, list, table, end;
 };
 
 __host__ __device__ inline size_t small_align(size_t x) { return (x + 15) & ~size_t(15); }
 
-__host__ __device__ inline SmallLayout small_layout(int n, int P, int M, int cap, int cs, int R) {
+__host__ __device__ inline SmallLayout small_layout(int n, int P, int M, int cap, int cs) {
     SmallLayout L;
     L.np = (n + cs - 1) / cs;
     L.kc = (P + cs - 1) / cs;
     L.tab = 2 * M + 1;
-    L.npg = (L.np + 31) / 32;
-    L.nks = kSmallWarps / L.npg;
     L.rec = 0;                                                       // uint4 [2][n]
     L.kv = L.rec + 32 * (size_t)n;                                   // uint4 [2][P]
-    L.part = L.kv + 32 * (size_t)P;                                  // float4 [R + nks][np]
-    L.list = L.part + 16 * (size_t)(R + L.nks) * L.np;               // u16 [np][cap]
+    L.own = L.kv + 32 * (size_t)P;                                   // uint4 [np]
+    L.frc = L.own + 16 * (size_t)L.np;                               // float4 [np]
+    L.list = L.frc + 16 * (size_t)L.np;                              // u16 [np][cap]
     L.table = L.list + small_align(2 * (size_t)L.np * cap);          // u32 [2M + 1]
     L.end = L.table + small_align(4 * (size_t)L.tab);
     return L;
@@ -190,17 +186,20 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     __shared__ float s_part[kSmallWarps][4];                    // structure-factor partials
     __shared__ int4 s_m[kSmallMaxKc];                           // this rank's wave vectors
     __shared__ uint4 s_token;                                   // from ranks without wave vectors
-    // from every rank's owner warps (at least its first warp): (particle moved,
-    // non-finite input, Nose-Hoover kinetic sum), by step parity
-    __shared__ uint4 s_msg[2][kSmallMaxCs * kSmallOwnWarps];
+    // from every rank, by step parity: (flags, 0, Nose-Hoover kinetic sum); flags:
+    // 1 a particle moved beyond half the skin, 2 non-finite input
+    __shared__ uint4 s_msg[2][kSmallMaxCs];
+    __shared__ unsigned long long s_k2;                         // this rank's kinetic sum
+    __shared__ int s_flags[2];                                  // its flags, by step parity
     const SysDev& S = a.S;
     const uint32_t rank = cluster_rank();
     const int cs = a.cs, n = a.n, P = S.P, tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
-    const SmallLayout L = small_layout(n, P, S.M, a.cap, cs, R);
+    const SmallLayout L = small_layout(n, P, S.M, a.cap, cs);
     uint4* rec = (uint4*)(smem + L.rec);
     uint4* kv = (uint4*)(smem + L.kv);              // [l]: -m and phi; [P + l]: R m and R
-    float4* part = (float4*)(smem + L.part);
+    uint4* own = (uint4*)(smem + L.own);            // owned records, to be sent
+    float4* frc = (float4*)(smem + L.frc);          // owned particles' total forces
     uint16_t* list = (uint16_t*)(smem + L.list);
     uint32_t* table = (uint32_t*)(smem + L.table);
     const int first = (int)rank * L.np;
@@ -224,8 +223,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         ref = a.sref[o];
     }
     for (int j = tid; j < L.tab; j += kSmallThreads) table[j] = (uint32_t)a.table[j];
-    for (int j = tid; j < 2 * kSmallMaxCs * kSmallOwnWarps; j += kSmallThreads)
-        (&s_msg[0][0])[j] = make_uint4(0, 0, 0, 0);
+    if (tid < 2 * kSmallMaxCs) (&s_msg[0][0])[tid] = make_uint4(0, 0, 0, 0);
     int cnt = 0;                                    // list entries of particle p
     if (pairs && !stale) {
         // the handle's list, in sorted indices of its last build
@@ -237,6 +235,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     NhState nh{};
     if (nhm) nh = *a.nh;
     if (tid == 0) {
+        s_k2 = 0ull;
+        s_flags[0] = s_flags[1] = 0;
         bar_init(bar_rec);
         bar_init(bar_kv);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -259,14 +259,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     const int wpp = kp > 0 ? kSmallWarps / kp : 0;
     const bool sums = warp < kp * wpp;              // this warp sums pair pr, share sub of wpp
     const int pr = sums ? warp % kp : 0, sub = sums ? warp / kp : 0;
-    const int pg = warp % L.npg, ks = warp / L.npg; // Fourier force: particle group, k share
-    // bytes a block receives per step: all records and all owner warps' messages
-    const int nfull = n / L.np, nrest = n - nfull * L.np;
-    const int nsend = nfull + (nrest > 0 ? 1 : 0);  // ranks with particles
-    const uint32_t rec_bytes =
-        16u * (uint32_t)(n + nfull * ((L.np + 31) / 32) + (nrest + 31) / 32 + (cs - nsend));
+    // bytes a block receives per step: all records and a message from every rank
+    const uint32_t rec_bytes = 16u * (uint32_t)(n + cs);
     const uint32_t kv_bytes = 32u * (uint32_t)P + 16u * (uint32_t)(cs - (P + L.kc - 1) / L.kc);
-    unsigned long long k2w = 0ull;                  // this owner warp's kinetic sum
     bool bad_seen = false;                          // some position or charge was not finite
     bool late = false;                              // a wait gave up: no more waiting
 
@@ -280,51 +275,56 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         }
         // ---- fixed-point records and displacement test, to every rank
         uint4 cur = make_uint4(0, 0, 0, 0);
-        if (warp * 32 < max(np, 1)) {
-            int moved = 0, bad = 0;
-            if (owner) {
-                cur = make_uint4(to_fixed(pos.x, S.fx_hi, S.fx_lo),
-                                 to_fixed(pos.y, S.fx_hi, S.fx_lo),
-                                 to_fixed(pos.z, S.fx_hi, S.fx_lo), __float_as_uint(pos.w));
-                const float dx = (float)(int32_t)(cur.x - ref.x) * S.L_over_2_32;
-                const float dy = (float)(int32_t)(cur.y - ref.y) * S.L_over_2_32;
-                const float dz = (float)(int32_t)(cur.z - ref.z) * S.L_over_2_32;
-                moved = (s == 0 && stale) || fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > S.f_half_skin2;
-                const uint32_t dst = local_addr(R_ + o);
-                for (int t = 0; t < cs; ++t) send(remote(dst, t), cur, remote(bar_rec, t));
-                bad = !(isfinite(pos.x) && isfinite(pos.y) && isfinite(pos.z) && isfinite(pos.w));
-                if (bad) atomicOr(a.err, kErrNonfinite);
+        int flags = 0;
+        if (owner) {
+            cur = make_uint4(to_fixed(pos.x, S.fx_hi, S.fx_lo), to_fixed(pos.y, S.fx_hi, S.fx_lo),
+                             to_fixed(pos.z, S.fx_hi, S.fx_lo), __float_as_uint(pos.w));
+            own[tid] = cur;
+            const float dx = (float)(int32_t)(cur.x - ref.x) * S.L_over_2_32;
+            const float dy = (float)(int32_t)(cur.y - ref.y) * S.L_over_2_32;
+            const float dz = (float)(int32_t)(cur.z - ref.z) * S.L_over_2_32;
+            if ((s == 0 && stale) || fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > S.f_half_skin2)
+                flags = 1;
+            if (!(isfinite(pos.x) && isfinite(pos.y) && isfinite(pos.z) && isfinite(pos.w))) {
+                flags |= 2;
+                atomicOr(a.err, kErrNonfinite);
             }
-            moved = __any_sync(0xffffffffu, moved);
-            bad = __any_sync(0xffffffffu, bad);
+        }
+        if (flags) atomicOr(&s_flags[par], flags);
+        __syncthreads();                            // own, s_flags, s_k2
+        for (int e = tid; e < np * cs; e += kSmallThreads) {
+            const int t = e / np, q = e - t * np;
+            send(remote(local_addr(R_ + first + q), t), own[q], remote(bar_rec, t));
+        }
+        if (warp == kSmallWarps / 2) {
+            // one message to every rank, from a warp of the middle (the first
+            // ones own particles, the last ones draw wave vectors)
+            const unsigned long long k2 = s_k2;
             if (lane < cs)
-                send(remote(local_addr(&s_msg[par][rank * kSmallOwnWarps + warp]), lane),
-                     make_uint4((uint32_t)moved, (uint32_t)bad, (uint32_t)k2w, (uint32_t)(k2w >> 32)),
+                send(remote(local_addr(&s_msg[par][rank]), lane),
+                     make_uint4((uint32_t)s_flags[par], 0u, (uint32_t)k2, (uint32_t)(k2 >> 32)),
                      remote(bar_rec, lane));
         }
-        // ---- this warp's wave vectors and the thermostat's noise meanwhile
-        int4 m0 = make_int4(0, 0, 0, 0), m1 = m0;
-        if (sums) {
-            warp_sample2(S, table, k0 + 2 * pr, k0 + min(2 * pr + 1, nk - 1), step, a.err, m0, m1);
-            if (sub == 0 && lane == 0) {
-                s_m[2 * pr] = m0;
-                s_m[2 * pr + 1] = m1;
+        // ---- this rank's wave vectors and the thermostat's noise meanwhile
+        if (kSmallWarps - 1 - warp < kp) {
+            const int q = 2 * (kSmallWarps - 1 - warp);
+            int4 m0, m1;
+            warp_sample2(S, table, k0 + q, k0 + min(q + 1, nk - 1), step, a.err, m0, m1);
+            if (lane == 0) {
+                s_m[q] = m0;
+                s_m[q + 1] = m1;
             }
         }
         MdNoise z{0.f, 0.f, 0.f, false};
         if (owner && !nhm) z = md_noise(S, step, o);
         if (!late && !bar_wait(bar_rec, par)) late = true;
-        bool rebuild = false;
-        for (int t = lane; t < kSmallMaxCs * kSmallOwnWarps; t += 32)
-        {
-            const uint4 v = s_msg[par][t];
-            rebuild |= v.x != 0u;
-            bad_seen |= v.y != 0u;
-        }
-        rebuild = __any_sync(0xffffffffu, rebuild);
-        bad_seen = __any_sync(0xffffffffu, bad_seen);
+        const uint32_t seen = __reduce_or_sync(0xffffffffu, lane < cs ? s_msg[par][lane].x : 0u);
+        const bool rebuild = (seen & 1u) != 0u;
+        bad_seen |= (seen & 2u) != 0u;
+        __syncthreads();                            // s_m
         // ---- structure factors of two wave vectors over a share of all records
         if (sums) {
+            const int4 m0 = s_m[2 * pr], m1 = s_m[2 * pr + 1];
             float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
 #pragma unroll 2
             for (int j = sub * 32 + lane; j < n; j += wpp * 32) {
@@ -352,16 +352,27 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             if ((lane & 7) == 0) s_part[sub * kp + pr][lane >> 3] = v;
         }
         __syncthreads();
-        if (tid < nk) {
+        if (tid == 0) {                             // (read above, written after the next barrier)
+            s_k2 = 0ull;
+            s_flags[par] = 0;
+        }
+        // ---- a warp per wave vector: its force coefficient, to every rank
+        for (int q = kSmallWarps - 1 - warp; q < nk; q += kSmallWarps) {
             float2 re = make_float2(0.f, 0.f), im = re;
-            for (int u = 0; u < wpp; ++u) {
-                const float* v = &s_part[u * kp + (tid >> 1)][(tid & 1) * 2];
-                const float2 x = two_sum(re.x, v[0]), y = two_sum(im.x, v[1]);
-                re = make_float2(x.x, re.y + x.y);
-                im = make_float2(y.x, im.y + y.y);
+            if (lane < wpp) {
+                const float* v = &s_part[lane * kp + (q >> 1)][(q & 1) * 2];
+                re.x = v[0];
+                im.x = v[1];
+            }
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) {
+                const float2 x = two_sum(re.x, __shfl_xor_sync(0xffffffffu, re.x, d));
+                re = make_float2(x.x, re.y + __shfl_xor_sync(0xffffffffu, re.y, d) + x.y);
+                const float2 y = two_sum(im.x, __shfl_xor_sync(0xffffffffu, im.x, d));
+                im = make_float2(y.x, im.y + __shfl_xor_sync(0xffffffffu, im.y, d) + y.y);
             }
             // c = coefficient scale / |m|^2 as a float pair (|m|^2 is exact)
-            const int4 m = s_m[tid];
+            const int4 m = s_m[q];
             const float m2 = (float)(m.x * m.x + m.y * m.y + m.z * m.z);
             const float ch = a.kscale_hi / m2;
             const float cl = (fmaf(-ch, m2, a.kscale_hi) + a.kscale_lo) / m2;
@@ -372,12 +383,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             const uint4 y = make_uint4(__float_as_uint(Rk * (float)m.x),
                                        __float_as_uint(Rk * (float)m.y),
                                        __float_as_uint(Rk * (float)m.z), __float_as_uint(Rk));
-            const uint32_t dst = local_addr(kv + k0 + tid);
-            for (int t = 0; t < cs; ++t) {
-                const uint32_t d = remote(dst, t), b = remote(bar_kv, t);
-                send(d, x, b);
-                send(d + 16u * (uint32_t)P, y, b);
-            }
+            const int t = lane & 15;                // lanes 0-15 send x, 16-31 send y
+            if (t < cs)
+                send(remote(local_addr(kv + (lane < 16 ? 0 : P) + k0 + q), t), lane < 16 ? x : y,
+                     remote(bar_kv, t));
         }
         if (nk == 0 && tid == 0)
             for (int t = 0; t < cs; ++t)
@@ -386,7 +395,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         if (nhm && owner) {
             // the friction, from the kinetic sums the messages carried
             unsigned long long k2 = 0ull;
-            for (int t = 0; t < kSmallMaxCs * kSmallOwnWarps; ++t) {
+            for (int t = 0; t < cs; ++t) {
                 const uint4 v = s_msg[par][t];
                 k2 += (unsigned long long)v.z | ((unsigned long long)v.w << 32);
             }
@@ -403,25 +412,33 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         if (rebuild) {
             const uint4 si = R_[min(pn, n - 1)];
             cnt = 0;
-            const int gl = lane - l;                // first lane of the particle's group
-            for (int jb = 0; jb < n; jb += R) {
-                const int j = jb + l;
-                bool near = false;
-                if (pairs && j < n) {
-                    const uint4 sj = R_[j];
-                    const float dx = (float)(int32_t)(sj.x - si.x) * S.L_over_2_32;
-                    const float dy = (float)(int32_t)(sj.y - si.y) * S.L_over_2_32;
-                    const float dz = (float)(int32_t)(sj.z - si.z) * S.L_over_2_32;
-                    near = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < S.f_list_cut2 && j != pn;
+            // 32 candidates per lane at a time, then the lanes' hits one after another
+            for (int jb = l; jb < n + l; jb += 32 * R) {
+                uint32_t bits = 0;
+                if (pairs)
+                    for (int b = 0, j = jb; b < 32 && j < n; ++b, j += R) {
+                        const uint4 sj = R_[j];
+                        const float dx = (float)(int32_t)(sj.x - si.x) * S.L_over_2_32;
+                        const float dy = (float)(int32_t)(sj.y - si.y) * S.L_over_2_32;
+                        const float dz = (float)(int32_t)(sj.z - si.z) * S.L_over_2_32;
+                        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                        if (r2 < S.f_list_cut2 && j != pn) bits |= 1u << b;
+                    }
+                int incl = __popc(bits), slot = cnt - incl;
+#pragma unroll
+                for (int d = 1; d < R; d <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, d, R);
+                    if (l >= d) incl += y;
                 }
-                const uint32_t bits = (__ballot_sync(0xffffffffu, near) >> gl) &
-                                      (R == 32 ? 0xffffffffu : (1u << (R & 31)) - 1u);
-                const int slot = cnt + __popc(bits & ((1u << l) - 1u));
-                if (near && slot < a.cap) {
-                    list[p * a.cap + slot] = (uint16_t)j;
-                    a.nbr[(size_t)slot * a.stride + pn] = j;
+                slot += incl;
+                cnt += __shfl_sync(0xffffffffu, incl, R - 1, R);
+                for (; bits; bits &= bits - 1, ++slot) {
+                    const int j = jb + (__ffs(bits) - 1) * R;
+                    if (slot < a.cap) {
+                        list[p * a.cap + slot] = (uint16_t)j;
+                        a.nbr[(size_t)slot * a.stride + pn] = j;
+                    }
                 }
-                cnt += __popc(bits);
             }
             if (pairs && l == 0) {
                 a.ncnt[pn] = min(cnt, a.cap);
@@ -440,52 +457,56 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             __syncwarp();
         }
         // ---- real-space pairs
+        float fx = 0.f, fy = 0.f, fz = 0.f;
+        uint4 si = make_uint4(0, 0, 0, 0);
         if (pairs) {
             PairAcc acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const uint4 si = R_[pn];
+            si = R_[pn];
             const float lbqi = kc.lB * __uint_as_float(si.w);
             for (int k = l; k < cnt; k += R)
                 pair_fixed(si, R_[list[p * a.cap + k]], S.L_over_2_32, lbqi, kc, acc);
-            part[l * L.np + p] = make_float4(acc.fx, acc.fy, acc.fz, 0.f);
+            fx = acc.fx;
+            fy = acc.fy;
+            fz = acc.fz;
         }
-        // ---- Fourier force: a lane per particle, a warp per share of the wave vectors
+        // ---- Fourier force
         if (!late && !bar_wait(bar_kv, par)) late = true;
-        const int pf = pg * 32 + lane;
-        if (ks < L.nks && pf < np) {
-            const uint4 si = R_[first + pf];
-            float fx = 0.f, fy = 0.f, fz = 0.f;
+        if (pairs) {
+            float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll 4
-            for (int k = ks; k < P; k += L.nks) {
+            for (int k = l; k < P; k += R) {
                 const uint4 A = kv[k], B = kv[P + k];
                 const uint32_t d = A.w + A.x * si.x + A.y * si.y + A.z * si.z;
                 const float sn = __sinf((float)(int32_t)d * kTurn);
-                fx = fmaf(sn, __uint_as_float(B.x), fx);
-                fy = fmaf(sn, __uint_as_float(B.y), fy);
-                fz = fmaf(sn, __uint_as_float(B.z), fz);
+                gx = fmaf(sn, __uint_as_float(B.x), gx);
+                gy = fmaf(sn, __uint_as_float(B.y), gy);
+                gz = fmaf(sn, __uint_as_float(B.z), gz);
             }
             const float sc = -__uint_as_float(si.w) * (float)(2.0 * M_PI) * S.f_invL;
-            part[(R + ks) * L.np + pf] = make_float4(sc * fx, sc * fy, sc * fz, 0.f);
+            fx = fmaf(sc, gx, fx);
+            fy = fmaf(sc, gy, fy);
+            fz = fmaf(sc, gz, fz);
         }
+#pragma unroll
+        for (int d = R / 2; d > 0; d >>= 1) {
+            fx += __shfl_down_sync(0xffffffffu, fx, d, R);
+            fy += __shfl_down_sync(0xffffffffu, fy, d, R);
+            fz += __shfl_down_sync(0xffffffffu, fz, d, R);
+        }
+        if (pairs && l == 0) frc[p] = make_float4(fx, fy, fz, 0.f);
         __syncthreads();
-        // ---- total force, thermostat and drift
+        // ---- thermostat and drift
         if (warp * 32 < np) {
             unsigned long long k2 = 0ull;
             if (owner) {
-                float fx = 0.f, fy = 0.f, fz = 0.f;
-#pragma unroll 8
-                for (int u = 0; u < R + L.nks; ++u) {
-                    const float4 v = part[u * L.np + tid];
-                    fx += v.x;
-                    fy += v.y;
-                    fz += v.z;
-                }
-                if (a.F_out && s == a.nsteps - 1) a.F_out[o] = make_float4(fx, fy, fz, 0.f);
-                if (nhm) k2 = nose_hoover_apply(S, nh.f_va, nh.f_vf, fx, fy, fz, vel, pos);
-                else md_apply(S, z, fx, fy, fz, vel, pos);
+                const float4 F = frc[tid];
+                if (a.F_out && s == a.nsteps - 1) a.F_out[o] = F;
+                if (nhm) k2 = nose_hoover_apply(S, nh.f_va, nh.f_vf, F.x, F.y, F.z, vel, pos);
+                else md_apply(S, z, F.x, F.y, F.z, vel, pos);
             }
             if (nhm) {
                 for (int d = 16; d > 0; d >>= 1) k2 += __shfl_xor_sync(0xffffffffu, k2, d);
-                k2w = k2;
+                if (lane == 0) atomicAdd(&s_k2, k2);
             }
         }
     }
@@ -496,11 +517,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     if (late && lane == 0) atomicOr(a.err, kErrWait);
     // the last step's kinetic sums, for the friction of the next call (slots
     // of the parity that no rank reads any more)
-    if (nhm && warp * 32 < np && lane == 0) {
-        const uint32_t d = remote(
-            local_addr(&s_msg[a.nsteps & 1][rank * kSmallOwnWarps + warp]), 0);
+    __syncthreads();
+    if (nhm && tid == 0) {
+        const uint32_t d = remote(local_addr(&s_msg[a.nsteps & 1][rank]), 0);
         asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(d + 8u),
-                     "r"((uint32_t)k2w), "r"((uint32_t)(k2w >> 32))
+                     "r"((uint32_t)s_k2), "r"((uint32_t)(s_k2 >> 32))
                      : "memory");
     }
     if (a.done_host) __threadfence_system();        // this thread's outputs
@@ -509,7 +530,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     if (rank == 0 && tid == 0) {
         if (nhm) {
             unsigned long long k2 = 0ull;
-            for (int t = 0; t < kSmallMaxCs * kSmallOwnWarps; ++t) {
+            for (int t = 0; t < cs; ++t) {
                 const uint4 v = s_msg[a.nsteps & 1][t];
                 k2 += (unsigned long long)v.z | ((unsigned long long)v.w << 32);
             }
@@ -573,8 +594,7 @@ bool small_md_fits(int n, int P, int M, int cap, int cs) {
     const int R = small_lanes(n, cs);
     if (n < 1 || (n + cs - 1) / cs * R > kSmallThreads) return false;
     if ((P + cs - 1) / cs > kSmallMaxKc || cs > kSmallMaxCs || M > 2000) return false;
-    if ((n + cs - 1) / cs > 32 * kSmallOwnWarps) return false;
-    const size_t smem = small_layout(n, P, M, cap, cs, R).end;
+    const size_t smem = small_layout(n, P, M, cap, cs).end;
     if (smem > 216 * 1024) return false;
     switch (R) {
         case 4: return small_fits<4>(cs, smem);
@@ -594,7 +614,7 @@ static cudaError_t small_launch(cudaStream_t st, const SmallArgs& a, size_t smem
 
 cudaError_t launch_small_md(cudaStream_t st, const SmallArgs& a) {
     const int R = small_lanes(a.n, a.cs);
-    const size_t smem = small_layout(a.n, a.S.P, a.S.M, a.cap, a.cs, R).end;
+    const size_t smem = small_layout(a.n, a.S.P, a.S.M, a.cap, a.cs).end;
     switch (R) {
         case 4: return small_launch<4>(st, a, smem);
         case 8: return small_launch<8>(st, a, smem);
