@@ -1380,7 +1380,7 @@ struct HostIO {
 // GPU, so its step grows with n P where the separate kernels' hardly does:
 // SMALL_RULE
 constexpr int kSmallStepsPerLaunch = 512;
-constexpr long long kSmallMaxNP = 1000000;
+constexpr long long kSmallMaxNP = 500000;
 
 bool small_steps(rbe_ctx* h, int n) {
     if (h->batch || h->mh || !h->list) return false;

@@ -11,14 +11,16 @@
 //   records    rank c owns n/16 particles (position, velocity and build record
 //              stay in registers of one thread each for the whole call); the
 //              block sends their fixed-point records to all ranks
-//   k-batch    rank c holds P/16 wave vectors, drawn while the records are
-//              under way; each warp sums the structure factors of two of them
+//   k-batch    rank c holds P/16 wave vectors, drawn a step ahead; each warp sums the structure factors of two of them
 //              over a share of all n records (no sum crosses blocks); then a
 //              warp per wave vector adds the shares, forms the force
 //              coefficient and sends it to all ranks
 //   pairs      meanwhile R lanes per owned particle walk its neighbour list,
 //              then (coefficients in) its wave vectors; the particle's thread
-//              applies the thermostat.
+//              applies the thermostat.  (A lane per particle with a warp per
+//              share of the wave vectors reads a coefficient once per warp, but
+//              needs another pass to add the shares: 7.2 against 7.0 us at
+//              N = 1000, P = 100, 12.5 against 13.5 at P = 500.)
 //
 // A block that runs ahead cannot overwrite what another still reads, nor count
 // on a barrier phase that has not begun: to send the records of step s + 1 it
@@ -184,7 +186,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_bar[2];        // records in, coefficients in
     __shared__ float s_part[kSmallWarps][4];                    // structure-factor partials
-    __shared__ int4 s_m[kSmallMaxKc];                           // this rank's wave vectors
+    __shared__ int4 s_m[2][kSmallMaxKc];                        // this rank's wave vectors and
+    __shared__ float2 s_c[2][kSmallMaxKc];                      // (float pairs) coef / rho, by parity
     __shared__ uint4 s_token;                                   // from ranks without wave vectors
     // from every rank, by step parity: (flags, 0, Nose-Hoover kinetic sum); flags:
     // 1 a particle moved beyond half the skin, 2 non-finite input
@@ -262,6 +265,31 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     // bytes a block receives per step: all records and a message from every rank
     const uint32_t rec_bytes = 16u * (uint32_t)(n + cs);
     const uint32_t kv_bytes = 32u * (uint32_t)P + 16u * (uint32_t)(cs - (P + L.kc - 1) / L.kc);
+    // the k-batch of a step: a warp per pair of wave vectors, from warp w0 on
+    auto draw = [&](uint64_t step, int w0) {
+        const int u = warp - w0;
+        if (u < 0 || u >= kp) return;
+        const int q = 2 * u, b = (int)(step & 1);
+        int4 m0, m1;
+        warp_sample2(S, table, k0 + q, k0 + min(q + 1, nk - 1), step, a.err, m0, m1);
+        if (lane < 2) {
+            // c = coefficient scale / |m|^2 as a float pair (|m|^2 is exact)
+            const int4 m = lane ? m1 : m0;
+            const float m2 = (float)(m.x * m.x + m.y * m.y + m.z * m.z);
+            const float ch = a.kscale_hi / m2;
+            s_m[b][q + lane] = m;
+            s_c[b][q + lane] =
+                make_float2(ch, (fmaf(-ch, m2, a.kscale_hi) + a.kscale_lo) / m2);
+        }
+    };
+    // (the warps below those that form the coefficients: the last ones hold few
+    // particles or none)
+    const int w_draw = max(0, kSmallWarps - min(nk, kSmallWarps) - kp);
+    draw(step0, w_draw);
+    // where this thread's first record of every step goes
+    const int q_snd = np > 0 ? tid % np : 0, t_snd = np > 0 ? tid / np : 0;
+    const uint32_t rec_snd = remote(local_addr(rec + first + q_snd), min(t_snd, cs - 1));
+    const uint32_t bar_snd = remote(bar_rec, min(t_snd, cs - 1));
     bool bad_seen = false;                          // some position or charge was not finite
     bool late = false;                              // a wait gave up: no more waiting
 
@@ -292,7 +320,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         }
         if (flags) atomicOr(&s_flags[par], flags);
         __syncthreads();                            // own, s_flags, s_k2
-        for (int e = tid; e < np * cs; e += kSmallThreads) {
+        if (tid < np * cs) send(rec_snd + 16u * (uint32_t)(par * n), own[q_snd], bar_snd);
+        for (int e = tid + kSmallThreads; e < np * cs; e += kSmallThreads) {
             const int t = e / np, q = e - t * np;
             send(remote(local_addr(R_ + first + q), t), own[q], remote(bar_rec, t));
         }
@@ -305,28 +334,15 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
                      make_uint4((uint32_t)s_flags[par], 0u, (uint32_t)k2, (uint32_t)(k2 >> 32)),
                      remote(bar_rec, lane));
         }
-        // ---- this rank's wave vectors and the thermostat's noise meanwhile
-        if (kSmallWarps - 1 - warp < kp) {
-            const int q = 2 * (kSmallWarps - 1 - warp);
-            int4 m0, m1;
-            warp_sample2(S, table, k0 + q, k0 + min(q + 1, nk - 1), step, a.err, m0, m1);
-            if (lane == 0) {
-                s_m[q] = m0;
-                s_m[q + 1] = m1;
-            }
-        }
-        MdNoise z{0.f, 0.f, 0.f, false};
-        if (owner && !nhm) z = md_noise(S, step, o);
         if (!late && !bar_wait(bar_rec, par)) late = true;
         const uint32_t seen = __reduce_or_sync(0xffffffffu, lane < cs ? s_msg[par][lane].x : 0u);
         const bool rebuild = (seen & 1u) != 0u;
         bad_seen |= (seen & 2u) != 0u;
-        __syncthreads();                            // s_m
         // ---- structure factors of two wave vectors over a share of all records
         if (sums) {
-            const int4 m0 = s_m[2 * pr], m1 = s_m[2 * pr + 1];
+            const int4 m0 = s_m[step & 1][2 * pr], m1 = s_m[step & 1][2 * pr + 1];
             float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
-#pragma unroll 2
+#pragma unroll 4
             for (int j = sub * 32 + lane; j < n; j += wpp * 32) {
                 const uint4 r = R_[j];
                 const float q = __uint_as_float(r.w);
@@ -358,28 +374,28 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         }
         // ---- a warp per wave vector: its force coefficient, to every rank
         for (int q = kSmallWarps - 1 - warp; q < nk; q += kSmallWarps) {
-            float2 re = make_float2(0.f, 0.f), im = re;
-            if (lane < wpp) {
-                const float* v = &s_part[lane * kp + (q >> 1)][(q & 1) * 2];
-                re.x = v[0];
-                im.x = v[1];
-            }
+            // lanes 0-15 add the shares' real parts, lanes 16-31 the imaginary
+            // ones, as float pairs
+            const int u = lane & 15, c = (q & 1) * 2 + (lane >> 4);
+            float2 v = make_float2(0.f, 0.f);
+            if (u < wpp) v.x = s_part[u * kp + (q >> 1)][c];
+            if (u + 16 < wpp) v = two_sum(v.x, s_part[(u + 16) * kp + (q >> 1)][c]);
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) {
-                const float2 x = two_sum(re.x, __shfl_xor_sync(0xffffffffu, re.x, d));
-                re = make_float2(x.x, re.y + __shfl_xor_sync(0xffffffffu, re.y, d) + x.y);
-                const float2 y = two_sum(im.x, __shfl_xor_sync(0xffffffffu, im.x, d));
-                im = make_float2(y.x, im.y + __shfl_xor_sync(0xffffffffu, im.y, d) + y.y);
+            for (int d = 8; d > 0; d >>= 1) {
+                const float2 x = two_sum(v.x, __shfl_xor_sync(0xffffffffu, v.x, d));
+                v = make_float2(x.x, v.y + __shfl_xor_sync(0xffffffffu, v.y, d) + x.y);
             }
-            // c = coefficient scale / |m|^2 as a float pair (|m|^2 is exact)
-            const int4 m = s_m[q];
-            const float m2 = (float)(m.x * m.x + m.y * m.y + m.z * m.z);
-            const float ch = a.kscale_hi / m2;
-            const float cl = (fmaf(-ch, m2, a.kscale_hi) + a.kscale_lo) / m2;
-            const float A = pair_mul(ch, cl, im), B = pair_mul(ch, cl, re), Rk = hypotf(A, B);
-            const float turns = atan2f(A, B) * 0.15915494309189535f;
+            const int4 m = s_m[step & 1][q];
+            const float2 cf = s_c[step & 1][q];
+            const float AB = pair_mul(cf.x, cf.y, v);
+            const float A = __shfl_sync(0xffffffffu, AB, 16), B = __shfl_sync(0xffffffffu, AB, 0);
+            const float Rk = hypotf(A, B);
+            // phi in 2^-32 turns; half a turn is 2^31 (the conversion saturates below it)
+            const float turns = atan2f(A, B) * 0.15915494309189535f * 4294967296.0f;
+            const uint32_t phi =
+                turns >= 2147483648.0f ? 0x80000000u : (uint32_t)__float2int_rn(turns);
             const uint4 x = make_uint4(0u - (uint32_t)m.x, 0u - (uint32_t)m.y, 0u - (uint32_t)m.z,
-                                       (uint32_t)(long long)llrintf(turns * 4294967296.0f));
+                                       phi);
             const uint4 y = make_uint4(__float_as_uint(Rk * (float)m.x),
                                        __float_as_uint(Rk * (float)m.y),
                                        __float_as_uint(Rk * (float)m.z), __float_as_uint(Rk));
@@ -388,6 +404,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
                 send(remote(local_addr(kv + (lane < 16 ? 0 : P) + k0 + q), t), lane < 16 ? x : y,
                      remote(bar_kv, t));
         }
+        if (s + 1 < a.nsteps) draw(step + 1, w_draw);   // the next step's wave vectors
+        MdNoise z{0.f, 0.f, 0.f, false};
+        if (owner && !nhm) z = md_noise(S, step, o);
         if (nk == 0 && tid == 0)
             for (int t = 0; t < cs; ++t)
                 send(remote(local_addr(&s_token), t), make_uint4(0u, 0u, 0u, 0u),
@@ -458,10 +477,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         }
         // ---- real-space pairs
         float fx = 0.f, fy = 0.f, fz = 0.f;
-        uint4 si = make_uint4(0, 0, 0, 0);
         if (pairs) {
             PairAcc acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            si = R_[pn];
+            const uint4 si = R_[pn];
             const float lbqi = kc.lB * __uint_as_float(si.w);
             for (int k = l; k < cnt; k += R)
                 pair_fixed(si, R_[list[p * a.cap + k]], S.L_over_2_32, lbqi, kc, acc);
@@ -472,6 +490,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         // ---- Fourier force
         if (!late && !bar_wait(bar_kv, par)) late = true;
         if (pairs) {
+            const uint4 si = R_[pn];
             float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll 4
             for (int k = l; k < P; k += R) {
