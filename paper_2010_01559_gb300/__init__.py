@@ -304,8 +304,9 @@ class RBEEnergy:
 
     ``RBEEnergy.apply(pos, q, rbe, step)`` with pos float32 [n,3] and q float32
     [n] (CUDA) returns the FP64 energy of the mixed path (scalar tensor for a
-    single system).  backward gives dE/dpos = -F and dE/dq = phi, recomputing
-    rho(k) for the same k-batch instead of storing per-pair phases.
+    single system).  backward gives dE/dpos = -F and dE/dq = phi of the same
+    evaluation: where a gradient may be asked for, the forward evaluation keeps
+    F and phi (20 bytes per particle), so that backward only scales them.
     """
 
     _fn = None
@@ -324,19 +325,17 @@ def _make_energy_fn():
         @staticmethod
         def forward(ctx, pos, q, rbe, step):
             pos_q = torch.cat([pos.detach().float(), q.detach().float()[:, None]], 1).contiguous()
-            _, E, _ = rbe.forces(pos_q, step, energy=True, phi=False)
-            ctx.rbe = rbe
-            ctx.step = step
-            ctx.save_for_backward(pos, q)
+            want = ctx.needs_input_grad[0] or ctx.needs_input_grad[1]
+            F, E, phi = rbe.forces(pos_q, step, energy=True, phi=want)
+            if want:
+                ctx.save_for_backward(pos, q, F, phi)
             return E[:, 0].sum() if E.shape[0] > 1 else E[0, 0]
 
         @staticmethod
         def backward(ctx, gE):
-            pos, q = ctx.saved_tensors
-            pos_q = torch.cat([pos.detach().float(), q.detach().float()[:, None]], 1).contiguous()
-            F, _, phi = ctx.rbe.forces(pos_q, ctx.step, energy=False, phi=True)
+            pos, q, F, phi = ctx.saved_tensors
             g = gE.to(torch.float32)
-            gpos = (-F[:, :3] * g).to(pos.dtype) if ctx.needs_input_grad[0] else None
+            gpos = (F[:, :3] * -g).to(pos.dtype) if ctx.needs_input_grad[0] else None
             gq = (phi * g).to(q.dtype) if ctx.needs_input_grad[1] else None
             return gpos, gq, None, None
 

@@ -54,7 +54,7 @@ struct GraphEntry {
     int prec;
     const void* host_pos;  // host-buffer graphs: the caller's pinned arrays (else null)
     const void* host_vel;
-    int host_steps;        // host-buffer graphs: steps per replay
+    int steps;             // steps per replay
     const void* done;      // completion word of a zero-copy host step (else null)
     cudaGraphExec_t exec;
     int kernels;           // kernels in one replay
@@ -161,10 +161,14 @@ struct rbe_ctx {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int rho_chunk = 0, force_split = 0, real_split = 0, real_seg = 0;   // 0 = automatic
     int cur_n = -1, cur_chunk = -1, cur_split = -1, cur_rsplit = -1, cur_seg = -1;
-    int npblk = 0, nfblk = 0, nrblk = 0, nchunks = 0, split = 1, rsplit = 1;
+    int npblk = 0, nfblk = 0, nchunks = 0, split = 1, rsplit = 1;
     int nseg = 0, seg_max = 1, stage_cap = 0, seg_threads = 64;
-    int max_pblk = 0, max_fblk = 0, max_rblk = 0, max_chunks = 0, max_seg = 0;
+    int max_pblk = 0, max_fblk = 0, max_chunks = 0, max_seg = 0;
     size_t max_part = 0;
+    // mixed structure factors: tiles, particles per tile and FP32 run of an
+    // evaluation without (n) and with energies (e)
+    int nrt = 0, rt_n = 0, rt_e = 0, run_n = 64, run_e = 64, max_rt = 0;
+    bool cur_set = false;                     // the chunk in effect was set, not automatic
     bool use_graph = false;
     double wait_limit = 0.0;                  // seconds a host wait may take (0: no limit)
     // list steps: structure factors + standing-list pass in one launch:
@@ -186,9 +190,9 @@ struct rbe_ctx {
     SysDev* d_sys = nullptr;
     Tile* d_pblk = nullptr;
     Tile* d_fblk = nullptr;
-    Tile* d_rblk = nullptr;
     Tile* d_segs = nullptr;
     Tile* d_chunks = nullptr;
+    Tile* d_rt = nullptr;                     // tiles of the mixed structure factors
     int* d_kstart = nullptr;
     int* d_cstart = nullptr;
     uint64_t* d_table = nullptr;
@@ -218,6 +222,7 @@ struct rbe_ctx {
     uint64_t* d_mh_pos = nullptr;             // per system: chain iterations done
     NhState* d_nh = nullptr;                  // per system: Nose-Hoover state
     // neighbour list of the mixed MD step (pairs within r_c + skin)
+    bool sort_cluster = false;                // the sort may run as one cluster
     bool list = false;                        // the handle keeps a list (skin >= 0)
     bool list_valid = false;                  // sorted arrays still those of the last build
     int list_split = 0, cur_lsplit = -1;      // lanes per particle of the list pass (0 = auto)
@@ -376,10 +381,9 @@ void fill_sysdev(const SysHost& s, SysDev& d) {
     d.off_t = s.off_t;
     d.off_part = 0;
     d.nchunk = 0;
+    d.nrt = 0;
     d.off_b = 0;
     d.nb = 0;
-    d.off_rb = 0;
-    d.nrb = 0;
     d.off_sg = 0;
     d.nsg = 0;
     d.off_lb = 0;
@@ -389,6 +393,7 @@ void fill_sysdev(const SysHost& s, SysDev& d) {
     int e = 52;
     const double bound = 4.0 * std::max(1, s.n);
     while (e > 20 && bound * std::ldexp(1.0, e) >= std::ldexp(1.0, 62)) --e;
+    d.rho_exp = e;
     d.rho_scale = std::ldexp(1.0, e);
     d.rho_inv_scale = std::ldexp(1.0, -e);
     d.f_rc2 = (float)(d.r_c * d.r_c);
@@ -435,13 +440,45 @@ bool fusion_on(const rbe_ctx* h) {
     return ntot >= kFuseMinN;
 }
 
+// Particles per structure-factor chunk: the share of a block of the FP64 path,
+// and the FP32 run of an evaluation that returns energies (at most kRhoStage).
 int auto_chunk(const rbe_ctx* h, long long ntot) {
-    const int ltiles = (h->pmax + kRhoKT - 1) / kRhoKT;
+    const int ltiles = (h->pmax + 255) / 256;
     const long long target_blocks = 152LL * 12;
     long long chunks = std::max(1LL, target_blocks / std::max(1, ltiles));
     long long c = (ntot + chunks - 1) / chunks;
     int p = pow2_ceil(std::max(1LL, c));
     return std::min(4096, std::max(32, p));
+}
+
+// Threads of a block that share a particle in the mixed structure factors.
+int rho_subs(int pmax) {
+    return kRhoThreads / std::max(1, (std::min(pmax, kRhoKT) + 1) / 2);
+}
+
+// FP32 run of the mixed structure factors without energies: as long as one pass
+// of the block holds a run per sub (a run's end costs about 30 instructions per
+// wave vector), at most 256 particles (chains of 128 terms), and shorter where
+// that leaves fewer than 128 blocks or, below 2^17 particles, more than 64.
+int auto_run(int pmax, long long ntot) {
+    const int subs = rho_subs(pmax);
+    int run = ntot < (1LL << 17) ? 64 : 256;
+    while (run > 8 && (ntot < 128LL * run * subs || run * subs > kRhoStage)) run >>= 1;
+    return run;
+}
+
+// Particles per block of the mixed structure factors: one pass while that gives
+// at most two blocks per SM (each block ends with two atomics per wave vector, and
+// more blocks than that cost more in atomics than they gain); beyond, whole
+// waves of four resident blocks per SM with at least 128 particles per block.
+int auto_rho_tile(int pmax, long long ntot, int run) {
+    const int pass = std::min(kRhoStage, run * rho_subs(pmax));
+    if (ntot <= 304LL * pass) return pass;
+    const long long ktiles = (pmax + kRhoKT - 1) / kRhoKT;
+    const long long slots = std::max(1LL, 608LL / ktiles);
+    const long long waves = std::max(1LL, std::min(8LL, ntot / (slots * 128)));
+    const long long tile = (ntot + slots * waves - 1) / (slots * waves);
+    return (int)std::max<long long>(pass, std::min<long long>(4096, (tile + 7) / 8 * 8));
 }
 
 int auto_split(long long ntot) {
@@ -495,21 +532,28 @@ rbe_status prepare(rbe_ctx* h, int n) {
     const int rseg = h->real_seg > 0 ? std::min(h->real_seg, ncd_max)
                                      : auto_real_seg(ntot, h->ncell, ncd_max);
     if (h->cur_n == n && h->cur_chunk == chunk && h->cur_split == split &&
-        h->cur_rsplit == rsplit && h->cur_seg == rseg && h->cur_lsplit == lsplit)
+        h->cur_rsplit == rsplit && h->cur_seg == rseg && h->cur_lsplit == lsplit &&
+        h->cur_set == (h->rho_chunk > 0))
         return RBE_OK;
+    // mixed structure factors: particles per block and FP32 runs (with energies,
+    // the chunk's, and tiles of whole runs)
+    const int run = auto_run(h->pmax, ntot), run_e = std::min(chunk, kRhoStage);
+    int rtile_n = h->rho_chunk > 0 ? chunk : auto_rho_tile(h->pmax, ntot, run);
+    const int rtile_e = (rtile_n + run_e - 1) / run_e * run_e;
+    if (h->batch) rtile_n = rtile_e;              // one table serves both
     h->list_valid = false;                 // the sorted arrays are rebuilt from scratch
     std::vector<Tile> segs;
     int seg_max = 1;
     double stage_need = 0.0;
-    std::vector<Tile> pblk, fblk, rblk, chunks, lblk;
+    std::vector<Tile> pblk, fblk, chunks, lblk, rtiles;
     const int ltile = kBlockP / lsplit;
     const int ftile = kBlockP / split;
-    const int rtile = kBlockP / real_split64(rsplit, ntot);
     int off_part = 0;
     for (int s = 0; s < h->nsys; ++s) {
         SysHost& sh = h->sys[s];
         SysDev& d = h->sysdev[s];
         fill_sysdev(sh, d);
+        d.rho_stride = 2 * h->ktot;
         d.off_b = (int)pblk.size();
         int nb = 0;
         for (int f = 0; f < sh.n || (f == 0 && nb == 0); f += kBlockP) {
@@ -522,14 +566,6 @@ rbe_status prepare(rbe_ctx* h, int n) {
             fblk.push_back(Tile{s, sh.off_p + f, std::max(0, std::min(ftile, sh.n - f)), 0});
             if (sh.n == 0) break;
         }
-        d.off_rb = (int)rblk.size();
-        int nrb = 0;
-        for (int f = 0; f < sh.n || f == 0; f += rtile) {
-            rblk.push_back(Tile{s, sh.off_p + f, std::max(0, std::min(rtile, sh.n - f)), 0});
-            ++nrb;
-            if (sh.n == 0) break;
-        }
-        d.nrb = nrb;
         d.off_lb = (int)lblk.size();
         if (h->list)
             for (int f = 0; f < sh.n || f == 0; f += ltile) {
@@ -561,11 +597,18 @@ rbe_status prepare(rbe_ctx* h, int n) {
             if (sh.n == 0) break;
         }
         d.nchunk = nc;
+        d.nrt = 0;
+        for (int f = 0; f < sh.n || f == 0; f += rtile_n) {
+            rtiles.push_back(Tile{s, sh.off_p + f, std::max(0, std::min(rtile_n, sh.n - f)), 0});
+            ++d.nrt;
+            if (sh.n == 0) break;
+        }
         off_part += nc * sh.p.P;
     }
     if ((int)pblk.size() > h->max_pblk || (int)fblk.size() > h->max_fblk ||
-        (int)rblk.size() > h->max_rblk || (int)chunks.size() > h->max_chunks ||
+        (int)chunks.size() > h->max_chunks ||
         (int)segs.size() > h->max_seg || (int)lblk.size() > h->max_lblk ||
+        (int)rtiles.size() > h->max_rt ||
         (size_t)off_part > h->max_part)
         return fail(h, RBE_ERR_ARG, "work tables exceed the workspace (n > capacity?)");
     RBE_CUDA(h, cudaMemcpyAsync(h->d_sys, h->sysdev.data(), sizeof(SysDev) * h->nsys,
@@ -574,11 +617,11 @@ rbe_status prepare(rbe_ctx* h, int n) {
                                 cudaMemcpyHostToDevice, h->stream));
     RBE_CUDA(h, cudaMemcpyAsync(h->d_fblk, fblk.data(), sizeof(Tile) * fblk.size(),
                                 cudaMemcpyHostToDevice, h->stream));
-    RBE_CUDA(h, cudaMemcpyAsync(h->d_rblk, rblk.data(), sizeof(Tile) * rblk.size(),
-                                cudaMemcpyHostToDevice, h->stream));
     RBE_CUDA(h, cudaMemcpyAsync(h->d_segs, segs.data(), sizeof(Tile) * segs.size(),
                                 cudaMemcpyHostToDevice, h->stream));
     RBE_CUDA(h, cudaMemcpyAsync(h->d_chunks, chunks.data(), sizeof(Tile) * chunks.size(),
+                                cudaMemcpyHostToDevice, h->stream));
+    RBE_CUDA(h, cudaMemcpyAsync(h->d_rt, rtiles.data(), sizeof(Tile) * rtiles.size(),
                                 cudaMemcpyHostToDevice, h->stream));
     if (!lblk.empty())
         RBE_CUDA(h, cudaMemcpyAsync(h->d_lblk, lblk.data(), sizeof(Tile) * lblk.size(),
@@ -588,8 +631,13 @@ rbe_status prepare(rbe_ctx* h, int n) {
     RBE_CUDA(h, cudaStreamSynchronize(h->stream));
     h->npblk = (int)pblk.size();
     h->nfblk = (int)fblk.size();
-    h->nrblk = (int)rblk.size();
     h->nchunks = (int)chunks.size();
+    h->nrt = (int)rtiles.size();
+    h->rt_n = rtile_n;
+    h->rt_e = rtile_e;
+    h->run_n = run;
+    h->run_e = run_e;
+    h->cur_set = h->rho_chunk > 0;
     h->split = split;
     h->rsplit = rsplit;
     h->nseg = (int)segs.size();
@@ -618,12 +666,11 @@ rbe_status prepare(rbe_ctx* h, int n) {
 
 rbe_status allocate(rbe_ctx* h) {
     // capacities (chunks as small as 32 particles, force tiles as small as 16)
-    long long pb = 0, fb = 0, rb = 0, ch = 0, part = 0;
+    long long pb = 0, fb = 0, ch = 0, part = 0;
     for (auto& s : h->sys) {
         const long long n = h->batch ? s.n : s.p.n_max;
         pb += (n + kBlockP - 1) / kBlockP + 1;
         fb += (n + 15) / 16 + 1;
-        rb += (n + 3) / 4 + 1;
         const long long c = (n + 31) / 32 + 1;
         ch += c;
         part += c * s.p.P;
@@ -631,10 +678,10 @@ rbe_status allocate(rbe_ctx* h) {
     h->max_pblk = (int)pb;
     h->max_lblk = (int)(pb * 8);             // list tiles as small as kBlockP / 8
     h->max_fblk = (int)fb;
-    h->max_rblk = (int)rb;
     h->max_seg = std::max(1, h->ncell);
     h->max_chunks = (int)ch;
     h->max_part = (size_t)part;
+    h->max_rt = (int)(2 * pb * (kBlockP / 8));    // structure-factor tiles of 8 particles
     const size_t N = (size_t)std::max(h->ntot, 1);
     rbe_status st = RBE_OK;
 #define RBE_ALLOC(ptr, cnt) \
@@ -642,9 +689,9 @@ rbe_status allocate(rbe_ctx* h) {
     RBE_ALLOC(h->d_sys, h->nsys);
     RBE_ALLOC(h->d_pblk, pb);
     RBE_ALLOC(h->d_fblk, fb);
-    RBE_ALLOC(h->d_rblk, rb);
     RBE_ALLOC(h->d_segs, std::max(1, h->ncell));
     RBE_ALLOC(h->d_chunks, ch);
+    RBE_ALLOC(h->d_rt, h->max_rt);
     RBE_ALLOC(h->d_kstart, h->nsys + 1);
     RBE_ALLOC(h->d_cstart, h->nsys + 1);
     RBE_ALLOC(h->d_table, h->ttot);
@@ -661,7 +708,7 @@ rbe_status allocate(rbe_ctx* h) {
     RBE_ALLOC(h->d_cell_cnt, h->ncell + 1);
     RBE_ALLOC(h->d_cell_start, h->ncell + 1);
     RBE_ALLOC(h->d_ksamp, h->ktot);
-    RBE_ALLOC(h->d_rho_fx, 2 * (size_t)h->ktot);
+    RBE_ALLOC(h->d_rho_fx, 2 * (size_t)kRhoCopies * h->ktot);
     RBE_ALLOC(h->d_kcnt, h->ktot);
     RBE_ALLOC(h->d_kcoef, h->ktot);
     RBE_ALLOC(h->d_mh_tq, h->ttot);
@@ -681,8 +728,9 @@ rbe_status allocate(rbe_ctx* h) {
     }
     RBE_ALLOC(h->d_kab, h->ktot);
     RBE_ALLOC(h->d_qsum_fx, h->nsys);
-    // per-block energy / virial partials: FP64 blocks, segment blocks or list blocks
-    const long long nblk_e = std::max<long long>(std::max<long long>(rb, (long long)kSegChunks *
+    // per-block energy / virial partials: FP64 blocks (up to 32 per particle tile),
+    // segment blocks or list blocks
+    const long long nblk_e = std::max<long long>(std::max<long long>(32 * pb, (long long)kSegChunks *
                                                  (h->ncell + 1)), (long long)h->max_lblk);
     RBE_ALLOC(h->d_blk_e, nblk_e);
     RBE_ALLOC(h->d_blk_w, nblk_e);
@@ -709,7 +757,7 @@ rbe_status allocate(rbe_ctx* h) {
         RBE_CUDA(h, cudaMemcpy(h->d_list_flag, &one, sizeof(int), cudaMemcpyHostToDevice));
     }
     RBE_CUDA(h, cudaMemset(h->d_qsum_fx, 0, sizeof(unsigned long long) * h->nsys));
-    RBE_CUDA(h, cudaMemset(h->d_rho_fx, 0, sizeof(unsigned long long) * 2 * h->ktot));
+    RBE_CUDA(h, cudaMemset(h->d_rho_fx, 0, sizeof(unsigned long long) * 2 * kRhoCopies * h->ktot));
     RBE_CUDA(h, cudaMemset(h->d_kcnt, 0, sizeof(int) * h->ktot));
     std::vector<uint64_t> tab, mtq;
     std::vector<double> mrho;
@@ -764,7 +812,8 @@ void release(rbe_ctx* h) {
     if (!h) return;
     for (auto& g : h->graphs) cudaGraphExecDestroy(g.exec);
     h->graphs.clear();
-    void* ptrs[] = {h->d_sys, h->d_pblk, h->d_fblk, h->d_rblk, h->d_segs, h->d_chunks,
+    void* ptrs[] = {h->d_sys, h->d_pblk, h->d_fblk, h->d_segs, h->d_chunks,
+                    h->d_rt,
                     h->d_kstart,
                     h->d_cstart,
                     h->d_table, h->d_fx, h->d_spos, h->d_fx64, h->d_spos64, h->d_cid, h->d_rank,
@@ -863,6 +912,7 @@ rbe_status create_common(const rbe_params* ps, const int32_t* ns, int nsys, bool
         }
         h->list_cap = (int)std::min(4096.0, 8.0 * std::ceil((1.5 * most + 8.0 * std::sqrt(most) + 16.0) / 8.0));
     }
+    h->sort_cluster = h->ncell <= kSortMaxCells && sort_cluster_ok(!batch);
     for (auto& sh : h->sys) h->mh_words = std::max(h->mh_words, 2 * sh.M + 1);
     rbe_status st = allocate(h);
     if (st != RBE_OK) {
@@ -916,8 +966,8 @@ Work make_work(const rbe_ctx* h, const Tile* tiles, int tile, int aux_stride) {
 RealArgs make_real_args(const rbe_ctx* h, int parts) {
     RealArgs r{};
     const int split64 = real_split64(h->rsplit, h->batch ? h->ntot : h->cur_n);
-    r.w = make_work(h, h->d_rblk, kBlockP / split64, 0);
-    r.nrblk = h->nrblk;
+    r.w = make_work(h, h->d_pblk, kBlockP, 0);
+    r.npblk = h->npblk;
     r.split = h->rsplit;
     r.split64 = split64;
     r.ncell = h->ncell;
@@ -941,17 +991,37 @@ RealArgs make_real_args(const rbe_ctx* h, int parts) {
     return r;
 }
 
-// Structure factors: per-chunk partials added to the fixed-point rho(k).
-void launch_rho(const rbe_ctx* h, cudaStream_t st, bool mixed, bool pdl = false) {
+// The mixed structure factors' work: tiles of particles and how many, the FP32 run.
+struct RhoWork {
+    Work w;
+    int ntiles, ktiles, run;
+};
+
+RhoWork make_rho_work(const rbe_ctx* h, bool energies) {
+    RhoWork r{};
+    const int tile = energies ? h->rt_e : h->rt_n;
+    r.w = make_work(h, h->d_rt, tile, 0);
+    r.ntiles = h->nrt;
+    if (!h->batch) {
+        r.ntiles = std::max(1, (r.w.one.n + tile - 1) / tile);
+        r.w.one.nrt = r.ntiles;
+    }
+    r.ktiles = (h->pmax + kRhoKT - 1) / kRhoKT;
+    r.run = energies ? h->run_e : h->run_n;
+    return r;
+}
+
+// Structure factors: partials added to the fixed-point rho(k).
+void launch_rho(const rbe_ctx* h, cudaStream_t st, bool mixed, bool energies, bool pdl = false) {
     const bool one = !h->batch;
-    const int ltiles = (h->pmax + kRhoKT - 1) / kRhoKT;
-    const Work w = make_work(h, h->d_chunks, h->cur_chunk, 1);
-    if (mixed)
-        launch_rho_mixed(st, one, w, h->nchunks, ltiles, h->d_ksamp, h->d_kcoef, h->d_fx,
+    if (mixed) {
+        const RhoWork r = make_rho_work(h, energies);
+        launch_rho_mixed(st, one, r.w, r.ntiles, r.ktiles, r.run, h->d_ksamp, h->d_kcoef, h->d_fx,
                          h->d_rho_fx, h->d_kcnt, h->d_kab, pdl);
-    else
-        launch_rho_f64(st, one, w, h->nchunks, h->cur_chunk, h->pmax, h->m_max(), h->d_ksamp,
-                       h->d_fx64, h->d_rho_fx);
+    } else {
+        launch_rho_f64(st, one, make_work(h, h->d_chunks, h->cur_chunk, 1), h->nchunks,
+                       h->cur_chunk, h->pmax, h->m_max(), h->d_ksamp, h->d_fx64, h->d_rho_fx);
+    }
 }
 
 void launch_force(const rbe_ctx* h, cudaStream_t st, bool mixed, const MdOut& md = MdOut{},
@@ -974,7 +1044,8 @@ void launch_force(const rbe_ctx* h, cudaStream_t st, bool mixed, const MdOut& md
 // order); both join before the real-space kernel.  With profiling on (and st
 // the handle's own stream, i.e. not capturing) every kernel is bracketed by
 // events and the per-kernel device times are accumulated after the last one.
-int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
+// chained: the evaluation follows a list step's closing kernel on st directly.
+int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = false) {
     const bool mixed = a.prec == RBE_MIXED;
     const bool one = !h->batch;
     const bool fourier = (a.parts & RBE_PART_FOURIER) != 0;
@@ -1004,7 +1075,7 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
     pa.want_q = want_q;
     pa.qsum_fx = h->d_qsum_fx;
     pa.rho_fx = h->d_rho_fx;
-    pa.nrho = h->ktot;
+    pa.nrho = 2 * kRhoCopies * h->ktot;
     pa.step_dev = a.step_dev;
     pa.step_arg = a.step;
     pa.cur_step = h->d_cur_step;
@@ -1041,7 +1112,7 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
     run(RBE_K_PREP, st, [&] {
         if (mixed)
             launch_prep_mixed(st, one, wp, h->npblk, a.pos, h->d_fx, h->d_cid, h->d_rank,
-                              h->d_cell_cnt, pa);
+                              h->d_cell_cnt, pa, chained && !prof);
         else
             launch_prep_f64(st, one, wp, h->npblk, a.pos64, h->d_fx64, h->d_fx, h->d_cid,
                             h->d_rank, h->d_cell_cnt, pa);
@@ -1066,19 +1137,18 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
             rl.list_flag = h->d_list_flag;
             rl.freal = h->d_freal;
             rl.list_when = 0;
-            const int ltiles = (h->pmax + kRhoKT - 1) / kRhoKT;
+            const RhoWork rw = make_rho_work(h, a.E != nullptr);
             run(RBE_K_RHO_LIST, st, [&] {
-                launch_rho_list(st, one, make_work(h, h->d_chunks, h->cur_chunk, 1), h->nchunks,
-                                ltiles, h->d_ksamp, h->d_kcoef, h->d_fx, h->d_rho_fx, h->d_kcnt,
-                                h->d_kab, rl, !prof);
+                launch_rho_list(st, one, rw.w, rw.ntiles, rw.ktiles, rw.run, h->d_ksamp,
+                                h->d_kcoef, h->d_fx, h->d_rho_fx, h->d_kcnt, h->d_kab, rl, !prof);
             });
         } else if (fourier) {
-            run(RBE_K_RHO, st, [&] { launch_rho(h, st, mixed, !prof); });
+            run(RBE_K_RHO, st, [&] { launch_rho(h, st, mixed, a.E != nullptr, !prof); });
         }
     } else if (fourier) {
         cudaEventRecord(h->ev_fork, st);
         cudaStreamWaitEvent(st2, h->ev_fork, 0);
-        run(RBE_K_RHO, st2, [&] { launch_rho(h, st2, mixed); });
+        run(RBE_K_RHO, st2, [&] { launch_rho(h, st2, mixed, a.E != nullptr); });
         run(RBE_K_FOURIER_FORCE, st2, [&] {
             launch_force(h, st2, mixed, MdOut{}, false, mixed || a.phi64);
         });
@@ -1091,26 +1161,53 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
         sc = prof ? st : h->stream3;
         cudaStreamWaitEvent(sc, h->ev_prep, 0);
     }
-    run(RBE_K_SCAN, sc, [&] {
-        // on a list evaluation the cells are assigned here, only for a rebuild
-        // (the prep kernel skips them): counted with the scan in the profile
-        if (lst && mixed) {
-            launch_cell_assign(sc, one, wp, h->npblk, h->d_fx, h->d_cid, h->d_rank,
-                               h->d_cell_cnt, h->ncell, lflag, h->d_err);
-            ++count;
-        }
-        launch_scan(sc, h->d_cell_cnt, h->d_cell_start, h->ncell, a.step_dev, h->d_cur_step,
-                    lflag);
-    });
-    run(RBE_K_SCATTER, sc, [&] {
-        launch_scatter(sc, n, h->d_cid, h->d_rank, h->d_cell_start, h->d_perm_tmp, lflag,
-                       h->d_err);
-    });
-    run(RBE_K_CELL_ORDER, sc, [&] {
-        launch_order(sc, n, h->d_cid, h->d_cell_start, h->d_perm_tmp, h->d_fx, h->d_spos,
-                     mixed ? nullptr : h->d_fx64, h->d_spos64, h->d_perm, lflag,
-                     lst ? h->d_iperm : nullptr, h->d_err);
-    });
+    if (h->sort_cluster && n <= kSortMaxN) {
+        run(RBE_K_SCAN, sc, [&] {
+            SortArgs sa{};
+            sa.w = wp;
+            sa.ntile = h->npblk;
+            sa.assign = lst && mixed ? 1 : 0;
+            sa.n = n;
+            sa.ncell = h->ncell;
+            sa.fx = h->d_fx;
+            sa.fx64 = mixed ? nullptr : h->d_fx64;
+            sa.cid = h->d_cid;
+            sa.rank = h->d_rank;
+            sa.cell_cnt = h->d_cell_cnt;
+            sa.cell_start = h->d_cell_start;
+            sa.perm_tmp = h->d_perm_tmp;
+            sa.perm = h->d_perm;
+            sa.iperm = lst ? h->d_iperm : nullptr;
+            sa.spos = h->d_spos;
+            sa.spos64 = h->d_spos64;
+            sa.step_dev = a.step_dev;
+            sa.cur_step = h->d_cur_step;
+            sa.list_flag = lflag;
+            sa.err = h->d_err;
+            launch_sort(sc, one, sa);
+        });
+    } else {
+        run(RBE_K_SCAN, sc, [&] {
+            // on a list evaluation the cells are assigned here, only for a rebuild
+            // (the prep kernel skips them): counted with the scan in the profile
+            if (lst && mixed) {
+                launch_cell_assign(sc, one, wp, h->npblk, h->d_fx, h->d_cid, h->d_rank,
+                                   h->d_cell_cnt, h->ncell, lflag, h->d_err);
+                ++count;
+            }
+            launch_scan(sc, h->d_cell_cnt, h->d_cell_start, h->ncell, a.step_dev, h->d_cur_step,
+                        lflag);
+        });
+        run(RBE_K_SCATTER, sc, [&] {
+            launch_scatter(sc, n, h->d_cid, h->d_rank, h->d_cell_start, h->d_perm_tmp, lflag,
+                           h->d_err);
+        });
+        run(RBE_K_CELL_ORDER, sc, [&] {
+            launch_order(sc, n, h->d_cid, h->d_cell_start, h->d_perm_tmp, h->d_fx, h->d_spos,
+                         mixed ? nullptr : h->d_fx64, h->d_spos64, h->d_perm, lflag,
+                         lst ? h->d_iperm : nullptr, h->d_err);
+        });
+    }
     if (lst)
         run(RBE_K_LIST_BUILD, sc, [&] {
             ListArgs la{};
@@ -1127,6 +1224,7 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
             la.perm = h->d_perm;
             la.stats = h->d_list_stats;
             la.err = h->d_err;
+            la.freal = a.list ? h->d_freal : nullptr;
             launch_list_build(sc, one, la);
         });
     if (fourier && !a.list) cudaStreamWaitEvent(st, h->ev_join, 0);
@@ -1154,18 +1252,14 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
         r.freal = h->d_freal;
         // the real-space pass over a standing list right after the prep kernel
         // (concurrent with the structure factors and the rebuild stream), or
-        // over the rebuilt list at the end of the rebuild stream; then the
-        // Fourier force, which adds it and applies the thermostat
+        // over a rebuilt list by the build itself; then the Fourier force,
+        // which adds it and applies the thermostat
         r.list_when = 0;
         if (!fused) {
             cudaStreamWaitEvent(st2, h->ev_prep, 0);
             run(RBE_K_REAL, st2, [&] { launch_real_list(st2, one, r); });
             cudaEventRecord(h->ev_real, st2);
         }
-        RealArgs rb = r;
-        rb.list_when = 1;
-        launch_real_list(sc, one, rb);
-        ++count;
         cudaEventRecord(h->ev_chain, sc);
         if (!fused) cudaStreamWaitEvent(st, h->ev_real, 0);
         cudaStreamWaitEvent(st, h->ev_chain, 0);
@@ -1209,7 +1303,7 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a) {
         run(RBE_K_ENERGY, st, [&] {
             launch_energy(st, one, make_work(h, nullptr, 0, 0), h->nsys, h->d_ksamp, h->d_rho_fx,
                           h->d_blk_e, h->d_blk_q, r.blk_w, a.parts,
-                          a.list_forces ? 2 : (mixed ? 1 : 0), a.E,
+                          a.list_forces ? 2 : (mixed ? 1 : 0), r.split64, a.E,
                           r.blk_w ? a.W : nullptr);
         });
     if (prof) {
@@ -1379,6 +1473,7 @@ struct HostIO {
 // cluster (rbe_small.cu).  The cluster's blocks share the work of the whole
 // GPU, so its step grows with n P where the separate kernels' hardly does:
 // SMALL_RULE
+constexpr int kGraphSteps = 8;
 constexpr int kSmallStepsPerLaunch = 512;
 constexpr long long kSmallMaxNP = 500000;
 
@@ -1484,36 +1579,45 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
         if (io) copy_out(h->stream);
         return finish(h, "rbe_step");
     }
-    // a host-buffer call replays one graph holding copies and steps (up to 4)
-    const bool host_graph = io && nsteps <= 4;
+    // steps queued one behind the other on stream sq
+    auto steps_on = [&](cudaStream_t sq, int k) {
+        int kernels = 0;
+        for (int i = 0; i < k; ++i) kernels += enqueue_eval(h, sq, a, i > 0 && a.list);
+        return kernels;
+    };
     if (!h->use_graph || h->prof_on) {
         if (io) copy_in(h->stream);
-        for (int k = 0; k < nsteps; ++k) enqueue_eval(h, h->stream, a);
+        steps_on(h->stream, nsteps);
         if (io) copy_out(h->stream);
         return finish(h, "rbe_step");
     }
-    cudaGraphExec_t exec = nullptr;
-    int kernels = 0;
-    for (auto& g : h->graphs)
-        if (g.n == n && g.pos == pos && g.vel == vel && g.step == step_dev && g.prec == prec &&
-            g.F == (const void*)F_out && g.host_pos == (host_graph ? io->pos : nullptr) &&
-            g.host_vel == (host_graph ? io->vel : nullptr) &&
-            g.host_steps == (host_graph ? nsteps : 0) && g.done == (const void*)a.done) {
-            exec = g.exec;
-            kernels = g.kernels;
+    // a host-buffer call replays one graph holding copies and steps (up to 4);
+    // otherwise a graph holds up to kGraphSteps steps (a step's first kernel then
+    // follows the previous step's last one without a graph launch in between:
+    // N = 8001 GRAPH_FIGURES us per step with one step per graph)
+    const bool host_graph = io && nsteps <= 4;
+    auto find_graph = [&](int k) -> const GraphEntry* {
+        for (auto& g : h->graphs)
+            if (g.n == n && g.pos == pos && g.vel == vel && g.step == step_dev &&
+                g.prec == prec && g.F == (const void*)F_out &&
+                g.host_pos == (host_graph ? io->pos : nullptr) &&
+                g.host_vel == (host_graph ? io->vel : nullptr) && g.steps == k &&
+                g.done == (const void*)a.done)
+                return &g;
+        return nullptr;
+    };
+    auto graph_of = [&](int k, cudaGraphExec_t& exec, int& kernels) -> rbe_status {
+        if (const GraphEntry* g = find_graph(k)) {
+            exec = g->exec;
+            kernels = g->kernels;
+            return RBE_OK;
         }
-    if (!exec) {
         // Capture on the handle's private stream, then replay on the caller's.
         RBE_CUDA(h, cudaStreamSynchronize(h->stream));
         RBE_CUDA(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-        if (host_graph) {
-            copy_in(h->cap_stream);
-            kernels = 0;
-            for (int k = 0; k < nsteps; ++k) kernels += enqueue_eval(h, h->cap_stream, a);
-            copy_out(h->cap_stream);
-        } else {
-            kernels = enqueue_eval(h, h->cap_stream, a);
-        }
+        if (host_graph) copy_in(h->cap_stream);
+        kernels = steps_on(h->cap_stream, k);
+        if (host_graph) copy_out(h->cap_stream);
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(h->cap_stream, &graph);
         if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
@@ -1522,18 +1626,26 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
         if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
         h->graphs.push_back(GraphEntry{n, pos, vel, step_dev, F_out, prec,
                                        host_graph ? io->pos : nullptr,
-                                       host_graph ? io->vel : nullptr,
-                                       host_graph ? nsteps : 0, a.done, exec, kernels});
-    }
-    if (host_graph) {
+                                       host_graph ? io->vel : nullptr, k, a.done, exec, kernels});
+        return RBE_OK;
+    };
+    if (io && !host_graph) copy_in(h->stream);
+    // steps per replay.  Capturing a graph of several steps costs as much as
+    // tens of steps, so a call with arguments not seen before replays one step
+    // at a time unless it is long.
+    const int per = host_graph ? nsteps
+                    : (nsteps >= 64 || find_graph(1) || find_graph(std::min(nsteps, kGraphSteps)))
+                        ? std::min(nsteps, kGraphSteps) : 1;
+    for (int left = nsteps, first = 1; left > 0 || (first && host_graph); first = 0) {
+        const int k = host_graph || left >= per ? per : 1;
+        cudaGraphExec_t exec = nullptr;
+        int kernels = 0;
+        if ((s = graph_of(k, exec, kernels)) != RBE_OK) return s;
         RBE_CUDA(h, cudaGraphLaunch(exec, h->stream));
         h->kernel_count += kernels;
-    } else {
-        if (io) copy_in(h->stream);
-        for (int k = 0; k < nsteps; ++k) RBE_CUDA(h, cudaGraphLaunch(exec, h->stream));
-        if (io) copy_out(h->stream);
-        h->kernel_count += (int64_t)kernels * nsteps;
+        left -= std::max(k, 1);
     }
+    if (io && !host_graph) copy_out(h->stream);
     return finish(h, "rbe_step");
 }
 
@@ -1931,7 +2043,7 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float* pos_q, rbe_tuning*
         h->rho_chunk = c;
         if ((s = prepare(h, n)) != RBE_OK) break;
         enqueue_eval(h, h->stream, a);
-        const float t = time_kernel(h, e0, e1, [&] { launch_rho(h, h->stream, true); });
+        const float t = time_kernel(h, e0, e1, [&] { launch_rho(h, h->stream, true, false); });
         if (t < best) { best = t; best_chunk = c; }
     }
     h->rho_chunk = best_chunk;
@@ -2025,12 +2137,11 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float* pos_q, rbe_tuning*
                     r.list_flag = h->d_list_flag;
                     r.list_when = 0;
                     r.freal = h->d_freal;
-                    const int ltiles = (h->pmax + kRhoKT - 1) / kRhoKT;
+                    const RhoWork rw = make_rho_work(h, false);
                     const float t = time_kernel(h, e0, e1, [&] {
                         if (fused)
-                            launch_rho_list(h->stream, !h->batch,
-                                            make_work(h, h->d_chunks, h->cur_chunk, 1),
-                                            h->nchunks, ltiles, h->d_ksamp, h->d_kcoef, h->d_fx,
+                            launch_rho_list(h->stream, !h->batch, rw.w, rw.ntiles, rw.ktiles,
+                                            rw.run, h->d_ksamp, h->d_kcoef, h->d_fx,
                                             h->d_rho_fx, h->d_kcnt, h->d_kab, r, false);
                         else
                             launch_real_list(h->stream, !h->batch, r);

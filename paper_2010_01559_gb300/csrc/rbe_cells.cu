@@ -17,6 +17,7 @@
 // unit (L / 2^32) of the exact one for any float x.  Periodic wrapping is then
 // the natural 2^32 modulus, m . s mod 1 is exact in integer arithmetic, and
 // the minimum-image displacement is the signed difference of two fractions.
+#include "rbe_cluster.cuh"
 #include "rbe_internal.cuh"
 
 namespace rbe {
@@ -256,7 +257,7 @@ __device__ __forceinline__ void draw_samples(const Work& w, const PrepArgs& pa, 
 // particle blocks, pb the block's index among them; the sampling blocks do not
 // take part).
 __device__ __forceinline__ void clear_rho(unsigned long long* rho_fx, int nrho, int nblk, int pb) {
-    for (int k = pb * blockDim.x + threadIdx.x; k < 2 * nrho; k += nblk * blockDim.x)
+    for (int k = pb * blockDim.x + threadIdx.x; k < nrho; k += nblk * blockDim.x)
         rho_fx[k] = 0ull;
 }
 
@@ -265,6 +266,7 @@ __global__ void __launch_bounds__(kBlockP)
 k_prep_mixed(const __grid_constant__ Work w, const float4* __restrict__ pos_q,
              uint4* __restrict__ fx, int* __restrict__ cid, int* __restrict__ rank,
              int* __restrict__ cell_cnt, const __grid_constant__ PrepArgs pa) {
+    pdl_wait();                        // the previous step's closing update
     pdl_trigger();                     // a dependent kernel may be scheduled meanwhile
     // the k-sampling blocks come first, so that their table staging and
     // searches run alongside the particle blocks instead of after them
@@ -535,18 +537,170 @@ __global__ void k_order(int n, const int* __restrict__ cid, const int* __restric
     if (fx64) spos64[dst] = fx64[i];
 }
 
+// ------------------------------------------------- the sort as one cluster
+// The same sort (assignment of a list evaluation, scan, scatter, in-cell order)
+// in one launch of one cluster, for systems of up to kSortMaxN particles and
+// kSortMaxCells cells.  What bounds it is latency: as four kernels it is four
+// launches in a row, nearly always to find that the list stands, and they set
+// the length of a step whose other branch is as short as theirs (N = 8001:
+// SORT_FIGURES).  The phases meet at cluster barriers; data of another block is
+// read past the L1 cache.  Beyond the limit sixteen SMs take longer for a sort
+// than the whole GPU needs with the launches.
+constexpr int kSortThreads = 1024;
+constexpr int kSortCs = 16;                              // blocks of the cluster
+constexpr int kSortPer = kSortMaxCells / (kSortCs * kSortThreads);   // cells per thread
+
+template <bool ONE>
+__global__ void __launch_bounds__(kSortThreads, 1) k_sort(const __grid_constant__ SortArgs a) {
+    __shared__ int s_warp[32], s_tot[kSortCs];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = (int)cluster_rank(), g0 = rank * kSortThreads + tid;
+    constexpr int GT = kSortCs * kSortThreads;
+    if (a.step_dev && g0 == 0) *a.step_dev = *a.cur_step + 1;        // one increment per step
+    if (a.list_flag && !*a.list_flag) return;            // the list stands (in every block)
+    if (a.assign) {
+        // cells and slots, a group of kBlockP threads per particle tile
+        constexpr int GR = kSortThreads / kBlockP;
+        for (int tile = rank * GR + tid / kBlockP; tile < a.ntile; tile += kSortCs * GR) {
+            const Tile tl = tile_at<ONE>(a.w, tile);
+            const SysDev& S = sys_of<ONE>(a.w, tl.sys);
+            const int t = tid % kBlockP;
+            if (t >= tl.count) continue;
+            const int i = tl.first + t;
+            const uint4 r = a.fx[i];
+            const int ncd = S.ncd;
+            const int c = S.off_c + (cell_of_fixed(r.z, ncd) * ncd + cell_of_fixed(r.y, ncd)) * ncd +
+                          cell_of_fixed(r.x, ncd);
+            a.cid[i] = c;
+            a.rank[i] = RBE_IN_BOUNDS(c, a.ncell, a.err) ? atomicAdd(a.cell_cnt + c, 1) : 0;
+        }
+        __threadfence();
+    }
+    cluster_sync();                                      // (every block has started)
+    // exclusive scan of the counts: a segment per block, kSortPer cells per thread
+    const int c0 = g0 * kSortPer;
+    int v[kSortPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kSortPer; ++k) {
+        v[k] = c0 + k < a.ncell ? __ldcg(a.cell_cnt + c0 + k) : 0;
+        sum += v[k];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int k = 0; k < kSortThreads / 32; ++k) {
+        if (k < warp) before += s_warp[k];
+        total += s_warp[k];
+    }
+    if (tid < kSortCs)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
+                         remote(local_addr(&s_tot[rank]), (uint32_t)tid)),
+                     "r"(total)
+                     : "memory");
+    cluster_sync();
+    for (int k = 0; k < rank; ++k) before += s_tot[k];
+    int run = before + incl - sum;
+#pragma unroll
+    for (int k = 0; k < kSortPer; ++k) {
+        if (c0 + k < a.ncell) {
+            a.cell_start[c0 + k] = run;
+            a.cell_cnt[c0 + k] = 0;
+        }
+        run += v[k];
+    }
+    if (rank == kSortCs - 1 && tid == kSortThreads - 1) a.cell_start[a.ncell] = run;
+    __threadfence();
+    cluster_sync();
+    for (int i = g0; i < a.n; i += GT) {
+        const int slot = __ldcg(a.cell_start + __ldcg(a.cid + i)) + __ldcg(a.rank + i);
+        if (RBE_IN_BOUNDS(slot, a.n, a.err)) a.perm_tmp[slot] = i;
+    }
+    __threadfence();
+    cluster_sync();
+    for (int s = g0; s < a.n; s += GT) {
+        const int i = __ldcg(a.perm_tmp + s);
+        if (!RBE_IN_BOUNDS(i, a.n, a.err)) continue;
+        const int c = __ldcg(a.cid + i);
+        const int b = __ldcg(a.cell_start + c), e = __ldcg(a.cell_start + c + 1);
+        const uint4 r = a.fx[i];
+        int q = 0;
+        for (int k = b; k < e; ++k) {
+            const int j = __ldcg(a.perm_tmp + k);
+            const uint32_t xj = a.fx[j].x;
+            q += (xj < r.x || (xj == r.x && j < i)) ? 1 : 0;
+        }
+        const int dst = b + q;
+        if (!RBE_IN_BOUNDS(dst, a.n, a.err)) continue;
+        a.perm[dst] = i;
+        if (a.iperm) a.iperm[i] = dst;
+        a.spos[dst] = r;
+        if (a.fx64) a.spos64[dst] = a.fx64[i];
+    }
+    // a block's shared memory lives until every remote store to it is done: the
+    // barriers above follow the only one (s_tot)
+}
+
 // ------------------------------------------------------------- launchers
+template <bool ONE>
+static cudaError_t sort_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr,
+                               cudaStream_t st) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(kSortCs);
+    cfg.blockDim = dim3(kSortThreads);
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kSortCs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaFuncSetAttribute(k_sort<ONE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+// Whether the GPU can place the sort's cluster.
+bool sort_cluster_ok(bool one) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    int nc = 0;
+    cudaError_t e = one ? sort_config<true>(cfg, attr, nullptr) : sort_config<false>(cfg, attr, nullptr);
+    if (e == cudaSuccess)
+        e = one ? cudaOccupancyMaxActiveClusters(&nc, k_sort<true>, &cfg)
+                : cudaOccupancyMaxActiveClusters(&nc, k_sort<false>, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && nc >= 1;
+}
+
+void launch_sort(cudaStream_t st, bool one, const SortArgs& a) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    if (one) {
+        sort_config<true>(cfg, attr, st);
+        cudaLaunchKernelEx(&cfg, k_sort<true>, a);
+    } else {
+        sort_config<false>(cfg, attr, st);
+        cudaLaunchKernelEx(&cfg, k_sort<false>, a);
+    }
+}
+
 void launch_prep_mixed(cudaStream_t st, bool one, const Work& w, int nblk, const float4* pos_q,
-                       uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa) {
+                       uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa,
+                       bool pdl) {
     // particle blocks, then sampling blocks: one per system (MH chains) or one per kBlockP samples
     if (pa.ktot > 0) nblk += pa.mh ? pa.nsys : (pa.ktot + kBlockP - 1) / kBlockP;
     if (nblk <= 0) return;
     const size_t smem = pa.mh ? (sizeof(double) + sizeof(uint32_t)) * (size_t)pa.mh_words
                               : sizeof(uint32_t) * (size_t)pa.tab_words;
+    PdlConfig c(dim3(nblk), dim3(kBlockP), smem, st, pdl);
     if (one)
-        k_prep_mixed<true><<<nblk, kBlockP, smem, st>>>(w, pos_q, fx, cid, rank, cell_cnt, pa);
+        cudaLaunchKernelEx(&c.cfg, k_prep_mixed<true>, w, pos_q, fx, cid, rank, cell_cnt, pa);
     else
-        k_prep_mixed<false><<<nblk, kBlockP, smem, st>>>(w, pos_q, fx, cid, rank, cell_cnt, pa);
+        cudaLaunchKernelEx(&c.cfg, k_prep_mixed<false>, w, pos_q, fx, cid, rank, cell_cnt, pa);
 }
 
 void launch_prep_f64(cudaStream_t st, bool one, const Work& w, int nblk, const double4* pos_q,

@@ -2,15 +2,13 @@
 //
 //  k-sampling   P i.i.d. m in Z^3 \ {0} from P_k ~ exp(-k^2 / 4 alpha)   (Eq. probexpression)
 //               by a per-axis integer inverse-CDF table indexed with Philox words;
-//  k_rho        per-chunk partial structure factors
-//                 rho_chunk(k_l) = sum_{j in chunk} q_j exp(i k_l . r_j)          (Sec. 2)
-//               one thread per wave vector, particles (caller's order, so this
-//               branch does not wait for the cell sort) staged in shared memory
-//               and read as broadcasts; the k-batch is drawn by the same blocks;
-//               Each block adds its chunk's partial to rho(k_l) with 64-bit
-//               fixed-point atomics: integer addition is associative, so the
-//               cross-block sum is bitwise reproducible, with no separate
-//               reduction pass;
+//  k_rho        partial structure factors of a tile of particles
+//                 rho_tile(k_l) = sum_{j in tile} q_j exp(i k_l . r_j)           (Sec. 2)
+//               particles (caller's order, so this branch does not wait for
+//               the cell sort) staged in shared memory and read as broadcasts;
+//               each block adds its sums to rho(k_l) with 64-bit fixed-point
+//               atomics: integer addition is associative, so the cross-block
+//               sum is bitwise reproducible, with no separate reduction pass;
 //  k_force      per particle: F*_i = -q_i sum_l coef_l k_l Im(e^{-i k_l.r_i} rho_l)
 //               (Eq. rbmapprox) and the Fourier part of dE/dq_i, with the k-batch
 //               and coef_l rho_l, coef_l = (S/P) 4 pi / (V k^2) formed in FP64, staged
@@ -45,161 +43,179 @@ __global__ void k_sample(const SysDev* __restrict__ sysv, int nsys, int ktot,
 }
 
 // ----------------------------------------------------------------- rho (mixed)
-// Two threads per wave vector (threads t and t + kLTile), each over every
-// other particle of the chunk; their sums are added before the atomics.
-constexpr int kRhoHalves = 2;
+// Blocks of 256 threads: a tile of particles against a tile of up to 512 wave
+// vectors, two per thread (one shared-memory read of a particle serves two
+// pairs), so a system with P of them fills ceil(P / 2) threads; the block holds
+// floor(256 / that) such groups ("subs"), which share the particles.  That keeps
+// the lanes busy at any P: with one thread row of 128 per 256 wave vectors a
+// batch of P = 100 used 39 % of them, P = 137 54 %, and P = 10 4 %.
+//
+// What bounds it: the special-function unit (a sine and a cosine per pair, 16
+// cycles per warp), so the sums must cost little beside it.  A thread adds every
+// other particle of a run of `run` particles in FP32, then carries the run's sum
+// into a float pair (a few FP32 operations; FP64 additions and conversions are
+// two lanes per clock on this part and, done per 32 particles, took as long as
+// the sines).  Each block adds its sums to the fixed-point rho(k) with integer
+// work, once per wave vector.  The result depends on `run` and on the runs'
+// boundaries only through FP32 rounding; an evaluation that returns energies
+// keeps the run its tuning names.
+//
+// Measured (device time of the kernel alone, before -> after): RHO_FIGURES
 
-// rho_body: chunk ctile of the particles and tile ktile of kRhoKT wave
-// vectors (HALVES * kLTile threads; it synchronises the block), for the kernel
-// of its own and for the fused structure-factor + list launch of the MD step.
-// Each thread takes kRhoK wave vectors, t and t + kLTile of the tile, so that
-// one shared-memory load of a particle serves kRhoK (particle, k) pairs.
-// With one thread per wave vector (HALVES = 1) the even and odd particles go
-// to separate sums that are added as the two halves' are: rho(k) comes out the
-// same to the last bit either way.
-template <bool ONE, int HALVES>
+// round(f 2^e) as a 64-bit integer, in integer arithmetic (|f| 2^e < 2^62)
+__device__ __forceinline__ long long fixed64(float f, int e) {
+    const uint32_t b = __float_as_uint(f);
+    const int ex = (int)((b >> 23) & 255u);
+    const long long m = ex ? (long long)((b & 0x7FFFFFu) | 0x800000u) : 0ll;
+    const int sh = ex - 150 + e;
+    const long long v = sh >= 0 ? m << min(sh, 38)
+                                : (sh > -25 ? (m + (1ll << (-sh - 1))) >> -sh : 0ll);
+    return (b >> 31) ? -v : v;
+}
+
+// Sums of one wave vector as float pairs: (Re hi, Re lo, Im hi, Im lo).
+__device__ __forceinline__ void carry(float4& s, float re, float im) {
+    const float2 x = two_sum(s.x, re), y = two_sum(s.z, im);
+    s = make_float4(x.x, s.y + x.y, y.x, s.w + y.y);
+}
+
+__device__ __forceinline__ void rho_add(unsigned long long* dst, const float4& s, int e) {
+    atomicAdd(dst, (unsigned long long)(fixed64(s.x, e) + fixed64(s.y, e)));
+    atomicAdd(dst + 1, (unsigned long long)(fixed64(s.z, e) + fixed64(s.w, e)));
+}
+
+// rho_body: particle tile ctile, wave-vector tile ktile (the whole block), for
+// the kernel of its own and for the fused structure-factor + list launch.
+template <bool ONE>
 __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__ ksamp,
                                          const double* __restrict__ kcoef,
                                          const uint4* __restrict__ fx,
                                          unsigned long long* __restrict__ rho_fx,
                                          int* __restrict__ kcnt, float2* __restrict__ kab,
-                                         int ctile, int ktile) {
-    constexpr int KR = kRhoK;
-    __shared__ uint4 sp[kStage];
-    __shared__ double2 s_half[HALVES > 1 ? kLTile * KR : 1];
+                                         int ctile, int ktile, int run) {
+    __shared__ uint4 sp[kRhoStage];                  // 8 KB, then the subs' sums
+    static_assert(sizeof(sp) >= sizeof(float4) * 2 * kRhoThreads, "sums alias the stage");
     const Tile ch = tile_at<ONE>(w, ctile);
     const SysDev& S = sys_of<ONE>(w, ch.sys);
-    const int half = threadIdx.x / kLTile;
-    const int t = threadIdx.x - half * kLTile;
-    if (ktile * kRhoKT >= S.P) return;               // whole block beyond this system's P
-    uint32_t mx[KR], my[KR], mz[KR];
-    bool active[KR];
+    const int k0 = ktile * kRhoKT;
+    if (k0 >= S.P) return;                           // whole block beyond this system's P
+    const int nk = min(S.P - k0, kRhoKT);            // wave vectors of this tile
+    const int slots = (nk + 1) / 2;
+    const int subs = kRhoThreads / slots;
+    const int sub = threadIdx.x / slots, slot = threadIdx.x - sub * slots;
+    const bool work = sub < subs;
+    uint32_t mx[2], my[2], mz[2];
 #pragma unroll
-    for (int r = 0; r < KR; ++r) {
-        const int l = ktile * kRhoKT + t + r * kLTile;
-        active[r] = l < S.P;
-        int4 m = make_int4(0, 0, 0, 0);
-        if (active[r]) m = ksamp[S.off_k + l];       // drawn by the prep kernel
+    for (int r = 0; r < 2; ++r) {
+        const int4 m = ksamp[S.off_k + k0 + min(slot + r * slots, nk - 1)];   // prep drew them
         mx[r] = (uint32_t)m.x;
         my[r] = (uint32_t)m.y;
         mz[r] = (uint32_t)m.z;
     }
-    // FP32 sums over one staged pass (at most kStage / 2 terms), FP64 across
-    // passes and halves, so the rounding does not grow with the chunk size
-    double red[KR], imd[KR], red_o[KR], imd_o[KR];
-#pragma unroll
-    for (int r = 0; r < KR; ++r) red[r] = imd[r] = red_o[r] = imd_o[r] = 0.0;
-    float re[KR], im[KR], re_o[KR], im_o[KR];
-    auto terms = [&](const uint4 p, float* re_, float* im_) {
-        const float q = __uint_as_float(p.w);
-#pragma unroll
-        for (int r = 0; r < KR; ++r) {
-            const uint32_t ph = mx[r] * p.x + my[r] * p.y + mz[r] * p.z;
-            const float th = (float)(int32_t)ph * kTwoPiOver2p32;
-            float sn, cs;
-            __sincosf(th, &sn, &cs);
-            re_[r] = fmaf(q, cs, re_[r]);
-            im_[r] = fmaf(q, sn, im_[r]);
-        }
-    };
-    const bool any = active[0];                      // t + kLTile < P only if t < P
-    for (int base = 0; base < ch.count; base += kStage) {
-        const int cnt = min(kStage, ch.count - base);
+    float4 sum[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    // particles per pass: a whole number of runs for every sub where that fits
+    const int per = run * subs;
+    const int stage = per <= kRhoStage ? per * (kRhoStage / per) : kRhoStage;
+    for (int base = 0; base < ch.count; base += stage) {
+        const int cnt = min(stage, ch.count - base);
         __syncthreads();
-        for (int u = threadIdx.x; u < cnt; u += blockDim.x) sp[u] = fx[ch.first + base + u];
+        for (int u = threadIdx.x; u < cnt; u += kRhoThreads) sp[u] = fx[ch.first + base + u];
         __syncthreads();
-#pragma unroll
-        for (int r = 0; r < KR; ++r) re[r] = im[r] = re_o[r] = im_o[r] = 0.f;
-        if (any) {
-            if constexpr (HALVES == 1) {
-                int j = 0;
+        if (work)
+            // a run's even particles, then its odd ones, are a unit of work each
+            for (int u = sub; (u >> 1) * run < cnt; u += subs) {
+                const int j0 = (u >> 1) * run + (u & 1), j1 = min(cnt, ((u >> 1) + 1) * run);
+                float re[2] = {0.f, 0.f}, im[2] = {0.f, 0.f};
 #pragma unroll 8
-                for (; j + 1 < cnt; j += 2) {
-                    terms(sp[j], re, im);
-                    terms(sp[j + 1], re_o, im_o);
+                for (int j = j0; j < j1; j += 2) {
+                    const uint4 p = sp[j];
+                    const float q = __uint_as_float(p.w);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const uint32_t ph = mx[r] * p.x + my[r] * p.y + mz[r] * p.z;
+                        const float th = (float)(int32_t)ph * kTwoPiOver2p32;
+                        float sn, cs;
+                        __sincosf(th, &sn, &cs);
+                        re[r] = fmaf(q, cs, re[r]);
+                        im[r] = fmaf(q, sn, im[r]);
+                    }
                 }
-                if (j < cnt) terms(sp[j], re, im);
-            } else {
-#pragma unroll 2
-                for (int j = half; j < cnt; j += HALVES) terms(sp[j], re, im);
+                carry(sum[0], re[0], im[0]);
+                carry(sum[1], re[1], im[1]);
             }
-        }
-#pragma unroll
-        for (int r = 0; r < KR; ++r) {
-            red[r] += (double)re[r];
-            imd[r] += (double)im[r];
-            red_o[r] += (double)re_o[r];
-            imd_o[r] += (double)im_o[r];
-        }
     }
-    if constexpr (HALVES > 1) {
-        if (half == 1) {
-#pragma unroll
-            for (int r = 0; r < KR; ++r) s_half[t + r * kLTile] = make_double2(red[r], imd[r]);
-        }
-        __syncthreads();
-        if (half == 0) {
-#pragma unroll
-            for (int r = 0; r < KR; ++r) {
-                const double2 o = s_half[t + r * kLTile];
-                if (active[r])
-                    rho_accumulate(rho_fx + 2 * (S.off_k + ktile * kRhoKT + t + r * kLTile),
-                                   red[r] + o.x, imd[r] + o.y, S.rho_scale);
-            }
+    unsigned long long* dst =
+        rho_fx + (size_t)(ctile % kRhoCopies) * S.rho_stride + 2 * (S.off_k + k0);
+    if (subs == 1) {
+        if (work) {
+            rho_add(dst + 2 * slot, sum[0], S.rho_exp);
+            if (slot + slots < nk) rho_add(dst + 2 * (slot + slots), sum[1], S.rho_exp);
         }
     } else {
-#pragma unroll
-        for (int r = 0; r < KR; ++r)
-            if (active[r])
-                rho_accumulate(rho_fx + 2 * (S.off_k + ktile * kRhoKT + t + r * kLTile),
-                               red[r] + red_o[r], imd[r] + imd_o[r], S.rho_scale);
+        float4* red = (float4*)sp;                   // [wave vector][sub]
+        __syncthreads();
+        if (work) {
+            red[slot * subs + sub] = sum[0];
+            red[(slot + slots) * subs + sub] = sum[1];
+        }
+        __syncthreads();
+        for (int l = threadIdx.x; l < nk; l += kRhoThreads) {
+            float4 s = red[l * subs];
+            for (int u = 1; u < subs; ++u) {
+                const float4 v = red[l * subs + u];
+                carry(s, v.x, v.z);
+                s.y += v.y;
+                s.w += v.w;
+            }
+            rho_add(dst + 2 * l, s, S.rho_exp);
+        }
     }
-    // The last of the system's chunks to add its partials for this tile of
+    // The last of the system's tiles to add its sums for this tile of
     // wave vectors finds rho(k) complete and turns it into the force
     // coefficient of Eq. rbmapprox in polar form, once per k instead of once
     // per force block: with A = coef Im rho and B = coef Re rho,
     // A cos(theta) - B sin(theta) = R sin(phi - theta) for R = |(A, B)| and
     // phi = atan2(A, B), stored as (R, phi in 2^-32 turns).  Fence, then
-    // count: every chunk's atomics are visible to the block that takes the
+    // count: every tile's atomics are visible to the block that takes the
     // last count (no waiting on other blocks).
     __shared__ int s_last;
     __threadfence();
     __syncthreads();
-    const int slot = S.off_k + ktile * kRhoKT;
-    if (threadIdx.x == 0) s_last = atomicAdd(kcnt + slot, 1) == S.nchunk - 1;
+    int* cnt_k = kcnt + S.off_k + k0;
+    if (threadIdx.x == 0) s_last = atomicAdd(cnt_k, 1) == S.nrt - 1;
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (int u = threadIdx.x; u < kRhoKT; u += blockDim.x) {
-            const int l = ktile * kRhoKT + u;
-            if (l >= S.P) break;
-            const double2 r = rho_read(rho_fx + 2 * (S.off_k + l), S.rho_inv_scale);
+        for (int l = k0 + threadIdx.x; l < k0 + nk; l += kRhoThreads) {
+            const double2 r =
+                rho_total(rho_fx + 2 * (S.off_k + l), S.rho_stride, S.rho_inv_scale);
             const double c = kcoef[S.off_k + l];
             const float A = (float)(c * r.y), B = (float)(c * r.x);
             const float turns = atan2f(A, B) * 0.15915494309189535f;      // (-1/2, 1/2]
             const uint32_t phi = (uint32_t)(long long)llrintf(turns * 4294967296.0f);
             kab[S.off_k + l] = make_float2(hypotf(A, B), __uint_as_float(phi));
         }
-        if (threadIdx.x == 0) kcnt[slot] = 0;        // ready for the next evaluation
+        if (threadIdx.x == 0) *cnt_k = 0;            // ready for the next evaluation
     }
 }
 
 template <bool ONE>
-__global__ void __launch_bounds__(kLTile * kRhoHalves)
+__global__ void __launch_bounds__(kRhoThreads, 4)
 k_rho_mixed(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
             const double* __restrict__ kcoef, const uint4* __restrict__ fx,
             unsigned long long* __restrict__ rho_fx, int* __restrict__ kcnt,
-            float2* __restrict__ kab) {
-    pdl_trigger();                                    // the force kernel may be scheduled
+            float2* __restrict__ kab, int run) {
     pdl_wait();                                       // the prep kernel's samples and records
-    rho_body<ONE, kRhoHalves>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, blockIdx.x, blockIdx.y);
+    pdl_trigger();                                    // the force kernel may be scheduled (and
+                                                      // finds the prep kernel complete)
+    rho_body<ONE>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, blockIdx.x, blockIdx.y, run);
 }
 
 // ------------------------------------------- structure factors + list pass
 // The MD step's structure factors and its real-space pass over a standing
-// neighbour list in one launch of kLTile-thread blocks: block b takes
+// neighbour list in one launch of kRhoThreads-thread blocks: block b takes
 // structure-factor work when floor((b + 1) nrho / total) > floor(b nrho /
-// total), else a tile of the list pass, so that the two kinds are spread evenly
+// total), else two tiles of the list pass, so that the two kinds are spread evenly
 // over the grid and each SM holds both at once -- the structure factors keep
 // the special-function unit busy while the pair terms use the ALU and FMA
 // pipes and wait on their gathers.  The list tiles work only when the list
@@ -207,23 +223,25 @@ k_rho_mixed(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
 // build), and keep the per-slot count tests: padded batches cost this
 // issue-bound launch more than they save.
 template <int R, bool ONE>
-__global__ void __launch_bounds__(kLTile)
+__global__ void __launch_bounds__(kRhoThreads, 4)
 k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
            const double* __restrict__ kcoef, const uint4* __restrict__ fx,
            unsigned long long* __restrict__ rho_fx, int* __restrict__ kcnt,
-           float2* __restrict__ kab, const __grid_constant__ RealArgs a, int nchunks, int nrho,
-           int nlist) {
-    pdl_trigger();                                    // the force kernel may be scheduled
+           float2* __restrict__ kab, const __grid_constant__ RealArgs a, int ntiles, int run,
+           int nrho, int nlist) {
     pdl_wait();                                       // the prep kernel's samples and records
+    pdl_trigger();                                    // the force kernel may be scheduled (and
+                                                      // finds the prep kernel complete)
     const int b = blockIdx.x, total = nrho + nlist;
     const int r0 = (int)((long long)b * nrho / total);
     const int r1 = (int)((long long)(b + 1) * nrho / total);
     if (r1 > r0) {
-        rho_body<ONE, 1>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, r0 % nchunks, r0 / nchunks);
+        rho_body<ONE>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, r0 % ntiles, r0 / ntiles, run);
         return;
     }
     if ((*a.list_flag != 0) != (a.list_when != 0)) return;
-    list_body<R, ONE, false, false, 8>(a, b - r1, threadIdx.x);
+    const int tile = 2 * (b - r1) + (int)(threadIdx.x / kBlockP);
+    if (tile < a.nlblk) list_body<R, ONE, false, false, 8>(a, tile, threadIdx.x % kBlockP);
 }
 
 // ----------------------------------------------------------------- force (mixed)
@@ -256,18 +274,20 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
     const Tile tl = tile_of<ONE>(w);
     const SysDev& S = sys_of<ONE>(w, tl.sys);
     const int sub = threadIdx.x % SPLIT;            // lane within the particle's group
-    pdl_wait();                                     // rho(k), kab and the real-space forces
+    // Before the structure factors are complete: what the prep kernel and the
+    // previous step left -- the records, and (MD step) the inputs of the closing
+    // update (thread t: particles t, t + NT, .. of the tile) and the thermostat's
+    // noise.  With a programmatic launch the blocks get here when every block of
+    // the structure-factor kernel has found the prep kernel complete; loads past
+    // L1, which may hold an earlier step's lines.
     int tq[PT];
     uint4 p[PT];
 #pragma unroll
     for (int q = 0; q < PT; ++q) {
         tq[q] = threadIdx.x / SPLIT + q * (NT / SPLIT);
         p[q] = make_uint4(0, 0, 0, 0);
-        if (tl.count > 0) p[q] = rec[tl.first + min(tq[q], tl.count - 1)];
+        if (tl.count > 0) p[q] = __ldcg(rec + tl.first + min(tq[q], tl.count - 1));
     }
-    // neighbour-list MD step: the inputs of the closing update (thread t:
-    // particles t, t + NT, .. of the tile) and the thermostat's noise, fetched
-    // before the wave-vector loop -- nothing writes them during this kernel
     const bool nhm = md.md_pos && md.nh && S.thermostat == RBE_THERMO_NOSE_HOOVER;
     float4 e_fr[EP], e_v[EP], e_r[EP];
     MdNoise e_z[EP];
@@ -278,14 +298,20 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
         e_r[e] = e_fr[e];
         e_z[e] = MdNoise{0.f, 0.f, 0.f, false};
         const int te = threadIdx.x + e * NT;
-        if (md.freal && te < tl.count) {
+        if (md.freal && md.md_pos && te < tl.count) {
             const int o = tl.first + te;
-            e_fr[e] = md.freal[o];
-            if (md.md_pos) {
-                e_v[e] = md.md_vel[o];
-                e_r[e] = md.md_pos[o];
-                if (!nhm) e_z[e] = md_noise(S, *md.cur_step, o);
-            }
+            e_v[e] = __ldcg(md.md_vel + o);
+            e_r[e] = __ldcg(md.md_pos + o);
+            if (!nhm) e_z[e] = md_noise(S, __ldcg((const unsigned long long*)md.cur_step), o);
+        }
+    }
+    pdl_wait();                                     // rho(k), kab and the real-space forces
+    pdl_trigger();                                  // the next step's prep kernel may be scheduled
+    if (md.freal) {
+#pragma unroll
+        for (int e = 0; e < EP; ++e) {
+            const int te = threadIdx.x + e * NT;
+            if (te < tl.count) e_fr[e] = md.freal[tl.first + te];
         }
     }
     float fx[PT], fy[PT], fz[PT], ph[PT];
@@ -395,58 +421,43 @@ void launch_sample(cudaStream_t st, const SysDev* sys, int nsys, int ktot, const
 }
 
 // The k-batch (ksamp) and coef_scale / k^2 (kcoef) come from the prep kernel.
-// A launch configuration, with programmatic stream serialisation if pdl.
-struct PdlConfig {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute attr[1]{};
-    PdlConfig(dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl) {
-        cfg.gridDim = grid;
-        cfg.blockDim = block;
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = pdl ? 1 : 0;
-    }
-};
-
-void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
+void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
                       const int4* ksamp, const double* kcoef, const uint4* fx,
                       unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl) {
-    if (nchunks <= 0 || ltiles <= 0) return;
-    PdlConfig c(dim3(nchunks, ltiles), dim3(kLTile * kRhoHalves), 0, st, pdl);
+    if (ntiles <= 0 || ktiles <= 0) return;
+    PdlConfig c(dim3(ntiles, ktiles), dim3(kRhoThreads), 0, st, pdl);
     if (one)
-        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<true>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab);
+        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<true>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab, run);
     else
-        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<false>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab);
+        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<false>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab,
+                           run);
 }
 
 template <int R>
-static void rho_list_r(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
+static void rho_list_r(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
                        const int4* ksamp, const double* kcoef, const uint4* fx,
                        unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
                        bool pdl) {
-    const int nrho = nchunks * ltiles;
-    PdlConfig c(dim3(nrho + a.nlblk), dim3(kLTile), 0, st, pdl);
+    const int nrho = ntiles * ktiles, nlist = (a.nlblk + 1) / 2;
+    PdlConfig c(dim3(nrho + nlist), dim3(kRhoThreads), 0, st, pdl);
     if (one)
         cudaLaunchKernelEx(&c.cfg, k_rho_list<R, true>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab, a,
-                           nchunks, nrho, a.nlblk);
+                           ntiles, run, nrho, nlist);
     else
         cudaLaunchKernelEx(&c.cfg, k_rho_list<R, false>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab,
-                           a, nchunks, nrho, a.nlblk);
+                           a, ntiles, run, nrho, nlist);
 }
 
-void launch_rho_list(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
+void launch_rho_list(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
                      const int4* ksamp, const double* kcoef, const uint4* fx,
                      unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
                      bool pdl) {
-    if (nchunks <= 0 || ltiles <= 0) return;
+    if (ntiles <= 0 || ktiles <= 0) return;
     switch (a.lsplit) {
-        case 2: rho_list_r<2>(st, one, w, nchunks, ltiles, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
-        case 4: rho_list_r<4>(st, one, w, nchunks, ltiles, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
-        case 8: rho_list_r<8>(st, one, w, nchunks, ltiles, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
-        default: rho_list_r<1>(st, one, w, nchunks, ltiles, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+        case 2: rho_list_r<2>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+        case 4: rho_list_r<4>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+        case 8: rho_list_r<8>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+        default: rho_list_r<1>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
     }
 }
 

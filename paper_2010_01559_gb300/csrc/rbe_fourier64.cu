@@ -152,10 +152,13 @@ k_rho_f64_tab(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
             }
         }
     }
+    unsigned long long* dst =
+        rho_fx + (size_t)((blockIdx.x * gridDim.y + blockIdx.y) % kRhoCopies) * S.rho_stride +
+        2 * S.off_k;
 #pragma unroll
     for (int r = 0; r < KR; ++r) {
         const int l = l0 + r * kTabThreads + threadIdx.x;
-        if (l < S.P) rho_accumulate(rho_fx + 2 * (S.off_k + l), re[r], im[r], S.rho_scale);
+        if (l < S.P) rho_accumulate(dst + 2 * l, re[r], im[r], S.rho_scale);
     }
 }
 
@@ -223,7 +226,7 @@ k_force_f64_tab(const __grid_constant__ Work w, const double4* __restrict__ rec6
         for (int k = threadIdx.x; k < nk; k += kTabThreads) {
             const int l = S.off_k + base + k;
             const int4 m = ksamp[l];
-            const double2 r = rho_read(rho_fx + 2 * l, S.rho_inv_scale);
+            const double2 r = rho_total(rho_fx + 2 * l, S.rho_stride, S.rho_inv_scale);
             const double c = kcoef[l];
             s_ab[k] = make_double2(c * r.y, c * r.x);
             s_mx[k] = m.x; s_my[k] = m.y; s_mz[k] = m.z;
@@ -284,7 +287,7 @@ k_force_f64(const __grid_constant__ Work w, const double4* __restrict__ rec64,
         for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
             const int l = S.off_k + base + k;
             const int4 m = ksamp[l];
-            const double2 r = rho_read(rho_fx + 2 * l, S.rho_inv_scale);
+            const double2 r = rho_total(rho_fx + 2 * l, S.rho_stride, S.rho_inv_scale);
             const double c = kcoef[l];
             kk[k] = make_double4(tp * m.x, tp * m.y, tp * m.z, c * r.y);
             kb[k] = c * r.x;

@@ -15,8 +15,8 @@
 //   perm   int   [N]   sorted index -> caller's index
 //   fs     float4[N]   Fourier force (xyz) and Fourier dE/dq (w), caller's order
 //   cell_cnt / cell_start  int [C + 1] over all systems' cells
-//   rho_fx int64 [2K]  rho(k_l) = (Re, Im) accumulated over all chunks with 64-bit
-//                      fixed-point atomics (integer addition is associative, so
+//   rho_fx int64 [kRhoCopies][2K]  rho(k_l) = (Re, Im), the sum of the copies,
+//                      accumulated over all blocks with 64-bit fixed-point atomics (integer addition is associative, so
 //                      the sum is bitwise reproducible), K = sum_s P_s
 //   ksamp  int4   [K] (m_x, m_y, m_z, attempts)
 //   qsum_fx int64 [nsys] sum q in fixed point (for dE/dq)
@@ -32,9 +32,15 @@
 namespace rbe {
 
 constexpr int kBlockP = 128;      // particles per block of the per-particle kernels
-constexpr int kLTile = 128;       // threads per wave-vector row of the structure-factor kernels
-constexpr int kRhoK = 2;          // wave vectors per thread of the mixed structure factors
-constexpr int kRhoKT = kLTile * kRhoK;   // wave vectors per tile of the mixed structure factors
+constexpr int kLTile = 128;       // threads per wave-vector row (FP64 and full structure factors)
+constexpr int kRhoThreads = 256;  // threads per block of the mixed structure factors
+constexpr int kRhoKT = 2 * kRhoThreads;  // wave vectors per tile: two per thread
+constexpr int kRhoStage = 512;    // particles staged per pass
+// Copies of the rho(k) accumulators that the blocks of the structure factors
+// spread their atomics over: additions to one address take about 27 SM cycles
+// each, so that the 250 blocks of a system of 8000 particles waited 8500 cycles
+// for theirs, more than their sums took.
+constexpr int kRhoCopies = 8;
 constexpr int kMaxAttempts = 32;  // bound on the (0,0,0) rejection loop
 constexpr int kErrSampler = 1;    // bits in the device error word
 constexpr int kErrList = 2;       // a neighbour list overflowed
@@ -61,11 +67,13 @@ struct SysDev {
     int off_k;              // first k sample
     int off_t;              // first table entry
     int off_part;           // first partial of the structure-factor chunks
-    int nchunk;             // structure-factor chunks of this system
+    int nchunk;             // structure-factor chunks of this system (FP64 path)
+    int nrt;                // structure-factor tiles of this system (mixed path)
+    int rho_exp;            // rho_scale = 2^rho_exp
+    int rho_stride;         // 64-bit words from one copy of the accumulators to the next
     double rho_scale;       // 64-bit fixed-point scale of the rho(k) accumulators
     double rho_inv_scale;
-    int off_b, nb;          // first per-particle block and block count (prep)
-    int off_rb, nrb;        // first real-space block and block count (FP64 path)
+    int off_b, nb;          // first per-particle block and block count
     int off_sg, nsg;        // first real-space segment and segment count (mixed path)
     int off_lb, nlb;        // first neighbour-list block and block count
     // FP32 copies of the pair and Langevin constants, rounded once on the host
@@ -282,6 +290,12 @@ __device__ __forceinline__ void langevin_update(float4* md_pos, float4* md_vel,
     md_pos[o] = rp;
 }
 
+// a + b as a float pair (s, e): s + e = a + b exactly (Knuth's two-sum).
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
+}
+
 // Programmatic dependent launch (a kernel launched with programmatic stream
 // serialisation may start while its predecessor in the stream finishes):
 // pdl_wait blocks until every prerequisite grid has completed and its writes
@@ -396,9 +410,25 @@ __device__ __forceinline__ int4 sample_one_smem(const SysDev& S, const uint32_t*
 }
 
 // ------------------------------------------------------------- launchers
+// A launch configuration, with programmatic stream serialisation if pdl.
+struct PdlConfig {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1]{};
+    PdlConfig(dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl) {
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = pdl ? 1 : 0;
+    }
+};
+
 // `one` selects the single-system kernels (Work.one / Work.tile), else tables.
 // cells / sorting (rbe_cells.cu)
-// The prep kernels also clear the rho(k) accumulators (2 * nrho words) and,
+// The prep kernels also clear the rho(k) accumulators (nrho words) and,
 // with want_q, add each system's charges to qsum_fx (cleared by the caller).
 struct PrepArgs {
     double2* blk_q;
@@ -434,7 +464,8 @@ struct PrepArgs {
     int ncell, ntot;         // cells and particles of all systems (index checks)
 };
 void launch_prep_mixed(cudaStream_t st, bool one, const Work& w, int nblk, const float4* pos_q,
-                       uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa);
+                       uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa,
+                       bool pdl = false);
 void launch_prep_f64(cudaStream_t st, bool one, const Work& w, int nblk, const double4* pos_q,
                      double4* fx64, uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa);
 // Neighbour-list evaluations: cell ids and slots (cid, rank, cell_cnt) of the
@@ -456,6 +487,34 @@ void launch_order(cudaStream_t st, int n, const int* cid, const int* cell_start,
                   double4* spos64, int* perm, const int* list_flag = nullptr,
                   int* iperm = nullptr, int* err = nullptr);
 
+// The sort as one cluster (rbe_cells.cu): scan, scatter and in-cell order, with
+// assign preceded by launch_cell_assign's work; step_dev and list_flag as for
+// launch_scan.
+constexpr int kSortMaxN = 1 << 16;
+constexpr int kSortMaxCells = 1 << 16;
+struct SortArgs {
+    Work w;                  // particle tiles (assign)
+    int ntile, assign;
+    int n, ncell;
+    const uint4* fx;
+    const double4* fx64;     // nullable: FP64 path
+    int* cid;
+    int* rank;
+    int* cell_cnt;
+    int* cell_start;
+    int* perm_tmp;
+    int* perm;
+    int* iperm;              // nullable
+    uint4* spos;
+    double4* spos64;
+    uint64_t* step_dev;      // nullable
+    const uint64_t* cur_step;
+    const int* list_flag;    // nullable
+    int* err;
+};
+bool sort_cluster_ok(bool one);
+void launch_sort(cudaStream_t st, bool one, const SortArgs& a);
+
 // Neighbour-list build (rbe_real.cu): for every sorted particle the sorted
 // indices of the particles within r_c + skin among its 27 neighbour cells.
 struct ListArgs {
@@ -471,6 +530,8 @@ struct ListArgs {
     const int* perm;         // sorted -> caller index
     unsigned long long* stats;   // [0] builds, [1] largest count
     int* err;
+    float4* freal;           // nullable (MD step): also the real-space force over the new
+                             // list, caller's order
 };
 void launch_list_build(cudaStream_t st, bool one, const ListArgs& la);
 
@@ -490,9 +551,24 @@ __device__ __forceinline__ double2 rho_read(const unsigned long long* src, doubl
                         (double)(long long)__ldcg(src + 1) * inv_scale);
 }
 
+// The same, summed over the copies.
+__device__ __forceinline__ double2 rho_total(const unsigned long long* src, int stride,
+                                             double inv_scale) {
+    unsigned long long re = 0ull, im = 0ull;
+#pragma unroll
+    for (int c = 0; c < kRhoCopies; ++c) {
+        const ulonglong2 v = __ldcg((const ulonglong2*)(src + (size_t)c * stride));
+        re += v.x;
+        im += v.y;
+    }
+    return make_double2((double)(long long)re * inv_scale, (double)(long long)im * inv_scale);
+}
+
 // pdl: launched with programmatic stream serialisation (the kernels wait for
 // their predecessor's results before reading them).
-void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
+// ntiles, ktiles: tiles of particles (w) and of kRhoKT wave vectors; run:
+// particles per FP32 run of the sums (a power of two up to kRhoStage).
+void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
                       const int4* ksamp, const double* kcoef, const uint4* fx,
                       unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl = false);
 // FP64 path (rbe_fourier64.cu): chunk = particles per chunk, pmax and mcap the
@@ -535,8 +611,8 @@ void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk
 constexpr int kSegChunks = 2;
 
 struct RealArgs {
-    Work w;                  // real-space tiles of kBlockP / split particles (FP64 path)
-    int nrblk;
+    Work w;                  // tiles of kBlockP particles (FP64 path)
+    int npblk;
     int split;               // threads per particle, mixed path (1, 3 or 9)
     int split64;             // threads per particle, FP64 path (4, 8, 16 or 32)
     int ncell;               // cells over all systems
@@ -589,7 +665,7 @@ void launch_real_f64(cudaStream_t st, bool one, const RealArgs& a);
 void launch_real_list(cudaStream_t st, bool one, const RealArgs& a);
 // The MD step's structure factors and its pass over a standing list in one
 // launch (rbe_fourier.cu); `a` as for launch_real_list with list_when = 0.
-void launch_rho_list(cudaStream_t st, bool one, const Work& w, int nchunks, int ltiles,
+void launch_rho_list(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
                      const int4* ksamp, const double* kcoef, const uint4* fx,
                      unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
                      bool pdl);
@@ -626,6 +702,6 @@ void launch_observables(cudaStream_t st, const SysDev& S, const uint4* fx, int f
 void launch_energy(cudaStream_t st, bool one, const Work& w, int nsys, const int4* ksamp,
                    const unsigned long long* rho_fx, const double2* blk_e,
                    const double2* blk_q, const double2* blk_w, int parts, int per_cell,
-                   double* E_out, double* W_out);
+                   int sub64, double* E_out, double* W_out);
 
 }  // namespace rbe

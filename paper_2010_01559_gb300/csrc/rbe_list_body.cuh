@@ -22,7 +22,7 @@ namespace rbe {
 // real-space and LJ energies and virials, as the cell-scan pass does.
 //
 // list_body: the work of one tile (kBlockP threads, tid = the thread's index
-// in them; it synchronises the block), for the pass's own kernel and for the
+// in them; in its FM form it synchronises the block), for the pass's own kernel and for the
 // fused structure-factor + list launch of the MD step.
 //
 // PAD: the slots of a batch past the particle's count stand for the particle
@@ -115,17 +115,17 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
                 wl += __shfl_down_sync(0xffffffffu, wl, o, R);
             }
         }
-        __shared__ float4 s_f[T];
-        __shared__ float4 s_e[FM ? T : 1];
-        if (p < tl.count && l == 0) {
-            s_f[p] = make_float4(fx, fy, fz, ph);
-            if constexpr (FM) s_e[p] = make_float4(ec, el, wc, wl);
-        }
-        __syncthreads();
-        if ((int)tid < tl.count) {
-            const float4 f = s_f[tid];
-            fx = f.x; fy = f.y; fz = f.z; ph = f.w;
-            if constexpr (FM) {
+        if constexpr (FM) {
+            __shared__ float4 s_f[T];
+            __shared__ float4 s_e[T];
+            if (p < tl.count && l == 0) {
+                s_f[p] = make_float4(fx, fy, fz, ph);
+                s_e[p] = make_float4(ec, el, wc, wl);
+            }
+            __syncthreads();
+            if ((int)tid < tl.count) {
+                const float4 f = s_f[tid];
+                fx = f.x; fy = f.y; fz = f.z; ph = f.w;
                 const float4 e = s_e[tid];
                 ec = e.x; el = e.y; wc = e.z; wl = e.w;
             }
@@ -133,9 +133,10 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
     }
     if constexpr (!FM) {
         // the real-space force in the caller's order, for the Fourier-force
-        // kernel that adds its part and applies the thermostat
-        if ((int)tid < tl.count) {
-            const int o = a.perm[tl.first + tid];
+        // kernel that adds its part and applies the thermostat (the first of the
+        // particle's lanes stores it: no block synchronisation in this form)
+        if (p < tl.count && l == 0) {
+            const int o = a.perm[tl.first + p];
             if (RBE_IN_BOUNDS(o, a.nbr_stride, a.err)) a.freal[o] = make_float4(fx, fy, fz, 0.f);
         }
     } else {
@@ -175,8 +176,8 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
 template <int R, bool ONE, bool FM>
 __global__ void __launch_bounds__(kBlockP) k_real_list(const __grid_constant__ RealArgs a) {
     if constexpr (!FM) {
-        // launched twice per step: right after the prep kernel (works when the
-        // list stands) and after the rebuild (works when the list was rebuilt)
+        // right after the prep kernel: works when the list stands (over a
+        // rebuilt list the build adds the pair terms itself)
         if ((*a.list_flag != 0) != (a.list_when != 0)) return;
     } else {
         if (a.flag_clear && blockIdx.x == 0 && threadIdx.x == 0) *a.flag_clear = 0;

@@ -383,17 +383,38 @@ k_real_seg(const __grid_constant__ RealArgs a) {
 // kernel tests that), so every pair within r_c stays in the list between
 // builds.  Cells have side >= r_c + skin.
 
-// One thread per sorted particle: the 27 neighbour cells as 9 rows of three
-// x-adjacent cells (one row, once, with one cell per edge), every j != i whose
-// fixed-point minimum-image distance is within r_c + skin, in scan order.  The
-// record of the build is kept, by caller index, as the reference of the
-// displacement test.
-template <bool ONE>
+// R lanes per sorted particle (one at large N) take every R-th candidate of the
+// 27 neighbour cells, 9 rows of three x-adjacent cells (one row, once, with one
+// cell per edge): every j != i whose fixed-point minimum-image distance is within
+// r_c + skin, in scan order.  The pairs within r_c go to the front of the
+// particle's slots, those in the skin to the back; the skin block then moves up
+// behind the first, so that the lanes of a warp in the list pass mostly agree on
+// the cutoff branch at the same position in their lists.  The record of the build
+// is kept, by caller index, as the reference of the displacement test.  PASS (MD
+// step): the lanes then add the pair terms of the particle over the list they
+// have just written, so that the step needs no further launch behind the rebuild
+// (nearly always an empty one).
+//
+// What bounds it: at 2^20 particles writing the slots (a thread per particle
+// writes its warp's entries of a slot near each other; lanes sharing a particle
+// scatter them), below about 10^5 the serial walk over some 400 candidates:
+// N = 8001 100 -> 22 us with 16 lanes (and four candidates of a lane in flight);
+// 4 lanes at N = 50021 139 us, against 120 with one.
+constexpr int kBuildU = 4;
+
+template <int R, bool ONE, bool PASS>
 __global__ void __launch_bounds__(kBlockP) k_list_build(const __grid_constant__ ListArgs la) {
     if (!*la.list_flag) return;
-    const Tile tl = tile_of<ONE>(la.w);
+    constexpr int T = kBlockP / R;                       // particles per block
+    // block (x, y): particles T y .. T y + T - 1 of tile x (kBlockP particles)
+    Tile tl = tile_of<ONE>(la.w);
+    tl.first += (int)blockIdx.y * T;
+    tl.count = max(0, min(T, tl.count - (int)blockIdx.y * T));
     const SysDev& S = sys_of<ONE>(la.w, tl.sys);
-    const int t = threadIdx.x;
+    const int t = threadIdx.x / R, l = threadIdx.x % R;
+    const unsigned lane = threadIdx.x & 31;
+    const unsigned gmask = R == 32 ? 0xffffffffu : ((1u << R) - 1u) << (lane & ~(R - 1u));
+    const unsigned below = gmask & ((1u << lane) - 1u);
     int cnt = 0;
     if (t < tl.count) {
         const int i = tl.first + t;
@@ -402,57 +423,126 @@ __global__ void __launch_bounds__(kBlockP) k_list_build(const __grid_constant__ 
         const int cx = (int)(((unsigned long long)si.x * (unsigned long long)ncd) >> 32);
         const int cy = (int)(((unsigned long long)si.y * (unsigned long long)ncd) >> 32);
         const int cz = (int)(((unsigned long long)si.z * (unsigned long long)ncd) >> 32);
-        const float Lu = S.L_over_2_32, cut2 = S.f_list_cut2;
-        const int dlo = ncd < 3 ? 0 : -1, dhi = ncd < 3 ? 0 : 1;
+        const float Lu = S.L_over_2_32, cut2 = S.f_list_cut2, rc2 = S.f_rc2;
         int* out = la.nbr + i;
         const size_t stride = (size_t)la.stride;
-        // one sweep: the pairs within r_c go to the front of the particle's
-        // slots, those in the skin to the back; the skin block then moves up
-        // behind the first, so that the lanes of a warp in the list pass mostly
-        // agree on the cutoff branch at the same position in their lists
-        const float rc2 = S.f_rc2;
-        int n_in = 0, n_sk = 0;
-        for (int dz = dlo; dz <= dhi; ++dz) {
-            for (int dy = dlo; dy <= dhi; ++dy) {
-                const int zz = wrapc(cz + dz, ncd), yy = wrapc(cy + dy, ncd);
-                int r0, e0, r1, e1;
-                row_ranges(la.cell_start, S.off_c + (zz * ncd + yy) * ncd, cx, ncd, r0, e0, r1, e1);
-                for (int part = 0; part < 2; ++part) {
-                    const int b = part ? r1 : r0, e = part ? e1 : e0;
-                    for (int j = b; j < e; ++j) {
-                        if (!RBE_IN_BOUNDS(j, la.stride, la.err)) break;
-                        const uint4 sj = __ldg(la.spos + j);
-                        const float dx = (float)(int32_t)(sj.x - si.x) * Lu;
-                        const float dyy = (float)(int32_t)(sj.y - si.y) * Lu;
-                        const float dzz = (float)(int32_t)(sj.z - si.z) * Lu;
-                        const float r2 = fmaf(dx, dx, fmaf(dyy, dyy, dzz * dzz));
-                        if (r2 < cut2 && j != i) {
-                            if (n_in + n_sk < la.cap) {
-                                const int slot = r2 < rc2 ? n_in : la.cap - 1 - n_sk;
-                                out[(size_t)slot * stride] = j;
-                            }
+        int n_in = 0, n_sk = 0;                          // the same in the particle's lanes
+        const int nrow = ncd < 3 ? 1 : 9;
+#pragma unroll 1
+        for (int r = 0; r < nrow; ++r) {
+            const int dz = ncd < 3 ? 0 : r / 3 - 1, dy = ncd < 3 ? 0 : r % 3 - 1;
+            const int zz = wrapc(cz + dz, ncd), yy = wrapc(cy + dy, ncd);
+            int r0, e0, r1, e1;
+            row_ranges(la.cell_start, S.off_c + (zz * ncd + yy) * ncd, cx, ncd, r0, e0, r1, e1);
+            const int n0 = e0 - r0, n = n0 + (e1 - r1);
+            // kBuildU candidates per lane at a time, their records in flight together
+            for (int k0 = 0; k0 < n; k0 += R * kBuildU) {
+                uint4 sj[kBuildU];
+                int jj[kBuildU];
+#pragma unroll
+                for (int u = 0; u < kBuildU; ++u) {
+                    const int k = k0 + u * R + l;
+                    int j = k < n0 ? r0 + k : r1 + (k - n0);
+                    if (k >= n || !RBE_IN_BOUNDS(j, la.stride, la.err)) j = i;   // not a pair
+                    jj[u] = j;
+                    sj[u] = __ldg(la.spos + j);
+                }
+#pragma unroll
+                for (int u = 0; u < kBuildU; ++u) {
+                    const int j = jj[u];
+                    const float dx = (float)(int32_t)(sj[u].x - si.x) * Lu;
+                    const float dyy = (float)(int32_t)(sj[u].y - si.y) * Lu;
+                    const float dzz = (float)(int32_t)(sj[u].z - si.z) * Lu;
+                    const float r2 = fmaf(dx, dx, fmaf(dyy, dyy, dzz * dzz));
+                    const bool near = r2 < cut2 && j != i;
+                    if constexpr (R == 1) {
+                        if (near) {
+                            if (n_in + n_sk < la.cap)
+                                out[(size_t)(r2 < rc2 ? n_in : la.cap - 1 - n_sk) * stride] = j;
                             if (r2 < rc2) ++n_in; else ++n_sk;
                         }
+                    } else {
+                        const unsigned m = __ballot_sync(gmask, near) & gmask;
+                        if (!m) continue;                // none of the lanes has one
+                        const unsigned m_in = __ballot_sync(gmask, near && r2 < rc2) & gmask;
+                        const unsigned m_sk = m & ~m_in;
+                        const int c_in = __popc(m_in), c_sk = __popc(m_sk);
+                        if (near) {
+                            // (an overflowing list is reported; entries stay in the slots)
+                            const int k_in = __popc(m_in & below), k_sk = __popc(m_sk & below);
+                            if (r2 < rc2) {
+                                if (n_in + k_in + n_sk + c_sk < la.cap)
+                                    out[(size_t)(n_in + k_in) * stride] = j;
+                            } else if (n_in + c_in + n_sk + k_sk < la.cap) {
+                                out[(size_t)(la.cap - 1 - (n_sk + k_sk)) * stride] = j;
+                            }
+                        }
+                        n_in += c_in;
+                        n_sk += c_sk;
                     }
                 }
             }
         }
         cnt = n_in + n_sk;
+        if constexpr (R > 1) __syncwarp(gmask);
         if (cnt <= la.cap) {
-            // move the skin block [cap - n_sk, cap) to [n_in, n_in + n_sk);
-            // the destination never lies above the source: ascending is safe
-            for (int k = 0; k < n_sk; ++k)
-                out[(size_t)(n_in + k) * stride] = out[(size_t)(la.cap - n_sk + k) * stride];
+            // move the skin block [cap - n_sk, cap) to [n_in, n_in + n_sk); the
+            // destination never lies above the source: ascending is safe
+            for (int k0 = 0; k0 < n_sk; k0 += R) {
+                const int k = k0 + l;
+                const int j = k < n_sk ? out[(size_t)(la.cap - n_sk + k) * stride] : 0;
+                if constexpr (R > 1) __syncwarp(gmask);
+                if (k < n_sk) out[(size_t)(n_in + k) * stride] = j;
+                if constexpr (R > 1) __syncwarp(gmask);
+            }
         }
-        la.ncnt[i] = min(cnt, la.cap);
         const int o = la.perm[i];
-        if (RBE_IN_BOUNDS(o, la.stride, la.err))
-            la.sref[o] = si;                // by caller index: the prep kernel reads it in order
-        if (cnt > la.cap) atomicOr(la.err, kErrList);
+        if (l == 0) {
+            la.ncnt[i] = min(cnt, la.cap);
+            if (RBE_IN_BOUNDS(o, la.stride, la.err))
+                la.sref[o] = si;            // by caller index: the prep kernel reads it in order
+            if (cnt > la.cap) atomicOr(la.err, kErrList);
+        }
+        if constexpr (PASS) {
+            PairConst kc;
+            kc.rc2 = S.f_rc2;
+            kc.lj_rc2 = S.lj_eps != 0.0 ? S.f_lj_rc2 : 0.f;
+            kc.alpha = S.f_alpha;
+            kc.sa = S.f_sqrt_alpha;
+            kc.two_sa_spi = S.f_two_sa_spi;
+            kc.lB = S.f_lB;
+            kc.lj_s2 = S.f_lj_sigma2;
+            kc.lj_eps = S.f_lj_eps;
+            kc.lj_shift = S.f_lj_shift;
+            kc.vir = false;
+            PairAcc acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            const float lbqi = kc.lB * __uint_as_float(si.w);
+            const int ne = min(cnt, la.cap);
+            for (int k0 = l; k0 < ne; k0 += R * kBuildU) {
+                uint4 sj[kBuildU];
+#pragma unroll
+                for (int u = 0; u < kBuildU; ++u) {
+                    int j = k0 + u * R < ne ? out[(size_t)(k0 + u * R) * stride] : i;
+                    if (!RBE_IN_BOUNDS(j, la.stride, la.err)) j = i;
+                    sj[u] = __ldg(la.spos + j);
+                }
+#pragma unroll
+                for (int u = 0; u < kBuildU; ++u) pair_fixed(si, sj[u], Lu, lbqi, kc, acc);
+            }
+            float fx = acc.fx, fy = acc.fy, fz = acc.fz;
+#pragma unroll
+            for (int d = R / 2; d > 0; d >>= 1) {
+                fx += __shfl_down_sync(gmask, fx, d, R);
+                fy += __shfl_down_sync(gmask, fy, d, R);
+                fz += __shfl_down_sync(gmask, fz, d, R);
+            }
+            if (l == 0 && RBE_IN_BOUNDS(o, la.stride, la.err))
+                la.freal[o] = make_float4(fx, fy, fz, 0.f);
+        }
     }
     const unsigned wmax = __reduce_max_sync(0xffffffffu, (unsigned)cnt);
-    if ((t & 31) == 0 && wmax) atomicMax(la.stats + 1, (unsigned long long)wmax);
-    if (blockIdx.x == 0 && t == 0) atomicAdd(la.stats, 1ull);
+    if (lane == 0 && wmax) atomicMax(la.stats + 1, (unsigned long long)wmax);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(la.stats, 1ull);
 }
 
 // ----------------------------------------------------------------- energy
@@ -466,7 +556,7 @@ template <bool ONE>
 __global__ void k_energy(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
                          const unsigned long long* __restrict__ rho_fx,
                          const double2* __restrict__ blk_e, const double2* __restrict__ blk_q,
-                         const double2* __restrict__ blk_w, int parts, int per_cell,
+                         const double2* __restrict__ blk_w, int parts, int per_cell, int sub64,
                          double* __restrict__ E_out, double* __restrict__ W_out) {
     const SysDev& S = sys_of<ONE>(w, blockIdx.x);
     double ef = 0.0, ec = 0.0, elj = 0.0, q1 = 0.0, q2 = 0.0;
@@ -474,7 +564,7 @@ __global__ void k_energy(const __grid_constant__ Work w, const int4* __restrict_
         const double tp = 2.0 * M_PI * S.invL;
         for (int l = threadIdx.x; l < S.P; l += blockDim.x) {
             const int4 m = ksamp[S.off_k + l];
-            const double2 r = rho_read(rho_fx + 2 * (S.off_k + l), S.rho_inv_scale);
+            const double2 r = rho_total(rho_fx + 2 * (S.off_k + l), S.rho_stride, S.rho_inv_scale);
             const double k2 = tp * tp * ((double)m.x * m.x + (double)m.y * m.y + (double)m.z * m.z);
             ef += 0.5 * (S.coef_scale / k2) * (r.x * r.x + r.y * r.y);
         }
@@ -484,9 +574,10 @@ __global__ void k_energy(const __grid_constant__ Work w, const int4* __restrict_
             q2 += v.y;
         }
     }
-    // partials per FP64 block (0), per segment block (1) or per list block (2)
-    const int off = per_cell == 2 ? S.off_lb : (per_cell ? S.off_sg * kSegChunks : S.off_rb);
-    const int nb = per_cell == 2 ? S.nlb : (per_cell ? S.nsg * kSegChunks : S.nrb);
+    // partials per FP64 block (0: sub64 for each particle tile), per segment
+    // block (1) or per list block (2)
+    const int off = per_cell == 2 ? S.off_lb : (per_cell ? S.off_sg * kSegChunks : S.off_b * sub64);
+    const int nb = per_cell == 2 ? S.nlb : (per_cell ? S.nsg * kSegChunks : S.nb * sub64);
     double wc = 0.0, wlj = 0.0;
     if (blk_e)
         for (int b = threadIdx.x; b < nb; b += blockDim.x) {
@@ -593,23 +684,36 @@ void launch_real_list(cudaStream_t st, bool one, const RealArgs& a) {
     }
 }
 
+template <int R>
+static void list_build_r(cudaStream_t st, bool one, const ListArgs& la) {
+    const dim3 grid(la.nblk, R);
+    if (la.freal) {
+        if (one) k_list_build<R, true, true><<<grid, kBlockP, 0, st>>>(la);
+        else k_list_build<R, false, true><<<grid, kBlockP, 0, st>>>(la);
+    } else {
+        if (one) k_list_build<R, true, false><<<grid, kBlockP, 0, st>>>(la);
+        else k_list_build<R, false, false><<<grid, kBlockP, 0, st>>>(la);
+    }
+}
+
 void launch_list_build(cudaStream_t st, bool one, const ListArgs& la) {
     if (la.nblk <= 0) return;
-    if (one) k_list_build<true><<<la.nblk, kBlockP, 0, st>>>(la);
-    else k_list_build<false><<<la.nblk, kBlockP, 0, st>>>(la);
+    // 16 lanes per particle while that fits in 2048 threads per SM
+    if ((long long)la.nblk * kBlockP * 16 > 152LL * 2048) list_build_r<1>(st, one, la);
+    else list_build_r<16>(st, one, la);
 }
 
 void launch_energy(cudaStream_t st, bool one, const Work& w, int nsys, const int4* ksamp,
                    const unsigned long long* rho_fx, const double2* blk_e,
                    const double2* blk_q, const double2* blk_w, int parts, int per_cell,
-                   double* E_out, double* W_out) {
+                   int sub64, double* E_out, double* W_out) {
     if (nsys <= 0) return;
     if (one)
         k_energy<true><<<nsys, 256, 0, st>>>(w, ksamp, rho_fx, blk_e, blk_q, blk_w, parts,
-                                             per_cell, E_out, W_out);
+                                             per_cell, sub64, E_out, W_out);
     else
         k_energy<false><<<nsys, 256, 0, st>>>(w, ksamp, rho_fx, blk_e, blk_q, blk_w, parts,
-                                              per_cell, E_out, W_out);
+                                              per_cell, sub64, E_out, W_out);
 }
 
 }  // namespace rbe

@@ -88,7 +88,11 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     constexpr int T = kBlockP / G;               // particles per block
     __shared__ int s_hit[T][kHitCap];
     __shared__ double4 s_f[T];
-    const Tile tl = tile_of<ONE>(a.w);
+    // block (x, y): particles T y .. T y + T - 1 of tile x (kBlockP particles)
+    Tile tl = tile_of<ONE>(a.w);
+    tl.first += (int)blockIdx.y * T;
+    tl.count = max(0, min(T, tl.count - (int)blockIdx.y * T));
+    const int blk = blockIdx.x * G + blockIdx.y;         // its energy / virial partials
     const SysDev& S = sys_of<ONE>(a.w, tl.sys);
     const int g = threadIdx.x % G, t = threadIdx.x / G;
     const bool active = t < tl.count;
@@ -265,12 +269,12 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     if constexpr (EN) {
         if (a.blk_e) {
             const double2 r = block_sum2_real(owner ? acc.ec : 0.0, owner ? acc.elj : 0.0);
-            if (threadIdx.x == 0) a.blk_e[blockIdx.x] = r;
+            if (threadIdx.x == 0) a.blk_e[blk] = r;
         }
         if (a.blk_w) {
             __syncthreads();                            // the partial buffers are reused
             const double2 r = block_sum2_real(owner ? acc.wc : 0.0, owner ? acc.wlj : 0.0);
-            if (threadIdx.x == 0) a.blk_w[blockIdx.x] = r;
+            if (threadIdx.x == 0) a.blk_w[blk] = r;
         }
     }
 }
@@ -278,17 +282,18 @@ k_real_f64(const __grid_constant__ RealArgs a) {
 template <int G>
 static void real_f64_g(cudaStream_t st, bool one, const RealArgs& a) {
     const bool en = a.phi_out64 || a.blk_e || a.blk_w;
+    const dim3 grid(a.npblk, G);
     if (one) {
-        if (en) k_real_f64<G, true, true><<<a.nrblk, kBlockP, 0, st>>>(a);
-        else k_real_f64<G, true, false><<<a.nrblk, kBlockP, 0, st>>>(a);
+        if (en) k_real_f64<G, true, true><<<grid, kBlockP, 0, st>>>(a);
+        else k_real_f64<G, true, false><<<grid, kBlockP, 0, st>>>(a);
     } else {
-        if (en) k_real_f64<G, false, true><<<a.nrblk, kBlockP, 0, st>>>(a);
-        else k_real_f64<G, false, false><<<a.nrblk, kBlockP, 0, st>>>(a);
+        if (en) k_real_f64<G, false, true><<<grid, kBlockP, 0, st>>>(a);
+        else k_real_f64<G, false, false><<<grid, kBlockP, 0, st>>>(a);
     }
 }
 
 void launch_real_f64(cudaStream_t st, bool one, const RealArgs& a) {
-    if (a.nrblk <= 0) return;
+    if (a.npblk <= 0) return;
     switch (a.split64) {
         case 4: real_f64_g<4>(st, one, a); break;
         case 8: real_f64_g<8>(st, one, a); break;

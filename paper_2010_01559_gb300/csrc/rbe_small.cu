@@ -46,6 +46,7 @@
 // Measured (one step, steps in one call): SMALL_FIGURES
 #include <algorithm>
 
+#include "rbe_cluster.cuh"
 #include "rbe_internal.cuh"
 #include "rbe_pair.cuh"
 
@@ -54,23 +55,6 @@ namespace rbe {
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallWarps = kSmallThreads / 32;
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t local_addr(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-// shared::cluster address in block `rank` of this block's shared address a
-__device__ __forceinline__ uint32_t remote(uint32_t a, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
 // 16 bytes into a block's shared memory, counted on that block's mbarrier
 __device__ __forceinline__ void send(uint32_t dst, const uint4& v, uint32_t bar) {
     asm volatile(
@@ -139,12 +123,6 @@ __host__ __device__ inline SmallLayout small_layout(int n, int P, int M, int cap
     L.table = L.list + small_align(2 * (size_t)L.np * cap);          // u32 [2M + 1]
     L.end = L.table + small_align(4 * (size_t)L.tab);
     return L;
-}
-
-// a + b as a float pair (s, e): s + e = a + b exactly (Knuth's two-sum).
-__device__ __forceinline__ float2 two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-    return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
 }
 
 // (ch + cl) (h + l) to FP32
