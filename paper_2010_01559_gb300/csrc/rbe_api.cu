@@ -168,6 +168,7 @@ struct rbe_ctx {
     // mixed structure factors: tiles, particles per tile and FP32 run of an
     // evaluation without (n) and with energies (e)
     int nrt = 0, rt_n = 0, rt_e = 0, run_n = 64, run_e = 64, max_rt = 0;
+    int rho_t = 256;                          // threads per block
     bool cur_set = false;                     // the chunk in effect was set, not automatic
     bool use_graph = false;
     double wait_limit = 0.0;                  // seconds a host wait may take (0: no limit)
@@ -451,31 +452,44 @@ int auto_chunk(const rbe_ctx* h, long long ntot) {
     return std::min(4096, std::max(32, p));
 }
 
-// Threads of a block that share a particle in the mixed structure factors.
-int rho_subs(int pmax) {
-    return kRhoThreads / std::max(1, (std::min(pmax, kRhoKT) + 1) / 2);
+// Mixed structure factors, for blocks of T threads (two wave vectors each):
+// threads of a block that share a particle, and the share of the lanes of the
+// warps in use that hold a wave vector.
+int rho_subs(int pmax, int T) { return T / std::max(1, (std::min(pmax, 2 * T) + 1) / 2); }
+
+double rho_fill(int pmax, int T) {
+    double lanes = 0.0;                                   // lanes in use per particle
+    for (int k0 = 0; k0 < pmax; k0 += 2 * T) {
+        const int nk = std::min(pmax - k0, 2 * T), subs = rho_subs(nk, T);
+        lanes += (double)((subs * ((nk + 1) / 2) + 31) / 32 * 32) / subs;
+    }
+    return 0.5 * pmax / std::max(lanes, 1e-9);
 }
 
-// FP32 run of the mixed structure factors without energies: as long as one pass
-// of the block holds a run per sub (a run's end costs about 30 instructions per
-// wave vector), at most 256 particles (chains of 128 terms), and shorter where
-// that leaves fewer than 128 blocks or, below 2^17 particles, more than 64.
-int auto_run(int pmax, long long ntot) {
-    const int subs = rho_subs(pmax);
+// Threads per block: 128 (more resident warps beside the list pass: the block's
+// registers come in smaller pieces) where that fills the lanes about as well.
+int auto_rho_threads(int pmax) { return rho_fill(pmax, 128) >= rho_fill(pmax, 256) - 0.05 ? 128 : 256; }
+
+// FP32 run without energies: as long as one pass of the block holds a run per
+// sub (a run's end costs about 30 instructions per wave vector), at most 256
+// particles (chains of 128 terms), and shorter where that leaves fewer than 128
+// blocks or, below 2^17 particles, more than 64.
+int auto_run(int pmax, long long ntot, int T) {
+    const int subs = rho_subs(pmax, T);
     int run = ntot < (1LL << 17) ? 64 : 256;
     while (run > 8 && (ntot < 128LL * run * subs || run * subs > kRhoStage)) run >>= 1;
     return run;
 }
 
-// Particles per block of the mixed structure factors: one pass while that gives
-// at most two blocks per SM (each block ends with two atomics per wave vector, and
-// more blocks than that cost more in atomics than they gain); beyond, whole
-// waves of four resident blocks per SM with at least 128 particles per block.
-int auto_rho_tile(int pmax, long long ntot, int run) {
-    const int pass = std::min(kRhoStage, run * rho_subs(pmax));
-    if (ntot <= 304LL * pass) return pass;
-    const long long ktiles = (pmax + kRhoKT - 1) / kRhoKT;
-    const long long slots = std::max(1LL, 608LL / ktiles);
+// Particles per block: one pass while that gives at most two blocks of 256
+// threads per SM (each block ends with two atomics per wave vector, and more
+// blocks than that cost more in atomics than they gain); beyond, whole waves of
+// resident blocks (1024 threads per SM) with at least 128 particles per block.
+int auto_rho_tile(int pmax, long long ntot, int run, int T) {
+    const int pass = std::min(kRhoStage, run * rho_subs(pmax, T));
+    const long long ktiles = (pmax + 2 * T - 1) / (2 * T);
+    if (ntot * ktiles <= 304LL * (256 / T) * pass) return pass;
+    const long long slots = std::max(1LL, 152LL * (1024 / T) / ktiles);
     const long long waves = std::max(1LL, std::min(8LL, ntot / (slots * 128)));
     const long long tile = (ntot + slots * waves - 1) / (slots * waves);
     return (int)std::max<long long>(pass, std::min<long long>(4096, (tile + 7) / 8 * 8));
@@ -537,8 +551,9 @@ rbe_status prepare(rbe_ctx* h, int n) {
         return RBE_OK;
     // mixed structure factors: particles per block and FP32 runs (with energies,
     // the chunk's, and tiles of whole runs)
-    const int run = auto_run(h->pmax, ntot), run_e = std::min(chunk, kRhoStage);
-    int rtile_n = h->rho_chunk > 0 ? chunk : auto_rho_tile(h->pmax, ntot, run);
+    const int rho_t = auto_rho_threads(h->pmax);
+    const int run = auto_run(h->pmax, ntot, rho_t), run_e = std::min(chunk, kRhoStage);
+    int rtile_n = h->rho_chunk > 0 ? chunk : auto_rho_tile(h->pmax, ntot, run, rho_t);
     const int rtile_e = (rtile_n + run_e - 1) / run_e * run_e;
     if (h->batch) rtile_n = rtile_e;              // one table serves both
     h->list_valid = false;                 // the sorted arrays are rebuilt from scratch
@@ -637,6 +652,7 @@ rbe_status prepare(rbe_ctx* h, int n) {
     h->rt_e = rtile_e;
     h->run_n = run;
     h->run_e = run_e;
+    h->rho_t = rho_t;
     h->cur_set = h->rho_chunk > 0;
     h->split = split;
     h->rsplit = rsplit;
@@ -991,23 +1007,24 @@ RealArgs make_real_args(const rbe_ctx* h, int parts) {
     return r;
 }
 
-// The mixed structure factors' work: tiles of particles and how many, the FP32 run.
+// The mixed structure factors' work and grid.
 struct RhoWork {
     Work w;
-    int ntiles, ktiles, run;
+    RhoGrid g;
 };
 
 RhoWork make_rho_work(const rbe_ctx* h, bool energies) {
     RhoWork r{};
     const int tile = energies ? h->rt_e : h->rt_n;
     r.w = make_work(h, h->d_rt, tile, 0);
-    r.ntiles = h->nrt;
+    r.g.ntiles = h->nrt;
     if (!h->batch) {
-        r.ntiles = std::max(1, (r.w.one.n + tile - 1) / tile);
-        r.w.one.nrt = r.ntiles;
+        r.g.ntiles = std::max(1, (r.w.one.n + tile - 1) / tile);
+        r.w.one.nrt = r.g.ntiles;
     }
-    r.ktiles = (h->pmax + kRhoKT - 1) / kRhoKT;
-    r.run = energies ? h->run_e : h->run_n;
+    r.g.threads = h->rho_t;
+    r.g.ktiles = (h->pmax + 2 * h->rho_t - 1) / (2 * h->rho_t);
+    r.g.run = energies ? h->run_e : h->run_n;
     return r;
 }
 
@@ -1016,8 +1033,8 @@ void launch_rho(const rbe_ctx* h, cudaStream_t st, bool mixed, bool energies, bo
     const bool one = !h->batch;
     if (mixed) {
         const RhoWork r = make_rho_work(h, energies);
-        launch_rho_mixed(st, one, r.w, r.ntiles, r.ktiles, r.run, h->d_ksamp, h->d_kcoef, h->d_fx,
-                         h->d_rho_fx, h->d_kcnt, h->d_kab, pdl);
+        launch_rho_mixed(st, one, r.w, r.g, h->d_ksamp, h->d_kcoef, h->d_fx, h->d_rho_fx,
+                         h->d_kcnt, h->d_kab, pdl);
     } else {
         launch_rho_f64(st, one, make_work(h, h->d_chunks, h->cur_chunk, 1), h->nchunks,
                        h->cur_chunk, h->pmax, h->m_max(), h->d_ksamp, h->d_fx64, h->d_rho_fx);
@@ -1139,8 +1156,8 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
             rl.list_when = 0;
             const RhoWork rw = make_rho_work(h, a.E != nullptr);
             run(RBE_K_RHO_LIST, st, [&] {
-                launch_rho_list(st, one, rw.w, rw.ntiles, rw.ktiles, rw.run, h->d_ksamp,
-                                h->d_kcoef, h->d_fx, h->d_rho_fx, h->d_kcnt, h->d_kab, rl, !prof);
+                launch_rho_list(st, one, rw.w, rw.g, h->d_ksamp, h->d_kcoef,
+                                h->d_fx, h->d_rho_fx, h->d_kcnt, h->d_kab, rl, !prof);
             });
         } else if (fourier) {
             run(RBE_K_RHO, st, [&] { launch_rho(h, st, mixed, a.E != nullptr, !prof); });
@@ -2140,9 +2157,8 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float* pos_q, rbe_tuning*
                     const RhoWork rw = make_rho_work(h, false);
                     const float t = time_kernel(h, e0, e1, [&] {
                         if (fused)
-                            launch_rho_list(h->stream, !h->batch, rw.w, rw.ntiles, rw.ktiles,
-                                            rw.run, h->d_ksamp, h->d_kcoef, h->d_fx,
-                                            h->d_rho_fx, h->d_kcnt, h->d_kab, r, false);
+                            launch_rho_list(h->stream, !h->batch, rw.w, rw.g, h->d_ksamp,
+                                            h->d_kcoef, h->d_fx, h->d_rho_fx, h->d_kcnt, h->d_kab, r, false);
                         else
                             launch_real_list(h->stream, !h->batch, r);
                     });

@@ -43,10 +43,10 @@ __global__ void k_sample(const SysDev* __restrict__ sysv, int nsys, int ktot,
 }
 
 // ----------------------------------------------------------------- rho (mixed)
-// Blocks of 256 threads: a tile of particles against a tile of up to 512 wave
-// vectors, two per thread (one shared-memory read of a particle serves two
-// pairs), so a system with P of them fills ceil(P / 2) threads; the block holds
-// floor(256 / that) such groups ("subs"), which share the particles.  That keeps
+// Blocks of T = 128 or 256 threads: a tile of particles against a tile of up to
+// 2 T wave vectors, two per thread (one shared-memory read of a particle serves
+// two pairs), so a system with P of them fills ceil(P / 2) threads; the block holds
+// floor(T / that) such groups ("subs"), which share the particles.  That keeps
 // the lanes busy at any P: with one thread row of 128 per 256 wave vectors a
 // batch of P = 100 used 39 % of them, P = 137 54 %, and P = 10 4 %.
 //
@@ -86,7 +86,7 @@ __device__ __forceinline__ void rho_add(unsigned long long* dst, const float4& s
 
 // rho_body: particle tile ctile, wave-vector tile ktile (the whole block), for
 // the kernel of its own and for the fused structure-factor + list launch.
-template <bool ONE>
+template <int T, bool ONE>
 __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__ ksamp,
                                          const double* __restrict__ kcoef,
                                          const uint4* __restrict__ fx,
@@ -94,14 +94,14 @@ __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__
                                          int* __restrict__ kcnt, float2* __restrict__ kab,
                                          int ctile, int ktile, int run) {
     __shared__ uint4 sp[kRhoStage];                  // 8 KB, then the subs' sums
-    static_assert(sizeof(sp) >= sizeof(float4) * 2 * kRhoThreads, "sums alias the stage");
+    static_assert(sizeof(sp) >= sizeof(float4) * 2 * T, "sums alias the stage");
     const Tile ch = tile_at<ONE>(w, ctile);
     const SysDev& S = sys_of<ONE>(w, ch.sys);
-    const int k0 = ktile * kRhoKT;
+    const int k0 = ktile * (2 * T);
     if (k0 >= S.P) return;                           // whole block beyond this system's P
-    const int nk = min(S.P - k0, kRhoKT);            // wave vectors of this tile
+    const int nk = min(S.P - k0, (2 * T));            // wave vectors of this tile
     const int slots = (nk + 1) / 2;
-    const int subs = kRhoThreads / slots;
+    const int subs = T / slots;
     const int sub = threadIdx.x / slots, slot = threadIdx.x - sub * slots;
     const bool work = sub < subs;
     uint32_t mx[2], my[2], mz[2];
@@ -119,30 +119,51 @@ __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__
     for (int base = 0; base < ch.count; base += stage) {
         const int cnt = min(stage, ch.count - base);
         __syncthreads();
-        for (int u = threadIdx.x; u < cnt; u += kRhoThreads) sp[u] = fx[ch.first + base + u];
+        for (int u = threadIdx.x; u < cnt; u += T) sp[u] = fx[ch.first + base + u];
         __syncthreads();
-        if (work)
+        auto terms = [&](const uint4 p, float* re, float* im) {
+            const float q = __uint_as_float(p.w);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const uint32_t ph = mx[r] * p.x + my[r] * p.y + mz[r] * p.z;
+                const float th = (float)(int32_t)ph * kTwoPiOver2p32;
+                float sn, cs;
+                __sincosf(th, &sn, &cs);
+                re[r] = fmaf(q, cs, re[r]);
+                im[r] = fmaf(q, sn, im[r]);
+            }
+        };
+        if (subs == 1) {
+            // one thread takes a run's even and odd particles side by side
+            if (work)
+                for (int j0 = 0; j0 < cnt; j0 += run) {
+                    const int j1 = min(cnt, j0 + run);
+                    float re[2] = {0.f, 0.f}, im[2] = {0.f, 0.f};
+                    float ro[2] = {0.f, 0.f}, io[2] = {0.f, 0.f};
+                    int j = j0;
+#pragma unroll 8
+                    for (; j + 1 < j1; j += 2) {
+                        terms(sp[j], re, im);
+                        terms(sp[j + 1], ro, io);
+                    }
+                    if (j < j1) terms(sp[j], re, im);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        carry(sum[r], re[r], im[r]);
+                        carry(sum[r], ro[r], io[r]);
+                    }
+                }
+        } else if (work) {
             // a run's even particles, then its odd ones, are a unit of work each
             for (int u = sub; (u >> 1) * run < cnt; u += subs) {
                 const int j0 = (u >> 1) * run + (u & 1), j1 = min(cnt, ((u >> 1) + 1) * run);
                 float re[2] = {0.f, 0.f}, im[2] = {0.f, 0.f};
 #pragma unroll 8
-                for (int j = j0; j < j1; j += 2) {
-                    const uint4 p = sp[j];
-                    const float q = __uint_as_float(p.w);
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const uint32_t ph = mx[r] * p.x + my[r] * p.y + mz[r] * p.z;
-                        const float th = (float)(int32_t)ph * kTwoPiOver2p32;
-                        float sn, cs;
-                        __sincosf(th, &sn, &cs);
-                        re[r] = fmaf(q, cs, re[r]);
-                        im[r] = fmaf(q, sn, im[r]);
-                    }
-                }
+                for (int j = j0; j < j1; j += 2) terms(sp[j], re, im);
                 carry(sum[0], re[0], im[0]);
                 carry(sum[1], re[1], im[1]);
             }
+        }
     }
     unsigned long long* dst =
         rho_fx + (size_t)(ctile % kRhoCopies) * S.rho_stride + 2 * (S.off_k + k0);
@@ -159,7 +180,7 @@ __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__
             red[(slot + slots) * subs + sub] = sum[1];
         }
         __syncthreads();
-        for (int l = threadIdx.x; l < nk; l += kRhoThreads) {
+        for (int l = threadIdx.x; l < nk; l += T) {
             float4 s = red[l * subs];
             for (int u = 1; u < subs; ++u) {
                 const float4 v = red[l * subs + u];
@@ -186,7 +207,7 @@ __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (int l = k0 + threadIdx.x; l < k0 + nk; l += kRhoThreads) {
+        for (int l = k0 + threadIdx.x; l < k0 + nk; l += T) {
             const double2 r =
                 rho_total(rho_fx + 2 * (S.off_k + l), S.rho_stride, S.rho_inv_scale);
             const double c = kcoef[S.off_k + l];
@@ -199,8 +220,8 @@ __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__
     }
 }
 
-template <bool ONE>
-__global__ void __launch_bounds__(kRhoThreads, 4)
+template <int T, bool ONE>
+__global__ void __launch_bounds__(T, 1024 / T)
 k_rho_mixed(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
             const double* __restrict__ kcoef, const uint4* __restrict__ fx,
             unsigned long long* __restrict__ rho_fx, int* __restrict__ kcnt,
@@ -208,22 +229,22 @@ k_rho_mixed(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
     pdl_wait();                                       // the prep kernel's samples and records
     pdl_trigger();                                    // the force kernel may be scheduled (and
                                                       // finds the prep kernel complete)
-    rho_body<ONE>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, blockIdx.x, blockIdx.y, run);
+    rho_body<T, ONE>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, blockIdx.x, blockIdx.y, run);
 }
 
 // ------------------------------------------- structure factors + list pass
 // The MD step's structure factors and its real-space pass over a standing
-// neighbour list in one launch of kRhoThreads-thread blocks: block b takes
+// neighbour list in one launch of T-thread blocks: block b takes
 // structure-factor work when floor((b + 1) nrho / total) > floor(b nrho /
-// total), else two tiles of the list pass, so that the two kinds are spread evenly
+// total), else T / kBlockP tiles of the list pass, so that the two kinds are spread evenly
 // over the grid and each SM holds both at once -- the structure factors keep
 // the special-function unit busy while the pair terms use the ALU and FMA
 // pipes and wait on their gathers.  The list tiles work only when the list
 // stands (over a rebuilt list the pass runs on the rebuild stream, after the
 // build), and keep the per-slot count tests: padded batches cost this
 // issue-bound launch more than they save.
-template <int R, bool ONE>
-__global__ void __launch_bounds__(kRhoThreads, 4)
+template <int T, int R, bool ONE>
+__global__ void __launch_bounds__(T, T == 128 ? 9 : 4)
 k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
            const double* __restrict__ kcoef, const uint4* __restrict__ fx,
            unsigned long long* __restrict__ rho_fx, int* __restrict__ kcnt,
@@ -236,11 +257,11 @@ k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
     const int r0 = (int)((long long)b * nrho / total);
     const int r1 = (int)((long long)(b + 1) * nrho / total);
     if (r1 > r0) {
-        rho_body<ONE>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, r0 % ntiles, r0 / ntiles, run);
+        rho_body<T, ONE>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, r0 % ntiles, r0 / ntiles, run);
         return;
     }
     if ((*a.list_flag != 0) != (a.list_when != 0)) return;
-    const int tile = 2 * (b - r1) + (int)(threadIdx.x / kBlockP);
+    const int tile = (T / kBlockP) * (b - r1) + (int)(threadIdx.x / kBlockP);
     if (tile < a.nlblk) list_body<R, ONE, false, false, 8>(a, tile, threadIdx.x % kBlockP);
 }
 
@@ -274,7 +295,9 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
     const Tile tl = tile_of<ONE>(w);
     const SysDev& S = sys_of<ONE>(w, tl.sys);
     const int sub = threadIdx.x % SPLIT;            // lane within the particle's group
-    // Before the structure factors are complete: what the prep kernel and the
+    if constexpr (SPLIT == 1) pdl_wait();           // rho(k), kab and the real-space forces
+    // Before the structure factors are complete (SPLIT > 1: in the large systems of
+    // SPLIT 1 there is nothing to hide, and the order costs registers): what the prep kernel and the
     // previous step left -- the records, and (MD step) the inputs of the closing
     // update (thread t: particles t, t + NT, .. of the tile) and the thermostat's
     // noise.  With a programmatic launch the blocks get here when every block of
@@ -305,7 +328,7 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
             if (!nhm) e_z[e] = md_noise(S, __ldcg((const unsigned long long*)md.cur_step), o);
         }
     }
-    pdl_wait();                                     // rho(k), kab and the real-space forces
+    if constexpr (SPLIT > 1) pdl_wait();
     pdl_trigger();                                  // the next step's prep kernel may be scheduled
     if (md.freal) {
 #pragma unroll
@@ -421,44 +444,67 @@ void launch_sample(cudaStream_t st, const SysDev* sys, int nsys, int ktot, const
 }
 
 // The k-batch (ksamp) and coef_scale / k^2 (kcoef) come from the prep kernel.
-void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
-                      const int4* ksamp, const double* kcoef, const uint4* fx,
-                      unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl) {
-    if (ntiles <= 0 || ktiles <= 0) return;
-    PdlConfig c(dim3(ntiles, ktiles), dim3(kRhoThreads), 0, st, pdl);
+template <int T>
+static void rho_mixed_t(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
+                        const int4* ksamp, const double* kcoef, const uint4* fx,
+                        unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl) {
+    PdlConfig c(dim3(ntiles, ktiles), dim3(T), 0, st, pdl);
     if (one)
-        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<true>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab, run);
+        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<T, true>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab,
+                           run);
     else
-        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<false>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab,
+        cudaLaunchKernelEx(&c.cfg, k_rho_mixed<T, false>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab,
                            run);
 }
 
-template <int R>
-static void rho_list_r(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
+void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
+                      const int4* ksamp, const double* kcoef, const uint4* fx,
+                      unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl) {
+    if (g.ntiles <= 0 || g.ktiles <= 0) return;
+    if (g.threads == 128)
+        rho_mixed_t<128>(st, one, w, g.ntiles, g.ktiles, g.run, ksamp, kcoef, fx, rho_fx, kcnt, kab, pdl);
+    else
+        rho_mixed_t<256>(st, one, w, g.ntiles, g.ktiles, g.run, ksamp, kcoef, fx, rho_fx, kcnt, kab, pdl);
+}
+
+template <int T, int R>
+static void rho_list_r(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
                        const int4* ksamp, const double* kcoef, const uint4* fx,
                        unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
                        bool pdl) {
-    const int nrho = ntiles * ktiles, nlist = (a.nlblk + 1) / 2;
-    PdlConfig c(dim3(nrho + nlist), dim3(kRhoThreads), 0, st, pdl);
+    constexpr int LT = T / kBlockP;
+    const int nrho = g.ntiles * g.ktiles, nlist = (a.nlblk + LT - 1) / LT;
+    PdlConfig c(dim3(nrho + nlist), dim3(T), 0, st, pdl);
     if (one)
-        cudaLaunchKernelEx(&c.cfg, k_rho_list<R, true>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab, a,
-                           ntiles, run, nrho, nlist);
+        cudaLaunchKernelEx(&c.cfg, k_rho_list<T, R, true>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab,
+                           a, g.ntiles, g.run, nrho, nlist);
     else
-        cudaLaunchKernelEx(&c.cfg, k_rho_list<R, false>, w, ksamp, kcoef, fx, rho_fx, kcnt, kab,
-                           a, ntiles, run, nrho, nlist);
+        cudaLaunchKernelEx(&c.cfg, k_rho_list<T, R, false>, w, ksamp, kcoef, fx, rho_fx, kcnt,
+                           kab, a, g.ntiles, g.run, nrho, nlist);
 }
 
-void launch_rho_list(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
+template <int T>
+static void rho_list_t(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
+                       const int4* ksamp, const double* kcoef, const uint4* fx,
+                       unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
+                       bool pdl) {
+    switch (a.lsplit) {
+        case 2: rho_list_r<T, 2>(st, one, w, g, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+        case 4: rho_list_r<T, 4>(st, one, w, g, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+        case 8: rho_list_r<T, 8>(st, one, w, g, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+        default: rho_list_r<T, 1>(st, one, w, g, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
+    }
+}
+
+void launch_rho_list(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
                      const int4* ksamp, const double* kcoef, const uint4* fx,
                      unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
                      bool pdl) {
-    if (ntiles <= 0 || ktiles <= 0) return;
-    switch (a.lsplit) {
-        case 2: rho_list_r<2>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
-        case 4: rho_list_r<4>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
-        case 8: rho_list_r<8>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
-        default: rho_list_r<1>(st, one, w, ntiles, ktiles, run, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl); break;
-    }
+    if (g.ntiles <= 0 || g.ktiles <= 0) return;
+    if (g.threads == 128)
+        rho_list_t<128>(st, one, w, g, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl);
+    else
+        rho_list_t<256>(st, one, w, g, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl);
 }
 
 template <int SPLIT, int PT>

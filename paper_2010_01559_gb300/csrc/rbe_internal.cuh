@@ -33,8 +33,6 @@ namespace rbe {
 
 constexpr int kBlockP = 128;      // particles per block of the per-particle kernels
 constexpr int kLTile = 128;       // threads per wave-vector row (FP64 and full structure factors)
-constexpr int kRhoThreads = 256;  // threads per block of the mixed structure factors
-constexpr int kRhoKT = 2 * kRhoThreads;  // wave vectors per tile: two per thread
 constexpr int kRhoStage = 512;    // particles staged per pass
 // Copies of the rho(k) accumulators that the blocks of the structure factors
 // spread their atomics over: additions to one address take about 27 SM cycles
@@ -566,9 +564,13 @@ __device__ __forceinline__ double2 rho_total(const unsigned long long* src, int 
 
 // pdl: launched with programmatic stream serialisation (the kernels wait for
 // their predecessor's results before reading them).
-// ntiles, ktiles: tiles of particles (w) and of kRhoKT wave vectors; run:
-// particles per FP32 run of the sums (a power of two up to kRhoStage).
-void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
+// The mixed structure factors' grid: tiles of particles (w) and of 2 threads wave
+// vectors, FP32 run of the sums (particles, at most kRhoStage), threads per block
+// (128 or 256).
+struct RhoGrid {
+    int ntiles, ktiles, run, threads;
+};
+void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
                       const int4* ksamp, const double* kcoef, const uint4* fx,
                       unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl = false);
 // FP64 path (rbe_fourier64.cu): chunk = particles per chunk, pmax and mcap the
@@ -665,7 +667,7 @@ void launch_real_f64(cudaStream_t st, bool one, const RealArgs& a);
 void launch_real_list(cudaStream_t st, bool one, const RealArgs& a);
 // The MD step's structure factors and its pass over a standing list in one
 // launch (rbe_fourier.cu); `a` as for launch_real_list with list_when = 0.
-void launch_rho_list(cudaStream_t st, bool one, const Work& w, int ntiles, int ktiles, int run,
+void launch_rho_list(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
                      const int4* ksamp, const double* kcoef, const uint4* fx,
                      unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,
                      bool pdl);
