@@ -419,6 +419,9 @@ void fill_sysdev(const SysHost& s, SysDev& d) {
     d.vsd = std::sqrt(p.kT / p.mass);
     d.f_vsd = (float)d.vsd;
     d.f_inv_Lu = (float)(4294967296.0 / L);
+    d.f_erfc_x = (float)(0.3275911 * d.sqrt_alpha);
+    d.f_gauss_ex2 = (float)(-d.alpha * 1.4426950408889634);
+    d.f_lj_rc2_on = p.lj_eps != 0.0 ? d.f_lj_rc2 : 0.0f;
     d.nh_rate = p.thermostat == RBE_THERMO_NOSE_HOOVER
                     ? p.dt / (3.0 * std::max(1, s.n) * p.nh_tau * p.nh_tau) : 0.0;
     d.nh_k2scale = p.kT > 0.0 ? p.mass / p.kT * 4294967296.0 : 0.0;

@@ -79,6 +79,11 @@ __device__ __forceinline__ void carry(float4& s, float re, float im) {
     s = make_float4(x.x, s.y + x.y, y.x, s.w + y.y);
 }
 
+__device__ __forceinline__ void carry(float4& s, f32x2 v) {
+    const float2 c = unpack2(v);
+    carry(s, c.x, c.y);
+}
+
 __device__ __forceinline__ void rho_add(unsigned long long* dst, const float4& s, int e) {
     atomicAdd(dst, (unsigned long long)(fixed64(s.x, e) + fixed64(s.y, e)));
     atomicAdd(dst + 1, (unsigned long long)(fixed64(s.z, e) + fixed64(s.w, e)));
@@ -121,47 +126,48 @@ __device__ __forceinline__ void rho_body(const Work& w, const int4* __restrict__
         __syncthreads();
         for (int u = threadIdx.x; u < cnt; u += T) sp[u] = fx[ch.first + base + u];
         __syncthreads();
-        auto terms = [&](const uint4 p, float* re, float* im) {
+        // (cos, sin) of both wave vectors for one particle, added times its charge
+        auto terms = [&](const uint4 p, f32x2* c) {
             const float q = __uint_as_float(p.w);
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const uint32_t ph = mx[r] * p.x + my[r] * p.y + mz[r] * p.z;
-                const float th = (float)(int32_t)ph * kTwoPiOver2p32;
-                float sn, cs;
-                __sincosf(th, &sn, &cs);
-                re[r] = fmaf(q, cs, re[r]);
-                im[r] = fmaf(q, sn, im[r]);
-            }
+            const f32x2 qq = pack2(q, q);
+            const float2 th = unpack2(
+                mul2(pack2((float)(int32_t)(mx[0] * p.x + my[0] * p.y + mz[0] * p.z),
+                           (float)(int32_t)(mx[1] * p.x + my[1] * p.y + mz[1] * p.z)),
+                     pack2(kTwoPiOver2p32, kTwoPiOver2p32)));
+            float sn, cs;
+            __sincosf(th.x, &sn, &cs);
+            c[0] = fma2(qq, pack2(cs, sn), c[0]);
+            __sincosf(th.y, &sn, &cs);
+            c[1] = fma2(qq, pack2(cs, sn), c[1]);
         };
         if (subs == 1) {
             // one thread takes a run's even and odd particles side by side
             if (work)
                 for (int j0 = 0; j0 < cnt; j0 += run) {
                     const int j1 = min(cnt, j0 + run);
-                    float re[2] = {0.f, 0.f}, im[2] = {0.f, 0.f};
-                    float ro[2] = {0.f, 0.f}, io[2] = {0.f, 0.f};
+                    f32x2 even[2] = {0ull, 0ull}, odd[2] = {0ull, 0ull};
                     int j = j0;
 #pragma unroll 8
                     for (; j + 1 < j1; j += 2) {
-                        terms(sp[j], re, im);
-                        terms(sp[j + 1], ro, io);
+                        terms(sp[j], even);
+                        terms(sp[j + 1], odd);
                     }
-                    if (j < j1) terms(sp[j], re, im);
+                    if (j < j1) terms(sp[j], even);
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
-                        carry(sum[r], re[r], im[r]);
-                        carry(sum[r], ro[r], io[r]);
+                        carry(sum[r], even[r]);
+                        carry(sum[r], odd[r]);
                     }
                 }
         } else if (work) {
             // a run's even particles, then its odd ones, are a unit of work each
             for (int u = sub; (u >> 1) * run < cnt; u += subs) {
                 const int j0 = (u >> 1) * run + (u & 1), j1 = min(cnt, ((u >> 1) + 1) * run);
-                float re[2] = {0.f, 0.f}, im[2] = {0.f, 0.f};
+                f32x2 c[2] = {0ull, 0ull};
 #pragma unroll 8
-                for (int j = j0; j < j1; j += 2) terms(sp[j], re, im);
-                carry(sum[0], re[0], im[0]);
-                carry(sum[1], re[1], im[1]);
+                for (int j = j0; j < j1; j += 2) terms(sp[j], c);
+                carry(sum[0], c[0]);
+                carry(sum[1], c[1]);
             }
         }
     }
@@ -262,7 +268,7 @@ k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
     }
     if ((*a.list_flag != 0) != (a.list_when != 0)) return;
     const int tile = (T / kBlockP) * (b - r1) + (int)(threadIdx.x / kBlockP);
-    if (tile < a.nlblk) list_body<R, ONE, false, false, 8>(a, tile, threadIdx.x % kBlockP);
+    if (tile < a.nlblk) list_step<R, ONE>(a, tile, threadIdx.x % kBlockP);
 }
 
 // ----------------------------------------------------------------- force (mixed)

@@ -80,6 +80,10 @@ struct SysDev {
     float f_lj_sigma2, f_lj_eps, f_lj_shift;
     float f_c1, f_c2, f_dt, f_dt_over_m, f_invL;
     float f_inv_Lu;         // 2^32 / L: length to fixed-point units
+    // pair constants of pair2_fixed
+    float f_erfc_x;         // 0.3275911 sqrt(alpha)
+    float f_gauss_ex2;      // -alpha log2 e
+    float f_lj_rc2_on;      // Lennard-Jones cutoff squared, 0 without Lennard-Jones
     int thermostat;         // RBE_THERMO_LANGEVIN, _ANDERSEN or _NOSE_HOOVER
     uint64_t andersen_thr;  // collision iff 32-bit Philox word < nu dt 2^32
     double vsd;             // sqrt(kT / m): Andersen velocity standard deviation
@@ -292,6 +296,30 @@ __device__ __forceinline__ void langevin_update(float4* md_pos, float4* md_vel,
 __device__ __forceinline__ float2 two_sum(float a, float b) {
     const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
     return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t)));
+}
+
+// Two FP32 lanes of one 64-bit register pair, one instruction for both (IEEE
+// rounding of each, subnormals to zero as in the rest of the library).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 // Programmatic dependent launch (a kernel launched with programmatic stream

@@ -35,8 +35,69 @@ namespace rbe {
 // once.  The pass on its own takes 4 (40 registers, more resident warps to
 // hide the gathers: 2^20 122 -> 111 us); the fused launch, whose registers
 // are set by its structure-factor blocks' company, takes 8.
-template <int R, bool ONE, bool FM, bool PAD = true, int U = 4>
+// The step form: one tile's real-space forces, entries two at a time (pair2_fixed),
+// stored in the caller's order for the Fourier-force kernel that adds its part and
+// applies the thermostat.  No block synchronisation.
+template <int R, bool ONE>
+__device__ __forceinline__ void list_step(const RealArgs& a, int tile, int tid) {
+    constexpr int U = 4;
+    const Tile tl = tile_at<ONE>(a.lw, tile);
+    const SysDev& S = sys_of<ONE>(a.lw, tl.sys);
+    const int p = tid / R, l = tid - p * R;
+    float3 f = make_float3(0.f, 0.f, 0.f);
+    if (p < tl.count) {
+        const int i = tl.first + p;
+        const uint4 si = a.spos[i];
+        const int* nb = a.nbr + i;
+        const size_t st = (size_t)a.nbr_stride;
+        const int cnt = __ldcs(a.ncnt + i);
+        Pair2Acc acc{0ull, 0ull, 0ull, 0.f, 0.f, 0.f};
+        int j[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int kk = l + q * R;
+            j[q] = kk < a.nbr_cap ? __ldcs(nb + (size_t)kk * st) : i;
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+            if (l + q * R >= cnt) j[q] = i;
+        for (int k0 = l;;) {
+            uint4 sj[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                if (!RBE_IN_BOUNDS(j[q], a.nbr_stride, a.err)) j[q] = i;
+                sj[q] = __ldg(a.spos + j[q]);
+            }
+            k0 += U * R;
+            if (k0 < cnt) {                      // the next batch's entries meanwhile
+#pragma unroll
+                for (int q = 0; q < U; ++q) {
+                    const int kk = k0 + q * R;
+                    j[q] = kk < cnt ? __ldcs(nb + (size_t)kk * st) : i;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < U; q += 2) pair2_fixed(si, sj[q], sj[q + 1], S, acc);
+            if (k0 >= cnt) break;
+        }
+        f = pair2_force(acc, si, S);
+    }
+#pragma unroll
+    for (int o = R / 2; o > 0; o >>= 1) {
+        f.x += __shfl_down_sync(0xffffffffu, f.x, o, R);
+        f.y += __shfl_down_sync(0xffffffffu, f.y, o, R);
+        f.z += __shfl_down_sync(0xffffffffu, f.z, o, R);
+    }
+    if (p < tl.count && l == 0) {
+        const int o = a.perm[tl.first + p];
+        if (RBE_IN_BOUNDS(o, a.nbr_stride, a.err)) a.freal[o] = make_float4(f.x, f.y, f.z, 0.f);
+    }
+}
+
+template <int R, bool ONE>
 __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) {
+    constexpr bool FM = true, PAD = true;
+    constexpr int U = 4;
     constexpr int T = kBlockP / R;               // particles per block
     const Tile tl = tile_at<ONE>(a.lw, tile);
     const int sys = tl.sys;
@@ -131,15 +192,7 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
             }
         }
     }
-    if constexpr (!FM) {
-        // the real-space force in the caller's order, for the Fourier-force
-        // kernel that adds its part and applies the thermostat (the first of the
-        // particle's lanes stores it: no block synchronisation in this form)
-        if (p < tl.count && l == 0) {
-            const int o = a.perm[tl.first + p];
-            if (RBE_IN_BOUNDS(o, a.nbr_stride, a.err)) a.freal[o] = make_float4(fx, fy, fz, 0.f);
-        }
-    } else {
+    {
         double e_c = 0.0, e_l = 0.0, w_c = 0.0, w_l = 0.0;
         if ((int)tid < tl.count) {
             const int i = tl.first + tid;
@@ -182,7 +235,8 @@ __global__ void __launch_bounds__(kBlockP) k_real_list(const __grid_constant__ R
     } else {
         if (a.flag_clear && blockIdx.x == 0 && threadIdx.x == 0) *a.flag_clear = 0;
     }
-    list_body<R, ONE, FM>(a, blockIdx.x, threadIdx.x);
+    if constexpr (FM) list_body<R, ONE>(a, blockIdx.x, threadIdx.x);
+    else list_step<R, ONE>(a, blockIdx.x, threadIdx.x);
 }
 
 }  // namespace rbe

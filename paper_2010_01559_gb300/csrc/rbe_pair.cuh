@@ -118,4 +118,74 @@ __device__ __forceinline__ void pair_fixed(const uint4& si, const uint4& sj, flo
     if (r2 > 0.f) pair_terms(dx, dy, dz, r2, __uint_as_float(sj.w), lbqi, kc, acc);
 }
 
+// ---- two pairs at a time (MD steps: the force alone)
+// The list pass of an MD step is bound by instruction issue: with two pairs per
+// packed FP32 instruction a pair takes about 32 instructions instead of 70.  Same
+// formulas as pair_terms (erfc as in erfc_as) from the same displacements and r^2
+// to the last bit, so that a pair at a cutoff falls on the same side (the truncated
+// force jumps by 7e-5 there at the parameters of the benchmark).  Pairs beyond the
+// cutoff and the particle itself (a zero displacement) get the factor 0.
+struct Pair2Acc {
+    f32x2 x, y, z;                               // Coulomb / (-lB q_i), the two pairs' sums apart
+    float lx, ly, lz;                            // Lennard-Jones
+};
+
+__device__ __forceinline__ void pair2_fixed(const uint4& si, const uint4& sa, const uint4& sb,
+                                            const SysDev& S, Pair2Acc& acc) {
+    const f32x2 Lu = pack2(S.L_over_2_32, S.L_over_2_32);
+    const f32x2 dx = mul2(pack2((float)(int32_t)(sa.x - si.x), (float)(int32_t)(sb.x - si.x)), Lu);
+    const f32x2 dy = mul2(pack2((float)(int32_t)(sa.y - si.y), (float)(int32_t)(sb.y - si.y)), Lu);
+    const f32x2 dz = mul2(pack2((float)(int32_t)(sa.z - si.z), (float)(int32_t)(sb.z - si.z)), Lu);
+    const f32x2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    const float2 q2 = unpack2(r2);
+    const bool ina = q2.x < S.f_rc2 && q2.x > 0.f, inb = q2.y < S.f_rc2 && q2.y > 0.f;
+    if (!(ina || inb)) return;
+    const float ia = rsqrtf(q2.x), ib = rsqrtf(q2.y);
+    const f32x2 inv = pack2(ia, ib), inv2 = mul2(inv, inv);
+    // t = 1 / (1 + 0.3275911 x), x = sqrt(alpha) r
+    const float2 den = unpack2(
+        fma2(mul2(r2, inv), pack2(S.f_erfc_x, S.f_erfc_x), pack2(1.f, 1.f)));
+    const f32x2 t = pack2(__fdividef(1.0f, den.x), __fdividef(1.0f, den.y));
+    const float2 e2 = unpack2(mul2(r2, pack2(S.f_gauss_ex2, S.f_gauss_ex2)));
+    const f32x2 ex = pack2(exp2f(e2.x), exp2f(e2.y));            // exp(-alpha r^2)
+    f32x2 p = fma2(t, pack2(1.061405429f, 1.061405429f), pack2(-1.453152027f, -1.453152027f));
+    p = fma2(p, t, pack2(1.421413741f, 1.421413741f));
+    p = fma2(p, t, pack2(-0.284496736f, -0.284496736f));
+    p = fma2(p, t, pack2(0.254829592f, 0.254829592f));
+    // q_j (erfc / r + 2 sqrt(alpha / pi) exp(-alpha r^2)) / r^2
+    const f32x2 g = mul2(fma2(mul2(p, t), inv, pack2(S.f_two_sa_spi, S.f_two_sa_spi)),
+                         mul2(ex, inv2));
+    const float2 f =
+        unpack2(mul2(g, pack2(__uint_as_float(sa.w), __uint_as_float(sb.w))));
+    const f32x2 s = pack2(ina ? f.x : 0.f, inb ? f.y : 0.f);
+    acc.x = fma2(s, dx, acc.x);
+    acc.y = fma2(s, dy, acc.y);
+    acc.z = fma2(s, dz, acc.z);
+    if (fminf(q2.x, q2.y) < S.f_lj_rc2_on) {     // a few pairs per particle, one at a time
+        const float2 x = unpack2(dx), y = unpack2(dy), z = unpack2(dz);
+        auto lj = [&](float r2s, float inv_r, float ux, float uy, float uz) {
+            if (r2s < S.f_lj_rc2_on && r2s > 0.f) {
+                const float inv_r2 = inv_r * inv_r;
+                const float sr2 = S.f_lj_sigma2 * inv_r2;
+                const float sr6 = sr2 * sr2 * sr2;
+                const float mag = 24.f * S.f_lj_eps * (2.f * sr6 * sr6 - sr6) * inv_r2;
+                acc.lx = fmaf(-mag, ux, acc.lx);
+                acc.ly = fmaf(-mag, uy, acc.ly);
+                acc.lz = fmaf(-mag, uz, acc.lz);
+            }
+        };
+        lj(q2.x, ia, x.x, y.x, z.x);
+        lj(q2.y, ib, x.y, y.y, z.y);
+    }
+}
+
+// The particle's force from its sums.
+__device__ __forceinline__ float3 pair2_force(const Pair2Acc& a, const uint4& si,
+                                              const SysDev& S) {
+    const float2 x = unpack2(a.x), y = unpack2(a.y), z = unpack2(a.z);
+    const float c = -S.f_lB * __uint_as_float(si.w);
+    return make_float3(fmaf(c, x.x + x.y, a.lx), fmaf(c, y.x + y.y, a.ly),
+                       fmaf(c, z.x + z.y, a.lz));
+}
+
 }  // namespace rbe
