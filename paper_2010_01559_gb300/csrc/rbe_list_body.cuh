@@ -8,37 +8,31 @@
 
 namespace rbe {
 
-// The MD step's real-space pass over the list: R lanes per particle (adjacent
-// lanes) take every R-th entry of the particle's list and the pair terms of
-// those within the cutoffs (U gathers in flight per lane); the lanes' sums
-// are added and stored per particle.  It needs nothing from the Fourier part,
-// so it runs concurrently with the structure factors (and, when the list
-// stands, with the no-op rebuild kernels); the Fourier-force kernel then
+// The real-space pass over the list: R lanes per particle (adjacent lanes) take
+// every R-th entry of the particle's list and the pair terms of those within the
+// cutoffs; the lanes' sums are added and stored per particle.  On an MD step it
+// needs nothing from the Fourier part, so it runs concurrently with the structure
+// factors (and with the no-op rebuild kernels); the Fourier-force kernel then
 // completes the step.
 //
-// FM (forces calls): the pass runs once, after the rebuild and the Fourier
-// force, and assembles per particle the total force (+ F^F), dE/dq (+ the
-// Fourier part, self and background terms) and per-block FP64 partials of the
-// real-space and LJ energies and virials, as the cell-scan pass does.
+// FM, for the pass's own kernel: 0, an MD step (list_step); 1, a forces call: the
+// pass runs once, after the rebuild and the Fourier force, and assembles per
+// particle the total force (+ F^F), dE/dq (+ the Fourier part, self and background
+// terms) and per-block FP64 partials of the real-space and LJ energies and
+// virials, as the cell-scan pass does (list_body); 2, a forces call that asks for
+// the force alone (list_step, + F^F).
 //
-// list_body: the work of one tile (kBlockP threads, tid = the thread's index
-// in them; in its FM form it synchronises the block), for the pass's own kernel and for the
-// fused structure-factor + list launch of the MD step.
+// The slots of a batch past the particle's count stand for the particle itself (a
+// zero displacement, which the pair terms skip) instead of being tested one by
+// one: the same sums, with lanes that stay converged.  U = 4 entries per lane and
+// batch, all gathers of a batch in flight at once and, in list_step, the next
+// batch's entries with them.
 //
-// PAD: the slots of a batch past the particle's count stand for the particle
-// itself (a zero displacement, which the pair terms skip) instead of being
-// tested one by one: the same sums, with lanes that stay converged.  Faster
-// for the pass on its own (2^20: 135 -> 122 us); inside the fused launch,
-// which is issue-bound, it gains nothing, and the fused launch keeps the tests.
-//
-// U: list entries per lane and batch, all gathers of a batch in flight at
-// once.  The pass on its own takes 4 (40 registers, more resident warps to
-// hide the gathers: 2^20 122 -> 111 us); the fused launch, whose registers
-// are set by its structure-factor blocks' company, takes 8.
 // The step form: one tile's real-space forces, entries two at a time (pair2_fixed),
 // stored in the caller's order for the Fourier-force kernel that adds its part and
 // applies the thermostat.  No block synchronisation.
-template <int R, bool ONE>
+// FORCES: in the caller's order to F_out, with the Fourier force added.
+template <int R, bool ONE, bool FORCES = false>
 __device__ __forceinline__ void list_step(const RealArgs& a, int tile, int tid) {
     constexpr int U = 4;
     const Tile tl = tile_at<ONE>(a.lw, tile);
@@ -90,13 +84,25 @@ __device__ __forceinline__ void list_step(const RealArgs& a, int tile, int tid) 
     }
     if (p < tl.count && l == 0) {
         const int o = a.perm[tl.first + p];
-        if (RBE_IN_BOUNDS(o, a.nbr_stride, a.err)) a.freal[o] = make_float4(f.x, f.y, f.z, 0.f);
+        if (!RBE_IN_BOUNDS(o, a.nbr_stride, a.err)) return;
+        if constexpr (FORCES) {
+            if (a.parts & kPartFourier) {
+                const float4 g = a.fs[o];
+                f.x += g.x;
+                f.y += g.y;
+                f.z += g.z;
+            }
+            a.F_out[o] = make_float4(f.x, f.y, f.z, 0.f);
+        } else {
+            a.freal[o] = make_float4(f.x, f.y, f.z, 0.f);
+        }
     }
 }
 
+// list_body: one tile of a forces call (kBlockP threads, tid = the thread's index
+// in them; it synchronises the block).
 template <int R, bool ONE>
 __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) {
-    constexpr bool FM = true, PAD = true;
     constexpr int U = 4;
     constexpr int T = kBlockP / R;               // particles per block
     const Tile tl = tile_at<ONE>(a.lw, tile);
@@ -115,7 +121,7 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
     kc.lj_s2 = S.f_lj_sigma2;
     kc.lj_eps = S.f_lj_eps;
     kc.lj_shift = S.f_lj_shift;
-    kc.vir = FM && a.blk_w != nullptr;
+    kc.vir = a.blk_w != nullptr;
     PairAcc acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (p < tl.count && (do_real || do_lj)) {
         const int i = tl.first + p;
@@ -134,13 +140,11 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const int kk = l + q * R;
-            j[q] = kk < a.nbr_cap ? __ldcs(nb + (size_t)kk * st) : (PAD ? i : 0);
+            j[q] = kk < a.nbr_cap ? __ldcs(nb + (size_t)kk * st) : i;
         }
-        if constexpr (PAD) {
 #pragma unroll
-            for (int q = 0; q < U; ++q)
-                if (l + q * R >= cnt) j[q] = i;
-        }
+        for (int q = 0; q < U; ++q)
+            if (l + q * R >= cnt) j[q] = i;
         for (int k0 = l;;) {
             uint4 sj[U];
 #pragma unroll
@@ -150,13 +154,13 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
             }
 #pragma unroll
             for (int q = 0; q < U; ++q)
-                if (PAD || k0 + q * R < cnt) pair_fixed(si, sj[q], Lu, lbqi, kc, acc);
+                pair_fixed(si, sj[q], Lu, lbqi, kc, acc);
             k0 += U * R;
             if (k0 >= cnt) break;
 #pragma unroll
             for (int q = 0; q < U; ++q) {
                 const int kk = k0 + q * R;
-                j[q] = kk < cnt ? __ldcs(nb + (size_t)kk * st) : (PAD ? i : 0);
+                j[q] = kk < cnt ? __ldcs(nb + (size_t)kk * st) : i;
             }
         }
     }
@@ -168,28 +172,24 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
             fx += __shfl_down_sync(0xffffffffu, fx, o, R);
             fy += __shfl_down_sync(0xffffffffu, fy, o, R);
             fz += __shfl_down_sync(0xffffffffu, fz, o, R);
-            if constexpr (FM) {
-                ph += __shfl_down_sync(0xffffffffu, ph, o, R);
-                ec += __shfl_down_sync(0xffffffffu, ec, o, R);
-                el += __shfl_down_sync(0xffffffffu, el, o, R);
-                wc += __shfl_down_sync(0xffffffffu, wc, o, R);
-                wl += __shfl_down_sync(0xffffffffu, wl, o, R);
-            }
+            ph += __shfl_down_sync(0xffffffffu, ph, o, R);
+            ec += __shfl_down_sync(0xffffffffu, ec, o, R);
+            el += __shfl_down_sync(0xffffffffu, el, o, R);
+            wc += __shfl_down_sync(0xffffffffu, wc, o, R);
+            wl += __shfl_down_sync(0xffffffffu, wl, o, R);
         }
-        if constexpr (FM) {
-            __shared__ float4 s_f[T];
-            __shared__ float4 s_e[T];
-            if (p < tl.count && l == 0) {
-                s_f[p] = make_float4(fx, fy, fz, ph);
-                s_e[p] = make_float4(ec, el, wc, wl);
-            }
-            __syncthreads();
-            if ((int)tid < tl.count) {
-                const float4 f = s_f[tid];
-                fx = f.x; fy = f.y; fz = f.z; ph = f.w;
-                const float4 e = s_e[tid];
-                ec = e.x; el = e.y; wc = e.z; wl = e.w;
-            }
+        __shared__ float4 s_f[T];
+        __shared__ float4 s_e[T];
+        if (p < tl.count && l == 0) {
+            s_f[p] = make_float4(fx, fy, fz, ph);
+            s_e[p] = make_float4(ec, el, wc, wl);
+        }
+        __syncthreads();
+        if ((int)tid < tl.count) {
+            const float4 f = s_f[tid];
+            fx = f.x; fy = f.y; fz = f.z; ph = f.w;
+            const float4 e = s_e[tid];
+            ec = e.x; el = e.y; wc = e.z; wl = e.w;
         }
     }
     {
@@ -226,17 +226,17 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
     }
 }
 
-template <int R, bool ONE, bool FM>
+template <int R, bool ONE, int FM>
 __global__ void __launch_bounds__(kBlockP) k_real_list(const __grid_constant__ RealArgs a) {
-    if constexpr (!FM) {
+    if constexpr (FM == 0) {
         // right after the prep kernel: works when the list stands (over a
         // rebuilt list the build adds the pair terms itself)
         if ((*a.list_flag != 0) != (a.list_when != 0)) return;
     } else {
         if (a.flag_clear && blockIdx.x == 0 && threadIdx.x == 0) *a.flag_clear = 0;
     }
-    if constexpr (FM) list_body<R, ONE>(a, blockIdx.x, threadIdx.x);
-    else list_step<R, ONE>(a, blockIdx.x, threadIdx.x);
+    if constexpr (FM == 1) list_body<R, ONE>(a, blockIdx.x, threadIdx.x);
+    else list_step<R, ONE, FM == 2>(a, blockIdx.x, threadIdx.x);
 }
 
 }  // namespace rbe

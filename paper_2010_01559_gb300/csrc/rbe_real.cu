@@ -504,19 +504,7 @@ __global__ void __launch_bounds__(kBlockP) k_list_build(const __grid_constant__ 
             if (cnt > la.cap) atomicOr(la.err, kErrList);
         }
         if constexpr (PASS) {
-            PairConst kc;
-            kc.rc2 = S.f_rc2;
-            kc.lj_rc2 = S.lj_eps != 0.0 ? S.f_lj_rc2 : 0.f;
-            kc.alpha = S.f_alpha;
-            kc.sa = S.f_sqrt_alpha;
-            kc.two_sa_spi = S.f_two_sa_spi;
-            kc.lB = S.f_lB;
-            kc.lj_s2 = S.f_lj_sigma2;
-            kc.lj_eps = S.f_lj_eps;
-            kc.lj_shift = S.f_lj_shift;
-            kc.vir = false;
-            PairAcc acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const float lbqi = kc.lB * __uint_as_float(si.w);
+            Pair2Acc acc{0ull, 0ull, 0ull, 0.f, 0.f, 0.f};
             const int ne = min(cnt, la.cap);
             for (int k0 = l; k0 < ne; k0 += R * kBuildU) {
                 uint4 sj[kBuildU];
@@ -527,9 +515,10 @@ __global__ void __launch_bounds__(kBlockP) k_list_build(const __grid_constant__ 
                     sj[u] = __ldg(la.spos + j);
                 }
 #pragma unroll
-                for (int u = 0; u < kBuildU; ++u) pair_fixed(si, sj[u], Lu, lbqi, kc, acc);
+                for (int u = 0; u < kBuildU; u += 2) pair2_fixed(si, sj[u], sj[u + 1], S, acc);
             }
-            float fx = acc.fx, fy = acc.fy, fz = acc.fz;
+            const float3 f = pair2_force(acc, si, S);
+            float fx = f.x, fy = f.y, fz = f.z;
 #pragma unroll
             for (int d = R / 2; d > 0; d >>= 1) {
                 fx += __shfl_down_sync(gmask, fx, d, R);
@@ -663,15 +652,20 @@ void launch_real_mixed(cudaStream_t st, bool one, const RealArgs& a) {
     }
 }
 
+template <int R, int FM>
+static void real_list_rf(cudaStream_t st, bool one, const RealArgs& a) {
+    if (one) k_real_list<R, true, FM><<<a.nlblk, kBlockP, 0, st>>>(a);
+    else k_real_list<R, false, FM><<<a.nlblk, kBlockP, 0, st>>>(a);
+}
+
 template <int R>
 static void real_list_r(cudaStream_t st, bool one, const RealArgs& a) {
-    if (a.fmode) {
-        if (one) k_real_list<R, true, true><<<a.nlblk, kBlockP, 0, st>>>(a);
-        else k_real_list<R, false, true><<<a.nlblk, kBlockP, 0, st>>>(a);
-    } else {
-        if (one) k_real_list<R, true, false><<<a.nlblk, kBlockP, 0, st>>>(a);
-        else k_real_list<R, false, false><<<a.nlblk, kBlockP, 0, st>>>(a);
-    }
+    // the force-only form takes both pair parts or none of a forces call's extras
+    const bool plain = !a.phi_out && !a.blk_e && !a.blk_w && a.F_out &&
+                       (a.parts & (kPartReal | kPartLJ)) == (kPartReal | kPartLJ);
+    if (!a.fmode) real_list_rf<R, 0>(st, one, a);
+    else if (plain) real_list_rf<R, 2>(st, one, a);
+    else real_list_rf<R, 1>(st, one, a);
 }
 
 void launch_real_list(cudaStream_t st, bool one, const RealArgs& a) {

@@ -225,17 +225,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     __syncthreads();
     cluster_sync();                                 // every rank's barriers are initialised
 
-    PairConst kc;
-    kc.rc2 = S.f_rc2;
-    kc.lj_rc2 = S.lj_eps != 0.0 ? S.f_lj_rc2 : 0.f;
-    kc.alpha = S.f_alpha;
-    kc.sa = S.f_sqrt_alpha;
-    kc.two_sa_spi = S.f_two_sa_spi;
-    kc.lB = S.f_lB;
-    kc.lj_s2 = S.f_lj_sigma2;
-    kc.lj_eps = S.f_lj_eps;
-    kc.lj_shift = S.f_lj_shift;
-    kc.vir = false;
     const int kp = (nk + 1) / 2;                    // pairs of wave vectors, a group of warps each
     const int wpp = kp > 0 ? kSmallWarps / kp : 0;
     const bool sums = warp < kp * wpp;              // this warp sums pair pr, share sub of wpp
@@ -456,14 +445,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         // ---- real-space pairs
         float fx = 0.f, fy = 0.f, fz = 0.f;
         if (pairs) {
-            PairAcc acc{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            Pair2Acc acc{0ull, 0ull, 0ull, 0.f, 0.f, 0.f};
             const uint4 si = R_[pn];
-            const float lbqi = kc.lB * __uint_as_float(si.w);
-            for (int k = l; k < cnt; k += R)
-                pair_fixed(si, R_[list[p * a.cap + k]], S.L_over_2_32, lbqi, kc, acc);
-            fx = acc.fx;
-            fy = acc.fy;
-            fz = acc.fz;
+            for (int k = l; k < cnt; k += 2 * R) {
+                const uint4 sb = k + R < cnt ? R_[list[p * a.cap + k + R]] : si;
+                pair2_fixed(si, R_[list[p * a.cap + k]], sb, S, acc);
+            }
+            const float3 f = pair2_force(acc, si, S);
+            fx = f.x;
+            fy = f.y;
+            fz = f.z;
         }
         // ---- Fourier force
         if (!late && !bar_wait(bar_kv, par)) late = true;
