@@ -498,10 +498,12 @@ int auto_rho_tile(int pmax, long long ntot, int run, int T) {
     return (int)std::max<long long>(pass, std::min<long long>(4096, (tile + 7) / 8 * 8));
 }
 
+// Threads per particle of the Fourier force: 45000 threads at least (measured,
+// us with 1, 2, 4, 8: N = 8001 9.3, 3.8, 3.1, 3.1; 30000 9.3, 6.2, 7.2, 9.2; 50021
+// 7.2, 7.2, 10.7, 11.3; 100003 7.2, 9.2, 13.3, 17.4).
 int auto_split(long long ntot) {
-    const long long target_threads = 152LL * 8 * kBlockP;
     int s = 1;
-    while (s < 8 && ntot * s < target_threads) s <<= 1;
+    while (s < 8 && ntot * s < 45000) s <<= 1;
     return s;
 }
 
@@ -1054,7 +1056,7 @@ void launch_force(const rbe_ctx* h, cudaStream_t st, bool mixed, const MdOut& md
     } else {
         const Work w = make_work(h, h->d_pblk, kBlockP, 0);
         launch_fourier_force_f64(st, one, w, h->npblk, h->m_max(), phi, h->d_fx64, h->d_ksamp,
-                                 h->d_kcoef, h->d_rho_fx, h->d_fs64);
+                                 h->d_kcoef, h->d_rho_fx, h->d_fs64, pdl);
     }
 }
 
@@ -1170,7 +1172,7 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
         cudaStreamWaitEvent(st2, h->ev_fork, 0);
         run(RBE_K_RHO, st2, [&] { launch_rho(h, st2, mixed, a.E != nullptr); });
         run(RBE_K_FOURIER_FORCE, st2, [&] {
-            launch_force(h, st2, mixed, MdOut{}, false, mixed || a.phi64);
+            launch_force(h, st2, mixed, MdOut{}, !mixed && !prof, mixed || a.phi64);
         });
         cudaEventRecord(h->ev_join, st2);
     }

@@ -268,7 +268,8 @@ k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
     }
     if ((*a.list_flag != 0) != (a.list_when != 0)) return;
     const int tile = (T / kBlockP) * (b - r1) + (int)(threadIdx.x / kBlockP);
-    if (tile < a.nlblk) list_step<R, ONE>(a, tile, threadIdx.x % kBlockP);
+    if (tile < a.nlblk)
+        list_step<R, ONE, false, T == 128 ? 4 : 8, T == 128>(a, tile, threadIdx.x % kBlockP);
 }
 
 // ----------------------------------------------------------------- force (mixed)
@@ -327,20 +328,25 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
         e_r[e] = e_fr[e];
         e_z[e] = MdNoise{0.f, 0.f, 0.f, false};
         const int te = threadIdx.x + e * NT;
-        if (md.freal && md.md_pos && te < tl.count) {
+        if (md.freal && te < tl.count) {
             const int o = tl.first + te;
-            e_v[e] = __ldcg(md.md_vel + o);
-            e_r[e] = __ldcg(md.md_pos + o);
-            if (!nhm) e_z[e] = md_noise(S, __ldcg((const unsigned long long*)md.cur_step), o);
+            if constexpr (SPLIT == 1) e_fr[e] = md.freal[o];
+            if (md.md_pos) {
+                e_v[e] = __ldcg(md.md_vel + o);
+                e_r[e] = __ldcg(md.md_pos + o);
+                if (!nhm) e_z[e] = md_noise(S, __ldcg((const unsigned long long*)md.cur_step), o);
+            }
         }
     }
-    if constexpr (SPLIT > 1) pdl_wait();
-    pdl_trigger();                                  // the next step's prep kernel may be scheduled
-    if (md.freal) {
+    if constexpr (SPLIT > 1) {
+        pdl_wait();
+        pdl_trigger();                              // the next step's prep kernel may be scheduled
+        if (md.freal) {
 #pragma unroll
-        for (int e = 0; e < EP; ++e) {
-            const int te = threadIdx.x + e * NT;
-            if (te < tl.count) e_fr[e] = md.freal[tl.first + te];
+            for (int e = 0; e < EP; ++e) {
+                const int te = threadIdx.x + e * NT;
+                if (te < tl.count) e_fr[e] = md.freal[tl.first + te];
+            }
         }
     }
     float fx[PT], fy[PT], fz[PT], ph[PT];

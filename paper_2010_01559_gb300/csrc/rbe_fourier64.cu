@@ -117,6 +117,7 @@ k_rho_f64_tab(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
     const int per = (ch.count + gridDim.y - 1) / gridDim.y;
     const int b0 = blockIdx.y * per, b1 = min(ch.count, b0 + per);
     if (l0 >= S.P || b0 >= b1) return;
+    pdl_trigger();                                  // the force kernel may build its tables
     const int mm = batch_mmax(ksamp + S.off_k, S.P), st = mm + 1;
     int ox[KR], oy[KR], oz[KR];
     uint32_t nx[KR], ny[KR], nz[KR];
@@ -141,6 +142,7 @@ k_rho_f64_tab(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
                 const double2* T = tab + 3 * p * st;
 #pragma unroll
                 for (int r = 0; r < KR; ++r) {
+                    if (l0 + r * kTabThreads + ((int)threadIdx.x & ~31) >= S.P) break;  // no lane
                     double2 X = T[ox[r]], Y = T[oy[r]], Z = T[oz[r]];
                     X.y = flip(X.y, nx[r]);
                     Y.y = flip(Y.y, ny[r]);
@@ -217,6 +219,7 @@ k_force_f64_tab(const __grid_constant__ Work w, const double4* __restrict__ rec6
     if (cnt <= 0) return;
     const int mm = batch_mmax(ksamp + S.off_k, S.P), st = mm + 1;
     build_tables(tab, mm, cnt, rec64 + tl.first + b0, S, false);
+    pdl_wait();                                     // rho(k)
     const int p = threadIdx.x / kTabLanes, sub = threadIdx.x % kTabLanes;
     const double2* T = tab + 3 * min(p, cnt - 1) * st;
     double fx = 0.0, fy = 0.0, fz = 0.0, ph = 0.0;
@@ -357,19 +360,19 @@ void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int c
 template <bool ONE, bool PHI>
 static void force_f64_tab(cudaStream_t st, const Work& w, int nblk, size_t smem,
                           const double4* fx64, const int4* ksamp, const double* kcoef,
-                          const unsigned long long* rho_fx, double4* fs64) {
+                          const unsigned long long* rho_fx, double4* fs64, bool pdl) {
     // + the staged wave vectors in static shared memory
     if (smem > 32 * 1024)
         cudaFuncSetAttribute(k_force_f64_tab<ONE, PHI>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_force_f64_tab<ONE, PHI><<<dim3(nblk, kBlockP / kTabP), kTabThreads, smem, st>>>(
-        w, fx64, ksamp, kcoef, rho_fx, fs64);
+    PdlConfig c(dim3(nblk, kBlockP / kTabP), dim3(kTabThreads), smem, st, pdl);
+    cudaLaunchKernelEx(&c.cfg, k_force_f64_tab<ONE, PHI>, w, fx64, ksamp, kcoef, rho_fx, fs64);
 }
 
 void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int mcap,
                               bool phi, const double4* fx64, const int4* ksamp,
                               const double* kcoef, const unsigned long long* rho_fx,
-                              double4* fs64) {
+                              double4* fs64, bool pdl) {
     if (nblk <= 0) return;
     if (mcap > kTabMaxM) {
         if (one)
@@ -380,11 +383,11 @@ void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk
     }
     const size_t sm = tab_smem(mcap);
     if (one) {
-        if (phi) force_f64_tab<true, true>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64);
-        else force_f64_tab<true, false>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64);
+        if (phi) force_f64_tab<true, true>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64, pdl);
+        else force_f64_tab<true, false>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64, pdl);
     } else {
-        if (phi) force_f64_tab<false, true>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64);
-        else force_f64_tab<false, false>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64);
+        if (phi) force_f64_tab<false, true>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64, pdl);
+        else force_f64_tab<false, false>(st, w, nblk, sm, fx64, ksamp, kcoef, rho_fx, fs64, pdl);
     }
 }
 

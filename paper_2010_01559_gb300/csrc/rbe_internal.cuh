@@ -602,7 +602,8 @@ void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, const RhoGrid& g
                       const int4* ksamp, const double* kcoef, const uint4* fx,
                       unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl = false);
 // FP64 path (rbe_fourier64.cu): chunk = particles per chunk, pmax and mcap the
-// largest P and sampler half width M over the systems; phi: also dE/dq.
+// largest P and sampler half width M over the systems; phi: also dE/dq; pdl: the
+// force follows launch_rho_f64 on the same stream, programmatically.
 void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int chunk, int pmax,
                     int mcap, const int4* ksamp, const double4* fx64,
                     unsigned long long* rho_fx);
@@ -631,7 +632,7 @@ void launch_fourier_force_mixed(cudaStream_t st, bool one, const Work& w, int nb
 void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int mcap,
                               bool phi, const double4* fx64, const int4* ksamp,
                               const double* kcoef, const unsigned long long* rho_fx,
-                              double4* fs64);
+                              double4* fs64, bool pdl = false);
 
 // real space, LJ, Langevin, energies (rbe_real.cu)
 // Blocks per real-space segment (mixed path): the first takes the particles

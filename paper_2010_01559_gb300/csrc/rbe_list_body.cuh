@@ -24,17 +24,20 @@ namespace rbe {
 //
 // The slots of a batch past the particle's count stand for the particle itself (a
 // zero displacement, which the pair terms skip) instead of being tested one by
-// one: the same sums, with lanes that stay converged.  U = 4 entries per lane and
-// batch, all gathers of a batch in flight at once and, in list_step, the next
-// batch's entries with them.
+// one: the same sums, with lanes that stay converged.
 //
 // The step form: one tile's real-space forces, entries two at a time (pair2_fixed),
 // stored in the caller's order for the Fourier-force kernel that adds its part and
 // applies the thermostat.  No block synchronisation.
 // FORCES: in the caller's order to F_out, with the Fourier force added.
-template <int R, bool ONE, bool FORCES = false>
+// U entries per lane and batch, all their gathers in flight together; AHEAD: the
+// next batch's entries are loaded while the pair terms run.  8 without is fastest
+// where the registers allow it (2^20: 122 us against 125 with 4 and 131 with 4
+// ahead; with 262144 particles 37, 39, 43), in the fused launch with 64 registers
+// too (P = 100: 171 against 183); within the 56 registers of its other form 4 ahead
+// is (P = 500: 314 us against 319, and 327 with 8).
+template <int R, bool ONE, bool FORCES = false, int U = 8, bool AHEAD = false>
 __device__ __forceinline__ void list_step(const RealArgs& a, int tile, int tid) {
-    constexpr int U = 4;
     const Tile tl = tile_at<ONE>(a.lw, tile);
     const SysDev& S = sys_of<ONE>(a.lw, tl.sys);
     const int p = tid / R, l = tid - p * R;
@@ -63,16 +66,18 @@ __device__ __forceinline__ void list_step(const RealArgs& a, int tile, int tid) 
                 sj[q] = __ldg(a.spos + j[q]);
             }
             k0 += U * R;
-            if (k0 < cnt) {                      // the next batch's entries meanwhile
+            auto next = [&] {
 #pragma unroll
                 for (int q = 0; q < U; ++q) {
                     const int kk = k0 + q * R;
                     j[q] = kk < cnt ? __ldcs(nb + (size_t)kk * st) : i;
                 }
-            }
+            };
+            if (AHEAD && k0 < cnt) next();
 #pragma unroll
             for (int q = 0; q < U; q += 2) pair2_fixed(si, sj[q], sj[q + 1], S, acc);
             if (k0 >= cnt) break;
+            if (!AHEAD) next();
         }
         f = pair2_force(acc, si, S);
     }
@@ -192,37 +197,35 @@ __device__ __forceinline__ void list_body(const RealArgs& a, int tile, int tid) 
             ec = e.x; el = e.y; wc = e.z; wl = e.w;
         }
     }
-    {
-        double e_c = 0.0, e_l = 0.0, w_c = 0.0, w_l = 0.0;
-        if ((int)tid < tl.count) {
-            const int i = tl.first + tid;
-            const int o = a.perm[i];
-            float phi = ph;
-            if (a.parts & kPartFourier) {
-                const float4 f = a.fs[o];
-                fx += f.x; fy += f.y; fz += f.z;
-                if (a.phi_out) {
-                    const double qi = (double)__uint_as_float(a.spos[i].w);
-                    const double qs = (double)(long long)__ldcg(a.qsum_fx + sys) / kQScale;
-                    phi += f.w - (float)(2.0 * S.self_coef * qi + S.bg_coef * qs);
-                }
+    double e_c = 0.0, e_l = 0.0, w_c = 0.0, w_l = 0.0;
+    if ((int)tid < tl.count) {
+        const int i = tl.first + tid;
+        const int o = a.perm[i];
+        float phi = ph;
+        if (a.parts & kPartFourier) {
+            const float4 f = a.fs[o];
+            fx += f.x; fy += f.y; fz += f.z;
+            if (a.phi_out) {
+                const double qi = (double)__uint_as_float(a.spos[i].w);
+                const double qs = (double)(long long)__ldcg(a.qsum_fx + sys) / kQScale;
+                phi += f.w - (float)(2.0 * S.self_coef * qi + S.bg_coef * qs);
             }
-            if (a.F_out) a.F_out[o] = make_float4(fx, fy, fz, 0.f);
-            if (a.phi_out) a.phi_out[o] = phi;
-            e_c = (double)ec;
-            e_l = (double)el;
-            w_c = (double)wc;
-            w_l = (double)wl;
         }
-        if (a.blk_e) {
-            const double2 r = block_sum2_real(e_c, e_l);
-            if (tid == 0) a.blk_e[tile] = r;
-        }
-        if (a.blk_w) {
-            __syncthreads();                            // the partial buffers are reused
-            const double2 r = block_sum2_real(w_c, w_l);
-            if (tid == 0) a.blk_w[tile] = r;
-        }
+        if (a.F_out) a.F_out[o] = make_float4(fx, fy, fz, 0.f);
+        if (a.phi_out) a.phi_out[o] = phi;
+        e_c = (double)ec;
+        e_l = (double)el;
+        w_c = (double)wc;
+        w_l = (double)wl;
+    }
+    if (a.blk_e) {
+        const double2 r = block_sum2_real(e_c, e_l);
+        if (tid == 0) a.blk_e[tile] = r;
+    }
+    if (a.blk_w) {
+        __syncthreads();                            // the partial buffers are reused
+        const double2 r = block_sum2_real(w_c, w_l);
+        if (tid == 0) a.blk_w[tile] = r;
     }
 }
 

@@ -11,8 +11,14 @@
 // the survivors' indices in shared memory; then the G lanes evaluate them
 // densely in FP64, which applies the cutoffs themselves.  erfc is
 // e^{-x^2} erfcx(x) with the Gaussian the force needs anyway, and one
-// reciprocal square root serves every division.  The closing MD update runs
-// one thread per particle after the block's pair sums.
+// reciprocal square root serves every division.
+//
+// Below some 10^4 particles the latency of an FP64 instruction (about a hundred
+// cycles) and of dependent loads bounds it instead: the lanes fetch the bounds of
+// a particle's nine neighbour rows side by side and walk them as one range with
+// kCand candidates in flight each, evaluate two listed pairs at a time, and a warp
+// of its own fetches what the closing update needs and draws the thermostat's
+// noise meanwhile.
 // Measured (events around the kernel, launch included): N = 1000, r_c = 5, MD
 // step: 298 -> 39 us; N = 8001, r_c = 6, forces with energy and dE/dq: 930 ->
 // 153 us.
@@ -24,6 +30,8 @@
 namespace rbe {
 
 constexpr int kHitCap = 96;           // listed candidates per particle before a flush
+constexpr int kCand = 2;              // candidates in flight per lane
+constexpr int kReal64Threads = kBlockP + 32;
 
 struct Pair64 {
     double fx, fy, fz, phr, ec, elj, wc, wlj;
@@ -38,28 +46,26 @@ __device__ __forceinline__ double min_image(double d, const Const64& c) {
     return fabs(d) > c.halfL ? d - copysign(c.L, d) : d;
 }
 
-// EN: also the potential, energies and virials.
+// EN: also the potential, energies and virials.  Without branches on the Coulomb
+// part, so that two calls in a row overlap; pj of a pair that is not one (live
+// false) is any record.
 template <bool EN>
-__device__ __forceinline__ void pair64(const double4& pi, const double4& pj, const Const64& c,
-                                       Pair64& a) {
+__device__ __forceinline__ void pair64(const double4& pi, const double4& pj, bool live,
+                                       const Const64& c, Pair64& a) {
     const double dx = min_image(pj.x - pi.x, c), dy = min_image(pj.y - pi.y, c),
                  dz = min_image(pj.z - pi.z, c);
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    const bool in = r2 < c.rc2, lj = r2 < c.lj_rc2;
-    if (!in && !lj) return;
+    const double r2 = live ? dx * dx + dy * dy + dz * dz : 1.0;
+    const bool in = live && r2 < c.rc2, lj = live && r2 < c.lj_rc2;
     const double inv_r = rsqrt(r2), inv_r2 = inv_r * inv_r;
-    double s = 0.0;
-    if (in) {
-        const double ex = exp(-c.alpha * r2);
-        const double pot = ex * erfcx(c.sqrt_alpha * (r2 * inv_r)) * inv_r;     // erfc / r
-        const double g = fma(c.two_sa_spi, ex, pot);
-        const double qq = c.lBqi * pj.w;
-        s = -qq * g * inv_r2;
-        if constexpr (EN) {
-            a.phr = fma(c.lB * pj.w, pot, a.phr);
-            a.ec = fma(0.5 * qq, pot, a.ec);
-            a.wc = fma(0.5 * qq, g, a.wc);
-        }
+    const double ex = exp(-c.alpha * r2);
+    const double pot = ex * erfcx(c.sqrt_alpha * (r2 * inv_r)) * inv_r;     // erfc / r
+    const double g = fma(c.two_sa_spi, ex, pot);
+    const double qq = in ? c.lBqi * pj.w : 0.0;
+    double s = -qq * g * inv_r2;
+    if constexpr (EN) {
+        a.phr = fma(in ? c.lB * pj.w : 0.0, pot, a.phr);
+        a.ec = fma(0.5 * qq, pot, a.ec);
+        a.wc = fma(0.5 * qq, g, a.wc);
     }
     if (lj) {
         const double sr2 = c.lj_sigma2 * inv_r2;
@@ -83,10 +89,11 @@ __device__ __forceinline__ double wrap_box(double r, double L) {
 }
 
 template <int G, bool ONE, bool EN>
-__global__ void __launch_bounds__(kBlockP)
+__global__ void __launch_bounds__(kReal64Threads)
 k_real_f64(const __grid_constant__ RealArgs a) {
     constexpr int T = kBlockP / G;               // particles per block
     __shared__ int s_hit[T][kHitCap];
+    __shared__ int s_pre[T][10], s_s0[T][9], s_n0[T][9], s_s1[T][9];   // rows as one range
     __shared__ double4 s_f[T];
     // block (x, y): particles T y .. T y + T - 1 of tile x (kBlockP particles)
     Tile tl = tile_of<ONE>(a.w);
@@ -94,173 +101,209 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     tl.count = max(0, min(T, tl.count - (int)blockIdx.y * T));
     const int blk = blockIdx.x * G + blockIdx.y;         // its energy / virial partials
     const SysDev& S = sys_of<ONE>(a.w, tl.sys);
-    const int g = threadIdx.x % G, t = threadIdx.x / G;
-    const bool active = t < tl.count;
-    const int i = tl.first + (tl.count > 0 ? min(t, tl.count - 1) : 0);
     const bool do_real = (a.parts & kPartReal) != 0;
     const bool do_lj = (a.parts & kPartLJ) != 0 && S.lj_eps != 0.0;
     Pair64 acc{0, 0, 0, 0, 0, 0, 0, 0};
-    if (tl.count > 0 && (do_real || do_lj)) {
-        const double4 pi = a.spos64[i];
-        Const64 c;
-        c.rc2 = do_real ? S.r_c * S.r_c : 0.0;
-        c.lj_rc2 = do_lj ? S.lj_rcut2 : 0.0;
-        c.lj_sigma2 = S.lj_sigma2;
-        c.lj_eps = S.lj_eps;
-        c.lj_shift = S.lj_shift;
-        c.alpha = S.alpha;
-        c.sqrt_alpha = S.sqrt_alpha;
-        c.two_sa_spi = 2.0 * S.sqrt_alpha * 0.5641895835477563;      // 1 / sqrt(pi)
-        c.lB = S.lB;
-        c.lBqi = S.lB * pi.w;
-        c.L = S.L;
-        c.halfL = 0.5 * S.L;
-        // the candidate test: fixed-point records are within a unit of the FP64
-        // positions, and the widened cutoff covers that and the FP32 rounding
-        const float Lu = S.L_over_2_32;
-        const float cut2 = fmaxf(do_real ? S.f_rc2 : 0.f, do_lj ? S.f_lj_rc2 : 0.f) * 1.0001f;
-        const uint4 si = a.spos[i];
-        const unsigned lane = threadIdx.x & 31;
-        const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane & ~(G - 1u));
-        const unsigned below = gmask & ((1u << lane) - 1u);
-        int* hit = s_hit[t];
-        int nhit = 0;                            // the same in every lane of the group
-        auto dense = [&](int n) {                // the first n listed pairs, G at a time
-            for (int k = g; k < n; k += G) pair64<EN>(pi, a.spos64[hit[k]], c, acc);
-        };
-        const int ncd = S.ncd;
-        auto cell = [&](double w) {
-            const double u = w * S.invL * (double)ncd;
-            return (u >= 0.0 && u < (double)ncd) ? (int)u : 0;
-        };
-        if (active) {
-            const int cx = cell(pi.x), cy = cell(pi.y), cz = cell(pi.z);
-            const int nrow = ncd < 3 ? 1 : 9;    // one cell: every pair once
-#pragma unroll 1
-            for (int r = 0; r < nrow; ++r) {
-                const int dz = ncd < 3 ? 0 : r / 3 - 1, dy = ncd < 3 ? 0 : r % 3 - 1;
-                const int zz = wrapc(cz + dz, ncd), yy = wrapc(cy + dy, ncd);
-                int s0, e0, s1, e1;
-                row_ranges(a.cell_start, S.off_c + (zz * ncd + yy) * ncd, cx, ncd, s0, e0, s1, e1);
-                const int n0 = e0 - s0, n = n0 + (e1 - s1);
-                for (int k0 = 0; k0 < n; k0 += G) {
-                    const int k = k0 + g;
-                    const int j = k < n0 ? s0 + k : s1 + (k - n0);
-                    bool near = false;
-                    if (k < n) {
-                        const uint4 sj = __ldg(a.spos + j);
-                        const float dx = (float)(int32_t)(sj.x - si.x) * Lu;
-                        const float dyy = (float)(int32_t)(sj.y - si.y) * Lu;
-                        const float dzz = (float)(int32_t)(sj.z - si.z) * Lu;
-                        near = fmaf(dx, dx, fmaf(dyy, dyy, dzz * dzz)) < cut2 && j != i;
+    bool owner = false;
+    if (threadIdx.x < kBlockP) {
+        // ---- the pair sums: G lanes per particle
+        const int g = threadIdx.x % G, t = threadIdx.x / G;
+        const bool active = t < tl.count;
+        owner = active && g == 0;
+        const int i = tl.first + (tl.count > 0 ? min(t, tl.count - 1) : 0);
+        if (tl.count > 0 && (do_real || do_lj)) {
+            const double4 pi = a.spos64[i];
+            Const64 c;
+            c.rc2 = do_real ? S.r_c * S.r_c : 0.0;
+            c.lj_rc2 = do_lj ? S.lj_rcut2 : 0.0;
+            c.lj_sigma2 = S.lj_sigma2;
+            c.lj_eps = S.lj_eps;
+            c.lj_shift = S.lj_shift;
+            c.alpha = S.alpha;
+            c.sqrt_alpha = S.sqrt_alpha;
+            c.two_sa_spi = 2.0 * S.sqrt_alpha * 0.5641895835477563;      // 1 / sqrt(pi)
+            c.lB = S.lB;
+            c.lBqi = S.lB * pi.w;
+            c.L = S.L;
+            c.halfL = 0.5 * S.L;
+            // the candidate test: fixed-point records are within a unit of the FP64
+            // positions, and the widened cutoff covers that and the FP32 rounding
+            const float Lu = S.L_over_2_32;
+            const float cut2 = fmaxf(do_real ? S.f_rc2 : 0.f, do_lj ? S.f_lj_rc2 : 0.f) * 1.0001f;
+            const uint4 si = a.spos[i];
+            const unsigned lane = threadIdx.x & 31;
+            const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane & ~(G - 1u));
+            const unsigned below = gmask & ((1u << lane) - 1u);
+            int* hit = s_hit[t];
+            int nhit = 0;                        // the same in every lane of the group
+            auto dense = [&](int k0, int n) {    // two listed pairs per lane from k0 on
+                const int ka = k0 + g, kb = ka + G;
+                const bool la = ka < n, lb = kb < n;
+                const double4 pa = a.spos64[la ? hit[ka] : i], pb = a.spos64[lb ? hit[kb] : i];
+                pair64<EN>(pi, pa, la, c, acc);
+                pair64<EN>(pi, pb, lb, c, acc);
+            };
+            const int ncd = S.ncd;
+            auto cell = [&](double w) {
+                const double u = w * S.invL * (double)ncd;
+                return (u >= 0.0 && u < (double)ncd) ? (int)u : 0;
+            };
+            if (active) {
+                const int cx = cell(pi.x), cy = cell(pi.y), cz = cell(pi.z);
+                const int nrow = ncd < 3 ? 1 : 9;         // one cell: every pair once
+                for (int r = g; r < nrow; r += G) {
+                    const int dz = ncd < 3 ? 0 : r / 3 - 1, dy = ncd < 3 ? 0 : r % 3 - 1;
+                    const int zz = wrapc(cz + dz, ncd), yy = wrapc(cy + dy, ncd);
+                    int b0, e0, b1, e1;
+                    row_ranges(a.cell_start, S.off_c + (zz * ncd + yy) * ncd, cx, ncd, b0, e0, b1,
+                               e1);
+                    s_s0[t][r] = b0;
+                    s_n0[t][r] = e0 - b0;
+                    s_s1[t][r] = b1;
+                    s_pre[t][r + 1] = (e0 - b0) + (e1 - b1);
+                }
+                __syncwarp(gmask);
+                if (g == 0) {
+                    int run = 0;
+                    s_pre[t][0] = 0;
+                    for (int r = 1; r <= nrow; ++r) s_pre[t][r] = run += s_pre[t][r];
+                }
+                __syncwarp(gmask);
+                const int tot = s_pre[t][nrow];
+                int r = 0;                                // row of this lane's candidate
+                for (int k0 = 0; k0 < tot; k0 += G * kCand) {
+                    uint4 sj[kCand];
+                    int jj[kCand];
+#pragma unroll
+                    for (int u = 0; u < kCand; ++u) {
+                        const int k = k0 + u * G + g;
+                        jj[u] = i;                        // not a pair
+                        if (k < tot) {
+                            while (k >= s_pre[t][r + 1]) ++r;
+                            const int o = k - s_pre[t][r], n0 = s_n0[t][r];
+                            jj[u] = o < n0 ? s_s0[t][r] + o : s_s1[t][r] + (o - n0);
+                        }
+                        sj[u] = __ldg(a.spos + jj[u]);
                     }
-                    const unsigned m = __ballot_sync(gmask, near) & gmask;
-                    if (near) hit[nhit + __popc(m & below)] = j;
-                    nhit += __popc(m);
-                    if (nhit > kHitCap - G) {    // crowded: evaluate what is listed
-                        __syncwarp(gmask);
-                        dense(nhit);
-                        __syncwarp(gmask);
-                        nhit = 0;
+#pragma unroll
+                    for (int u = 0; u < kCand; ++u) {
+                        const float dx = (float)(int32_t)(sj[u].x - si.x) * Lu;
+                        const float dyy = (float)(int32_t)(sj[u].y - si.y) * Lu;
+                        const float dzz = (float)(int32_t)(sj[u].z - si.z) * Lu;
+                        const bool near =
+                            fmaf(dx, dx, fmaf(dyy, dyy, dzz * dzz)) < cut2 && jj[u] != i;
+                        const unsigned m = __ballot_sync(gmask, near) & gmask;
+                        if (near) hit[nhit + __popc(m & below)] = jj[u];
+                        nhit += __popc(m);
+                        if (nhit > kHitCap - G) {         // crowded: evaluate what is listed
+                            __syncwarp(gmask);
+                            for (int k = 0; k < nhit; k += 2 * G) dense(k, nhit);
+                            __syncwarp(gmask);
+                            nhit = 0;
+                        }
                     }
                 }
             }
+            __syncwarp();
+            // dense rounds, the warp's groups together
+            const int rounds =
+                (int)__reduce_max_sync(0xffffffffu, (unsigned)(nhit + 2 * G - 1) / (2 * G));
+            for (int q = 0; q < rounds; ++q) dense(q * 2 * G, nhit);
         }
-        __syncwarp();
-        // dense rounds, the warp's groups together
-        const int rounds = (int)__reduce_max_sync(0xffffffffu, (unsigned)(nhit + G - 1) / G);
-        for (int q = 0; q < rounds; ++q) {
-            const int k = q * G + g;
-            if (k < nhit) pair64<EN>(pi, a.spos64[hit[k]], c, acc);
-        }
-    }
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        acc.fx += __shfl_down_sync(0xffffffffu, acc.fx, o, G);
-        acc.fy += __shfl_down_sync(0xffffffffu, acc.fy, o, G);
-        acc.fz += __shfl_down_sync(0xffffffffu, acc.fz, o, G);
-        if constexpr (EN) {
-            acc.phr += __shfl_down_sync(0xffffffffu, acc.phr, o, G);
-            acc.ec += __shfl_down_sync(0xffffffffu, acc.ec, o, G);
-            acc.elj += __shfl_down_sync(0xffffffffu, acc.elj, o, G);
-            acc.wc += __shfl_down_sync(0xffffffffu, acc.wc, o, G);
-            acc.wlj += __shfl_down_sync(0xffffffffu, acc.wlj, o, G);
+        for (int o = G / 2; o > 0; o >>= 1) {
+            acc.fx += __shfl_down_sync(0xffffffffu, acc.fx, o, G);
+            acc.fy += __shfl_down_sync(0xffffffffu, acc.fy, o, G);
+            acc.fz += __shfl_down_sync(0xffffffffu, acc.fz, o, G);
+            if constexpr (EN) {
+                acc.phr += __shfl_down_sync(0xffffffffu, acc.phr, o, G);
+                acc.ec += __shfl_down_sync(0xffffffffu, acc.ec, o, G);
+                acc.elj += __shfl_down_sync(0xffffffffu, acc.elj, o, G);
+                acc.wc += __shfl_down_sync(0xffffffffu, acc.wc, o, G);
+                acc.wlj += __shfl_down_sync(0xffffffffu, acc.wlj, o, G);
+            }
         }
+        if (owner) s_f[t] = make_double4(acc.fx, acc.fy, acc.fz, acc.phr);
     }
-    const bool owner = active && g == 0;
-    if (owner) s_f[t] = make_double4(acc.fx, acc.fy, acc.fz, acc.phr);
-    __syncthreads();
-    if ((int)threadIdx.x < min(T, tl.count)) {
-        // one thread per particle: total force, outputs, MD update
-        const int ii = tl.first + threadIdx.x;
-        const double4 fr = s_f[threadIdx.x];
-        double fx = fr.x, fy = fr.y, fz = fr.z, phi = fr.w;
-        const int o = a.perm[ii];
+    // ---- the closing warp, a lane per particle: what does not depend on the sums
+    const int tc = (int)threadIdx.x - kBlockP;
+    const bool closes = tc >= 0 && tc < tl.count;
+    const bool nhm = a.md_pos64 && a.nh && S.thermostat == RBE_THERMO_NOSE_HOOVER;
+    const bool andersen = S.thermostat == RBE_THERMO_ANDERSEN;
+    int o = 0;
+    double4 f = make_double4(0, 0, 0, 0), v = f, rp = f;
+    double xi[3] = {0.0, 0.0, 0.0};
+    bool coll = false;
+    if (closes) {
+        o = a.perm[tl.first + tc];
         if (a.parts & kPartFourier) {
-            const double4 f = a.fs64[o];
-            fx += f.x; fy += f.y; fz += f.z;
+            f = a.fs64[o];
             if (a.phi_out64) {
                 const double qs = (double)(long long)__ldcg(a.qsum_fx + tl.sys) / kQScale;
-                phi += f.w - 2.0 * S.self_coef * a.spos64[ii].w - S.bg_coef * qs;
+                f.w -= 2.0 * S.self_coef * a.spos64[tl.first + tc].w + S.bg_coef * qs;
+            }
+        } else {
+            f.w = 0.0;
+        }
+        if (a.md_pos64) {
+            v = a.md_vel64[o];
+            rp = a.md_pos64[o];
+            if (!nhm) {
+                // Langevin: normals of the OU step; Andersen: collision word, then normals
+                const uint64_t step = *a.cur_step;
+                const uint2 key = make_uint2((uint32_t)S.seed, (uint32_t)(S.seed >> 32));
+                const uint32_t pid = (uint32_t)(o - S.off_p);
+                const uint4 cw =
+                    philox4x32_10(make_uint4(pid, 0u, (uint32_t)step,
+                                             (S.stream << 8) | (andersen ? 0x07u : 0x02u)), key);
+                coll = andersen && (uint64_t)cw.x < S.andersen_thr;
+                if (!andersen || coll) {
+                    const uint4 w = andersen
+                                        ? philox4x32_10(make_uint4(pid, 1u, (uint32_t)step,
+                                                                   (S.stream << 8) | 0x07u), key)
+                                        : cw;
+                    const double u1 = ((double)w.x + 1.0) * 0x1p-32, u2 = (double)w.y * 0x1p-32;
+                    const double u3 = ((double)w.z + 1.0) * 0x1p-32, u4 = (double)w.w * 0x1p-32;
+                    const double r1 = sqrt(-2.0 * log(u1)), r3 = sqrt(-2.0 * log(u3));
+                    double s2, c2;
+                    sincospi(2.0 * u2, &s2, &c2);
+                    xi[0] = r1 * c2;
+                    xi[1] = r1 * s2;
+                    xi[2] = r3 * cospi(2.0 * u4);
+                }
             }
         }
-        if (a.F_out64) a.F_out64[o] = make_double4(fx, fy, fz, 0.0);
-        if (a.phi_out64) a.phi_out64[o] = phi;
-        if (a.md_pos64 && a.nh && S.thermostat == RBE_THERMO_NOSE_HOOVER) {
-            // Nose-Hoover leapfrog: v <- (v a + (dt/m) F) b, drift, wrap
-            const double na = a.nh[tl.sys].a, nb = a.nh[tl.sys].b;
-            const double F3[3] = {fx, fy, fz};
-            double4 v = a.md_vel64[o];
-            double4 rp = a.md_pos64[o];
+    }
+    __syncthreads();
+    if (closes) {
+        const double4 fr = s_f[tc];
+        const double F3[3] = {fr.x + f.x, fr.y + f.y, fr.z + f.z};
+        if (a.F_out64) a.F_out64[o] = make_double4(F3[0], F3[1], F3[2], 0.0);
+        if (a.phi_out64) a.phi_out64[o] = fr.w + f.w;
+        if (a.md_pos64) {
             double* vv[3] = {&v.x, &v.y, &v.z};
             double* rr[3] = {&rp.x, &rp.y, &rp.z};
-            double v2 = 0.0;
+            if (nhm) {
+                // Nose-Hoover leapfrog: v <- (v a + (dt/m) F) b, drift, wrap
+                const double na = a.nh[tl.sys].a, nb = a.nh[tl.sys].b;
+                double v2 = 0.0;
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const double vd = (*vv[d] * na + S.dt_over_m * F3[d]) * nb;
-                *rr[d] = wrap_box(*rr[d] + S.dt * vd, S.L);
-                *vv[d] = vd;
-                v2 += vd * vd;
-            }
-            a.md_vel64[o] = v;
-            a.md_pos64[o] = rp;
-            atomicAdd(&a.nh[tl.sys].k2, __double2ull_rn(v2 * S.nh_k2scale));
-        } else if (a.md_pos64) {
-            const uint64_t step = *a.cur_step;
-            const uint2 key = make_uint2((uint32_t)S.seed, (uint32_t)(S.seed >> 32));
-            const uint32_t pid = (uint32_t)(o - S.off_p);
-            const bool andersen = S.thermostat == RBE_THERMO_ANDERSEN;
-            // Langevin: normals of the OU step; Andersen: collision word, then normals
-            const uint4 cw = philox4x32_10(make_uint4(pid, 0u, (uint32_t)step,
-                                                      (S.stream << 8) | (andersen ? 0x07u : 0x02u)),
-                                           key);
-            const bool coll = andersen && (uint64_t)cw.x < S.andersen_thr;
-            double xi[3] = {0.0, 0.0, 0.0};
-            if (!andersen || coll) {
-                const uint4 w = andersen ? philox4x32_10(make_uint4(pid, 1u, (uint32_t)step,
-                                                                    (S.stream << 8) | 0x07u), key)
-                                         : cw;
-                const double u1 = ((double)w.x + 1.0) * 0x1p-32, u2 = (double)w.y * 0x1p-32;
-                const double u3 = ((double)w.z + 1.0) * 0x1p-32, u4 = (double)w.w * 0x1p-32;
-                const double r1 = sqrt(-2.0 * log(u1)), r3 = sqrt(-2.0 * log(u3));
-                double s2, c2;
-                sincospi(2.0 * u2, &s2, &c2);
-                xi[0] = r1 * c2;
-                xi[1] = r1 * s2;
-                xi[2] = r3 * cospi(2.0 * u4);
-            }
-            const double F3[3] = {fx, fy, fz};
-            double4 v = a.md_vel64[o];
-            double4 rp = a.md_pos64[o];
-            double* vv[3] = {&v.x, &v.y, &v.z};
-            double* rr[3] = {&rp.x, &rp.y, &rp.z};
+                for (int d = 0; d < 3; ++d) {
+                    const double vd = (*vv[d] * na + S.dt_over_m * F3[d]) * nb;
+                    *rr[d] = wrap_box(*rr[d] + S.dt * vd, S.L);
+                    *vv[d] = vd;
+                    v2 += vd * vd;
+                }
+                atomicAdd(&a.nh[tl.sys].k2, __double2ull_rn(v2 * S.nh_k2scale));
+            } else {
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                double vd = *vv[d] + S.dt_over_m * F3[d];
-                if (!andersen) vd = S.c1 * vd + S.c2 * xi[d];
-                *rr[d] = wrap_box(*rr[d] + S.dt * vd, S.L);
-                if (coll) vd = S.vsd * xi[d];          // Andersen collision after the drift
-                *vv[d] = vd;
+                for (int d = 0; d < 3; ++d) {
+                    double vd = *vv[d] + S.dt_over_m * F3[d];
+                    if (!andersen) vd = S.c1 * vd + S.c2 * xi[d];
+                    *rr[d] = wrap_box(*rr[d] + S.dt * vd, S.L);
+                    if (coll) vd = S.vsd * xi[d];          // Andersen collision after the drift
+                    *vv[d] = vd;
+                }
             }
             a.md_vel64[o] = v;
             a.md_pos64[o] = rp;
@@ -284,11 +327,11 @@ static void real_f64_g(cudaStream_t st, bool one, const RealArgs& a) {
     const bool en = a.phi_out64 || a.blk_e || a.blk_w;
     const dim3 grid(a.npblk, G);
     if (one) {
-        if (en) k_real_f64<G, true, true><<<grid, kBlockP, 0, st>>>(a);
-        else k_real_f64<G, true, false><<<grid, kBlockP, 0, st>>>(a);
+        if (en) k_real_f64<G, true, true><<<grid, kReal64Threads, 0, st>>>(a);
+        else k_real_f64<G, true, false><<<grid, kReal64Threads, 0, st>>>(a);
     } else {
-        if (en) k_real_f64<G, false, true><<<grid, kBlockP, 0, st>>>(a);
-        else k_real_f64<G, false, false><<<grid, kBlockP, 0, st>>>(a);
+        if (en) k_real_f64<G, false, true><<<grid, kReal64Threads, 0, st>>>(a);
+        else k_real_f64<G, false, false><<<grid, kReal64Threads, 0, st>>>(a);
     }
 }
 
