@@ -56,6 +56,7 @@ struct GraphEntry {
     const void* host_vel;
     int steps;             // steps per replay
     const void* done;      // completion word of a zero-copy host step (else null)
+    const void* pos_from;  // positions the prep kernel reads (mixed path)
     cudaGraphExec_t exec;
     int kernels;           // kernels in one replay
 };
@@ -246,6 +247,8 @@ struct rbe_ctx {
     unsigned int* d_done_cnt = nullptr;       // blocks of the closing kernel finished
     cudaEvent_t ev_real = nullptr;            // list step: real-space pass done
     cudaStream_t stream3 = nullptr;           // list step: the rebuild branch
+    cudaStream_t stream4 = nullptr;           // list step on host arrays: the velocities' copy
+    cudaEvent_t ev_vel = nullptr;             // list step on host arrays: velocities fetched
     cudaEvent_t ev_chain = nullptr;           // list step: rebuild branch done
     cudaEvent_t ev_prep = nullptr;            // list step: prep kernel done
     unsigned long long* d_qsum_fx = nullptr;  // sum q per system (fixed point)
@@ -821,6 +824,8 @@ rbe_status allocate(rbe_ctx* h) {
     RBE_CUDA(h, cudaEventCreateWithFlags(&h->ev_chain, cudaEventDisableTiming));
     RBE_CUDA(h, cudaEventCreateWithFlags(&h->ev_prep, cudaEventDisableTiming));
     RBE_CUDA(h, cudaStreamCreateWithFlags(&h->stream3, cudaStreamNonBlocking));
+    RBE_CUDA(h, cudaStreamCreateWithFlags(&h->stream4, cudaStreamNonBlocking));
+    RBE_CUDA(h, cudaEventCreateWithFlags(&h->ev_vel, cudaEventDisableTiming));
     RBE_CUDA(h, cudaHostAlloc((void**)&h->h_pin, 4 * sizeof(uint64_t), cudaHostAllocMapped));
     h->h_pin[0] = h->h_pin[1] = h->h_pin[2] = h->h_pin[3] = 0;
     RBE_CUDA(h, cudaHostGetDevicePointer((void**)&h->h_pin_dev, h->h_pin, 0));
@@ -857,6 +862,8 @@ void release(rbe_ctx* h) {
     if (h->ev_chain) cudaEventDestroy(h->ev_chain);
     if (h->ev_prep) cudaEventDestroy(h->ev_prep);
     if (h->stream3) cudaStreamDestroy(h->stream3);
+    if (h->stream4) cudaStreamDestroy(h->stream4);
+    if (h->ev_vel) cudaEventDestroy(h->ev_vel);
     if (h->h_pin) cudaFreeHost(h->h_pin);
     for (int k = 0; k < RBE_K_COUNT; ++k) {
         if (h->ev_beg[k]) cudaEventDestroy(h->ev_beg[k]);
@@ -967,6 +974,13 @@ struct EvalArgs {
     bool list;                // mixed MD step over the neighbour list
     bool list_forces;         // mixed forces call over the neighbour list
     unsigned long long* done; // list step, nullable: completion word (mapped host memory)
+    // list step on page-locked host arrays (md_pos, md_vel), else null: the device
+    // copies the closing update reads, what the prep kernel has to fill of them,
+    // and the host velocities to fetch while the structure factors run
+    const float4* pos_in;
+    float4* vel_in;
+    float4* pos_copy;
+    const float4* vel_fetch;
 };
 
 // Kernel work descriptor: tables for a batch, by-value constants and a tile
@@ -1119,6 +1133,7 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
     pa.ncell = h->ncell;
     pa.ntot = n;
     pa.nh = (a.md_pos || a.md_pos64) ? h->d_nh : nullptr;
+    pa.pos_copy = a.pos_copy;
     const bool lst = a.list || a.list_forces;     // the evaluation keeps the list
     if (lst) {
         pa.sref = h->d_sref;
@@ -1145,6 +1160,13 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
         // while the previous one drains); the list pass and the rebuild fork
         // off after prep
         cudaEventRecord(h->ev_prep, st);
+        if (a.vel_fetch) {
+            cudaStream_t sv = prof ? st : h->stream4;
+            cudaStreamWaitEvent(sv, h->ev_prep, 0);
+            cudaMemcpyAsync(a.vel_in, a.vel_fetch, sizeof(float4) * (size_t)n,
+                            cudaMemcpyDefault, sv);
+            cudaEventRecord(h->ev_vel, sv);
+        }
         if (fused) {
             // the structure factors and the pass over a standing list in one
             // launch whose blocks take either kind of work
@@ -1285,11 +1307,14 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
         cudaEventRecord(h->ev_chain, sc);
         if (!fused) cudaStreamWaitEvent(st, h->ev_real, 0);
         cudaStreamWaitEvent(st, h->ev_chain, 0);
+        if (a.vel_fetch) cudaStreamWaitEvent(st, h->ev_vel, 0);
         MdOut md{};
         md.freal = h->d_freal;
         md.F_out = a.F;
         md.md_pos = a.md_pos;
         md.md_vel = a.md_vel;
+        md.pos_in = a.pos_in ? a.pos_in : a.md_pos;
+        md.vel_in = a.vel_in ? a.vel_in : a.md_vel;
         md.nh = pa.nh;
         md.cur_step = h->d_cur_step;
         md.list_flag = h->d_list_flag;
@@ -1491,6 +1516,12 @@ struct HostIO {
     float* vel;
 };
 
+// A list step whose pos and vel are page-locked host arrays: it reads them there
+// (both; the positions by its prep kernel, the velocities by a copy while the
+// structure factors run) or finds them in the staging buffers (out), and writes
+// them there.
+enum class ZeroCopy { none, both, out };
+
 // Whether the MD steps of a single list system of n particles run as one
 // cluster (rbe_small.cu).  The cluster's blocks share the work of the whole
 // GPU, so its step grows with n P where the separate kernels' hardly does:
@@ -1514,7 +1545,7 @@ bool small_steps(rbe_ctx* h, int n) {
 
 rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nsteps,
                      uint64_t* step_dev, float* F_out = nullptr, const HostIO* io = nullptr,
-                     unsigned long long* done = nullptr) {
+                     unsigned long long* done = nullptr, ZeroCopy zc = ZeroCopy::none) {
     if (!h) return fail(nullptr, RBE_ERR_ARG, "null handle");
     rbe_status s = check_n(h, n);
     if (s != RBE_OK) return s;
@@ -1533,6 +1564,16 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
         a.F = (float4*)F_out;
         a.list = h->list;
         a.done = h->list ? done : nullptr;
+        if (zc != ZeroCopy::none && !small_steps(h, n)) {
+            a.pos_in = h->d_stage_pos;
+            a.vel_in = h->d_stage_vel;
+            if (zc == ZeroCopy::both) {
+                a.pos_copy = h->d_stage_pos;
+                a.vel_fetch = (const float4*)vel;
+            } else {
+                a.pos = h->d_stage_pos;
+            }
+        }
     } else {
         a.pos64 = (const double4*)pos;
         a.md_pos64 = (double4*)pos;
@@ -1624,7 +1665,7 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
                 g.prec == prec && g.F == (const void*)F_out &&
                 g.host_pos == (host_graph ? io->pos : nullptr) &&
                 g.host_vel == (host_graph ? io->vel : nullptr) && g.steps == k &&
-                g.done == (const void*)a.done)
+                g.done == (const void*)a.done && g.pos_from == (const void*)a.pos)
                 return &g;
         return nullptr;
     };
@@ -1648,7 +1689,8 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
         if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
         h->graphs.push_back(GraphEntry{n, pos, vel, step_dev, F_out, prec,
                                        host_graph ? io->pos : nullptr,
-                                       host_graph ? io->vel : nullptr, k, a.done, exec, kernels});
+                                       host_graph ? io->vel : nullptr, k, a.done, a.pos, exec,
+                                       kernels});
         return RBE_OK;
     };
     if (io && !host_graph) copy_in(h->stream);
@@ -1924,17 +1966,35 @@ rbe_status rbe_step_host(rbe_handle h, int32_t n, float* pos_q, float* vel, int3
     void* dpos = n > 0 ? mapped_host(pos_q) : nullptr;
     void* dvel = n > 0 ? mapped_host(vel) : nullptr;
     if (n > 0 && dpos && dvel) {
-        // page-locked arrays: the step's kernels read and write them in place
-        // over the host link (no staging copies); the step index advances in
-        // the pinned word.  A list step's closing kernel also delivers the
+        // page-locked arrays: a list step's prep kernel reads the positions over the
+        // host link and leaves a copy on the device, the velocities are fetched
+        // while the structure factors run, and the closing kernel writes both in
+        // place (it read them there too: N = 262144 225 us per step, HOST_NOW now).
+        // Without a list the kernels read and write in place.  The step index
+        // advances in the pinned word.  A list step's closing kernel also delivers the
         // error word and then a completion word there, which this thread
         // polls instead of waiting on the stream.
         const bool signal = h->list && nsteps > 0;
         const uint64_t want = step0 + (uint64_t)nsteps;
         uint64_t* done = h->h_pin + 2;
         if (signal) __atomic_store_n(done, ~want, __ATOMIC_RELAXED);
-        s = step_impl(h, n, RBE_MIXED, dpos, dvel, nsteps, h->h_pin_dev, nullptr, nullptr,
-                      signal ? (unsigned long long*)(h->h_pin_dev + 2) : nullptr);
+        unsigned long long* word = signal ? (unsigned long long*)(h->h_pin_dev + 2) : nullptr;
+        if (signal && nsteps > 1 && !small_steps(h, n)) {
+            // the steps before the last stay on the device
+            const size_t bytes = sizeof(float4) * (size_t)n;
+            RBE_CUDA(h, cudaMemcpyAsync(h->d_stage_pos, pos_q, bytes, cudaMemcpyHostToDevice,
+                                        h->stream));
+            RBE_CUDA(h, cudaMemcpyAsync(h->d_stage_vel, vel, bytes, cudaMemcpyHostToDevice,
+                                        h->stream));
+            s = step_impl(h, n, RBE_MIXED, h->d_stage_pos, h->d_stage_vel, nsteps - 1,
+                          h->h_pin_dev);
+            if (s == RBE_OK)
+                s = step_impl(h, n, RBE_MIXED, dpos, dvel, 1, h->h_pin_dev, nullptr, nullptr, word,
+                              ZeroCopy::out);
+        } else {
+            s = step_impl(h, n, RBE_MIXED, dpos, dvel, nsteps, h->h_pin_dev, nullptr, nullptr,
+                          word, signal ? ZeroCopy::both : ZeroCopy::none);
+        }
         if (s != RBE_OK) return s;
         if (signal) {
             // acquire: the outputs and the error word, stored before the word

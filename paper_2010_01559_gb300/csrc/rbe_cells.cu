@@ -313,6 +313,7 @@ k_prep_mixed(const __grid_constant__ Work w, const float4* __restrict__ pos_q,
         }
         const uint4 rec = make_uint4(sx, sy, sz, __float_as_uint(p.w));
         fx[i] = rec;
+        if (pa.pos_copy) pa.pos_copy[i] = p;
         if (pa.want_q) {
             qs = (double)p.w;
             q2s = (double)p.w * (double)p.w;

@@ -332,8 +332,8 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
             const int o = tl.first + te;
             if constexpr (SPLIT == 1) e_fr[e] = md.freal[o];
             if (md.md_pos) {
-                e_v[e] = __ldcg(md.md_vel + o);
-                e_r[e] = __ldcg(md.md_pos + o);
+                e_v[e] = __ldcg(md.vel_in + o);
+                e_r[e] = __ldcg(md.pos_in + o);
                 if (!nhm) e_z[e] = md_noise(S, __ldcg((const unsigned long long*)md.cur_step), o);
             }
         }

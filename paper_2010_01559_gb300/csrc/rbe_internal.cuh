@@ -488,6 +488,8 @@ struct PrepArgs {
     uint4* spos;             // [sorted] current records
     int* list_flag;          // set: rebuild the list in this step
     int ncell, ntot;         // cells and particles of all systems (index checks)
+    float4* pos_copy;        // nullable: the positions as read, for the closing update of a
+                             // step on page-locked host arrays
 };
 void launch_prep_mixed(cudaStream_t st, bool one, const Work& w, int nblk, const float4* pos_q,
                        uint4* fx, int* cid, int* rank, int* cell_cnt, const PrepArgs& pa,
@@ -612,8 +614,10 @@ void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int c
 struct MdOut {
     const float4* freal;     // real-space force, caller's order (null: no MD stage)
     float4* F_out;           // nullable: total force
-    float4* md_pos;          // nullable: positions / velocities updated in place
+    float4* md_pos;          // nullable: updated positions / velocities
     float4* md_vel;
+    const float4* pos_in;    // positions / velocities before the update (md_pos and md_vel,
+    const float4* vel_in;    // or device copies where those are in host memory)
     NhState* nh;
     const uint64_t* cur_step;
     int* list_flag;          // nullable: cleared (the step's rebuild flag is consumed)
