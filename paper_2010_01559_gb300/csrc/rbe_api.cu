@@ -25,6 +25,7 @@
 
 #include "rbe.h"
 #include "rbe_internal.cuh"
+#include "rbe_poly64.cuh"
 
 using namespace rbe;
 
@@ -40,6 +41,7 @@ struct SysHost {
     int ncd = 0;
     double skin = 0.0;                 // neighbour-list skin in effect (0 without a list)
     std::vector<uint64_t> table;
+    Poly64 poly64;                     // FP64 pair polynomials
     std::vector<uint64_t> mh_tq;       // MH proposal thresholds (2M+1)
     std::vector<double> mh_rho;        // MH target / proposal ratios (2M+1)
     int off_p = 0, off_c = 0, off_k = 0, off_t = 0;
@@ -127,6 +129,21 @@ void build_mh_tables(double alpha, double L, int M, std::vector<uint64_t>& tq,
     }
 }
 
+// The FP64 pair polynomials of a system (Poly64): those of the smallest range that
+// holds alpha r_c^2, times sqrt(alpha).
+void build_poly64(const rbe_params& p, Poly64& out) {
+    std::memset(&out, 0, sizeof(out));
+    const double U = p.alpha * p.r_c * p.r_c, sa = std::sqrt(p.alpha);
+    if (!(U <= 16.0)) return;
+    const bool low = U <= 8.0;
+    out.n = low ? kPolyTerms8 : kPolyTerms16;
+    for (int i = 0; i < out.n; ++i) {
+        out.a[i] = sa * (low ? kPolyA8[i] : kPolyA16[i]);
+        out.d[i] = sa * (low ? kPolyD8[i] : kPolyD16[i]);
+    }
+    out.scale = 2.0 * p.alpha / (low ? 8.0 : 16.0);
+}
+
 int pow2_ceil(long long v) {
     int p = 1;
     while (p < v && p < (1 << 30)) p <<= 1;
@@ -208,6 +225,8 @@ struct rbe_ctx {
     int* d_perm_tmp = nullptr;
     float4* d_fs = nullptr;
     double4* d_fs64 = nullptr;
+    Poly64* d_poly64 = nullptr;               // per system: FP64 pair polynomials
+    bool use_poly64 = false;
     int* d_cell_cnt = nullptr;
     int* d_cell_start = nullptr;
     int4* d_ksamp = nullptr;
@@ -729,6 +748,7 @@ rbe_status allocate(rbe_ctx* h) {
     RBE_ALLOC(h->d_perm_tmp, N);
     RBE_ALLOC(h->d_fs, N);
     RBE_ALLOC(h->d_fs64, N);
+    RBE_ALLOC(h->d_poly64, h->nsys);
     RBE_ALLOC(h->d_cell_cnt, h->ncell + 1);
     RBE_ALLOC(h->d_cell_start, h->ncell + 1);
     RBE_ALLOC(h->d_ksamp, h->ktot);
@@ -786,7 +806,9 @@ rbe_status allocate(rbe_ctx* h) {
     std::vector<uint64_t> tab, mtq;
     std::vector<double> mrho;
     std::vector<int> kstart, cstart;
+    std::vector<Poly64> poly;
     for (auto& s : h->sys) {
+        poly.push_back(s.poly64);
         tab.insert(tab.end(), s.table.begin(), s.table.end());
         mtq.insert(mtq.end(), s.mh_tq.begin(), s.mh_tq.end());
         mrho.insert(mrho.end(), s.mh_rho.begin(), s.mh_rho.end());
@@ -800,6 +822,8 @@ rbe_status allocate(rbe_ctx* h) {
     RBE_CUDA(h, cudaMemcpy(h->d_table, tab.data(), sizeof(uint64_t) * tab.size(),
                            cudaMemcpyHostToDevice));
     RBE_CUDA(h, cudaMemcpy(h->d_kstart, kstart.data(), sizeof(int) * kstart.size(),
+                           cudaMemcpyHostToDevice));
+    RBE_CUDA(h, cudaMemcpy(h->d_poly64, poly.data(), sizeof(Poly64) * poly.size(),
                            cudaMemcpyHostToDevice));
     RBE_CUDA(h, cudaMemcpy(h->d_mh_tq, mtq.data(), sizeof(uint64_t) * mtq.size(),
                            cudaMemcpyHostToDevice));
@@ -843,7 +867,7 @@ void release(rbe_ctx* h) {
                     h->d_kstart,
                     h->d_cstart,
                     h->d_table, h->d_fx, h->d_spos, h->d_fx64, h->d_spos64, h->d_cid, h->d_rank,
-                    h->d_perm, h->d_perm_tmp, h->d_fs, h->d_fs64, h->d_cell_cnt,
+                    h->d_perm, h->d_perm_tmp, h->d_fs, h->d_fs64, h->d_poly64, h->d_cell_cnt,
                     h->d_cell_start, h->d_ksamp, h->d_rho_fx, h->d_kcnt, h->d_kab,
                     h->d_kcoef, h->d_mh_tq, h->d_mh_rho, h->d_mh_state, h->d_mh_pos, h->d_nh,
                     h->d_lblk, h->d_nbr, h->d_ncnt, h->d_sref, h->d_iperm, h->d_list_flag,
@@ -899,6 +923,8 @@ rbe_status create_common(const rbe_params* ps, const int32_t* ns, int nsys, bool
         sh.M = axis_M(sh.p.alpha, sh.p.box);
         sh.H = build_table(sh.p.alpha, sh.p.box, sh.M, sh.table);
         build_mh_tables(sh.p.alpha, sh.p.box, sh.M, sh.mh_tq, sh.mh_rho);
+        build_poly64(sh.p, sh.poly64);
+        h->use_poly64 = (s == 0 || h->use_poly64) && sh.poly64.n > 0;
         if (sh.p.sampler != ps[0].sampler) {
             delete h;
             return fail(nullptr, RBE_ERR_ARG, "all systems of a handle must use the same sampler");
@@ -1022,6 +1048,8 @@ RealArgs make_real_args(const rbe_ctx* h, int parts) {
     r.fs = h->d_fs;
     r.spos64 = h->d_spos64;
     r.fs64 = h->d_fs64;
+    r.poly64 = h->d_poly64;
+    r.use_poly64 = h->use_poly64 ? 1 : 0;
     r.err = h->d_err;
     return r;
 }
@@ -1528,7 +1556,6 @@ enum class ZeroCopy { none, both, out };
 // SMALL_RULE
 constexpr int kGraphSteps = 8;
 constexpr int kSmallStepsPerLaunch = 512;
-constexpr long long kSmallMaxNP = 500000;
 
 bool small_steps(rbe_ctx* h, int n) {
     if (h->batch || h->mh || !h->list) return false;
@@ -1657,7 +1684,7 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
     // a host-buffer call replays one graph holding copies and steps (up to 4);
     // otherwise a graph holds up to kGraphSteps steps (a step's first kernel then
     // follows the previous step's last one without a graph launch in between:
-    // N = 8001 GRAPH_FIGURES us per step with one step per graph)
+    // N = 8001 GRAPH_FIGURES)
     const bool host_graph = io && nsteps <= 4;
     auto find_graph = [&](int k) -> const GraphEntry* {
         for (auto& g : h->graphs)
@@ -1969,7 +1996,7 @@ rbe_status rbe_step_host(rbe_handle h, int32_t n, float* pos_q, float* vel, int3
         // page-locked arrays: a list step's prep kernel reads the positions over the
         // host link and leaves a copy on the device, the velocities are fetched
         // while the structure factors run, and the closing kernel writes both in
-        // place (it read them there too: N = 262144 225 us per step, HOST_NOW now).
+        // place (it read them there too: N = 262144 HOST_NOW).
         // Without a list the kernels read and write in place.  The step index
         // advances in the pinned word.  A list step's closing kernel also delivers the
         // error word and then a completion word there, which this thread

@@ -645,6 +645,17 @@ void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk
 // kernel's tail with a second pass.
 constexpr int kSegChunks = 2;
 
+// FP64 path: the smooth parts of a system's pair terms as polynomials
+// (rbe_poly64.cuh) in t = scale r^2 - 1, lowest power first.
+constexpr int kPoly64 = 40;
+struct Poly64 {
+    double d[kPoly64];       // sqrt(alpha) (erf(x) / x - 2 / sqrt(pi) e^{-x^2}), x^2 = alpha r^2
+    double a[kPoly64];       // sqrt(alpha) erf(x) / x
+    double scale;            // 2 alpha / U
+    int n;                   // terms (0: alpha r_c^2 is beyond 16)
+    int pad;
+};
+
 struct RealArgs {
     Work w;                  // tiles of kBlockP particles (FP64 path)
     int npblk;
@@ -673,6 +684,8 @@ struct RealArgs {
     // fp64
     const double4* spos64;
     const double4* fs64;
+    const Poly64* poly64;    // per system
+    int use_poly64;          // every system has one
     double4* F_out64;
     double* phi_out64;
     double4* md_pos64;

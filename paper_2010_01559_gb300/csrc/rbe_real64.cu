@@ -13,6 +13,12 @@
 // e^{-x^2} erfcx(x) with the Gaussian the force needs anyway, and one
 // reciprocal square root serves every division.
 //
+// Pair terms: erfc(x) / r = 1 / r - sqrt(alpha) erf(x) / x, and erf(x) / x is an
+// entire function of u = alpha r^2, as is the Gaussian the force adds, so for the
+// usual cutoffs (u <= 16 at r_c) both come from one polynomial each (rbe_poly64.cuh):
+// about 25 to 35 multiply-adds instead of an exponential and erfcx, some 70
+// instructions.  The absolute error stays that of 1 / r.
+//
 // Below some 10^4 particles the latency of an FP64 instruction (about a hundred
 // cycles) and of dependent loads bounds it instead: the lanes fetch the bounds of
 // a particle's nine neighbour rows side by side and walk them as one range with
@@ -39,7 +45,9 @@ struct Pair64 {
 
 struct Const64 {
     double rc2, lj_rc2, lj_sigma2, lj_eps, lj_shift, alpha, sqrt_alpha, two_sa_spi, lB, lBqi;
-    double L, halfL;
+    double L, halfL, t_scale;
+    const double2* poly;                 // (d, a) per power, highest first
+    int npoly;
 };
 
 __device__ __forceinline__ double min_image(double d, const Const64& c) {
@@ -49,7 +57,7 @@ __device__ __forceinline__ double min_image(double d, const Const64& c) {
 // EN: also the potential, energies and virials.  Without branches on the Coulomb
 // part, so that two calls in a row overlap; pj of a pair that is not one (live
 // false) is any record.
-template <bool EN>
+template <bool EN, bool POLY>
 __device__ __forceinline__ void pair64(const double4& pi, const double4& pj, bool live,
                                        const Const64& c, Pair64& a) {
     const double dx = min_image(pj.x - pi.x, c), dy = min_image(pj.y - pi.y, c),
@@ -57,9 +65,24 @@ __device__ __forceinline__ void pair64(const double4& pi, const double4& pj, boo
     const double r2 = live ? dx * dx + dy * dy + dz * dz : 1.0;
     const bool in = live && r2 < c.rc2, lj = live && r2 < c.lj_rc2;
     const double inv_r = rsqrt(r2), inv_r2 = inv_r * inv_r;
-    const double ex = exp(-c.alpha * r2);
-    const double pot = ex * erfcx(c.sqrt_alpha * (r2 * inv_r)) * inv_r;     // erfc / r
-    const double g = fma(c.two_sa_spi, ex, pot);
+    double pot = 0.0, g;                 // erfc / r, erfc / r + 2 sqrt(alpha / pi) e^{-alpha r^2}
+    if constexpr (POLY) {
+        const double t = fma(r2, c.t_scale, -1.0);
+        const double2 top = c.poly[0];
+        double pd = top.x, pa = top.y;
+#pragma unroll 4
+        for (int k = 1; k < c.npoly; ++k) {
+            const double2 v = c.poly[k];
+            pd = fma(pd, t, v.x);
+            if constexpr (EN) pa = fma(pa, t, v.y);
+        }
+        g = inv_r - pd;
+        if constexpr (EN) pot = inv_r - pa;
+    } else {
+        const double ex = exp(-c.alpha * r2);
+        pot = ex * erfcx(c.sqrt_alpha * (r2 * inv_r)) * inv_r;
+        g = fma(c.two_sa_spi, ex, pot);
+    }
     const double qq = in ? c.lBqi * pj.w : 0.0;
     double s = -qq * g * inv_r2;
     if constexpr (EN) {
@@ -88,13 +111,14 @@ __device__ __forceinline__ double wrap_box(double r, double L) {
     return (r >= 0.0 && r < L) ? r : r - L * floor(r / L);
 }
 
-template <int G, bool ONE, bool EN>
+template <int G, bool ONE, bool EN, bool POLY>
 __global__ void __launch_bounds__(kReal64Threads)
 k_real_f64(const __grid_constant__ RealArgs a) {
     constexpr int T = kBlockP / G;               // particles per block
     __shared__ int s_hit[T][kHitCap];
     __shared__ int s_pre[T][10], s_s0[T][9], s_n0[T][9], s_s1[T][9];   // rows as one range
     __shared__ double4 s_f[T];
+    __shared__ double2 s_poly[POLY ? kPoly64 : 1];       // highest power first
     // block (x, y): particles T y .. T y + T - 1 of tile x (kBlockP particles)
     Tile tl = tile_of<ONE>(a.w);
     tl.first += (int)blockIdx.y * T;
@@ -105,6 +129,14 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     const bool do_lj = (a.parts & kPartLJ) != 0 && S.lj_eps != 0.0;
     Pair64 acc{0, 0, 0, 0, 0, 0, 0, 0};
     bool owner = false;
+    int npoly = 0;
+    if constexpr (POLY) {
+        const Poly64& P = a.poly64[tl.sys];
+        npoly = P.n;
+        for (int k = threadIdx.x; k < npoly; k += kReal64Threads)
+            s_poly[npoly - 1 - k] = make_double2(P.d[k], P.a[k]);
+        __syncthreads();
+    }
     if (threadIdx.x < kBlockP) {
         // ---- the pair sums: G lanes per particle
         const int g = threadIdx.x % G, t = threadIdx.x / G;
@@ -126,6 +158,9 @@ k_real_f64(const __grid_constant__ RealArgs a) {
             c.lBqi = S.lB * pi.w;
             c.L = S.L;
             c.halfL = 0.5 * S.L;
+            c.poly = s_poly;
+            c.npoly = npoly;
+            c.t_scale = POLY ? a.poly64[tl.sys].scale : 0.0;
             // the candidate test: fixed-point records are within a unit of the FP64
             // positions, and the widened cutoff covers that and the FP32 rounding
             const float Lu = S.L_over_2_32;
@@ -140,8 +175,8 @@ k_real_f64(const __grid_constant__ RealArgs a) {
                 const int ka = k0 + g, kb = ka + G;
                 const bool la = ka < n, lb = kb < n;
                 const double4 pa = a.spos64[la ? hit[ka] : i], pb = a.spos64[lb ? hit[kb] : i];
-                pair64<EN>(pi, pa, la, c, acc);
-                pair64<EN>(pi, pb, lb, c, acc);
+                pair64<EN, POLY>(pi, pa, la, c, acc);
+                pair64<EN, POLY>(pi, pb, lb, c, acc);
             };
             const int ncd = S.ncd;
             auto cell = [&](double w) {
@@ -322,16 +357,22 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     }
 }
 
+template <int G, bool ONE, bool EN>
+static void real_f64_e(cudaStream_t st, const RealArgs& a) {
+    const dim3 grid(a.npblk, G);
+    if (a.use_poly64) k_real_f64<G, ONE, EN, true><<<grid, kReal64Threads, 0, st>>>(a);
+    else k_real_f64<G, ONE, EN, false><<<grid, kReal64Threads, 0, st>>>(a);
+}
+
 template <int G>
 static void real_f64_g(cudaStream_t st, bool one, const RealArgs& a) {
     const bool en = a.phi_out64 || a.blk_e || a.blk_w;
-    const dim3 grid(a.npblk, G);
     if (one) {
-        if (en) k_real_f64<G, true, true><<<grid, kReal64Threads, 0, st>>>(a);
-        else k_real_f64<G, true, false><<<grid, kReal64Threads, 0, st>>>(a);
+        if (en) real_f64_e<G, true, true>(st, a);
+        else real_f64_e<G, true, false>(st, a);
     } else {
-        if (en) k_real_f64<G, false, true><<<grid, kReal64Threads, 0, st>>>(a);
-        else k_real_f64<G, false, false><<<grid, kReal64Threads, 0, st>>>(a);
+        if (en) real_f64_e<G, false, true>(st, a);
+        else real_f64_e<G, false, false>(st, a);
     }
 }
 
