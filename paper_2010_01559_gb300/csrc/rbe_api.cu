@@ -545,7 +545,8 @@ int auto_list_split(long long ntot) {
 
 // Threads per particle of the FP64 real-space pass, from the mixed path's: with
 // 9 of those, 32 up to 16 warps per SM (fewer serial rounds where latency
-// bounds the pass: N = 1000 REAL32) and 16 above (fuller rounds).
+// bounds the pass: five steps of N = 1000 227 us with 16, 188 with 32) and
+// 16 above (fuller rounds: N = 8001 forces 278 us with 32, 260 with 16).
 int real_split64(int r, long long ntot) {
     return r >= 8 ? (ntot <= 152LL * 16 ? 32 : 16) : (r >= 2 ? 8 : 4);
 }
@@ -1550,17 +1551,26 @@ struct HostIO {
 // them there.
 enum class ZeroCopy { none, both, out };
 
-// Whether the MD steps of a single list system of n particles run as one
-// cluster (rbe_small.cu).  The cluster's blocks share the work of the whole
-// GPU, so its step grows with n P where the separate kernels' hardly does:
-// SMALL_RULE
+// Whether the MD steps of a single list system of n particles run as one cluster
+// (rbe_small.cu).  Its sixteen SMs share the work of the whole GPU, so its step
+// grows with n and n P, about (3 + 0.0022 n + 1.6e-5 n P) us, where the separate
+// kernels' grows only with P, (10.3 + 0.009 P) us at these sizes: measured, one
+// cluster / separate, N = 1000: 5.4 / 10.4 (P = 10), 6.7 / 10.8 (100), 13.8 / 14.7
+// (500); N = 1500, P = 500: 17.4 / 15.4; N = 2000: 7.7 / 10.7 (10), 9.8 / 11.4 (100),
+// 12.5 / 12.2 (200), 21.3 / 16.4 (500); N = 3000: 10.1 / 11.2 (10), 14.0 / 12.1
+// (100), 30.5 / 18.3 (500).  The line through these leaves some near it on the slower
+// side by up to a tenth (N = 1500, P = 300: 12.8 / 14.1, taken as separate kernels).
+bool small_pays(long long n, long long P) {
+    return n * (1100 + 8 * P) <= 3650000 + 4500 * P;
+}
+
 constexpr int kGraphSteps = 8;
 constexpr int kSmallStepsPerLaunch = 512;
 
 bool small_steps(rbe_ctx* h, int n) {
     if (h->batch || h->mh || !h->list) return false;
     const SysHost& sh = h->sys[0];
-    if ((long long)n * sh.p.P > kSmallMaxNP) return false;
+    if (!small_pays(n, sh.p.P)) return false;
     if (h->small_n != n) {                       // asked once per particle count
         h->small_n = n;
         h->small_cs = 0;
@@ -1684,7 +1694,8 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
     // a host-buffer call replays one graph holding copies and steps (up to 4);
     // otherwise a graph holds up to kGraphSteps steps (a step's first kernel then
     // follows the previous step's last one without a graph launch in between:
-    // N = 8001 GRAPH_FIGURES)
+    // ten steps of N = 8001, P = 50 149 us with one step per graph, 132 with
+    // eight; N = 50021, P = 137 154 and 143)
     const bool host_graph = io && nsteps <= 4;
     auto find_graph = [&](int k) -> const GraphEntry* {
         for (auto& g : h->graphs)
@@ -1996,7 +2007,7 @@ rbe_status rbe_step_host(rbe_handle h, int32_t n, float* pos_q, float* vel, int3
         // page-locked arrays: a list step's prep kernel reads the positions over the
         // host link and leaves a copy on the device, the velocities are fetched
         // while the structure factors run, and the closing kernel writes both in
-        // place (it read them there too: N = 262144 HOST_NOW).
+        // place (it read them there too: N = 262144 222 us per step, 201 now).
         // Without a list the kernels read and write in place.  The step index
         // advances in the pinned word.  A list step's closing kernel also delivers the
         // error word and then a completion word there, which this thread

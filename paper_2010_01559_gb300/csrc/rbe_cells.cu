@@ -543,9 +543,12 @@ __global__ void k_order(int n, const int* __restrict__ cid, const int* __restric
 // in one launch of one cluster, for systems of up to kSortMaxN particles and
 // kSortMaxCells cells.  What bounds it is latency: as four kernels it is four
 // launches in a row, nearly always to find that the list stands, and they set
-// the length of a step whose other branch is as short as theirs (N = 8001:
-// SORT_FIGURES).  The phases meet at cluster barriers; data of another block is
-// read past the L1 cache.  Beyond the limit sixteen SMs take longer for a sort
+// the length of a step whose other branch is as short as theirs.
+// Measured, ten steps, four kernels / one cluster: N = 4001, P = 100 154 / 128 us;
+// 8001, P = 50 163 / 132; 60000, P = 100 281 / 263.  Where the structure factors are
+// the longer branch it gives nothing: N = 8001, P = 200 174 / 174; 20000, P = 100
+// 205 / 205; 50021, P = 137 142 / 143.  The phases meet at cluster barriers; data of
+// another block is read past the L1 cache.  Beyond the limit sixteen SMs take longer for a sort
 // than the whole GPU needs with the launches.
 constexpr int kSortThreads = 1024;
 constexpr int kSortCs = 16;                              // blocks of the cluster

