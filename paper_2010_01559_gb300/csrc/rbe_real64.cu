@@ -64,7 +64,10 @@ __device__ __forceinline__ void pair64(const double4& pi, const double4& pj, boo
                  dz = min_image(pj.z - pi.z, c);
     const double r2 = live ? dx * dx + dy * dy + dz * dz : 1.0;
     const bool in = live && r2 < c.rc2, lj = live && r2 < c.lj_rc2;
-    const double inv_r = rsqrt(r2), inv_r2 = inv_r * inv_r;
+    // the square of rsqrt's last-place error would enter the Lennard-Jones force
+    // seven times: one Newton step makes 1 / r^2 good to its rounding
+    const double inv_r = rsqrt(r2), sq = inv_r * inv_r;
+    const double inv_r2 = fma(sq, fma(-r2, sq, 1.0), sq);
     double pot = 0.0, g;                 // erfc / r, erfc / r + 2 sqrt(alpha / pi) e^{-alpha r^2}
     if constexpr (POLY) {
         const double t = fma(r2, c.t_scale, -1.0);

@@ -70,3 +70,28 @@ def test_wide_sampling_table_takes_the_direct_form(rbe):
     assert h.info().M > 560
     h.close()
     _check(rbe, wl)
+
+
+@pytest.mark.parametrize("u", [7.9, 8.0, 8.1, 15.9, 16.0, 16.1, 30.0])
+def test_pair_terms_where_the_polynomials_change(rbe, u):
+    """alpha r_c^2 at the two polynomials' ends and beyond them, and one system
+    beyond them in a batch, which takes the library functions for all."""
+    import torch
+    def wl_of(u, seed):
+        return workloads.electrolyte_1to1(250, 0.064, u / 25.0, 5.0, 40, seed=seed)
+    wl = wl_of(u, 3)
+    pos = torch.from_numpy(wl.pos_q().astype(np.float64)).cuda()
+    ref = oracle_eval(wl, 5, want_phi=True)
+    h = rbe.RBE(rbe.params_from(wl.params, n_max=wl.n))
+    F, E, phi = h.forces_f64(pos, 5, phi=True)
+    h.sync()
+    assert rel_rms(F[:, :3].cpu().numpy(), ref["F"]) <= TOL
+    assert rel_rms(phi.cpu().numpy(), ref["phi"]) <= TOL
+    h.close()
+    both = [wl, wl_of(30.0, 4)]
+    hb = rbe.RBEBatch([rbe.params_from(w.params) for w in both], [w.n for w in both])
+    posb = torch.from_numpy(np.concatenate([w.pos_q() for w in both]).astype(np.float64)).cuda()
+    Fb, _, _ = hb.forces_f64(posb, 5)
+    hb.sync()
+    assert rel_rms(Fb[:250, :3].cpu().numpy(), ref["F"]) <= TOL
+    hb.close()
