@@ -547,7 +547,9 @@ __global__ void k_order(int n, const int* __restrict__ cid, const int* __restric
 // Measured, ten steps, four kernels / one cluster: N = 4001, P = 100 154 / 128 us;
 // 8001, P = 50 163 / 132; 60000, P = 100 281 / 263.  Where the structure factors are
 // the longer branch it gives nothing: N = 8001, P = 200 174 / 174; 20000, P = 100
-// 205 / 205; 50021, P = 137 142 / 143.  The phases meet at cluster barriers; data of
+// 205 / 205; 50021, P = 137 142 / 143.  A step that does sort is longer with it above
+// some 10^4 particles (N = 8001 69 / 65 us, 20000 110 / 114, 50021 129 / 139), which one
+// step in fifty does.  The phases meet at cluster barriers; data of
 // another block is read past the L1 cache.  Beyond the limit sixteen SMs take longer for a sort
 // than the whole GPU needs with the launches.
 constexpr int kSortThreads = 1024;

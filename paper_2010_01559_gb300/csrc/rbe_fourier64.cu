@@ -21,8 +21,10 @@
 // particles per block a system of 1000 is 125 blocks, so that most SMs work
 // (one thread per particle left 8 blocks of 128).
 // Measured (events around one kernel, launch included), structure factors and
-// force: N = 1000, P = 100: 41 -> 13 and 133 -> 14 us against one sincos per
-// pair; N = 8001, P = 200: 132 -> 47 and 261 -> 67 us.
+// force: N = 1000, P = 100: 41 -> 12 and 133 -> 14 us against one sincos per
+// pair; N = 8001, P = 200: 132 -> 41 and 261 -> 67 us.  Error of forces / dE/dq
+// against an 80-bit evaluation, geometric mean over 16 systems of 9000 to 20000:
+// 0.56 / 0.79 of the direct form's.
 #include <algorithm>
 
 #include "rbe_internal.cuh"

@@ -398,8 +398,10 @@ k_real_seg(const __grid_constant__ RealArgs a) {
 // What bounds it: at 2^20 particles writing the slots (a thread per particle
 // writes its warp's entries of a slot near each other; lanes sharing a particle
 // scatter them), below about 10^5 the serial walk over some 400 candidates:
-// N = 8001 100 -> 22 us with 16 lanes (and four candidates of a lane in flight);
-// 4 lanes at N = 50021 139 us, against 120 with one.
+// N = 8001 59 us with one lane, 24 with 16.  4 lanes take 144 us at N = 50021 and 449
+// at 262144, one lane 77 and 182 (with the pair terms).  Candidates in flight, one
+// lane: 1 / 2 / 4 / 8 / 12 at N = 262144 257 / 214 / 182 / 185 / 213 us, at 2^20 814 /
+// 695 / 612 / 642 / 765.
 constexpr int kBuildU = 4;
 
 template <int R, bool ONE, bool PASS>
