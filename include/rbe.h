@@ -63,7 +63,10 @@ typedef enum {
     RBE_ERR_OOM = 3,        /* device allocation failed                                */
     RBE_ERR_SAMPLER = 4,    /* a k-sample hit (0,0,0) on 32 attempts in a row           */
     RBE_ERR_TIMEOUT = 5,    /* a host wait ran past the handle's wait limit
-                               (rbe_set_wait_limit); the work is still queued          */
+                               (rbe_set_wait_limit); the work is still queued.  Also,
+                               latched: the blocks of a small system's step (see
+                               rbe_step) did not hear from each other within 2 s and
+                               gave the step up                                       */
     RBE_ERR_NONFINITE = 6,  /* a position or charge of an input was NaN or infinite
                                (latched on the device, reported at the next sync)     */
     RBE_ERR_STATE = 7,      /* call not valid for this handle (e.g. wrong n for a batch) */
@@ -217,7 +220,10 @@ rbe_status rbe_forces_f64(rbe_handle h, int32_t n, const double *pos_q, uint64_t
  * in place.  step_dev (device uint64) holds the index of the next step; each
  * step reads it to select its k-batch and noise and increments it on the
  * device, so a captured replay advances the stream.  The step sequence is
- * replayed from a CUDA graph when use_graph was enabled (rbe_set_graph). */
+ * replayed from a CUDA graph when use_graph was enabled (rbe_set_graph).
+ * A single list system (inverse-CDF sampler) small enough that
+ * n (1100 + 8 P) <= 3.65e6 + 4500 P runs all steps of a call as one
+ * thread-block cluster, with or without graphs and whatever the tuning. */
 rbe_status rbe_step(rbe_handle h, int32_t n, float *pos_q, float *vel, int32_t nsteps,
                     uint64_t *step_dev);
 
@@ -257,7 +263,8 @@ rbe_status rbe_step_f64(rbe_handle h, int32_t n, double *pos_q, double *vel, int
 rbe_status rbe_nose_hoover_xi(rbe_handle h, double *xi, int32_t set);
 
 /* Enable (1) or disable (0) CUDA-graph replay of rbe_step.  The first
- * rbe_step call after enabling captures one step per distinct argument set. */
+ * rbe_step call with a set of arguments captures one step; later ones, and a
+ * first of 64 steps or more, capture up to eight steps per graph. */
 rbe_status rbe_set_graph(rbe_handle h, int32_t use_graph);
 
 /* Host-memory variants: copy the inputs from host (preferably pinned)
@@ -265,8 +272,11 @@ rbe_status rbe_set_graph(rbe_handle h, int32_t use_graph);
  * the handle's own.  rbe_forces_host: pos_q float4[n] in, F_out float4[n]
  * out, E_out (nullable) double[4 n_systems] out.  rbe_step_host: pos_q and
  * vel float4[n] in/out, steps step0 .. step0 + nsteps - 1; when both arrays
- * are page-locked (cudaHostAlloc, cudaHostRegister) the step's kernels read
- * and write them in place over the host link instead of staging copies, and
+ * are page-locked (cudaHostAlloc, cudaHostRegister) a single list step's
+ * first kernel reads the positions over the host link and keeps them on the
+ * device, the velocities are fetched meanwhile and the closing kernel writes
+ * both in place (of several steps the last one's; without a list every kernel
+ * works in place), and
  * on a neighbour-list handle the call returns as soon as the step's closing
  * kernel has written a completion word to the handle's mapped host memory
  * (every output store is visible to the host by then; the kernel's last

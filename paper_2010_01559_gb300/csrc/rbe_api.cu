@@ -854,8 +854,6 @@ rbe_status allocate(rbe_ctx* h) {
     int prio_low = 0, prio_high = 0;
     RBE_CUDA(h, cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
     RBE_CUDA(h, cudaStreamCreateWithPriority(&h->stream3, cudaStreamNonBlocking, prio_high));
-    RBE_CUDA(h, cudaStreamCreateWithFlags(&h->stream4, cudaStreamNonBlocking));
-    RBE_CUDA(h, cudaEventCreateWithFlags(&h->ev_vel, cudaEventDisableTiming));
     RBE_CUDA(h, cudaHostAlloc((void**)&h->h_pin, 4 * sizeof(uint64_t), cudaHostAllocMapped));
     h->h_pin[0] = h->h_pin[1] = h->h_pin[2] = h->h_pin[3] = 0;
     RBE_CUDA(h, cudaHostGetDevicePointer((void**)&h->h_pin_dev, h->h_pin, 0));
@@ -1610,6 +1608,10 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
             a.pos_in = h->d_stage_pos;
             a.vel_in = h->d_stage_vel;
             if (zc == ZeroCopy::both) {
+                if (!h->stream4)                // only handles stepped this way have one
+                    RBE_CUDA(h, cudaStreamCreateWithFlags(&h->stream4, cudaStreamNonBlocking));
+                if (!h->ev_vel)
+                    RBE_CUDA(h, cudaEventCreateWithFlags(&h->ev_vel, cudaEventDisableTiming));
                 a.pos_copy = h->d_stage_pos;
                 a.vel_fetch = (const float4*)vel;
             } else {
