@@ -47,6 +47,7 @@ struct Pair64 {
 struct Const64 {
     double rc2, lj_rc2, lj_sigma2, lj_eps, lj_shift, alpha, sqrt_alpha, two_sa_spi, lB, lBqi;
     double L, halfL, t_scale;
+    double far2;                         // r_c^2
     const double2* poly;                 // (d, a) per power, highest first
     int npoly;
 };
@@ -57,13 +58,14 @@ __device__ __forceinline__ double min_image(double d, const Const64& c) {
 
 // EN: also the potential, energies and virials.  Without branches on the Coulomb
 // part, so that two calls in a row overlap; pj of a pair that is not one (live
-// false) is any record.
+// false) is any record, and its distance stands at r_c: within the polynomials'
+// range in any unit of length (a charge of 0 does not cancel an infinity).
 template <bool EN, bool POLY>
 __device__ __forceinline__ void pair64(const double4& pi, const double4& pj, bool live,
                                        const Const64& c, Pair64& a) {
     const double dx = min_image(pj.x - pi.x, c), dy = min_image(pj.y - pi.y, c),
                  dz = min_image(pj.z - pi.z, c);
-    const double r2 = live ? dx * dx + dy * dy + dz * dz : 1.0;
+    const double r2 = live ? dx * dx + dy * dy + dz * dz : c.far2;
     const bool in = live && r2 < c.rc2, lj = live && r2 < c.lj_rc2;
     // the square of rsqrt's last-place error would enter the Lennard-Jones force
     // seven times: one Newton step makes 1 / r^2 good to its rounding
@@ -150,7 +152,8 @@ k_real_f64(const __grid_constant__ RealArgs a) {
         if (tl.count > 0 && (do_real || do_lj)) {
             const double4 pi = a.spos64[i];
             Const64 c;
-            c.rc2 = do_real ? S.r_c * S.r_c : 0.0;
+            c.far2 = S.r_c * S.r_c;
+            c.rc2 = do_real ? c.far2 : 0.0;
             c.lj_rc2 = do_lj ? S.lj_rcut2 : 0.0;
             c.lj_sigma2 = S.lj_sigma2;
             c.lj_eps = S.lj_eps;
