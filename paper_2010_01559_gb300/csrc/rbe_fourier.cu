@@ -64,13 +64,14 @@ __global__ void k_sample(const SysDev* __restrict__ sysv, int nsys, int ktot,
 // N = 8001, P = 200 14.3 -> 11.2 us; 50021, P = 137 39.3 -> 14.0; 100003, P = 200 40.9 ->
 // 20.8; 2^20, P = 100 129 -> 60.5; 262144, P = 500 70.6 -> 70.2 (full lanes already).
 
-// round(f 2^e) as a 64-bit integer, in integer arithmetic (|f| 2^e < 2^62)
+// round(f 2^e) as a 64-bit integer, in integer arithmetic (|f| 2^e < 2^63; beyond, the
+// words saturate as a conversion of the double would)
 __device__ __forceinline__ long long fixed64(float f, int e) {
     const uint32_t b = __float_as_uint(f);
     const int ex = (int)((b >> 23) & 255u);
     const long long m = ex ? (long long)((b & 0x7FFFFFu) | 0x800000u) : 0ll;
     const int sh = ex - 150 + e;
-    const long long v = sh >= 0 ? m << min(sh, 38)
+    const long long v = sh >= 0 ? (sh <= 39 ? m << sh : 0x7FFFFFFFFFFFFFFFll)
                                 : (sh > -25 ? (m + (1ll << (-sh - 1))) >> -sh : 0ll);
     return (b >> 31) ? -v : v;
 }
