@@ -169,9 +169,12 @@ k_real_f64(const __grid_constant__ RealArgs a) {
             c.npoly = npoly;
             c.t_scale = POLY ? a.poly64[tl.sys].scale : 0.0;
             // the candidate test: fixed-point records are within a unit of the FP64
-            // positions, and the widened cutoff covers that and the FP32 rounding
+            // positions (a displacement within two, whatever the box measures in
+            // cutoffs), and the cutoff widened by 5e-5 covers the FP32 rounding
             const float Lu = S.L_over_2_32;
-            const float cut2 = fmaxf(do_real ? S.f_rc2 : 0.f, do_lj ? S.f_lj_rc2 : 0.f) * 1.0001f;
+            const float cut = fmaf(sqrtf(fmaxf(do_real ? S.f_rc2 : 0.f,
+                                               do_lj ? S.f_lj_rc2 : 0.f)), 1.00005f, 2.f * Lu);
+            const float cut2 = cut * cut;
             const uint4 si = a.spos[i];
             const unsigned lane = threadIdx.x & 31;
             const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (lane & ~(G - 1u));
