@@ -41,7 +41,7 @@ struct SysHost {
     int ncd = 0;
     double skin = 0.0;                 // neighbour-list skin in effect (0 without a list)
     std::vector<uint64_t> table;
-    Poly64 poly64;                     // FP64 pair polynomials
+    Poly64 poly64;                     // erfcx of the FP64 pair terms
     std::vector<uint64_t> mh_tq;       // MH proposal thresholds (2M+1)
     std::vector<double> mh_rho;        // MH target / proposal ratios (2M+1)
     int off_p = 0, off_c = 0, off_k = 0, off_t = 0;
@@ -129,19 +129,16 @@ void build_mh_tables(double alpha, double L, int M, std::vector<uint64_t>& tq,
     }
 }
 
-// The FP64 pair polynomials of a system (Poly64): those of the smallest range that
-// holds alpha r_c^2, times sqrt(alpha).
+// The polynomial of a system's FP64 pair terms (Poly64): that of the smallest range
+// that holds alpha r_c^2.
 void build_poly64(const rbe_params& p, Poly64& out) {
     std::memset(&out, 0, sizeof(out));
-    const double U = p.alpha * p.r_c * p.r_c, sa = std::sqrt(p.alpha);
-    if (!(U <= 16.0)) return;
-    const bool low = U <= 8.0;
+    const double u = p.alpha * p.r_c * p.r_c;
+    if (!(u <= 16.0)) return;
+    const bool low = u <= 8.0;
     out.n = low ? kPolyTerms8 : kPolyTerms16;
-    for (int i = 0; i < out.n; ++i) {
-        out.a[i] = sa * (low ? kPolyA8[i] : kPolyA16[i]);
-        out.d[i] = sa * (low ? kPolyD8[i] : kPolyD16[i]);
-    }
-    out.scale = 2.0 * p.alpha / (low ? 8.0 : 16.0);
+    std::copy_n(low ? kErfcx8 : kErfcx16, out.n, out.c);
+    out.scale = 2.0 * std::sqrt(p.alpha / (low ? 8.0 : 16.0));
 }
 
 int pow2_ceil(long long v) {
@@ -225,7 +222,7 @@ struct rbe_ctx {
     int* d_perm_tmp = nullptr;
     float4* d_fs = nullptr;
     double4* d_fs64 = nullptr;
-    Poly64* d_poly64 = nullptr;               // per system: FP64 pair polynomials
+    Poly64* d_poly64 = nullptr;               // per system: erfcx of the FP64 pairs
     bool use_poly64 = false;
     int* d_cell_cnt = nullptr;
     int* d_cell_start = nullptr;

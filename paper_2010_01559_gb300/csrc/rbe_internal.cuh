@@ -645,13 +645,12 @@ void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk
 // kernel's tail with a second pass.
 constexpr int kSegChunks = 2;
 
-// FP64 path: the smooth parts of a system's pair terms as polynomials
-// (rbe_poly64.cuh) in t = scale r^2 - 1, lowest power first.
-constexpr int kPoly64 = 40;
+// FP64 path: erfcx(sqrt(alpha) r) up to a system's cutoff as a polynomial
+// (rbe_poly64.cuh) in t = scale r - 1, lowest power first.
+constexpr int kPoly64 = 32;
 struct Poly64 {
-    double d[kPoly64];       // sqrt(alpha) (erf(x) / x - 2 / sqrt(pi) e^{-x^2}), x^2 = alpha r^2
-    double a[kPoly64];       // sqrt(alpha) erf(x) / x
-    double scale;            // 2 alpha / U
+    double c[kPoly64];
+    double scale;            // 2 sqrt(alpha / U)
     int n;                   // terms (0: alpha r_c^2 is beyond 16)
     int pad;
 };

@@ -13,11 +13,11 @@
 // e^{-x^2} erfcx(x) with the Gaussian the force needs anyway, and one
 // reciprocal square root serves every division.
 //
-// Pair terms: erfc(x) / r = 1 / r - sqrt(alpha) erf(x) / x, and erf(x) / x is an
-// entire function of u = alpha r^2, as is the Gaussian the force adds, so for the
-// usual cutoffs (u <= 16 at r_c) both come from one polynomial each (rbe_poly64.cuh):
-// about 25 to 35 multiply-adds instead of an exponential and erfcx, some 70
-// instructions.  The absolute error stays that of 1 / r.
+// erfcx is a polynomial of about 30 terms for the usual cutoffs (alpha r_c^2 <= 16,
+// rbe_poly64.cuh), the library's beyond.  Every factor of a term keeps its relative
+// accuracy, so that a pair near the cutoff, where erfc has fallen by up to seven
+// orders, is as good as a close one (1 / r minus a polynomial of erf(x) / x takes a
+// term less, but is good to 1e-16 / r only).
 //
 // Below some 10^4 particles the latency of an FP64 instruction (about a hundred
 // cycles) and of dependent loads bounds it instead: the lanes fetch the bounds of
@@ -48,7 +48,7 @@ struct Const64 {
     double rc2, lj_rc2, lj_sigma2, lj_eps, lj_shift, alpha, sqrt_alpha, two_sa_spi, lB, lBqi;
     double L, halfL, t_scale;
     double far2;                         // r_c^2
-    const double2* poly;                 // (d, a) per power, highest first
+    const double* poly;                  // highest power first
     int npoly;
 };
 
@@ -71,24 +71,19 @@ __device__ __forceinline__ void pair64(const double4& pi, const double4& pj, boo
     // seven times: one Newton step makes 1 / r^2 good to its rounding
     const double inv_r = rsqrt(r2), sq = inv_r * inv_r;
     const double inv_r2 = fma(sq, fma(-r2, sq, 1.0), sq);
-    double pot = 0.0, g;                 // erfc / r, erfc / r + 2 sqrt(alpha / pi) e^{-alpha r^2}
+    const double r = r2 * inv_r;
+    double ecx;                          // erfcx(sqrt(alpha) r)
     if constexpr (POLY) {
-        const double t = fma(r2, c.t_scale, -1.0);
-        const double2 top = c.poly[0];
-        double pd = top.x, pa = top.y;
+        const double t = fma(r, c.t_scale, -1.0);
+        ecx = c.poly[0];
 #pragma unroll 4
-        for (int k = 1; k < c.npoly; ++k) {
-            const double2 v = c.poly[k];
-            pd = fma(pd, t, v.x);
-            if constexpr (EN) pa = fma(pa, t, v.y);
-        }
-        g = inv_r - pd;
-        if constexpr (EN) pot = inv_r - pa;
+        for (int k = 1; k < c.npoly; ++k) ecx = fma(ecx, t, c.poly[k]);
     } else {
-        const double ex = exp(-c.alpha * r2);
-        pot = ex * erfcx(c.sqrt_alpha * (r2 * inv_r)) * inv_r;
-        g = fma(c.two_sa_spi, ex, pot);
+        ecx = erfcx(c.sqrt_alpha * r);
     }
+    const double ex = exp(-c.alpha * r2);
+    const double pot = ex * ecx * inv_r;                       // erfc / r
+    const double g = fma(c.two_sa_spi, ex, pot);               // + 2 sqrt(alpha / pi) e^{-alpha r^2}
     const double qq = in ? c.lBqi * pj.w : 0.0;
     double s = -qq * g * inv_r2;
     if constexpr (EN) {
@@ -124,7 +119,7 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     __shared__ int s_hit[T][kHitCap];
     __shared__ int s_pre[T][10], s_s0[T][9], s_n0[T][9], s_s1[T][9];   // rows as one range
     __shared__ double4 s_f[T];
-    __shared__ double2 s_poly[POLY ? kPoly64 : 1];       // highest power first
+    __shared__ double s_poly[POLY ? kPoly64 : 1];        // highest power first
     // block (x, y): particles T y .. T y + T - 1 of tile x (kBlockP particles)
     Tile tl = tile_of<ONE>(a.w);
     tl.first += (int)blockIdx.y * T;
@@ -140,7 +135,7 @@ k_real_f64(const __grid_constant__ RealArgs a) {
         const Poly64& P = a.poly64[tl.sys];
         npoly = P.n;
         for (int k = threadIdx.x; k < npoly; k += kReal64Threads)
-            s_poly[npoly - 1 - k] = make_double2(P.d[k], P.a[k]);
+            s_poly[npoly - 1 - k] = P.c[k];
         __syncthreads();
     }
     if (threadIdx.x < kBlockP) {

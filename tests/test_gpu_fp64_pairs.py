@@ -1,5 +1,6 @@
-"""The FP64 real-space pair terms of isolated pairs at the cutoff's edge, in a box a
-million cutoffs wide.
+"""The FP64 real-space pair terms to their own relative accuracy: isolated pairs up
+to the cutoff, where erfc has fallen by seven orders, and pairs at the cutoff's edge
+in a box a million cutoffs wide.
 
 Bounds: a pair term's relative error is that of e^{-u} (u = alpha r^2, the
 exponent's two roundings: 2 u 2^-53) and about ten more roundings, in the kernel and
@@ -70,6 +71,16 @@ def _check(rbe, box, alpha, r_c, pos, q):
     assert rel.max() <= 1e-13, rel.max()
     assert abs(E[0, 2].item() - re.sum()) <= 1e-13 * np.abs(re).sum()
     h.close()
+
+
+@pytest.mark.parametrize("u", [4.0, 7.9, 8.1, 15.9, 16.1, 30.0])
+def test_relative_accuracy_up_to_the_cutoff(rbe, u):
+    rng = np.random.default_rng(5)
+    dist = 5.0 * np.linspace(0.9, 0.99999, 64)
+    pos = _pairs(60.0, 15.0, 4, dist, rng)
+    q = np.tile([1.0, 1.0, 1.0, -1.0], 32)
+    q[::2] *= np.linspace(0.5, 2.0, 64)
+    _check(rbe, 60.0, u / 25.0, 5.0, pos, q)
 
 
 def test_cutoff_far_below_the_box(rbe):
