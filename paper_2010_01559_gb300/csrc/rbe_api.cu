@@ -223,7 +223,7 @@ struct rbe_ctx {
     float4* d_fs = nullptr;
     double4* d_fs64 = nullptr;
     Poly64* d_poly64 = nullptr;               // per system: erfcx of the FP64 pairs
-    bool use_poly64 = false;
+    int npoly64 = 0;                          // systems within its range
     int* d_cell_cnt = nullptr;
     int* d_cell_start = nullptr;
     int4* d_ksamp = nullptr;
@@ -925,7 +925,7 @@ rbe_status create_common(const rbe_params* ps, const int32_t* ns, int nsys, bool
         sh.H = build_table(sh.p.alpha, sh.p.box, sh.M, sh.table);
         build_mh_tables(sh.p.alpha, sh.p.box, sh.M, sh.mh_tq, sh.mh_rho);
         build_poly64(sh.p, sh.poly64);
-        h->use_poly64 = (s == 0 || h->use_poly64) && sh.poly64.n > 0;
+        h->npoly64 += sh.poly64.n > 0;
         if (sh.p.sampler != ps[0].sampler) {
             delete h;
             return fail(nullptr, RBE_ERR_ARG, "all systems of a handle must use the same sampler");
@@ -1050,7 +1050,7 @@ RealArgs make_real_args(const rbe_ctx* h, int parts) {
     r.spos64 = h->d_spos64;
     r.fs64 = h->d_fs64;
     r.poly64 = h->d_poly64;
-    r.use_poly64 = h->use_poly64 ? 1 : 0;
+    r.poly64_form = h->npoly64 == 0 ? 0 : (h->npoly64 == h->nsys ? 1 : 2);
     r.err = h->d_err;
     return r;
 }

@@ -684,7 +684,7 @@ struct RealArgs {
     const double4* spos64;
     const double4* fs64;
     const Poly64* poly64;    // per system
-    int use_poly64;          // every system has one
+    int poly64_form;         // systems that have one: 0 none, 1 all, 2 some
     double4* F_out64;
     double* phi_out64;
     double4* md_pos64;

@@ -56,11 +56,16 @@ __device__ __forceinline__ double min_image(double d, const Const64& c) {
     return fabs(d) > c.halfL ? d - copysign(c.L, d) : d;
 }
 
+// How a launch's systems get erfcx: a system alone by its polynomial or, beyond its
+// range, the library's function; a batch of either kind alone likewise, a batch of
+// both by each block's own system, so that no system's results depend on the others.
+enum { kErfcxLib, kErfcxPoly, kErfcxEach };             // RealArgs.poly64_form
+
 // EN: also the potential, energies and virials.  Without branches on the Coulomb
 // part, so that two calls in a row overlap; pj of a pair that is not one (live
 // false) is any record, and its distance stands at r_c: within the polynomials'
 // range in any unit of length (a charge of 0 does not cancel an infinity).
-template <bool EN, bool POLY>
+template <bool EN, int POLY>
 __device__ __forceinline__ void pair64(const double4& pi, const double4& pj, bool live,
                                        const Const64& c, Pair64& a) {
     const double dx = min_image(pj.x - pi.x, c), dy = min_image(pj.y - pi.y, c),
@@ -73,7 +78,7 @@ __device__ __forceinline__ void pair64(const double4& pi, const double4& pj, boo
     const double inv_r2 = fma(sq, fma(-r2, sq, 1.0), sq);
     const double r = r2 * inv_r;
     double ecx;                          // erfcx(sqrt(alpha) r)
-    if constexpr (POLY) {
+    if (POLY == kErfcxPoly || (POLY == kErfcxEach && c.npoly > 0)) {
         const double t = fma(r, c.t_scale, -1.0);
         ecx = c.poly[0];
 #pragma unroll 4
@@ -112,7 +117,7 @@ __device__ __forceinline__ double wrap_box(double r, double L) {
     return (r >= 0.0 && r < L) ? r : r - L * floor(r / L);
 }
 
-template <int G, bool ONE, bool EN, bool POLY>
+template <int G, bool ONE, bool EN, int POLY>
 __global__ void __launch_bounds__(kReal64Threads)
 k_real_f64(const __grid_constant__ RealArgs a) {
     constexpr int T = kBlockP / G;               // particles per block
@@ -365,8 +370,15 @@ k_real_f64(const __grid_constant__ RealArgs a) {
 template <int G, bool ONE, bool EN>
 static void real_f64_e(cudaStream_t st, const RealArgs& a) {
     const dim3 grid(a.npblk, G);
-    if (a.use_poly64) k_real_f64<G, ONE, EN, true><<<grid, kReal64Threads, 0, st>>>(a);
-    else k_real_f64<G, ONE, EN, false><<<grid, kReal64Threads, 0, st>>>(a);
+    if constexpr (!ONE)
+        if (a.poly64_form == kErfcxEach) {
+            k_real_f64<G, ONE, EN, kErfcxEach><<<grid, kReal64Threads, 0, st>>>(a);
+            return;
+        }
+    if (a.poly64_form == kErfcxPoly)
+        k_real_f64<G, ONE, EN, kErfcxPoly><<<grid, kReal64Threads, 0, st>>>(a);
+    else
+        k_real_f64<G, ONE, EN, kErfcxLib><<<grid, kReal64Threads, 0, st>>>(a);
 }
 
 template <int G>
