@@ -304,7 +304,9 @@ rbe_status rbe_set_wait_limit(rbe_handle h, double seconds);
 
 /* Launch shapes of the per-particle kernels (0 = automatic for every field). */
 typedef struct {
-    int32_t rho_chunk;     /* particles per structure-factor chunk: power of two in [32, 8192] */
+    int32_t rho_chunk;     /* particles per structure-factor chunk: power of two in [32, 8192];
+                              0 or the automatic chunk's value: the mixed path's tiles are
+                              automatic too (any number of particles)                      */
     int32_t force_split;   /* threads per particle in the Fourier-force pass: 1, 2, 4 or 8     */
     int32_t real_split;    /* threads per particle in the mixed real-space pass: 1, 3 or 9,
                               each scanning 9 / real_split of the 9 neighbour rows (the FP64

@@ -184,7 +184,7 @@ struct rbe_ctx {
     // evaluation without (n) and with energies (e)
     int nrt = 0, rt_n = 0, rt_e = 0, run_n = 64, run_e = 64, max_rt = 0;
     int rho_t = 256;                          // threads per block
-    bool cur_set = false;                     // the chunk in effect was set, not automatic
+    bool cur_set = false;                     // the chunk in effect is not the automatic one
     bool use_graph = false;
     double wait_limit = 0.0;                  // seconds a host wait may take (0: no limit)
     // list steps: structure factors + standing-list pass in one launch:
@@ -562,7 +562,11 @@ int auto_real_seg(long long ntot, long long ncell, int ncd) {
 rbe_status prepare(rbe_ctx* h, int n) {
     if (!h->batch) h->sys[0].n = n;
     const long long ntot = h->batch ? h->ntot : n;
-    const int chunk = h->rho_chunk > 0 ? h->rho_chunk : auto_chunk(h, ntot);
+    // naming the automatic chunk names the automatic shapes of the mixed path with it:
+    // a chunk read by rbe_get_tuning can be set again, and rbe_autotune tries them
+    const int achunk = auto_chunk(h, ntot);
+    const int chunk = h->rho_chunk > 0 ? h->rho_chunk : achunk;
+    const bool named = chunk != achunk;
     const int split = h->force_split > 0 ? h->force_split : auto_split(ntot);
     const int rsplit = h->real_split > 0 ? h->real_split : auto_real_split(ntot);
     const int lsplit = h->list_split > 0 ? h->list_split : auto_list_split(ntot);
@@ -572,13 +576,13 @@ rbe_status prepare(rbe_ctx* h, int n) {
                                      : auto_real_seg(ntot, h->ncell, ncd_max);
     if (h->cur_n == n && h->cur_chunk == chunk && h->cur_split == split &&
         h->cur_rsplit == rsplit && h->cur_seg == rseg && h->cur_lsplit == lsplit &&
-        h->cur_set == (h->rho_chunk > 0))
+        h->cur_set == named)
         return RBE_OK;
     // mixed structure factors: particles per block and FP32 runs (with energies,
     // the chunk's, and tiles of whole runs)
     const int rho_t = auto_rho_threads(h->pmax);
     const int run = auto_run(h->pmax, ntot, rho_t), run_e = std::min(chunk, kRhoStage);
-    int rtile_n = h->rho_chunk > 0 ? chunk : auto_rho_tile(h->pmax, ntot, run, rho_t);
+    int rtile_n = named ? chunk : auto_rho_tile(h->pmax, ntot, run, rho_t);
     const int rtile_e = (rtile_n + run_e - 1) / run_e * run_e;
     if (h->batch) rtile_n = rtile_e;              // one table serves both
     h->list_valid = false;                 // the sorted arrays are rebuilt from scratch
@@ -678,7 +682,7 @@ rbe_status prepare(rbe_ctx* h, int n) {
     h->run_n = run;
     h->run_e = run_e;
     h->rho_t = rho_t;
-    h->cur_set = h->rho_chunk > 0;
+    h->cur_set = named;
     h->split = split;
     h->rsplit = rsplit;
     h->nseg = (int)segs.size();
