@@ -666,7 +666,8 @@ static cudaError_t sort_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* att
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaFuncSetAttribute(k_sort<ONE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    static KernelLimits limits;
+    return limits.set((const void*)k_sort<ONE>, true);
 }
 
 // Whether the GPU can place the sort's cluster.

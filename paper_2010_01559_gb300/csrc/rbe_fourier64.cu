@@ -325,9 +325,8 @@ constexpr int kTabMaxM = 560;               // 8 * 3 * 561 * 16 B = 210 KB
 template <bool ONE, int KR>
 static void rho_f64_kr(cudaStream_t st, const Work& w, dim3 grid, size_t smem, const int4* ksamp,
                        const double4* fx64, unsigned long long* rho_fx) {
-    if (smem > 40 * 1024)
-        cudaFuncSetAttribute(k_rho_f64_tab<ONE, KR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    static KernelLimits limits;
+    limits.set((const void*)k_rho_f64_tab<ONE, KR>);
     k_rho_f64_tab<ONE, KR><<<grid, kTabThreads, smem, st>>>(w, ksamp, fx64, rho_fx);
 }
 
@@ -363,10 +362,8 @@ template <bool ONE, bool PHI>
 static void force_f64_tab(cudaStream_t st, const Work& w, int nblk, size_t smem,
                           const double4* fx64, const int4* ksamp, const double* kcoef,
                           const unsigned long long* rho_fx, double4* fs64, bool pdl) {
-    // + the staged wave vectors in static shared memory
-    if (smem > 32 * 1024)
-        cudaFuncSetAttribute(k_force_f64_tab<ONE, PHI>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static KernelLimits limits;
+    limits.set((const void*)k_force_f64_tab<ONE, PHI>);
     PdlConfig c(dim3(nblk, kBlockP / kTabP), dim3(kTabThreads), smem, st, pdl);
     cudaLaunchKernelEx(&c.cfg, k_force_f64_tab<ONE, PHI>, w, fx64, ksamp, kcoef, rho_fx, fs64);
 }

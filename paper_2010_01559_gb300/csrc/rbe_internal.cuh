@@ -24,6 +24,7 @@
 // and the same with double4 / double2 records for the FP64 path.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -449,6 +450,42 @@ struct PdlConfig {
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = pdl ? 1 : 0;
+    }
+};
+
+// The launch limits of one kernel: as much dynamic shared memory as its static part
+// leaves and, with clusters, more than eight blocks of one.  A kernel's attributes
+// belong to the process: set to the size of one handle's launch, they had another
+// thread's refused between the two calls.  So they are raised once per device, to
+// all there is, and a launch names its own size alone.  (Threads that meet here set
+// the same values.)
+class KernelLimits {
+    static constexpr int kDevices = 64;
+    std::atomic<bool> done_[kDevices] = {};
+    static cudaError_t raise(const void* kernel, int device, bool clusters) {
+        int smem = 0;
+        cudaFuncAttributes at{};
+        cudaError_t e = cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin,
+                                               device);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     smem - (int)at.sharedSizeBytes);
+        if (e == cudaSuccess && clusters)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        return e;
+    }
+
+public:
+    cudaError_t set(const void* kernel, bool clusters = false) {
+        int device = 0;
+        cudaError_t e = cudaGetDevice(&device);
+        if (e != cudaSuccess) return e;
+        if (device < kDevices && done_[device].load(std::memory_order_acquire)) return cudaSuccess;
+        e = raise(kernel, device, clusters);
+        if (e == cudaSuccess && device < kDevices)
+            done_[device].store(true, std::memory_order_release);
+        return e;
     }
 };
 

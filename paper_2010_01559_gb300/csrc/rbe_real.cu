@@ -622,18 +622,18 @@ size_t real_seg_smem(int stage_cap, int seg_max, int nt) {
            sizeof(int) * 9 * (size_t)(seg_max + 3) + sizeof(uint32_t) * (size_t)(seg_max + 1);
 }
 
+template <int R, bool ONE, int NT>
+static void real_mixed_ro(cudaStream_t st, const RealArgs& a) {
+    static KernelLimits limits;
+    limits.set((const void*)k_real_seg<R, ONE, NT>);
+    k_real_seg<R, ONE, NT><<<a.nseg * kSegChunks, NT, real_seg_smem(a.stage_cap, a.seg_max, NT),
+                             st>>>(a);
+}
+
 template <int R, int NT>
 static void real_mixed_rn(cudaStream_t st, bool one, const RealArgs& a) {
-    const size_t smem = real_seg_smem(a.stage_cap, a.seg_max, NT);
-    if (one) {
-        cudaFuncSetAttribute(k_real_seg<R, true, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-        k_real_seg<R, true, NT><<<a.nseg * kSegChunks, NT, smem, st>>>(a);
-    } else {
-        cudaFuncSetAttribute(k_real_seg<R, false, NT>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_real_seg<R, false, NT><<<a.nseg * kSegChunks, NT, smem, st>>>(a);
-    }
+    if (one) real_mixed_ro<R, true, NT>(st, a);
+    else real_mixed_ro<R, false, NT>(st, a);
 }
 
 // Block size: enough warps for the particles of a typical segment, 64 .. 256.

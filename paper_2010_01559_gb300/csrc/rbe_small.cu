@@ -547,7 +547,7 @@ static int small_lanes(int n, int cs) {
 }
 
 template <int R>
-static bool small_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, cudaStream_t st,
+static cudaError_t small_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, cudaStream_t st,
                          int cs, size_t smem) {
     cfg = cudaLaunchConfig_t{};
     cfg.gridDim = dim3(cs);
@@ -560,10 +560,8 @@ static bool small_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, cud
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaFuncSetAttribute(k_small_md<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem) == cudaSuccess &&
-           cudaFuncSetAttribute(k_small_md<R>, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                                1) == cudaSuccess;
+    static KernelLimits limits;
+    return limits.set((const void*)k_small_md<R>, true);
 }
 
 template <int R>
@@ -571,7 +569,7 @@ static bool small_fits(int cs, size_t smem) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     int clusters = 0;
-    const bool ok = small_config<R>(cfg, attr, nullptr, cs, smem) &&
+    const bool ok = small_config<R>(cfg, attr, nullptr, cs, smem) == cudaSuccess &&
                     cudaOccupancyMaxActiveClusters(&clusters, k_small_md<R>, &cfg) == cudaSuccess;
     if (!ok) cudaGetLastError();
     return ok && clusters >= 1;
@@ -598,7 +596,8 @@ template <int R>
 static cudaError_t small_launch(cudaStream_t st, const SmallArgs& a, size_t smem) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    if (!small_config<R>(cfg, attr, st, a.cs, smem)) return cudaGetLastError();
+    const cudaError_t e = small_config<R>(cfg, attr, st, a.cs, smem);
+    if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, k_small_md<R>, a);
 }
 
