@@ -202,6 +202,11 @@ struct rbe_ctx {
     double prof_ms[RBE_K_COUNT] = {};
     int64_t prof_cnt[RBE_K_COUNT] = {};
     int64_t kernel_count = 0;
+    // a launch of the current call was refused (the call's other evaluations are
+    // skipped), and the first error of the call (some runtime calls that succeed
+    // clear the thread's last error, so it is kept here)
+    bool refused = false;
+    cudaError_t call_err = cudaSuccess;
 
     SysDev* d_sys = nullptr;
     Tile* d_pblk = nullptr;
@@ -560,8 +565,30 @@ int auto_real_seg(long long ntot, long long ncell, int ncd) {
     return std::max(1, std::min(seg, ncd));
 }
 
+// Keeps the first error of a call; true if there was a new one.
+bool note_error(rbe_ctx* h) {
+    const cudaError_t e = cudaGetLastError();
+    if (h->call_err == cudaSuccess) h->call_err = e;
+    return e != cudaSuccess;
+}
+
+// Ends a call's error state.  After a refused launch the kernels behind it were left
+// out: the cell counts that the prep kernel made are cleared (the scan does so
+// otherwise) and the sorted arrays count as unbuilt.
+cudaError_t end_call(rbe_ctx* h) {
+    if (h->refused) {
+        h->list_valid = false;
+        cudaMemsetAsync(h->d_cell_cnt, 0, sizeof(int) * (h->ncell + 1), h->stream);
+    }
+    const cudaError_t e = h->call_err;
+    h->refused = false;
+    h->call_err = cudaSuccess;
+    return e;
+}
+
 // (Re)build the work tables for the current particle counts and tuning.
 rbe_status prepare(rbe_ctx* h, int n) {
+    end_call(h);                       // of a call that returned early
     if (!h->batch) h->sys[0].n = n;
     const long long ntot = h->batch ? h->ntot : n;
     // naming the automatic chunk names the automatic shapes of the mixed path with it:
@@ -1132,9 +1159,12 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
     const bool fused = a.list && mixed && (a.parts & RBE_PART_FOURIER) && fusion_on(h);
     bool used[RBE_K_COUNT] = {};
     int count = 0;
+    note_error(h);                     // (of something else in this thread)
     auto run = [&](int kid, cudaStream_t s, auto&& launch) {
+        if (h->refused) return;
         if (prof) cudaEventRecord(h->ev_beg[kid], s);
         launch();
+        h->refused = note_error(h);
         if (prof) {
             cudaEventRecord(h->ev_end[kid], s);
             used[kid] = true;
@@ -1415,7 +1445,8 @@ rbe_status check_n(rbe_ctx* h, int n) {
 }
 
 rbe_status finish(rbe_ctx* h, const char* where) {
-    cudaError_t e = cudaGetLastError();
+    note_error(h);
+    const cudaError_t e = end_call(h);
     if (e != cudaSuccess) return cuda_fail(h, e, where);
     return RBE_OK;
 }
@@ -1732,6 +1763,10 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
         if (host_graph) copy_out(h->cap_stream);
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(h->cap_stream, &graph);
+        if (h->refused) {                           // no graph of whole steps
+            if (graph) cudaGraphDestroy(graph);
+            return finish(h, "rbe_step");
+        }
         if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
         e = cudaGraphInstantiate(&exec, graph, 0);
         cudaGraphDestroy(graph);
