@@ -66,7 +66,9 @@ typedef enum {
                                (rbe_set_wait_limit); the work is still queued.  Also,
                                latched: the blocks of a small system's step (see
                                rbe_step) did not hear from each other within 2 s and
-                               gave the step up                                       */
+                               gave it up: positions, velocities and step index are
+                               those before it (before the last 512 steps at most of
+                               a longer call)                                         */
     RBE_ERR_NONFINITE = 6,  /* a position or charge of an input was NaN or infinite
                                (latched on the device, reported at the next sync)     */
     RBE_ERR_STATE = 7,      /* call not valid for this handle (e.g. wrong n for a batch) */

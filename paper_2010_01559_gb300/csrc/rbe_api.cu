@@ -18,6 +18,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <thread>
@@ -1602,6 +1603,17 @@ bool small_pays(long long n, long long P) {
     return n * (1100 + 8 * P) <= 3650000 + 4500 * P;
 }
 
+// Longest wait of a block of the cluster for another one's message, in ns (a step
+// takes microseconds).  The bounds-checked build takes it from the environment, so
+// that a test can make it run out.
+unsigned long long cluster_wait_ns() {
+#ifdef RBE_CHECK_BOUNDS
+    if (const char* v = std::getenv("RBE_TEST_CLUSTER_WAIT_NS"))
+        return std::strtoull(v, nullptr, 10);
+#endif
+    return 2000000000ull;
+}
+
 constexpr int kGraphSteps = 8;
 constexpr int kSmallStepsPerLaunch = 512;
 
@@ -1686,8 +1698,11 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
         // a small system: the steps of the call as one cluster, a few hundred
         // steps per launch so that no launch holds its SMs for long
         if (io) copy_in(h->stream);
+        // (the host call that polls the word holds the step index in the pinned one)
+        const unsigned long long done_value = a.done ? h->h_pin[0] + (uint64_t)nsteps : 0ull;
         for (int k = 0; k < nsteps; k += kSmallStepsPerLaunch) {
             SmallArgs sa{};
+            sa.wait_ns = cluster_wait_ns();
             sa.S = h->sysdev[0];
             sa.n = n;
             sa.cs = h->small_cs;
@@ -1714,6 +1729,7 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
             if (a.done && k + sa.nsteps == nsteps) {
                 sa.done_host = a.done;
                 sa.err_host = (int*)(a.done - 1);
+                sa.done_value = done_value;
             }
             RBE_CUDA(h, launch_small_md(h->stream, sa));
             ++h->kernel_count;
@@ -1857,8 +1873,8 @@ rbe_status report_err(rbe_ctx* h) {
                                               "meaningful)");
         if (err & kErrWait)
             return fail(h, RBE_ERR_TIMEOUT, "the blocks of a one-cluster MD step did not hear "
-                                            "from each other (the results of that call are not "
-                                            "meaningful)");
+                                            "from each other and gave it up (the state and the "
+                                            "step index are those before it)");
         if (err & kErrBounds)
             return fail(h, RBE_ERR_BOUNDS, "the bounds-checked build found an index outside its "
                                            "array (the access was skipped)");

@@ -773,8 +773,10 @@ struct SmallArgs {
     int stride, cap;
     unsigned long long* stats;
     int* err;
-    unsigned long long* done_host;   // nullable: completion word (as in MdOut)
-    int* err_host;
+    unsigned long long* done_host;   // nullable: completion word (as in MdOut), written with
+    int* err_host;                   // done_value when the call's steps are done or given up
+    unsigned long long done_value;
+    unsigned long long wait_ns;      // longest wait for another block's message
 };
 bool small_md_fits(int n, int P, int M, int cap, int cs);
 cudaError_t launch_small_md(cudaStream_t st, const SmallArgs& a);

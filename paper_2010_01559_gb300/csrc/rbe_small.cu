@@ -73,17 +73,25 @@ __device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                  : "memory");
 }
-// Waits for the phase of the given parity, for two seconds at most (a step takes
-// microseconds): false if it did not complete.
 __device__ __forceinline__ unsigned long long now_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
-    unsigned long long t0 = 0ull;
-    for (unsigned t = 0;; ++t) {
-        uint32_t done;
+// Whether the phase of the given parity has completed, at once (test_wait) or after a
+// wait of the hardware's choosing (try_wait).
+template <bool TEST>
+__device__ __forceinline__ bool bar_poll(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    if constexpr (TEST)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    else
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -91,11 +99,20 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
             : "=r"(done)
             : "r"(bar), "r"(parity)
             : "memory");
-        if (done) return true;
+    return done != 0u;
+}
+// Waits for the phase of the given parity, limit_ns at most (a step takes
+// microseconds; 0: one look): false if it did not complete.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity,
+                                         unsigned long long limit_ns) {
+    if (limit_ns == 0ull) return bar_poll<true>(bar, parity);
+    unsigned long long t0 = 0ull;
+    for (unsigned t = 0;; ++t) {
+        if (bar_poll<false>(bar, parity)) return true;
         if ((t & 63u) == 0u) {
             const unsigned long long now = now_ns();
             if (t == 0u) t0 = now;
-            else if (now - t0 > 2000000000ull) return false;
+            else if (now - t0 > limit_ns) return false;
         }
     }
 }
@@ -174,6 +191,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     __shared__ uint4 s_msg[2][kSmallMaxCs];
     __shared__ unsigned long long s_k2;                         // this rank's kinetic sum
     __shared__ int s_flags[2];                                  // its flags, by step parity
+    __shared__ int s_late[kSmallMaxCs];                         // the ranks that gave up
     const SysDev& S = a.S;
     const uint32_t rank = cluster_rank();
     const int cs = a.cs, n = a.n, P = S.P, tid = threadIdx.x;
@@ -260,7 +278,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     const uint32_t rec_snd = remote(local_addr(rec + first + q_snd), min(t_snd, cs - 1));
     const uint32_t bar_snd = remote(bar_rec, min(t_snd, cs - 1));
     bool bad_seen = false;                          // some position or charge was not finite
-    bool late = false;                              // a wait gave up: no more waiting
+    bool gave_up = false;                           // a wait of this block ran out
 
     for (int s = 0; s < a.nsteps; ++s) {
         const uint64_t step = step0 + (uint64_t)s;
@@ -303,7 +321,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
                      make_uint4((uint32_t)s_flags[par], 0u, (uint32_t)k2, (uint32_t)(k2 >> 32)),
                      remote(bar_rec, lane));
         }
-        if (!late && !bar_wait(bar_rec, par)) late = true;
+        const bool rec_in = bar_wait(bar_rec, par, a.wait_ns);
         const uint32_t seen = __reduce_or_sync(0xffffffffu, lane < cs ? s_msg[par][lane].x : 0u);
         const bool rebuild = (seen & 1u) != 0u;
         bad_seen |= (seen & 2u) != 0u;
@@ -336,7 +354,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             v += __shfl_xor_sync(0xffffffffu, v, 1);
             if ((lane & 7) == 0) s_part[sub * kp + pr][lane >> 3] = v;
         }
-        __syncthreads();
+        if (__syncthreads_or(!rec_in)) {            // the whole block leaves the steps, before
+            gave_up = true;                         // it uses or sends anything of this one
+            break;
+        }
         if (tid == 0) {                             // (read above, written after the next barrier)
             s_k2 = 0ull;
             s_flags[par] = 0;
@@ -459,7 +480,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             fz = f.z;
         }
         // ---- Fourier force
-        if (!late && !bar_wait(bar_kv, par)) late = true;
+        const bool kv_in = bar_wait(bar_kv, par, a.wait_ns);
         if (pairs) {
             const uint4 si = R_[pn];
             float gx = 0.f, gy = 0.f, gz = 0.f;
@@ -484,13 +505,15 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             fz += __shfl_down_sync(0xffffffffu, fz, d, R);
         }
         if (pairs && l == 0) frc[p] = make_float4(fx, fy, fz, 0.f);
-        __syncthreads();
+        if (__syncthreads_or(!kv_in)) {
+            gave_up = true;
+            break;
+        }
         // ---- thermostat and drift
         if (warp * 32 < np) {
             unsigned long long k2 = 0ull;
             if (owner) {
                 const float4 F = frc[tid];
-                if (a.F_out && s == a.nsteps - 1) a.F_out[o] = F;
                 if (nhm) k2 = nose_hoover_apply(S, nh.f_va, nh.f_vf, F.x, F.y, F.z, vel, pos);
                 else md_apply(S, z, F.x, F.y, F.z, vel, pos);
             }
@@ -500,13 +523,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             }
         }
     }
-    if (owner) {
-        a.pos[o] = pos;
-        a.vel[o] = vel;
-    }
-    if (late && lane == 0) atomicOr(a.err, kErrWait);
     // the last step's kinetic sums, for the friction of the next call (slots
-    // of the parity that no rank reads any more)
+    // of the parity that no rank reads any more), and whether this rank gave up
     __syncthreads();
     if (nhm && tid == 0) {
         const uint32_t d = remote(local_addr(&s_msg[a.nsteps & 1][rank]), 0);
@@ -514,26 +532,54 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
                      "r"((uint32_t)s_k2), "r"((uint32_t)(s_k2 >> 32))
                      : "memory");
     }
+    if (tid < cs)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
+                         remote(local_addr(&s_late[rank]), (uint32_t)tid)),
+                     "r"((int)gave_up)
+                     : "memory");
+    cluster_sync();
+    int any = 0;
+    for (int t = 0; t < cs; ++t) any |= s_late[t];
+    if (!any) {
+        if (owner) {
+            a.pos[o] = pos;
+            a.vel[o] = vel;
+            if (a.F_out) a.F_out[o] = frc[tid];
+        }
+    } else if (tid == 0) {
+        // some rank gave up: none stores its state.  No rank sends any more; what is
+        // still under way to this one lands before the block goes
+        const unsigned long long t0 = now_ns();
+        while (now_ns() - t0 < 100000ull) {
+        }
+    }
     if (a.done_host) __threadfence_system();        // this thread's outputs
     // orders those stores, and keeps every rank's shared memory alive until all are done
     cluster_sync();
     if (rank == 0 && tid == 0) {
-        if (nhm) {
-            unsigned long long k2 = 0ull;
-            for (int t = 0; t < cs; ++t) {
-                const uint4 v = s_msg[a.nsteps & 1][t];
-                k2 += (unsigned long long)v.z | ((unsigned long long)v.w << 32);
+        if (any) {
+            // positions, velocities, friction and step index stay as they were; the
+            // list may have been rebuilt in part
+            atomicOr(a.err, kErrWait);
+            *a.list_flag = 1;
+        } else {
+            if (nhm) {
+                unsigned long long k2 = 0ull;
+                for (int t = 0; t < cs; ++t) {
+                    const uint4 v = s_msg[a.nsteps & 1][t];
+                    k2 += (unsigned long long)v.z | ((unsigned long long)v.w << 32);
+                }
+                nh.k2 = k2;
+                *a.nh = nh;
             }
-            nh.k2 = k2;
-            *a.nh = nh;
+            *a.list_flag = 0;
+            *a.step_dev = step0 + (uint64_t)a.nsteps;
         }
-        *a.list_flag = 0;
-        *a.step_dev = step0 + (uint64_t)a.nsteps;
         if (a.done_host) {
             __threadfence_system();
             *(volatile int*)a.err_host = *(const volatile int*)a.err;
             __threadfence_system();
-            *(volatile unsigned long long*)a.done_host = step0 + (uint64_t)a.nsteps;
+            *(volatile unsigned long long*)a.done_host = a.done_value;
         }
     }
 }
