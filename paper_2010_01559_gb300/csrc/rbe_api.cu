@@ -1086,6 +1086,7 @@ RealArgs make_real_args(const rbe_ctx* h, int parts) {
     r.fs64 = h->d_fs64;
     r.poly64 = h->d_poly64;
     r.poly64_form = h->npoly64 == 0 ? 0 : (h->npoly64 == h->nsys ? 1 : 2);
+    r.nbr_stride = std::max(h->ntot, 1);
     r.err = h->d_err;
     return r;
 }
@@ -1243,7 +1244,6 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
             rl.lsplit = h->lsplit;
             rl.nbr = h->d_nbr;
             rl.ncnt = h->d_ncnt;
-            rl.nbr_stride = std::max(h->ntot, 1);
             rl.nbr_cap = h->list_cap;
             rl.list_flag = h->d_list_flag;
             rl.freal = h->d_freal;
@@ -1357,7 +1357,6 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
         r.lsplit = h->lsplit;
         r.nbr = h->d_nbr;
         r.ncnt = h->d_ncnt;
-        r.nbr_stride = std::max(h->ntot, 1);
         r.nbr_cap = h->list_cap;
         r.list_flag = h->d_list_flag;
         r.freal = h->d_freal;
@@ -1405,7 +1404,6 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
         r.lsplit = h->lsplit;
         r.nbr = h->d_nbr;
         r.ncnt = h->d_ncnt;
-        r.nbr_stride = std::max(h->ntot, 1);
         r.nbr_cap = h->list_cap;
         r.list_flag = h->d_list_flag;
         r.list_when = 2;
@@ -2314,7 +2312,6 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float* pos_q, rbe_tuning*
                     r.lsplit = h->lsplit;
                     r.nbr = h->d_nbr;
                     r.ncnt = h->d_ncnt;
-                    r.nbr_stride = std::max(h->ntot, 1);
                     r.nbr_cap = h->list_cap;
                     r.list_flag = h->d_list_flag;
                     r.list_when = 0;

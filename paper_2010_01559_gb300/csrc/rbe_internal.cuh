@@ -733,7 +733,7 @@ struct RealArgs {
     int nlblk, lsplit;
     const int* nbr;
     const int* ncnt;
-    int nbr_stride, nbr_cap;
+    int nbr_stride, nbr_cap; // nbr_stride: particles in the arrays (also of the FP64 pass)
     const int* list_flag;    // rebuild flag of this step
     int list_when;           // the list kernel works only when (*list_flag != 0) == list_when
                              // (2: always)

@@ -227,6 +227,7 @@ k_real_f64(const __grid_constant__ RealArgs a) {
                             while (k >= s_pre[t][r + 1]) ++r;
                             const int o = k - s_pre[t][r], n0 = s_n0[t][r];
                             jj[u] = o < n0 ? s_s0[t][r] + o : s_s1[t][r] + (o - n0);
+                            if (!RBE_IN_BOUNDS(jj[u], a.nbr_stride, a.err)) jj[u] = i;
                         }
                         sj[u] = __ldg(a.spos + jj[u]);
                     }
@@ -272,7 +273,7 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     }
     // ---- the closing warp, a lane per particle: what does not depend on the sums
     const int tc = (int)threadIdx.x - kBlockP;
-    const bool closes = tc >= 0 && tc < tl.count;
+    bool closes = tc >= 0 && tc < tl.count;
     const bool nhm = a.md_pos64 && a.nh && S.thermostat == RBE_THERMO_NOSE_HOOVER;
     const bool andersen = S.thermostat == RBE_THERMO_ANDERSEN;
     int o = 0;
@@ -281,6 +282,9 @@ k_real_f64(const __grid_constant__ RealArgs a) {
     bool coll = false;
     if (closes) {
         o = a.perm[tl.first + tc];
+        if (!RBE_IN_BOUNDS(o, a.nbr_stride, a.err)) closes = false;
+    }
+    if (closes) {
         if (a.parts & kPartFourier) {
             f = a.fs64[o];
             if (a.phi_out64) {

@@ -229,9 +229,12 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     if (pairs && !stale) {
         // the handle's list, in sorted indices of its last build
         const int i = a.iperm[pn];
-        cnt = min(a.ncnt[i], a.cap);
-        for (int k = l; k < cnt; k += R)
-            list[p * a.cap + k] = (uint16_t)a.perm[a.nbr[(size_t)k * a.stride + i]];
+        cnt = RBE_IN_BOUNDS(i, a.stride, a.err) ? min(a.ncnt[i], a.cap) : 0;
+        for (int k = l; k < cnt; k += R) {
+            const int j = a.nbr[(size_t)k * a.stride + i];
+            const int c = RBE_IN_BOUNDS(j, a.stride, a.err) ? a.perm[j] : pn;
+            list[p * a.cap + k] = (uint16_t)(RBE_IN_BOUNDS(c, n, a.err) ? c : pn);
+        }
     }
     NhState nh{};
     if (nhm) nh = *a.nh;
@@ -470,9 +473,13 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         if (pairs) {
             Pair2Acc acc{0ull, 0ull, 0ull, 0.f, 0.f, 0.f};
             const uint4 si = R_[pn];
+            auto rec_of = [&](int k) {              // (the particle itself is no pair)
+                const int j = list[p * a.cap + k];
+                return RBE_IN_BOUNDS(j, n, a.err) ? R_[j] : si;
+            };
             for (int k = l; k < cnt; k += 2 * R) {
-                const uint4 sb = k + R < cnt ? R_[list[p * a.cap + k + R]] : si;
-                pair2_fixed(si, R_[list[p * a.cap + k]], sb, S, acc);
+                const uint4 sb = k + R < cnt ? rec_of(k + R) : si;
+                pair2_fixed(si, rec_of(k), sb, S, acc);
             }
             const float3 f = pair2_force(acc, si, S);
             fx = f.x;
