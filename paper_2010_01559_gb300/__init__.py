@@ -305,8 +305,9 @@ class RBEEnergy:
     ``RBEEnergy.apply(pos, q, rbe, step)`` with pos float32 [n,3] and q float32
     [n] (CUDA) returns the FP64 energy of the mixed path (scalar tensor for a
     single system).  backward gives dE/dpos = -F and dE/dq = phi of the same
-    evaluation: where a gradient may be asked for, the forward evaluation keeps
-    F and phi (20 bytes per particle), so that backward only scales them.
+    evaluation: the forward evaluation keeps F where pos requires a gradient and
+    computes and keeps phi where q does (16 and 4 bytes per particle), so that
+    backward only scales them; without gradients (torch.no_grad) it keeps nothing.
     """
 
     _fn = None
@@ -315,7 +316,7 @@ class RBEEnergy:
     def apply(cls, pos, q, rbe, step):
         if cls._fn is None:
             cls._fn = _make_energy_fn()
-        return cls._fn.apply(pos, q, rbe, step)
+        return cls._fn.apply(pos, q, rbe, step, _torch().is_grad_enabled())
 
 
 def _make_energy_fn():
@@ -323,12 +324,12 @@ def _make_energy_fn():
 
     class _Fn(torch.autograd.Function):
         @staticmethod
-        def forward(ctx, pos, q, rbe, step):
+        def forward(ctx, pos, q, rbe, step, grad):
             pos_q = torch.cat([pos.detach().float(), q.detach().float()[:, None]], 1).contiguous()
-            want = ctx.needs_input_grad[0] or ctx.needs_input_grad[1]
-            F, E, phi = rbe.forces(pos_q, step, energy=True, phi=want)
-            if want:
-                ctx.save_for_backward(pos, q, F, phi)
+            want_F, want_phi = (grad and need for need in ctx.needs_input_grad[:2])
+            F, E, phi = rbe.forces(pos_q, step, energy=True, phi=want_phi)
+            if want_F or want_phi:
+                ctx.save_for_backward(pos, q, F if want_F else None, phi)
             return E[:, 0].sum() if E.shape[0] > 1 else E[0, 0]
 
         @staticmethod
@@ -337,6 +338,6 @@ def _make_energy_fn():
             g = gE.to(torch.float32)
             gpos = (F[:, :3] * -g).to(pos.dtype) if ctx.needs_input_grad[0] else None
             gq = (phi * g).to(q.dtype) if ctx.needs_input_grad[1] else None
-            return gpos, gq, None, None
+            return gpos, gq, None, None, None
 
     return _Fn
