@@ -144,6 +144,40 @@ __host__ __device__ inline SmallLayout small_layout(int n, int P, int M, int cap
     return L;
 }
 
+// A warp's structure factors: FP32 chains per lane, then the lanes' sums.  Their
+// rounding is kept at that of chains of 16 terms added exactly, a variance of 8 n in
+// units of one term's (c / 2 per term of a chain of c, one per term and level of a
+// sum of the lanes).  Up to kSmallPlain terms per lane an FP32 sum over the five levels
+// stays at it, (6 / 2 + 5) n; beyond, the lanes' sums are float pairs, of chains of
+// kSmallChain terms at most.  Fourier force against 64 bits (RMS, 16 to 24 systems),
+// FP32 sums throughout / now: N = 2000, P = 100 2.83e-7 / 2.74e-7; 1150, 500 3.25e-7 /
+// 3.14e-7; 890, 1000 2.88e-7 / 2.72e-7.
+constexpr int kSmallPlain = 6, kSmallChain = 16;
+
+__device__ __forceinline__ float sum_of(float a, float b) { return a + b; }
+__device__ __forceinline__ float2 sum_of(float2 a, float2 b) {
+    const float2 x = two_sum(a.x, b.x);
+    return make_float2(x.x, a.y + b.y + x.y);
+}
+__device__ __forceinline__ float lane_xor(float v, int d) {
+    return __shfl_xor_sync(0xffffffffu, v, d);
+}
+__device__ __forceinline__ float2 lane_xor(float2 v, int d) {
+    return make_float2(lane_xor(v.x, d), lane_xor(v.y, d));
+}
+// Four sums over the warp, halving the values with the lanes: lanes 0, 8, 16, 24 end
+// with re0, im0, re1, im1.
+template <class V>
+__device__ __forceinline__ V warp_sum4(V re0, V im0, V re1, V im1, int lane) {
+    const bool up = lane & 16, up2 = lane & 8;
+    const V a = sum_of(up ? re1 : re0, lane_xor(up ? re0 : re1, 16));
+    const V b = sum_of(up ? im1 : im0, lane_xor(up ? im0 : im1, 16));
+    V v = sum_of(up2 ? b : a, lane_xor(up2 ? a : b, 8));
+    v = sum_of(v, lane_xor(v, 4));
+    v = sum_of(v, lane_xor(v, 2));
+    return sum_of(v, lane_xor(v, 1));
+}
+
 // (ch + cl) (h + l) to FP32
 __device__ __forceinline__ float pair_mul(float ch, float cl, float2 v) {
     const float p = __fmul_rn(ch, v.x);
@@ -182,7 +216,7 @@ template <int R>
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_constant__ SmallArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(8) unsigned long long s_bar[2];        // records in, coefficients in
-    __shared__ float s_part[kSmallWarps][4];                    // structure-factor partials
+    __shared__ float2 s_part[kSmallWarps][4];                   // structure-factor partials (pairs)
     __shared__ int4 s_m[2][kSmallMaxKc];                        // this rank's wave vectors and
     __shared__ float2 s_c[2][kSmallMaxKc];                      // (float pairs) coef / rho, by parity
     __shared__ uint4 s_token;                                   // from ranks without wave vectors
@@ -331,30 +365,42 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
         // ---- structure factors of two wave vectors over a share of all records
         if (sums) {
             const int4 m0 = s_m[step & 1][2 * pr], m1 = s_m[step & 1][2 * pr + 1];
-            float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
+            const int stride = wpp * 32, j0 = sub * 32 + lane;
+            // the sums of a lane's records j0 .. je - 1 (every stride-th): q cos, q sin of
+            // both wave vectors
+            auto chain = [&](int jb, int je) {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-            for (int j = sub * 32 + lane; j < n; j += wpp * 32) {
-                const uint4 r = R_[j];
-                const float q = __uint_as_float(r.w);
-                float sn, cn;
-                __sincosf((float)(int32_t)((uint32_t)m0.x * r.x + (uint32_t)m0.y * r.y +
-                                           (uint32_t)m0.z * r.z) * kTurn, &sn, &cn);
-                re0 = fmaf(q, cn, re0);
-                im0 = fmaf(q, sn, im0);
-                __sincosf((float)(int32_t)((uint32_t)m1.x * r.x + (uint32_t)m1.y * r.y +
-                                           (uint32_t)m1.z * r.z) * kTurn, &sn, &cn);
-                re1 = fmaf(q, cn, re1);
-                im1 = fmaf(q, sn, im1);
+                for (int j = jb; j < je; j += stride) {
+                    const uint4 r = R_[j];
+                    const float q = __uint_as_float(r.w);
+                    float sn, cn;
+                    __sincosf((float)(int32_t)((uint32_t)m0.x * r.x + (uint32_t)m0.y * r.y +
+                                               (uint32_t)m0.z * r.z) * kTurn, &sn, &cn);
+                    a.x = fmaf(q, cn, a.x);
+                    a.y = fmaf(q, sn, a.y);
+                    __sincosf((float)(int32_t)((uint32_t)m1.x * r.x + (uint32_t)m1.y * r.y +
+                                               (uint32_t)m1.z * r.z) * kTurn, &sn, &cn);
+                    a.z = fmaf(q, cn, a.z);
+                    a.w = fmaf(q, sn, a.w);
+                }
+                return a;
+            };
+            float2 v;
+            if (n <= kSmallPlain * stride) {
+                const float4 a = chain(j0, n);
+                v = make_float2(warp_sum4(a.x, a.y, a.z, a.w, lane), 0.f);
+            } else {
+                float2 re0{}, im0{}, re1{}, im1{};
+                for (int jb = j0; jb < n; jb += kSmallChain * stride) {
+                    const float4 a = chain(jb, min(n, jb + kSmallChain * stride));
+                    re0 = sum_of(re0, make_float2(a.x, 0.f));
+                    im0 = sum_of(im0, make_float2(a.y, 0.f));
+                    re1 = sum_of(re1, make_float2(a.z, 0.f));
+                    im1 = sum_of(im1, make_float2(a.w, 0.f));
+                }
+                v = warp_sum4(re0, im0, re1, im1, lane);
             }
-            // the four sums over the warp, halving the values with the lanes:
-            // lanes 0, 8, 16, 24 end with re0, im0, re1, im1
-            const bool up = lane & 16, up2 = lane & 8;
-            const float a0 = (up ? re1 : re0) + __shfl_xor_sync(0xffffffffu, up ? re0 : re1, 16);
-            const float a1 = (up ? im1 : im0) + __shfl_xor_sync(0xffffffffu, up ? im0 : im1, 16);
-            float v = (up2 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up2 ? a0 : a1, 8);
-            v += __shfl_xor_sync(0xffffffffu, v, 4);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
             if ((lane & 7) == 0) s_part[sub * kp + pr][lane >> 3] = v;
         }
         if (__syncthreads_or(!rec_in)) {            // the whole block leaves the steps, before
@@ -371,13 +417,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
             // ones, as float pairs
             const int u = lane & 15, c = (q & 1) * 2 + (lane >> 4);
             float2 v = make_float2(0.f, 0.f);
-            if (u < wpp) v.x = s_part[u * kp + (q >> 1)][c];
-            if (u + 16 < wpp) v = two_sum(v.x, s_part[(u + 16) * kp + (q >> 1)][c]);
+            if (u < wpp) v = s_part[u * kp + (q >> 1)][c];
+            if (u + 16 < wpp) v = sum_of(v, s_part[(u + 16) * kp + (q >> 1)][c]);
 #pragma unroll
-            for (int d = 8; d > 0; d >>= 1) {
-                const float2 x = two_sum(v.x, __shfl_xor_sync(0xffffffffu, v.x, d));
-                v = make_float2(x.x, v.y + __shfl_xor_sync(0xffffffffu, v.y, d) + x.y);
-            }
+            for (int d = 8; d > 0; d >>= 1) v = sum_of(v, lane_xor(v, d));
             const int4 m = s_m[step & 1][q];
             const float2 cf = s_c[step & 1][q];
             const float AB = pair_mul(cf.x, cf.y, v);
