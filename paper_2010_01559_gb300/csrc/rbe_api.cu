@@ -185,6 +185,7 @@ struct rbe_ctx {
     // evaluation without (n) and with energies (e)
     int nrt = 0, rt_n = 0, rt_e = 0, run_n = 64, run_e = 64, max_rt = 0;
     int rho_t = 256;                          // threads per block
+    int force_sums = 1;                       // partial sums per thread of the mixed force
     bool cur_set = false;                     // the chunk in effect is not the automatic one
     bool use_graph = false;
     double wait_limit = 0.0;                  // seconds a host wait may take (0: no limit)
@@ -525,13 +526,26 @@ int auto_rho_tile(int pmax, long long ntot, int run, int T) {
     return (int)std::max<long long>(pass, std::min<long long>(4096, (tile + 7) / 8 * 8));
 }
 
-// Threads per particle of the Fourier force: 45000 threads at least (measured,
+// Threads per particle of the Fourier force: 56000 threads at least (measured,
 // us with 1, 2, 4, 8: N = 8001 9.3, 3.8, 3.1, 3.1; 30000 9.3, 6.2, 7.2, 9.2; 50021
-// 7.2, 7.2, 10.7, 11.3; 100003 7.2, 9.2, 13.3, 17.4).
+// 7.2, 7.2, 10.7, 11.3; 100003 7.2, 9.2, 13.3, 17.4; with the partial sums below, five
+// steps of N = 50021 147.2 with 1, 145.3 with 2, 168 with 4).
 int auto_split(long long ntot) {
     int s = 1;
-    while (s < 8 && ntot * s < 45000) s <<= 1;
+    while (s < 8 && ntot * s < 56000) s <<= 1;
     return s;
+}
+
+// Partial sums of each of those threads.  The pass had 155648 threads (8 warps for each
+// scheduler of 152 SMs) before it was found faster with fewer; the sums of the threads
+// that one took over stay apart, so that the FP32 chains are no longer than they were.
+// Fourier force against 64 bits (RMS), that many threads / one chain / now: N = 50021,
+// P = 137 2.62e-7 / 3.09e-7 / 2.62e-7; 100003, 200 3.64 / 4.01 / 3.62; 140001, 128 3.03 /
+// 3.53 / 3.03; 30000, 50 2.99 / 3.06 / 2.99.
+int auto_force_sums(long long ntot, int split) {
+    int s = 1;
+    while (s < 8 && ntot * s < 152LL * 8 * kBlockP) s <<= 1;
+    return std::max(1, std::min(4, s / split));
 }
 
 // Threads per particle of the mixed real-space pass (each takes 9/R of the 9
@@ -715,6 +729,8 @@ rbe_status prepare(rbe_ctx* h, int n) {
     h->rho_t = rho_t;
     h->cur_set = named;
     h->split = split;
+    // (a split that was set, and is not the automatic one, takes its shares in one sum)
+    h->force_sums = split == auto_split(ntot) ? auto_force_sums(ntot, split) : 1;
     h->rsplit = rsplit;
     h->nseg = (int)segs.size();
     h->seg_max = seg_max;
@@ -1131,7 +1147,7 @@ void launch_force(const rbe_ctx* h, cudaStream_t st, bool mixed, const MdOut& md
     if (mixed) {
         const Work w = make_work(h, h->split == 1 ? h->d_pblk : h->d_fblk, kBlockP / h->split, 0);
         launch_fourier_force_mixed(st, one, w, h->split == 1 ? h->npblk : h->nfblk, h->split,
-                                   h->d_fx, h->d_ksamp, h->d_kab, h->d_fs, md, pdl);
+                                   h->force_sums, h->d_fx, h->d_ksamp, h->d_kab, h->d_fs, md, pdl);
     } else {
         const Work w = make_work(h, h->d_pblk, kBlockP, 0);
         launch_fourier_force_f64(st, one, w, h->npblk, h->m_max(), phi, h->d_fx64, h->d_ksamp,

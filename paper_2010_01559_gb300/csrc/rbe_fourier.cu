@@ -284,13 +284,14 @@ k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
 // same SFU pair, the dE/dq term R cos(phi - theta)).
 struct KPhase { uint32_t nmx, nmy, nmz, phi; };
 struct KForce { float rmx, rmy, rmz, R; };
-
 // SPLIT threads per particle (each a 1/SPLIT share of the wave vectors), or
 // with SPLIT = 1 PT = 2 particles per thread, which share each wave vector's
 // shared-memory loads and the loop overhead (the pass is issue-bound at large
 // N).  A block holds a tile of kBlockP / SPLIT particles and kBlockP / PT
-// threads.  PHI: also dE/dq (the forces path); MD steps need only the force.
-template <int SPLIT, int PT, bool PHI, bool ONE>
+// threads.  A: sums of its own per thread, each over every A-th term of its share, so
+// that fewer threads per particle do not mean longer FP32 chains.  PHI: also dE/dq (the
+// forces path); MD steps need only the force.
+template <int SPLIT, int PT, int A, bool PHI, bool ONE>
 __global__ void __launch_bounds__(kBlockP / PT)
 k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
               const int4* __restrict__ ksamp, const float2* __restrict__ kab,
@@ -352,9 +353,11 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
             }
         }
     }
-    float fx[PT], fy[PT], fz[PT], ph[PT];
+    float cx[PT][A], cy[PT][A], cz[PT][A], cp[PT][A];      // sums of every A-th term
 #pragma unroll
-    for (int q = 0; q < PT; ++q) fx[q] = fy[q] = fz[q] = ph[q] = 0.f;
+    for (int q = 0; q < PT; ++q)
+#pragma unroll
+        for (int u = 0; u < A; ++u) cx[q][u] = cy[q][u] = cz[q][u] = cp[q][u] = 0.f;
     for (int base = 0; base < S.P; base += kKT) {
         const int cnt = min(kKT, S.P - base);
         __syncthreads();
@@ -366,8 +369,7 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
             kf[k] = KForce{rp.x * (float)m.x, rp.x * (float)m.y, rp.x * (float)m.z, rp.x};
         }
         __syncthreads();
-#pragma unroll 8
-        for (int k = sub; k < cnt; k += SPLIT) {
+        auto term = [&](int k, int u) {
             const KPhase a = kp[k];
             const KForce f = kf[k];
 #pragma unroll
@@ -378,15 +380,40 @@ k_force_mixed(const __grid_constant__ Work w, const uint4* __restrict__ rec,
                 if constexpr (PHI) {
                     float cs;
                     __sincosf(t, &sn, &cs);
-                    ph[q] = fmaf(f.R, cs, ph[q]);           // Re(e^{-i theta} rho) * coef
+                    cp[q][u] = fmaf(f.R, cs, cp[q][u]);     // Re(e^{-i theta} rho) * coef
                 } else {
                     sn = __sinf(t);
                 }
-                fx[q] = fmaf(sn, f.rmx, fx[q]);
-                fy[q] = fmaf(sn, f.rmy, fy[q]);
-                fz[q] = fmaf(sn, f.rmz, fz[q]);
+                cx[q][u] = fmaf(sn, f.rmx, cx[q][u]);
+                cy[q][u] = fmaf(sn, f.rmy, cy[q][u]);
+                cz[q][u] = fmaf(sn, f.rmz, cz[q][u]);
             }
-        }
+        };
+        int k = sub;
+#pragma unroll 8 / A
+        for (; k + (A - 1) * SPLIT < cnt; k += A * SPLIT)
+#pragma unroll
+            for (int u = 0; u < A; ++u) term(k + u * SPLIT, u);
+#pragma unroll
+        for (int u = 0; u < A - 1; ++u)
+            if (k + u * SPLIT < cnt) term(k + u * SPLIT, u);
+    }
+    float fx[PT], fy[PT], fz[PT], ph[PT];
+#pragma unroll
+    for (int q = 0; q < PT; ++q) {
+#pragma unroll
+        for (int d = A / 2; d > 0; d >>= 1)
+#pragma unroll
+            for (int u = 0; u < d; ++u) {
+                cx[q][u] += cx[q][u + d];
+                cy[q][u] += cy[q][u + d];
+                cz[q][u] += cz[q][u + d];
+                cp[q][u] += cp[q][u + d];
+            }
+        fx[q] = cx[q][0];
+        fy[q] = cy[q][0];
+        fz[q] = cz[q][0];
+        ph[q] = cp[q][0];
     }
 #pragma unroll
     for (int o = SPLIT / 2; o > 0; o >>= 1) {
@@ -522,29 +549,40 @@ void launch_rho_list(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
         rho_list_t<256>(st, one, w, g, ksamp, kcoef, fx, rho_fx, kcnt, kab, a, pdl);
 }
 
-template <int SPLIT, int PT>
-static void force_mixed_split(cudaStream_t st, bool one, const Work& w, int nblk, const uint4* fx,
-                              const int4* ksamp, const float2* kab, float4* fs,
-                              const MdOut& md, bool pdl) {
+template <int SPLIT, int PT, int A>
+static void force_mixed_a(cudaStream_t st, bool one, const Work& w, int nblk, const uint4* fx,
+                          const int4* ksamp, const float2* kab, float4* fs, const MdOut& md,
+                          bool pdl) {
     PdlConfig c(dim3(nblk), dim3(kBlockP / PT), 0, st, pdl);
     if (md.freal) {
-        if (one) cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, false, true>, w, fx, ksamp, kab, fs, md);
-        else cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, false, false>, w, fx, ksamp, kab, fs, md);
+        if (one) cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, A, false, true>, w, fx, ksamp, kab, fs, md);
+        else cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, A, false, false>, w, fx, ksamp, kab, fs, md);
     } else {
-        if (one) cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, true, true>, w, fx, ksamp, kab, fs, md);
-        else cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, true, false>, w, fx, ksamp, kab, fs, md);
+        if (one) cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, A, true, true>, w, fx, ksamp, kab, fs, md);
+        else cudaLaunchKernelEx(&c.cfg, k_force_mixed<SPLIT, PT, A, true, false>, w, fx, ksamp, kab, fs, md);
     }
 }
 
+template <int SPLIT, int PT>
+static void force_mixed_split(cudaStream_t st, bool one, const Work& w, int nblk, int sums,
+                              const uint4* fx, const int4* ksamp, const float2* kab, float4* fs,
+                              const MdOut& md, bool pdl) {
+    if constexpr (SPLIT <= 2)
+        if (sums >= 4) return force_mixed_a<SPLIT, PT, 4>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl);
+    if constexpr (SPLIT <= 4)
+        if (sums >= 2) return force_mixed_a<SPLIT, PT, 2>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl);
+    force_mixed_a<SPLIT, PT, 1>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl);
+}
+
 void launch_fourier_force_mixed(cudaStream_t st, bool one, const Work& w, int nblk, int split,
-                                const uint4* fx, const int4* ksamp, const float2* kab,
+                                int sums, const uint4* fx, const int4* ksamp, const float2* kab,
                                 float4* fs, const MdOut& md, bool pdl) {
     if (nblk <= 0) return;
     switch (split) {
-        case 2: force_mixed_split<2, 1>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl); break;
-        case 4: force_mixed_split<4, 1>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl); break;
-        case 8: force_mixed_split<8, 1>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl); break;
-        default: force_mixed_split<1, 2>(st, one, w, nblk, fx, ksamp, kab, fs, md, pdl); break;
+        case 2: force_mixed_split<2, 1>(st, one, w, nblk, sums, fx, ksamp, kab, fs, md, pdl); break;
+        case 4: force_mixed_split<4, 1>(st, one, w, nblk, sums, fx, ksamp, kab, fs, md, pdl); break;
+        case 8: force_mixed_split<8, 1>(st, one, w, nblk, sums, fx, ksamp, kab, fs, md, pdl); break;
+        default: force_mixed_split<1, 2>(st, one, w, nblk, sums, fx, ksamp, kab, fs, md, pdl); break;
     }
 }
 

@@ -667,9 +667,10 @@ struct MdOut {
     int* err_host;
     const int* err;
 };
+// split: threads per particle; sums: partial sums per thread (1, 2 or 4)
 void launch_fourier_force_mixed(cudaStream_t st, bool one, const Work& w, int nblk, int split,
-                                const uint4* fx, const int4* ksamp, const float2* kab,
-                                float4* fs, const MdOut& md = MdOut{}, bool pdl = false);
+                                int sums, const uint4* fx, const int4* ksamp, const float2* kab,
+                                float4* fs, const MdOut& md, bool pdl);
 void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int mcap,
                               bool phi, const double4* fx64, const int4* ksamp,
                               const double* kcoef, const unsigned long long* rho_fx,
