@@ -223,9 +223,11 @@ rbe_status rbe_forces_f64(rbe_handle h, int32_t n, const double *pos_q, uint64_t
  * step reads it to select its k-batch and noise and increments it on the
  * device, so a captured replay advances the stream.  The step sequence is
  * replayed from a CUDA graph when use_graph was enabled (rbe_set_graph).
- * A single list system (inverse-CDF sampler) small enough that
- * n (1100 + 8 P) <= 3.65e6 + 4500 P runs all steps of a call as one
- * thread-block cluster, with or without graphs and whatever the tuning. */
+ * A single list system (inverse-CDF sampler) that is small enough runs all steps
+ * of a call as one thread-block cluster, with or without graphs and whatever the
+ * tuning: with m neighbours within r_c + skin on average,
+ * n (33 + 1.32 P + 2.3 m) <= 574000 + 580 P + 840 m, and its list fits in shared
+ * memory. */
 rbe_status rbe_step(rbe_handle h, int32_t n, float *pos_q, float *vel, int32_t nsteps,
                     uint64_t *step_dev);
 

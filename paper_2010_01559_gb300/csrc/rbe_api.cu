@@ -1605,16 +1605,20 @@ struct HostIO {
 enum class ZeroCopy { none, both, out };
 
 // Whether the MD steps of a single list system of n particles run as one cluster
-// (rbe_small.cu).  Its sixteen SMs share the work of the whole GPU, so its step
-// grows with n and n P, about (3 + 0.0022 n + 1.6e-5 n P) us, where the separate
-// kernels' grows only with P, (10.3 + 0.009 P) us at these sizes: measured, one
-// cluster / separate, N = 1000: 5.4 / 10.4 (P = 10), 6.7 / 10.8 (100), 13.8 / 14.7
-// (500); N = 1500, P = 500: 17.4 / 15.4; N = 2000: 7.7 / 10.7 (10), 9.8 / 11.4 (100),
-// 12.5 / 12.2 (200), 21.3 / 16.4 (500); N = 3000: 10.1 / 11.2 (10), 14.0 / 12.1
-// (100), 30.5 / 18.3 (500).  The line through these leaves some near it on the slower
-// side by up to a tenth (N = 1500, P = 300: 12.8 / 14.1, taken as separate kernels).
-bool small_pays(long long n, long long P) {
-    return n * (1100 + 8 * P) <= 3650000 + 4500 * P;
+// (rbe_small.cu): P wave vectors, m neighbours within r_c + skin on average.  Its sixteen
+// SMs share the work of the whole GPU, so its step grows with n P and n m, about
+// (3.1 + 0.00033 n + 1.32e-5 n P + 2.4e-5 n m + 0.0047 P + 0.004 m) us, where the
+// separate kernels' hardly grows with n, (9.3 + 0.0105 P + 0.0124 m) us at these sizes.
+// The line is where these meet, half a microsecond early.  Measured, one cluster /
+// separate, at (n, P, m):
+//   1000, 10, 45     5.3 / 10.2    2000, 100, 45   9.5 / 10.8    2000, 200, 45  12.5 / 12.2
+//   1000, 500, 45   14.1 / 14.5    3000, 10, 45    8.3 / 11.6    3000, 100, 45  14.0 / 12.1
+//   1000, 100, 107   7.9 / 11.3    2000, 10, 107   9.4 / 11.1    2000, 100, 107 12.3 / 11.6
+//   1500, 10, 183    9.8 / 11.6    1500, 100, 183 11.8 / 12.2    2000, 10, 183  12.1 / 11.6
+//   600, 100, 305   10.0 / 14.3    1000, 50, 348  15.5 / 14.6    801, 50, 407   13.8 / 16.0
+//   999, 10, 508    19.3 / 16.3    999, 300, 508  24.2 / 18.5    1200, 100, 558 26.5 / 17.8
+bool small_pays(double n, double P, double m) {
+    return n * (0.00033 + 1.32e-5 * P + 2.3e-5 * m) <= 5.74 + 0.0058 * P + 0.0084 * m;
 }
 
 // Longest wait of a block of the cluster for another one's message, in ns (a step
@@ -1634,7 +1638,8 @@ constexpr int kSmallStepsPerLaunch = 512;
 bool small_steps(rbe_ctx* h, int n) {
     if (h->batch || h->mh || !h->list) return false;
     const SysHost& sh = h->sys[0];
-    if (!small_pays(n, sh.p.P)) return false;
+    const double rr = sh.p.r_c + sh.skin, L = sh.p.box;
+    if (!small_pays(n, sh.p.P, 4.0 / 3.0 * M_PI * rr * rr * rr * n / (L * L * L))) return false;
     if (h->small_n != n) {                       // asked once per particle count
         h->small_n = n;
         h->small_cs = 0;
