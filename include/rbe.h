@@ -351,7 +351,8 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float *pos_q, rbe_tuning 
 /* Kernels of one evaluation, in launch order (per-kernel profile indices). */
 enum {
     RBE_K_PREP = 0,          /* fixed-point coordinates, cell ids, charge sums      */
-    RBE_K_SCAN = 1,          /* exclusive scan of cell counts, step latch           */
+    RBE_K_SCAN = 1,          /* exclusive scan of cell counts, step latch; up to 2^16
+                                particles and cells the whole sort, in one launch  */
     RBE_K_SCATTER = 2,       /* counting-sort scatter                               */
     RBE_K_CELL_ORDER = 3,    /* order inside each cell by original index            */
     RBE_K_RHO = 4,           /* k-sampling, per-chunk structure factors, and (last

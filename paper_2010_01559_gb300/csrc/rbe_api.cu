@@ -1263,7 +1263,6 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
             rl.nbr_cap = h->list_cap;
             rl.list_flag = h->d_list_flag;
             rl.freal = h->d_freal;
-            rl.list_when = 0;
             const RhoWork rw = make_rho_work(h, a.E != nullptr);
             run(RBE_K_RHO_LIST, st, [&] {
                 launch_rho_list(st, one, rw.w, rw.g, h->d_ksamp, h->d_kcoef,
@@ -1380,7 +1379,6 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
         // (concurrent with the structure factors and the rebuild stream), or
         // over a rebuilt list by the build itself; then the Fourier force,
         // which adds it and applies the thermostat
-        r.list_when = 0;
         if (!fused) {
             cudaStreamWaitEvent(st2, h->ev_prep, 0);
             run(RBE_K_REAL, st2, [&] { launch_real_list(st2, one, r); });
@@ -1422,7 +1420,6 @@ int enqueue_eval(rbe_ctx* h, cudaStream_t st, const EvalArgs& a, bool chained = 
         r.ncnt = h->d_ncnt;
         r.nbr_cap = h->list_cap;
         r.list_flag = h->d_list_flag;
-        r.list_when = 2;
         r.fmode = 1;
         r.flag_clear = h->d_list_flag;
         run(RBE_K_REAL, st, [&] { launch_real_list(st, one, r); });
@@ -2335,7 +2332,6 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float* pos_q, rbe_tuning*
                     r.ncnt = h->d_ncnt;
                     r.nbr_cap = h->list_cap;
                     r.list_flag = h->d_list_flag;
-                    r.list_when = 0;
                     r.freal = h->d_freal;
                     const RhoWork rw = make_rho_work(h, false);
                     const float t = time_kernel(h, e0, e1, [&] {

@@ -61,8 +61,8 @@ __global__ void k_sample(const SysDev* __restrict__ sysv, int nsys, int ktot,
 // keeps the run its tuning names.
 //
 // Measured (events around the kernel, about 5 us of them launch, before -> now):
-// N = 8001, P = 200 14.3 -> 11.2 us; 50021, P = 137 39.3 -> 14.0; 100003, P = 200 40.9 ->
-// 20.8; 2^20, P = 100 129 -> 60.5; 262144, P = 500 70.6 -> 70.2 (full lanes already).
+// N = 8001, P = 200 14.3 -> 10.9 us; 50021, P = 137 39.3 -> 13.9; 100003, P = 200 40.9 ->
+// 20.9; 2^20, P = 100 129 -> 60.7; 262144, P = 500 70.6 -> 70.2 (full lanes already).
 
 // round(f 2^e) as a 64-bit integer, in integer arithmetic (|f| 2^e < 2^63; beyond, the
 // words saturate as a conversion of the double would)
@@ -249,9 +249,9 @@ k_rho_mixed(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
 // over the grid and each SM holds both at once -- the structure factors keep
 // the special-function unit busy while the pair terms use the ALU and FMA
 // pipes and wait on their gathers.  The list tiles work only when the list
-// stands (over a rebuilt list the pass runs on the rebuild stream, after the
-// build), and keep the per-slot count tests: padded batches cost this
-// issue-bound launch more than they save.
+// stands (over a rebuilt list the build adds the pair terms itself).  The list
+// pass is that of its own kernel (list_step), with as many entries in flight as the
+// registers beside the structure factors allow.
 template <int T, int R, bool ONE>
 __global__ void __launch_bounds__(T, T == 128 ? 9 : 4)
 k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
@@ -269,7 +269,7 @@ k_rho_list(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
         rho_body<T, ONE>(w, ksamp, kcoef, fx, rho_fx, kcnt, kab, r0 % ntiles, r0 / ntiles, run);
         return;
     }
-    if ((*a.list_flag != 0) != (a.list_when != 0)) return;
+    if (*a.list_flag) return;
     const int tile = (T / kBlockP) * (b - r1) + (int)(threadIdx.x / kBlockP);
     if (tile < a.nlblk)
         list_step<R, ONE, false, T == 128 ? 4 : 8, T == 128>(a, tile, threadIdx.x % kBlockP);

@@ -735,9 +735,8 @@ struct RealArgs {
     const int* nbr;
     const int* ncnt;
     int nbr_stride, nbr_cap; // nbr_stride: particles in the arrays (also of the FP64 pass)
-    const int* list_flag;    // rebuild flag of this step
-    int list_when;           // the list kernel works only when (*list_flag != 0) == list_when
-                             // (2: always)
+    const int* list_flag;    // rebuild flag of this step: the MD step's pass works when it is 0
+                             // (over a rebuilt list the build adds the pair terms)
     int fmode;               // forces call: assemble F, phi, energy and virial partials
     int* flag_clear;         // forces call: the rebuild flag to clear
     float4* freal;           // list kernel output: real-space force, caller's order
@@ -749,7 +748,7 @@ void launch_real_mixed(cudaStream_t st, bool one, const RealArgs& a);
 void launch_real_f64(cudaStream_t st, bool one, const RealArgs& a);
 void launch_real_list(cudaStream_t st, bool one, const RealArgs& a);
 // The MD step's structure factors and its pass over a standing list in one
-// launch (rbe_fourier.cu); `a` as for launch_real_list with list_when = 0.
+// launch (rbe_fourier.cu); `a` as for launch_real_list on an MD step.
 void launch_rho_list(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
                      const int4* ksamp, const double* kcoef, const uint4* fx,
                      unsigned long long* rho_fx, int* kcnt, float2* kab, const RealArgs& a,

@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kBlockP) k_real_list(const __grid_constant__ R
     if constexpr (FM == 0) {
         // right after the prep kernel: works when the list stands (over a
         // rebuilt list the build adds the pair terms itself)
-        if ((*a.list_flag != 0) != (a.list_when != 0)) return;
+        if (*a.list_flag) return;
     } else {
         if (a.flag_clear && blockIdx.x == 0 && threadIdx.x == 0) *a.flag_clear = 0;
     }

@@ -28,11 +28,12 @@
 // records (a rank without particles or wave vectors sends a message all the
 // same), and the records alternate between two buffers.
 //
-// Serial chains are what counts.  FP64 instructions are kept out of the loop
-// (their latency on this part is over a hundred cycles; summing a wave vector's
-// shares and its coefficient in FP64 took 3500 to 10700 cycles a step); one
-// thread sending to 16 ranks in turn or adding 32 partial forces took 1200 to
-// 4000, which a thread per message and shuffles take to a few hundred.  Partial sums are added as float pairs, and the coefficient
+// Serial chains are what counts.  FP64 instructions are kept out of the loop but for
+// the Nose-Hoover friction and kinetic energies (their latency on this part is over a
+// hundred cycles; summing a wave vector's shares and its coefficient in FP64 took 3500
+// to 10700 cycles a step); one thread sending to 16 ranks in turn or adding 32 partial
+// forces took 1200 to 4000, which a thread per message and shuffles take to a few
+// hundred.  Partial sums are added as float pairs, and the coefficient
 // (lB S/P 4 pi / V) / k^2 is a float-pair constant over the integer |m|^2.
 //
 // Neighbour list: the owned particles' neighbours within r_c + skin as 16-bit
@@ -44,8 +45,8 @@
 // of the handle.
 //
 // Measured (us per step, 64 steps in a call, replayed kernels before -> now):
-// N = 300, P = 10 15.4 -> 4.1; N = 1000, P = 100 16.3 -> 6.7 and P = 500 18.3 -> 13.8;
-// N = 2000, P = 100 16.3 -> 9.8.
+// N = 300, P = 10 15.4 -> 4.1; N = 1000, P = 100 16.3 -> 6.5 and P = 500 18.3 -> 14.0;
+// N = 2000, P = 100 16.3 -> 9.5.
 #include <algorithm>
 
 #include "rbe_cluster.cuh"
