@@ -2234,15 +2234,18 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float* pos_q, rbe_tuning*
     a.F = h->d_stage_F;
     const bool prof = h->prof_on;
     h->prof_on = false;
-    // structure-factor chunk
-    float best = 1e30f;
-    int best_chunk = 32;
+    // structure-factor chunk: named ones, and the automatic shapes under the automatic
+    // chunk's value
+    const int achunk = auto_chunk(h, h->batch ? h->ntot : n);
+    float best = 1e30f, best_nt = 1e30f;
+    int best_chunk = 32, best_named = 32;
     for (int c = 32; c <= 4096; c <<= 1) {
         h->rho_chunk = c;
         if ((s = prepare(h, n)) != RBE_OK) break;
         enqueue_eval(h, h->stream, a);
         const float t = time_kernel(h, e0, e1, [&] { launch_rho(h, h->stream, true, false); });
         if (t < best) { best = t; best_chunk = c; }
+        if (c != achunk && t < best_nt) { best_nt = t; best_named = c; }
     }
     h->rho_chunk = best_chunk;
     // Fourier-force split, timed in the form the handle's MD steps run it
@@ -2311,8 +2314,9 @@ rbe_status rbe_autotune(rbe_handle h, int32_t n, const float* pos_q, rbe_tuning*
             h->fusion_mode = fused ? 1 : 0;
             std::vector<int> chunks{rho_best_chunk};
             if (fused) {
-                if (rho_best_chunk / 2 >= 32) chunks.insert(chunks.begin(), rho_best_chunk / 2);
-                if (rho_best_chunk * 2 <= 4096) chunks.push_back(rho_best_chunk * 2);
+                chunks = {achunk};
+                for (int c : {best_named / 2, best_named, best_named * 2})
+                    if (c >= 32 && c <= 4096 && c != achunk) chunks.push_back(c);
             }
             float bt = 1e30f;
             out_chunk = rho_best_chunk;
