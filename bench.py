@@ -4,7 +4,7 @@
 One benchmark step = one MD step of the whole hot path on the large 1:1
 electrolyte (N = 2^20 ions, 2^19 of each sign, number density 0.064,
 alpha = 0.3, r_c = 5, P = 500, WCA LJ, Langevin T = 1, gamma = 1, dt = 1e-3):
-k-sampling, structure factors with FP64 rho(k), Fourier forces, neighbour
+k-sampling, structure factors with fixed-point rho(k), Fourier forces, neighbour
 list (rebuilt on the device when a particle has moved more than skin/2), real
 space + LJ and the Langevin update, mixed precision, replayed from a CUDA graph.
 
@@ -871,7 +871,7 @@ def run_ours(args):
             "config": {"workload": wl.name, "N": wl.n, "P": wl.params.P,
                        "alpha": wl.params.alpha, "r_c": wl.params.r_c,
                        "box": round(wl.params.box, 4), "density": 0.064,
-                       "path": "mixed (FP32 phases/forces, FP64 rho(k) and energy sums), "
+                       "path": "mixed (FP32 phases/forces, 64-bit fixed-point rho(k), FP64 energy sums), "
                                "neighbour-list MD steps, Langevin", "graph": True,
                        "l2": "flushed between timed steps (256 MiB write, untimed)",
                        "timed_region": f"{hl['reps']} x {K} steps, each block bracketed by "
@@ -899,10 +899,11 @@ def run_ours(args):
             "list_stats": stats,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": bytes_io,
                     "d2h_bytes_per_step": bytes_io, "steps": K,
-                    "api": "rbe_step_host on pinned host pos/vel (float32 [N, 4] each): every "
-                           "step's kernels read and write the page-locked arrays in place over "
-                           "the host link; the call returns when the closing kernel's "
-                           "completion word reaches mapped host memory"},
+                    "api": "rbe_step_host on pinned host pos/vel (float32 [N, 4] each): the "
+                           "step's first kernel reads the positions over the host link, the "
+                           "velocities are copied meanwhile, the closing kernel writes both "
+                           "in place; the call returns when its completion word reaches "
+                           "mapped host memory"},
             "fp64_path": same["fp64"],
             "speedup_vs_fp64": value / v64,
             "speedup_same_algorithm": {
