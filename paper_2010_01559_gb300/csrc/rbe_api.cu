@@ -1137,7 +1137,7 @@ void launch_rho(const rbe_ctx* h, cudaStream_t st, bool mixed, bool energies, bo
                          h->d_kcnt, h->d_kab, pdl);
     } else {
         launch_rho_f64(st, one, make_work(h, h->d_chunks, h->cur_chunk, 1), h->nchunks,
-                       h->cur_chunk, h->pmax, h->m_max(), h->d_ksamp, h->d_fx64, h->d_rho_fx);
+                       h->cur_chunk, h->cur_n, h->pmax, h->m_max(), h->d_ksamp, h->d_fx64, h->d_rho_fx);
     }
 }
 
@@ -1150,7 +1150,7 @@ void launch_force(const rbe_ctx* h, cudaStream_t st, bool mixed, const MdOut& md
                                    h->force_sums, h->d_fx, h->d_ksamp, h->d_kab, h->d_fs, md, pdl);
     } else {
         const Work w = make_work(h, h->d_pblk, kBlockP, 0);
-        launch_fourier_force_f64(st, one, w, h->npblk, h->m_max(), phi, h->d_fx64, h->d_ksamp,
+        launch_fourier_force_f64(st, one, w, h->npblk, h->cur_n, h->pmax, h->m_max(), phi, h->d_fx64, h->d_ksamp,
                                  h->d_kcoef, h->d_rho_fx, h->d_fs64, pdl);
     }
 }

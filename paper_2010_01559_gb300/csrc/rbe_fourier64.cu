@@ -36,7 +36,7 @@ constexpr int kTabThreads = 128;
 constexpr int kTabLanes = kTabThreads / kTabP;     // lanes per particle of the force
 constexpr int kTabK = 128;          // wave vectors staged per pass of the force
 
-// Direct form: tables that do not fit in shared memory (very large alpha L^2).
+// Direct form: tables that do not fit in shared memory or do not pay (large alpha L^2).
 constexpr int kDirectStage = 256;
 
 size_t tab_smem(int mcap) { return sizeof(double2) * kTabP * 3 * (size_t)(mcap + 1); }
@@ -166,7 +166,7 @@ k_rho_f64_tab(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
     }
 }
 
-// Direct form, one sincos per pair: only where the tables do not fit.
+// Direct form, one sincos per pair: where the tables do not fit or do not pay.
 template <bool ONE>
 __global__ void __launch_bounds__(kLTile)
 k_rho_f64(const __grid_constant__ Work w, const int4* __restrict__ ksamp,
@@ -269,7 +269,7 @@ k_force_f64_tab(const __grid_constant__ Work w, const double4* __restrict__ rec6
     }
 }
 
-// Direct form, one thread per particle: only where the tables do not fit.
+// Direct form, one thread per particle: where the tables do not fit or do not pay.
 template <bool ONE>
 __global__ void __launch_bounds__(kBlockP)
 k_force_f64(const __grid_constant__ Work w, const double4* __restrict__ rec64,
@@ -317,10 +317,28 @@ k_force_f64(const __grid_constant__ Work w, const double4* __restrict__ rec64,
 }
 
 // ------------------------------------------------------------- launchers
-// Tables whenever those of kTabP particles fit in a block's shared memory
-// (half width M of the sampler up to kTabMaxM): even a batch far smaller than
-// the table costs no more than its sines and cosines would.
+// Tables where they fit in a block's shared memory (half width M of the sampler up to
+// kTabMaxM) and cost less than a sine and a cosine per pair.  A table's cost grows with
+// M (its length and, by the shared memory it takes, the blocks that share an SM), the
+// direct form's with P, in whole warps for the structure factors.  Fitted and measured
+// (us, table / direct; events around the kernel):
+//                             structure factors    force
+//   N = 1000, M = 168, P = 5      13 / 38           12 / 13
+//   20000, 79, 10                 38 / 52           43 / 31
+//   20000, 250, 40               123 / 91          109 / 106
+//   140000, 151, 20              406 / 272         448 / 206
+//   2^20, 295, 50               5453 / 3749       9838 / 3365
+//   2^20, 295, 500             12944 / 29389     25147 / 33453
 constexpr int kTabMaxM = 560;               // 8 * 3 * 561 * 16 B = 210 KB
+
+static bool rho_tables_pay(double n, int P, int M) {
+    return M <= kTabMaxM && 11.0 + n * (1.9e-5 * M + 1.7e-5 * P) <=
+                                30.0 + 1.73e-3 * n * ((P + 31) / 32);
+}
+
+static bool force_tables_pay(double n, int P, int M) {
+    return M <= kTabMaxM && 8.0 + n * (1.8e-5 * M + 3.6e-5 * P) <= 6.0 + P * (1.1 + 7e-5 * n);
+}
 
 template <bool ONE, int KR>
 static void rho_f64_kr(cudaStream_t st, const Work& w, dim3 grid, size_t smem, const int4* ksamp,
@@ -330,11 +348,11 @@ static void rho_f64_kr(cudaStream_t st, const Work& w, dim3 grid, size_t smem, c
     k_rho_f64_tab<ONE, KR><<<grid, kTabThreads, smem, st>>>(w, ksamp, fx64, rho_fx);
 }
 
-void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int chunk, int pmax,
-                    int mcap, const int4* ksamp, const double4* fx64,
+void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int chunk, int n,
+                    int pmax, int mcap, const int4* ksamp, const double4* fx64,
                     unsigned long long* rho_fx) {
     if (nchunks <= 0 || pmax <= 0) return;
-    if (mcap > kTabMaxM) {
+    if (!rho_tables_pay(n, pmax, mcap)) {
         dim3 grid(nchunks, (pmax + kLTile - 1) / kLTile);
         if (one) k_rho_f64<true><<<grid, kLTile, 0, st>>>(w, ksamp, fx64, rho_fx);
         else k_rho_f64<false><<<grid, kLTile, 0, st>>>(w, ksamp, fx64, rho_fx);
@@ -368,12 +386,12 @@ static void force_f64_tab(cudaStream_t st, const Work& w, int nblk, size_t smem,
     cudaLaunchKernelEx(&c.cfg, k_force_f64_tab<ONE, PHI>, w, fx64, ksamp, kcoef, rho_fx, fs64);
 }
 
-void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int mcap,
-                              bool phi, const double4* fx64, const int4* ksamp,
+void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int n,
+                              int pmax, int mcap, bool phi, const double4* fx64, const int4* ksamp,
                               const double* kcoef, const unsigned long long* rho_fx,
                               double4* fs64, bool pdl) {
     if (nblk <= 0) return;
-    if (mcap > kTabMaxM) {
+    if (!force_tables_pay(n, pmax, mcap)) {
         if (one)
             k_force_f64<true><<<nblk, kBlockP, 0, st>>>(w, fx64, ksamp, kcoef, rho_fx, fs64);
         else

@@ -640,11 +640,11 @@ struct RhoGrid {
 void launch_rho_mixed(cudaStream_t st, bool one, const Work& w, const RhoGrid& g,
                       const int4* ksamp, const double* kcoef, const uint4* fx,
                       unsigned long long* rho_fx, int* kcnt, float2* kab, bool pdl = false);
-// FP64 path (rbe_fourier64.cu): chunk = particles per chunk, pmax and mcap the
+// FP64 path (rbe_fourier64.cu): chunk = particles per chunk, n the particles, pmax and mcap the
 // largest P and sampler half width M over the systems; phi: also dE/dq; pdl: the
 // force follows launch_rho_f64 on the same stream, programmatically.
-void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int chunk, int pmax,
-                    int mcap, const int4* ksamp, const double4* fx64,
+void launch_rho_f64(cudaStream_t st, bool one, const Work& w, int nchunks, int chunk, int n,
+                    int pmax, int mcap, const int4* ksamp, const double4* fx64,
                     unsigned long long* rho_fx);
 // The last stage of a neighbour-list MD step, run by the Fourier-force
 // kernel: total force = Fourier + freal, then the thermostat.
@@ -671,8 +671,8 @@ struct MdOut {
 void launch_fourier_force_mixed(cudaStream_t st, bool one, const Work& w, int nblk, int split,
                                 int sums, const uint4* fx, const int4* ksamp, const float2* kab,
                                 float4* fs, const MdOut& md, bool pdl);
-void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int mcap,
-                              bool phi, const double4* fx64, const int4* ksamp,
+void launch_fourier_force_f64(cudaStream_t st, bool one, const Work& w, int nblk, int n,
+                              int pmax, int mcap, bool phi, const double4* fx64, const int4* ksamp,
                               const double* kcoef, const unsigned long long* rho_fx,
                               double4* fs64, bool pdl = false);
 
