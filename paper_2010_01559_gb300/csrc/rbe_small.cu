@@ -47,6 +47,12 @@
 // Measured (us per step, 64 steps in a call, replayed kernels before -> now):
 // N = 300, P = 10 15.4 -> 4.1; N = 1000, P = 100 16.3 -> 6.5 and P = 500 18.3 -> 14.0;
 // N = 2000, P = 100 16.3 -> 9.5.
+// A call costs about 10 us beside its steps (the cluster's launch, the list taken over,
+// a first pass through the code), the price of a path that does not depend on how many
+// steps a call has (calls of any length give the same bits).  One step per call, back to
+// back, replayed kernels before -> now: N = 300, P = 10 14.4 -> 13.6; 1000, 100 16.8 -> 16.9;
+// 2000, 100 20.6 -> 21.2; 3000, 10 18.6 -> 20.8 (22.7 with the list's entries taken over one
+// by one); 1000, 500 20.6 -> 25.1.
 #include <algorithm>
 
 #include "rbe_cluster.cuh"
@@ -262,13 +268,39 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_md(const __grid_cons
     if (tid < 2 * kSmallMaxCs) (&s_msg[0][0])[tid] = make_uint4(0, 0, 0, 0);
     int cnt = 0;                                    // list entries of particle p
     if (pairs && !stale) {
-        // the handle's list, in sorted indices of its last build
+        // the handle's list, in sorted indices of its last build: kTake entries per lane
+        // in flight at a time, the first ones alongside the count (slots within the
+        // capacity always hold valid indices)
+        constexpr int kTake = 8;
         const int i = a.iperm[pn];
-        cnt = RBE_IN_BOUNDS(i, a.stride, a.err) ? min(a.ncnt[i], a.cap) : 0;
-        for (int k = l; k < cnt; k += R) {
-            const int j = a.nbr[(size_t)k * a.stride + i];
-            const int c = RBE_IN_BOUNDS(j, a.stride, a.err) ? a.perm[j] : pn;
-            list[p * a.cap + k] = (uint16_t)(RBE_IN_BOUNDS(c, n, a.err) ? c : pn);
+        if (RBE_IN_BOUNDS(i, a.stride, a.err)) {
+            const int* nb = a.nbr + i;
+            int j[kTake], c[kTake];
+            const int have = a.ncnt[i];
+#pragma unroll
+            for (int u = 0; u < kTake; ++u) {
+                const int k = l + u * R;
+                j[u] = k < a.cap ? nb[(size_t)k * a.stride] : 0;
+            }
+            cnt = min(have, a.cap);
+            for (int k0 = l; k0 < cnt; k0 += kTake * R) {
+                if (k0 > l) {
+#pragma unroll
+                    for (int u = 0; u < kTake; ++u) {
+                        const int k = k0 + u * R;
+                        j[u] = k < cnt ? nb[(size_t)k * a.stride] : 0;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kTake; ++u)
+                    c[u] = RBE_IN_BOUNDS(j[u], a.stride, a.err) ? a.perm[j[u]] : pn;
+#pragma unroll
+                for (int u = 0; u < kTake; ++u) {
+                    const int k = k0 + u * R;
+                    if (k < cnt)
+                        list[p * a.cap + k] = (uint16_t)(RBE_IN_BOUNDS(c[u], n, a.err) ? c[u] : pn);
+                }
+            }
         }
     }
     NhState nh{};
