@@ -278,7 +278,7 @@ rbe_status rbe_set_graph(rbe_handle h, int32_t use_graph);
  * vel float4[n] in/out, steps step0 .. step0 + nsteps - 1; when both arrays
  * are page-locked (cudaHostAlloc, cudaHostRegister) a single list step's
  * first kernel reads the positions over the host link and keeps them on the
- * device, the velocities are fetched meanwhile and the closing kernel writes
+ * device, the velocities are read or copied meanwhile and the closing kernel writes
  * both in place (of several steps the last one's; without a list every kernel
  * works in place), and
  * on a neighbour-list handle the call returns as soon as the step's closing

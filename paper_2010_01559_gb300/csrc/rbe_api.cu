@@ -1596,10 +1596,16 @@ struct HostIO {
 };
 
 // A list step whose pos and vel are page-locked host arrays: it reads them there
-// (both; the positions by its prep kernel, the velocities by a copy while the
-// structure factors run) or finds them in the staging buffers (out), and writes
-// them there.
+// (both; the positions by its prep kernel, the velocities meanwhile) or finds them in
+// the staging buffers (out), and writes them there.
 enum class ZeroCopy { none, both, out };
+
+// Particles from which such a step's velocities are copied to the device while the
+// structure factors run; below, the closing kernel reads them over the host link before
+// those are done, which hides the same reads without a copy in the step (us per step,
+// read / copied: N = 4000 23 / 31, 16000 31 / 37, 65536 56 / 57, 131072 99 / 100 with a
+// graph and 108 / 98 without, 262144 205 / 200).
+constexpr int kVelCopyMinN = 1 << 17;
 
 // Whether the MD steps of a single list system of n particles run as one cluster
 // (rbe_small.cu): P wave vectors, m neighbours within r_c + skin on average.  Its sixteen
@@ -1671,12 +1677,16 @@ rbe_status step_impl(rbe_ctx* h, int n, int prec, void* pos, void* vel, int nste
             a.pos_in = h->d_stage_pos;
             a.vel_in = h->d_stage_vel;
             if (zc == ZeroCopy::both) {
-                if (!h->stream4)                // only handles stepped this way have one
-                    RBE_CUDA(h, cudaStreamCreateWithFlags(&h->stream4, cudaStreamNonBlocking));
-                if (!h->ev_vel)
-                    RBE_CUDA(h, cudaEventCreateWithFlags(&h->ev_vel, cudaEventDisableTiming));
                 a.pos_copy = h->d_stage_pos;
-                a.vel_fetch = (const float4*)vel;
+                if (n >= kVelCopyMinN) {
+                    if (!h->stream4)            // only handles stepped this way have one
+                        RBE_CUDA(h, cudaStreamCreateWithFlags(&h->stream4, cudaStreamNonBlocking));
+                    if (!h->ev_vel)
+                        RBE_CUDA(h, cudaEventCreateWithFlags(&h->ev_vel, cudaEventDisableTiming));
+                    a.vel_fetch = (const float4*)vel;
+                } else {
+                    a.vel_in = (float4*)vel;
+                }
             } else {
                 a.pos = h->d_stage_pos;
             }
@@ -2083,9 +2093,10 @@ rbe_status rbe_step_host(rbe_handle h, int32_t n, float* pos_q, float* vel, int3
     void* dvel = n > 0 ? mapped_host(vel) : nullptr;
     if (n > 0 && dpos && dvel) {
         // page-locked arrays: a list step's prep kernel reads the positions over the
-        // host link and leaves a copy on the device, the velocities are fetched
-        // while the structure factors run, and the closing kernel writes both in
-        // place (it read them there too: N = 262144 222 us per step, 201 now).
+        // host link and leaves a copy on the device, the velocities are read or copied
+        // meanwhile (kVelCopyMinN), and the closing kernel writes both in place (it
+        // read the positions there too: N = 262144 220 us per step, 200 now; 16000 42
+        // and 30).
         // Without a list the kernels read and write in place.  The step index
         // advances in the pinned word.  A list step's closing kernel also delivers the
         // error word and then a completion word there, which this thread
