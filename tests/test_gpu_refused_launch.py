@@ -1,4 +1,4 @@
-"""A launch that the driver refuses is reported by the call that made it, whatever
+"""A launch that CUDA refuses is reported by the call that made it, whatever
 other runtime calls succeed after it: the direct FP64 structure factors of a batch of
 2^23 wave vectors need 65536 rows of blocks, one more than a grid has."""
 import pytest
